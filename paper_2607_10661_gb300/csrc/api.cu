@@ -90,6 +90,23 @@ int64_t cache_rows_per_layer(const ptd_kv_cache* c, int batch) {
   return c->page_size > 0 ? (int64_t)c->num_pages * c->page_size : (int64_t)batch * c->seq_capacity;
 }
 
+// Tensor map of a cache's K or V as [rows of all layers][KV heads][D], boxes of `cols` columns of
+// one head and `box_rows` rows.
+bool encode_cache(CUtensorMap* map, const ptd_kv_cache* c, int batch, void* base, uint32_t cols, uint32_t box_rows,
+                  bool swizzle) {
+  PFN_cuTensorMapEncodeTiled_v12000 enc = encode_fn();
+  if (!enc) return false;
+  const size_t es = dtype_size(c->dtype);
+  const cuuint64_t gdim[3] = {(cuuint64_t)c->head_dim, (cuuint64_t)c->num_kv_heads,
+                              (cuuint64_t)(cache_rows_per_layer(c, batch) * c->num_layers)};
+  const cuuint64_t gstride[2] = {(cuuint64_t)c->head_dim * es, (cuuint64_t)c->num_kv_heads * c->head_dim * es};
+  const cuuint32_t box[3] = {cols, 1, box_rows}, estride[3] = {1, 1, 1};
+  return enc(map, c->dtype == PTD_BF16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, base,
+             gdim, gstride, box, estride, CU_TENSOR_MAP_INTERLEAVE_NONE,
+             swizzle ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 bool use_tensor_cores(const ptd_kv_cache* c) { return c->dtype == PTD_BF16 && c->head_dim == 128; }
 
 // Number of 256-row M-tile pairs per (tree, KV head) and work units of the tensor-core path.
@@ -264,8 +281,13 @@ static ptd_status tree_attention(const ptd_tree* tree, const ptd_kv_cache* cache
 
   if (cache->dtype == PTD_F32) {
     if (D != 32 && D != 64 && D != 128) return PTD_ERR_UNSUPPORTED;
-    p.pairs = 1;
-    st = cuda_status(ptd::launch_tree_attn_simt(p, s));
+    CUtensorMap map_k, map_v;
+    const uint32_t rows = (uint32_t)ptd::simt_box_rows(cache->page_size);
+    if (!encode_cache(&map_k, cache, tree->batch, cache->k, 32, rows, true) ||
+        !encode_cache(&map_v, cache, tree->batch, cache->v, (uint32_t)D, rows, false))
+      return PTD_ERR_CUDA;
+    st = cuda_status(
+        ptd::launch_tree_attn_simt(map_k, map_v, p, tree->max_ctx, num_sms_of_current_device(), s));
     if (st == PTD_OK) g_last_launches = 1;
     return st;
   }
@@ -296,27 +318,18 @@ static ptd_status tree_attention(const ptd_tree* tree, const ptd_kv_cache* cache
     grid = dim3((unsigned)units, 1, 1);
   }
 
-  PFN_cuTensorMapEncodeTiled_v12000 enc = encode_fn();
-  if (!enc) return PTD_ERR_CUDA;
-  const int64_t rows_per_layer = cache_rows_per_layer(cache, tree->batch);
-  const cuuint64_t gdim[3] = {(cuuint64_t)D, (cuuint64_t)cache->num_kv_heads,
-                              (cuuint64_t)(rows_per_layer * cache->num_layers)};
-  const cuuint64_t gstride[2] = {(cuuint64_t)D * 2, (cuuint64_t)cache->num_kv_heads * D * 2};
-  const cuuint32_t box[3] = {64, 1, (cuuint32_t)(cache->page_size > 0 ? cache->page_size : 128)};
-  const cuuint32_t estride[3] = {1, 1, 1};
+  const uint32_t box_rows = (uint32_t)(cache->page_size > 0 ? cache->page_size : 128);
   CUtensorMap map_k, map_v;
-  if (enc(&map_k, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, cache->k, gdim, gstride, box, estride,
-          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-    return PTD_ERR_CUDA;
-  if (enc(&map_v, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, cache->v, gdim, gstride, box, estride,
-          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+  if (!encode_cache(&map_k, cache, tree->batch, cache->k, 64, box_rows, true) ||
+      !encode_cache(&map_v, cache, tree->batch, cache->v, 64, box_rows, true))
     return PTD_ERR_CUDA;
 
   // Q tiles by TMA: one M tile is 128 / G nodes x G heads, a 3-D box over [rows][Hq][D]
   CUtensorMap map_q;
   std::memset(&map_q, 0, sizeof(map_q));
+  PFN_cuTensorMapEncodeTiled_v12000 enc = encode_fn();
+  if (!enc) return PTD_ERR_CUDA;
+  const cuuint32_t estride[3] = {1, 1, 1};
   const int G = p.group;
   p.q_tma = 0;
   if (G >= 1 && G <= 128 && 128 % G == 0 && aligned16(q)) {

@@ -45,7 +45,11 @@ size_t tc_smem_bytes();
 // before its first global access.
 cudaError_t launch_tree_attn_tc(const CUtensorMap& map_k, const CUtensorMap& map_v, const CUtensorMap& map_q,
                                 const AttnParams& p, dim3 grid, cudaStream_t stream);
-cudaError_t launch_tree_attn_simt(const AttnParams& p, cudaStream_t stream);
+// fp32 attention.  map_k: boxes of 32 columns (128-byte swizzle), map_v: of D columns, both of one
+// KV head and simt_box_rows(page_size) rows.
+cudaError_t launch_tree_attn_simt(const CUtensorMap& map_k, const CUtensorMap& map_v, const AttnParams& p, int max_ctx,
+                                  int sms, cudaStream_t stream);
+inline int simt_box_rows(int page_size) { return page_size > 0 ? 16 : 64; }
 // The merge of the units the persistent cut split, after the attention kernel (programmatic
 // dependent launch): one CTA per unit, the pieces' partials combined in CTA order.
 cudaError_t launch_tree_attn_merge(const AttnParams& p, int units, int sms, cudaStream_t stream);

@@ -2,217 +2,550 @@
 // the result keeps full fp32 accuracy).
 //
 // Same operation as the tensor-core kernel (Sec. 3.1 ancestor-only visibility over the
-// committed prefix plus the tree, Sec. 3.2): one CTA of 4 warps per (layer, node, query
-// head).  The keys are cut into chunks of 32 and warp w takes chunks w, w + 4, ...: in a
-// chunk lane j scores key j (its K row read with independent 16-byte loads), the warp keeps
-// an online softmax (running max m, sum l), and every lane accumulates D/32 output columns
-// from the chunk's 32 V rows, all of whose loads are issued before the first multiply.  The
-// four warps' (m, l, O) are combined in shared memory at the end.
+// committed prefix plus the tree, Sec. 3.2), and the same dense view of it: the T nodes times
+// the G query heads of a KV head form M = T * G rows that share every K/V row.  A unit is one
+// (layer, tree, KV head, block of BM rows); a cluster of `csize` CTAs computes it, CTA r taking
+// the r-th share of the keys, and the CTAs' partial softmax states (m, l, O) are combined
+// through distributed shared memory, so the split needs no scratch and no second launch.
+//
+// In a CTA (128 threads as 8 row groups x 16 lanes) keys come in tiles of 64 whose K and V one
+// thread brings in by TMA (K of the next tile during this tile's P V, V during its Q K^T; row
+// copies issued by a warp's lanes held the other warps up at the next barrier).  Thread (row
+// group, lane g) scores its RM = BM / 8 rows against keys g + 16 j (packed fp32 pairs over two
+// columns, fma.rn.f32x2, so Q and K are used as they lie; K in 32-column boxes with the 128-byte
+// swizzle, so that eight consecutive keys' 16-byte reads hit distinct banks), the row maxima
+// reduce over the 16 lanes, P goes transposed to shared memory, and the thread accumulates RM
+// rows x D / 16 columns of O (pairs over two rows).
+//
+// What bounds it: shared-memory reads and the fp32 FMA pipe (an 8 x 4 tile of S reads 12 floats
+// per 32 FMAs, an 8 x 8 tile of O 16 per 64; the pipe gives ~110 FMA per cycle and SM) for many
+// rows, the latency of a tile's chain and the K/V stream for few.  Measured (GB300, one layer,
+// against one CTA per (node, head) over all keys, which read every K/V row T * G times): 32 query
+// / 8 KV heads, D 128, 2048 + 63 keys, 63 nodes 628 -> 69.5 us (31 TFLOP/s); the same with one
+// node 86 -> 26 us; 8 heads, D 64, 256 + 15 keys, 15 nodes 14.5 -> 6.6 us.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include <cmath>
 #include <cstdint>
+#include <type_traits>
 
 #include "attention.cuh"
 #include "ptd_device.cuh"
 
+namespace cg = cooperative_groups;
+
 namespace ptd {
 namespace simt {
 
-constexpr int kWarps = 4;
+constexpr int kThreads = 128;
+constexpr int kWarps = kThreads / 32;
+constexpr int kLanes = 16;                   // lanes that share a row group
+constexpr int kGroups = kThreads / kLanes;   // row groups
+constexpr int kBN = 64;                      // keys per tile
+constexpr int kKeys = kBN / kLanes;          // keys per lane and tile
+constexpr int kMaxCluster = 8;
+constexpr int kMaxNodes = 128;
 
+constexpr int kBoxRows = 16;                 // rows of a box of a paged cache (a tile starts on a multiple of 16)
+
+// Shared memory (floats) of a block of kGroups * RM rows (D = 128, 64 rows: two CTAs per SM).
+template <int D, int RM>
+struct Layout {
+  static constexpr int BM = kGroups * RM;
+  static constexpr int kK = 0;                // K [D / 32][kBN][32], 128-byte swizzle
+  static constexpr int kV = kK + kBN * D;     // V [kBN][D]
+  static constexpr int kP = kV + kBN * D;     // P^T [kBN][BM], 16-byte chunk c of row n at c ^ p_swizzle(n)
+  static constexpr int kQ = kP + kBN * BM;    // Q [BM][D]
+  static constexpr int kBar = kQ + BM * D;    // Q, K and V barriers, abort flag
+  static constexpr int kEnd = kBar + 8;
+  static constexpr int kPar = kP;             // set-up: the tree's parents (before P is written)
+  static constexpr int kO = kV;               // end: the partial rows [BM][D] (over V: BM <= kBN)
+  static constexpr int kMl = kP;              // end: [BM][2] running maximum and row sum (over P)
+  static constexpr size_t kBytes = (size_t)kEnd * sizeof(float);
+  static_assert(BM <= kBN && kBN * BM >= kMaxNodes && 2 * (kBytes + 1024) <= 233472, "shared memory");
+  // eight consecutive keys' stores of the same rows hit distinct banks
+  static __device__ __forceinline__ int p_swizzle(int n) { return BM >= 32 ? n & 7 : (n >> 1) & 3; }
+};
+
+// Maximum / sum over the 16 lanes that share a row group.
+__device__ __forceinline__ float group_max(float v) {
+#pragma unroll
+  for (int o = kLanes / 2; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+  return v;
+}
+__device__ __forceinline__ float group_sum(float v) {
+#pragma unroll
+  for (int o = kLanes / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
 __device__ __forceinline__ float warp_max(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
   return v;
 }
-
 __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
 
-template <int D>
-__global__ void __launch_bounds__(kWarps * 32) tree_attn_simt_kernel(const AttnParams p) {
-  constexpr int DPL = D / 32;   // output columns per lane
-  __shared__ int par_s[128];
-  __shared__ __align__(16) float q_s[D];
-  __shared__ uint32_t anc_s[4];
-  __shared__ float m_s[kWarps], l_s[kWarps];
-  __shared__ float o_s[kWarps][D];
-  __shared__ int meta_s[3];     // tree b, node within the tree, invalid
-
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int h = blockIdx.x, n = blockIdx.y, lq = blockIdx.z;
-  const int layer = p.layer_begin + lq;
-  const int hkv = h / p.group;
-  float* O = static_cast<float*>(p.out);
-  const size_t qrow = (((size_t)lq * p.n_total + n) * p.hq + h) * D;
-
-  if (threadIdx.x == 0) {
-    int lo = 0, hi = p.batch;   // tree b with node_offsets[b] <= n < node_offsets[b + 1]
-    while (hi - lo > 1) {
-      const int mid = (lo + hi) >> 1;
-      if (p.node_offsets[mid] <= n) lo = mid; else hi = mid;
+// N consecutive floats (1, or 2 or a multiple of 4 with the alignment of a 16-byte load).
+template <int N>
+__device__ __forceinline__ void load_n(const float* p, float (&x)[N]) {
+  if constexpr (N == 1) {
+    x[0] = *p;
+  } else if constexpr (N == 2) {
+    const float2 a = *reinterpret_cast<const float2*>(p);
+    x[0] = a.x, x[1] = a.y;
+  } else {
+#pragma unroll
+    for (int i = 0; i < N; i += 4) {
+      const float4 a = *reinterpret_cast<const float4*>(p + i);
+      x[i] = a.x, x[i + 1] = a.y, x[i + 2] = a.z, x[i + 3] = a.w;
     }
-    meta_s[0] = lo;
   }
-  __syncthreads();
-  const int b = meta_s[0];
+}
+template <int N>
+__device__ __forceinline__ void store_n(float* p, const float (&x)[N]) {
+  if constexpr (N == 1) {
+    *p = x[0];
+  } else if constexpr (N == 2) {
+    *reinterpret_cast<float2*>(p) = make_float2(x[0], x[1]);
+  } else {
+#pragma unroll
+    for (int i = 0; i < N; i += 4) *reinterpret_cast<float4*>(p + i) = make_float4(x[i], x[i + 1], x[i + 2], x[i + 3]);
+  }
+}
+// A lane's DC = D / 16 columns: two runs of four (D = 128), or one run.
+template <int D>
+__device__ __forceinline__ void load_cols(const float* row, int g, float (&x)[D / kLanes]) {
+  if constexpr (D == 128) {
+    const float4 a = *reinterpret_cast<const float4*>(row + 4 * g);
+    const float4 c = *reinterpret_cast<const float4*>(row + 64 + 4 * g);
+    x[0] = a.x, x[1] = a.y, x[2] = a.z, x[3] = a.w, x[4] = c.x, x[5] = c.y, x[6] = c.z, x[7] = c.w;
+  } else {
+    load_n<D / kLanes>(row + D / kLanes * g, x);
+  }
+}
+
+// One tile of K or V, rows [k0, min(k0 + kBN, k_hi)), by one thread; bar receives the bytes.  A
+// contiguous cache's tile is whole rows of the tensor whatever the share's end (rows past it are
+// some other slot's, or zeros past the tensor); a paged one's comes in boxes of 16 rows, those at
+// or past k_hi left out.
+template <int D, bool kIsK>
+__device__ __forceinline__ void load_tile(const AttnParams& p, const CUtensorMap* map, float* dst_f, uint32_t bar, int b,
+                                          int layer, int hkv, int k0, int k_hi) {
+  constexpr int kCols = kIsK ? 32 : D;   // columns of a box
+  const uint32_t dst = smem_u32(dst_f);
+  if (p.page_size == 0) {
+    const int row0 = (layer * p.batch + b) * p.seq_capacity + k0;
+    mbar_arrive_expect_tx(bar, kBN * D * 4);
+#pragma unroll
+    for (int c = 0; c < D / kCols; ++c) tma_load_3d(dst + (uint32_t)(c * kBN * kCols) * 4u, map, bar, c * kCols, hkv, row0);
+  } else {
+    const int shift = __ffs(p.page_size) - 1;   // pages are powers of two
+    const int* table = p.block_table + (size_t)b * p.max_pages;
+    const int n = min(kBN, (k_hi - k0 + kBoxRows - 1) & ~(kBoxRows - 1));
+    mbar_arrive_expect_tx(bar, (uint32_t)(n * D * 4));
+#pragma unroll 1
+    for (int r = 0; r < n; r += kBoxRows) {
+      const int row0 = ((layer * p.num_pages + table[(k0 + r) >> shift]) << shift) + ((k0 + r) & (p.page_size - 1));
+#pragma unroll
+      for (int c = 0; c < D / kCols; ++c)
+        tma_load_3d(dst + (uint32_t)((c * kBN + r) * kCols) * 4u, map, bar, c * kCols, hkv, row0);
+    }
+  }
+}
+
+template <int D, int RM>
+__global__ void __launch_bounds__(kThreads, 2)
+    tree_attn_simt_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
+                          const __grid_constant__ AttnParams p, int csize, int m_blocks, uint32_t inv_group) {
+  using L = Layout<D, RM>;
+  constexpr int BM = L::BM;
+  constexpr int DC = D / kLanes;            // output columns per thread
+  extern __shared__ __align__(1024) float sm[];
+  cg::cluster_group cluster = cg::this_cluster();
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int g = lane & (kLanes - 1);        // key / column lane
+  const int rg = tid / kLanes;              // row group
+  const int rank = blockIdx.x % csize;
+  int u = blockIdx.x / csize;
+  const int mb = u % m_blocks;
+  u /= m_blocks;
+  const int hkv = u % p.hkv;
+  u /= p.hkv;
+  const int b = u % p.batch;
+  const int lq = u / p.batch;
+  const int layer = p.layer_begin + lq;
+  const int G = p.group;
+  // row m's node: m / G by a multiplication (m < 2^16; inv_group = ceil(2^32 / G), 0 for G = 1)
+  auto node_of = [&](int m) { return inv_group != 0u ? (int)__umulhi((uint32_t)m, inv_group) : m; };
+  const uint32_t bar_q = smem_u32(sm + L::kBar), bar_k = bar_q + 8, bar_v = bar_q + 16;
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(sm + L::kBar + 6);
+
+  if (tid == 0) {
+    mbar_init(bar_q, 1);
+    mbar_init(bar_k, 1);
+    mbar_init(bar_v, 1);
+    *abort_flag = 0;
+    fence_mbar_init();
+    prefetch_tensormap(&map_k);
+    prefetch_tensormap(&map_v);
+    grid_launch_dependents();   // the next grid may be placed now; it waits for this one
+  }
+  grid_dependency_wait();   // the trees, Q, the cache and the output belong to the stream's previous work
+  // ---- the tree (every CTA of the cluster decides alike, so all of them leave here or none)
   const int node0 = p.node_offsets[b];
   const int T = p.node_offsets[b + 1] - node0;
   const int C = p.ctx_lens[b];
   const int N = C + T;
-  const int i = n - node0;
-  bool bad_shape = T < 1 || T > p.max_nodes || node0 < 0 || node0 + T > p.n_total || C < 0 || i < 0 || i >= T;
+  bool bad_shape = T < 1 || T > p.max_nodes || T > kMaxNodes || node0 < 0 || node0 + T > p.n_total || C < 0;
   if (!bad_shape) bad_shape = p.page_size > 0 ? N > p.max_pages * p.page_size : N > p.seq_capacity;
+  // nodes that no tree owns
+  if (tid == 0 && ((b == 0 && node0 != 0) || (b == p.batch - 1 && node0 + T != p.n_total)))
+    atomicMax(p.dev_status, (int)PTD_ERR_INVALID_TREE);
   if (bad_shape) {
-    if (threadIdx.x == 0) atomicMax(p.dev_status, (int)PTD_ERR_INVALID_TREE);
+    if (tid == 0) atomicMax(p.dev_status, (int)PTD_ERR_INVALID_TREE);
     return;
   }
-  bool bad = false;
-  if (threadIdx.x < T) {
-    const int pp = p.parents[node0 + threadIdx.x];
-    par_s[threadIdx.x] = pp;
-    bad = threadIdx.x == 0 ? (pp != -1) : (pp < 0 || pp >= (int)threadIdx.x);
-  }
-  const int invalid = __syncthreads_or(bad);
-  if (invalid) {
-    if (threadIdx.x == 0) atomicMax(p.dev_status, (int)PTD_ERR_INVALID_TREE);
-    for (int d = threadIdx.x; d < D; d += blockDim.x) O[qrow + d] = 0.f;
-    return;
-  }
-  if (threadIdx.x == 0) {
-    uint32_t m[4] = {0, 0, 0, 0};
-    for (int a = i; a >= 0; a = par_s[a]) m[a >> 5] |= 1u << (a & 31);
-    for (int w = 0; w < 4; ++w) anc_s[w] = m[w];
-  }
-  const float* Q = static_cast<const float*>(p.q);
-  for (int d = threadIdx.x; d < D; d += blockDim.x) q_s[d] = Q[qrow + d];
-  __syncthreads();
-  const uint32_t a0 = anc_s[0], a1 = anc_s[1], a2 = anc_s[2], a3 = anc_s[3];
-
-  const float* Kc = static_cast<const float*>(p.k);
-  const float* Vc = static_cast<const float*>(p.v);
-  const size_t slot_elems = (size_t)p.hkv * D;
-  auto slot_row = [&](int slot) -> size_t {
-    size_t r;
-    if (p.page_size > 0) {
-      const int pg = p.block_table[(size_t)b * p.max_pages + slot / p.page_size];
-      r = ((size_t)layer * p.num_pages + pg) * p.page_size + slot % p.page_size;
-    } else {
-      r = ((size_t)layer * p.batch + b) * p.seq_capacity + slot;
-    }
-    return r * slot_elems + (size_t)hkv * D;
+  const int M = T * G;
+  const int row0 = mb * BM;
+  if (row0 >= M) return;
+  const int rows = min(BM, M - row0);
+  const size_t out_row0 = ((size_t)lq * p.n_total + node0) * p.hq + (size_t)hkv * G;   // + node * hq + head
+  auto q_row = [&](int r) {   // row r of the block in q and out
+    const int m = row0 + r, node = node_of(m);
+    return out_row0 + (size_t)node * p.hq + (m - node * G);
   };
 
-  float m = -INFINITY, l = 0.f;
-  float acc[DPL];
-#pragma unroll
-  for (int c = 0; c < DPL; ++c) acc[c] = 0.f;
-  for (int k0 = warp * 32; k0 < N; k0 += kWarps * 32) {
-    const int key = k0 + lane;
-    bool vis = key < C;
-    if (!vis && key < N) {
-      const int a = key - C;
-      const uint32_t w = a < 32 ? a0 : a < 64 ? a1 : a < 96 ? a2 : a3;
-      vis = (w >> (a & 31)) & 1u;
-    }
-    float s = -INFINITY;
-    if (vis) {
-      const float4* kr = reinterpret_cast<const float4*>(Kc + slot_row(key));
-      const float4* qr = reinterpret_cast<const float4*>(q_s);
-      float4 kv[D / 4];
-#pragma unroll
-      for (int c = 0; c < D / 4; ++c) kv[c] = __ldg(kr + c);
-      float d0 = 0.f, d1 = 0.f;
-#pragma unroll
-      for (int c = 0; c < D / 4; c += 2) {
-        const float4 q0 = qr[c], q1 = qr[c + 1];
-        d0 = fmaf(q0.x, kv[c].x, d0);
-        d0 = fmaf(q0.y, kv[c].y, d0);
-        d0 = fmaf(q0.z, kv[c].z, d0);
-        d0 = fmaf(q0.w, kv[c].w, d0);
-        d1 = fmaf(q1.x, kv[c + 1].x, d1);
-        d1 = fmaf(q1.y, kv[c + 1].y, d1);
-        d1 = fmaf(q1.z, kv[c + 1].z, d1);
-        d1 = fmaf(q1.w, kv[c + 1].w, d1);
+  // this CTA's keys: the rank-th of csize shares, in steps of 16
+  const int per = ((N + csize - 1) / csize + 15) & ~15;
+  const int k_lo = min(N, rank * per), k_hi = min(N, k_lo + per);
+  const int n_tiles = (k_hi - k_lo + kBN - 1) / kBN;
+  // the tree is checked before any copy starts, so that leaving needs no drain
+  int* const par_s = reinterpret_cast<int*>(sm + L::kPar);
+  bool bad = false;
+  if (tid < T) {
+    const int pp = p.parents[node0 + tid];
+    par_s[tid] = pp;
+    bad = tid == 0 ? (pp != -1) : (pp < 0 || pp >= tid);
+  }
+  if (__syncthreads_or(bad)) {
+    if (tid == 0) atomicMax(p.dev_status, (int)PTD_ERR_INVALID_TREE);
+    if (rank == 0)
+      for (int e = tid; e < rows * (D / 4); e += kThreads) {
+        const int r = e / (D / 4);
+        reinterpret_cast<float4*>(static_cast<float*>(p.out) + q_row(r) * D)[e % (D / 4)] = make_float4(0.f, 0.f, 0.f, 0.f);
       }
-      s = (d0 + d1) * p.scale;
-    }
-    const float m_new = fmaxf(m, warp_max(s));
-    if (m_new == -INFINITY) continue;   // nothing visible yet (warp-uniform)
-    const float alpha = m == -INFINITY ? 0.f : expf(m - m_new);
-    const float pj = vis ? expf(s - m_new) : 0.f;
-    l = l * alpha + warp_sum(pj);
-#pragma unroll
-    for (int c = 0; c < DPL; ++c) acc[c] *= alpha;
-    // all 32 V rows of the chunk at once (rows past the sequence are not read)
-    const int nk = min(32, N - k0);
-    float v[32][DPL];
-#pragma unroll
-    for (int j = 0; j < 32; ++j) {
-      const float* vr = Vc + slot_row(j < nk ? k0 + j : k0);
-#pragma unroll
-      for (int c = 0; c < DPL; ++c) v[j][c] = j < nk ? __ldg(vr + c * 32 + lane) : 0.f;
-    }
-#pragma unroll
-    for (int j = 0; j < 32; ++j) {
-      const float pjj = __shfl_sync(0xffffffffu, pj, j);
-#pragma unroll
-      for (int c = 0; c < DPL; ++c) acc[c] = fmaf(pjj, v[j][c], acc[c]);
-    }
-    m = m_new;
+    return;
   }
-  // combine the four warps' partial softmax states
-  if (lane == 0) {
-    m_s[warp] = m;
-    l_s[warp] = l;
+  if (n_tiles > 0) {
+    if (tid == 0) load_tile<D, true>(p, &map_k, sm + L::kK, bar_k, b, layer, hkv, k_lo, k_hi);
+    if (tid == 32) load_tile<D, false>(p, &map_v, sm + L::kV, bar_v, b, layer, hkv, k_lo, k_hi);
+    if (warp == 2) {   // Q rows of the block (padding rows keep what is there: their results are not written)
+      if (lane == 0) mbar_arrive_expect_tx(bar_q, (uint32_t)(rows * D * 4));
+      __syncwarp();
+      for (int r = lane; r < rows; r += 32)
+        bulk_load(smem_u32(sm + L::kQ + r * D), static_cast<const float*>(p.q) + q_row(r) * D, D * 4, bar_q);
+    }
   }
+  // ancestor masks (walk up the strictly decreasing parents), for tiles past the context: lane i
+  // of a half warp holds its row group's row i
+  uint32_t am[4] = {0, 0, 0, 0};
+  if (k_hi > C && g < RM && rg * RM + g < rows)
+    for (int a = node_of(row0 + rg * RM + g); a >= 0; a = par_s[a]) {
+      const uint32_t bit = 1u << (a & 31);
 #pragma unroll
-  for (int c = 0; c < DPL; ++c) o_s[warp][c * 32 + lane] = acc[c];
+      for (int w = 0; w < 4; ++w) am[w] |= (a >> 5) == w ? bit : 0u;
+    }
+
+  float m_run[RM], l_run[RM];           // running maximum (log2 units), this thread's share of the row sum
+  unsigned long long o[DC][RM / 2];     // O, pairs of rows
+#pragma unroll
+  for (int i = 0; i < RM; ++i) m_run[i] = -INFINITY, l_run[i] = 0.f;
+#pragma unroll
+  for (int c = 0; c < DC; ++c)
+#pragma unroll
+    for (int i = 0; i < RM / 2; ++i) o[c][i] = 0ull;
+  const float sl2 = p.scale_log2;
+  // A wait that gave up (the status says so) leaves the walk going without further waits, so
+  // that every thread meets every barrier.
+  bool ok = true;
+
+  if (n_tiles > 0) ok = mbar_wait(bar_q, 0, abort_flag, p.dev_status);
+  for (int t = 0; t < n_tiles; ++t) {
+    const int k0 = k_lo + t * kBN;
+    const int nk = min(kBN, k_hi - k0);
+    __syncthreads();   // the previous tile's V is read, the parents are read
+    if (t > 0 && tid == 32 && ok) load_tile<D, false>(p, &map_v, sm + L::kV, bar_v, b, layer, hkv, k0, k_hi);
+    if (ok) ok = mbar_wait(bar_k, (uint32_t)(t & 1), abort_flag, p.dev_status);
+    // ---- S = Q K^T, pairs over columns
+    float pr[kKeys][RM];
+    {
+      unsigned long long s[kKeys][RM];
+#pragma unroll
+      for (int j = 0; j < kKeys; ++j)
+#pragma unroll
+        for (int i = 0; i < RM; ++i) s[j][i] = 0ull;
+      const float* kp = sm + L::kK + g * 32;
+      const int x = (smem_u32(kp) >> 7) & 7;   // the swizzle of keys g + 16 j: chunk c lies at c ^ x
+      const float* qp = sm + L::kQ + rg * RM * D;
+      auto dot = [&](auto keys) {
+        constexpr int NK = decltype(keys)::value;
+#pragma unroll 4
+        for (int d = 0; d < D; d += 4) {
+          ulonglong2 kf[NK];
+#pragma unroll
+          for (int j = 0; j < NK; ++j) kf[j] = *reinterpret_cast<const ulonglong2*>(kp + (d >> 5) * (kBN * 32) + j * kLanes * 32 + (((d >> 2) & 7) ^ x) * 4);
+#pragma unroll
+          for (int i = 0; i < RM; ++i) {
+            const ulonglong2 q = *reinterpret_cast<const ulonglong2*>(qp + i * D + d);
+#pragma unroll
+            for (int j = 0; j < NK; ++j) s[j][i] = f2_fma(q.y, kf[j].y, f2_fma(q.x, kf[j].x, s[j][i]));
+          }
+        }
+      };
+      if (nk > kBN / 2)
+        dot(std::integral_constant<int, kKeys>{});
+      else   // a share's last tile may hold few keys
+        dot(std::integral_constant<int, kKeys / 2>{});
+#pragma unroll
+      for (int j = 0; j < kKeys; ++j)
+#pragma unroll
+        for (int i = 0; i < RM; ++i) {
+          float a, c;
+          f2_unpack(s[j][i], a, c);
+          pr[j][i] = a + c;
+        }
+    }
+    // ---- mask, row maxima, P
+    if (k0 + nk > C || nk < kBN) {
+#pragma unroll
+      for (int i = 0; i < RM; ++i) {
+        uint32_t w[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) w[q] = __shfl_sync(0xffffffffu, am[q], (lane & kLanes) + i);
+#pragma unroll
+        for (int j = 0; j < kKeys; ++j) {
+          const int key = g + kLanes * j, a = k0 + key - C;
+          const uint32_t word = a < 32 ? w[0] : a < 64 ? w[1] : a < 96 ? w[2] : w[3];
+          if (key >= nk || (a >= 0 && !((word >> (a & 31)) & 1u))) pr[j][i] = -INFINITY;
+        }
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < RM; i += 2) {
+      float alpha[2];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        float mx = pr[0][i + h];
+#pragma unroll
+        for (int j = 1; j < kKeys; ++j) mx = fmaxf(mx, pr[j][i + h]);
+        mx = group_max(mx) * sl2;
+        const float m_new = fmaxf(m_run[i + h], mx);
+        const float m_use = m_new == -INFINITY ? 0.f : m_new;   // -inf only while nothing is visible
+        alpha[h] = exp2f(m_run[i + h] - m_use);                 // 0 from the first visible key's tile
+        m_run[i + h] = m_new;
+        float sum = 0.f;
+#pragma unroll
+        for (int j = 0; j < kKeys; ++j) {
+          pr[j][i + h] = exp2f(fmaf(pr[j][i + h], sl2, -m_use));
+          sum += pr[j][i + h];
+        }
+        l_run[i + h] = fmaf(l_run[i + h], alpha[h], sum);
+      }
+      const unsigned long long a2 = f2_pack(alpha[0], alpha[1]);
+#pragma unroll
+      for (int c = 0; c < DC; ++c) o[c][i / 2] = f2_mul(o[c][i / 2], a2);
+    }
+    // P^T (a row group is one half warp: it reads only what it wrote here)
+    constexpr int RC = RM < 4 ? RM : 4;   // rows per store
+#pragma unroll
+    for (int j = 0; j < kKeys; ++j) {
+      const int key = g + kLanes * j;
+#pragma unroll
+      for (int i = 0; i < RM; i += RC) {
+        const int r = rg * RM + i;
+        float x[RC];
+#pragma unroll
+        for (int e = 0; e < RC; ++e) x[e] = pr[j][i + e];
+        store_n<RC>(sm + L::kP + key * BM + ((r >> 2) ^ L::p_swizzle(key)) * 4 + (r & 3), x);
+      }
+    }
+    __syncthreads();   // K is read
+    if (t + 1 < n_tiles && tid == 0 && ok)
+      load_tile<D, true>(p, &map_k, sm + L::kK, bar_k, b, layer, hkv, k0 + kBN, k_hi);
+    if (ok) ok = mbar_wait(bar_v, (uint32_t)(t & 1), abort_flag, p.dev_status);
+    if (nk < kBN) {   // the share's last tile: P is 0 past its keys, and 0 must not meet a NaN of V
+      for (int r = nk; r < ((nk + 3) & ~3); ++r)
+        for (int d = tid; d < D; d += kThreads) sm[L::kV + r * D + d] = 0.f;
+      __syncthreads();
+    }
+    // ---- O += P V, pairs over rows
+    const float* vp = sm + L::kV;
+#pragma unroll 1
+    for (int k4 = 0; k4 < nk; k4 += 4) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const int k = k4 + e;
+        float pk[RM], v[DC];
+#pragma unroll
+        for (int i = 0; i < RM; i += RC) {
+          const int r = rg * RM + i;
+          float x[RC];
+          load_n<RC>(sm + L::kP + k * BM + ((r >> 2) ^ L::p_swizzle(k)) * 4 + (r & 3), x);
+#pragma unroll
+          for (int q = 0; q < RC; ++q) pk[i + q] = x[q];
+        }
+        load_cols<D>(vp + k * D, g, v);
+#pragma unroll
+        for (int c = 0; c < DC; ++c) {
+          const unsigned long long vv = f2_pack(v[c], v[c]);
+#pragma unroll
+          for (int i = 0; i < RM / 2; ++i) o[c][i] = f2_fma(f2_pack(pk[2 * i], pk[2 * i + 1]), vv, o[c][i]);
+        }
+      }
+    }
+  }
+
+  if (!ok) {   // copies in flight land (bounded) before shared memory is reused or given up
+    for (int ph = 0; ph < 2; ++ph) {
+      mbar_drain(bar_q, (uint32_t)ph, 50000000ull);
+      mbar_drain(bar_k, (uint32_t)ph, 50000000ull);
+      mbar_drain(bar_v, (uint32_t)ph, 50000000ull);
+    }
+  }
+  // ---- this CTA's partial rows into shared memory (over V and P)
   __syncthreads();
-  if (warp == 0) {
-    float M = -INFINITY;
 #pragma unroll
-    for (int w = 0; w < kWarps; ++w) M = fmaxf(M, m_s[w]);
-    float L = 0.f, wgt[kWarps];
+  for (int i = 0; i < RM; ++i) {
+    const float l = group_sum(l_run[i]);
+    if (g == 0) *reinterpret_cast<float2*>(sm + L::kMl + (rg * RM + i) * 2) = make_float2(m_run[i], l);
+  }
 #pragma unroll
-    for (int w = 0; w < kWarps; ++w) {
-      wgt[w] = (m_s[w] == -INFINITY) ? 0.f : expf(m_s[w] - M);
-      L += l_s[w] * wgt[w];
+  for (int i = 0; i < RM; ++i) {
+    float x[DC];
+#pragma unroll
+    for (int c = 0; c < DC; ++c) {
+      float lo, hi;
+      f2_unpack(o[c][i / 2], lo, hi);
+      x[c] = i & 1 ? hi : lo;
     }
-    const float inv = L > 0.f ? 1.f / L : 0.f;
-#pragma unroll
-    for (int c = 0; c < DPL; ++c) {
-      float o = 0.f;
-#pragma unroll
-      for (int w = 0; w < kWarps; ++w) o = fmaf(wgt[w], o_s[w][c * 32 + lane], o);
-      O[qrow + c * 32 + lane] = o * inv;
+    float* dst = sm + L::kO + (rg * RM + i) * D;
+    if constexpr (D == 128) {
+      *reinterpret_cast<float4*>(dst + 4 * g) = make_float4(x[0], x[1], x[2], x[3]);
+      *reinterpret_cast<float4*>(dst + 64 + 4 * g) = make_float4(x[4], x[5], x[6], x[7]);
+    } else {
+      store_n<DC>(dst + DC * g, x);
     }
+  }
+  cluster.sync();
+  // ---- combine: CTA r writes the r-th share of the rows, one row per warp at a time
+  constexpr int WC = D / 32;   // columns per lane of a whole warp
+  const int r_lo = rank * rows / csize, r_hi = (rank + 1) * rows / csize;
+#pragma unroll 1
+  for (int r = r_lo + warp; r < r_hi; r += kWarps) {
+    float part[kMaxCluster][WC];
+#pragma unroll
+    for (int c = 0; c < kMaxCluster; ++c)
+      if (c < csize) load_n<WC>(cluster.map_shared_rank(sm + L::kO, c) + r * D + WC * lane, part[c]);
+    float m = -INFINITY, l = 0.f;
+    if (lane < csize) {
+      const float2 ml = *reinterpret_cast<const float2*>(cluster.map_shared_rank(sm + L::kMl, lane) + 2 * r);
+      m = ml.x, l = ml.y;
+    }
+    const float mm = warp_max(m);
+    const float w = l > 0.f ? exp2f(m - mm) : 0.f;
+    const float lw = warp_sum(l * w);
+    const float inv = lw > 0.f ? 1.f / lw : 0.f;
+    float acc[WC];
+#pragma unroll
+    for (int e = 0; e < WC; ++e) acc[e] = 0.f;
+#pragma unroll
+    for (int c = 0; c < kMaxCluster; ++c) {
+      const float wc = __shfl_sync(0xffffffffu, w, c);
+      if (c < csize) {
+#pragma unroll
+        for (int e = 0; e < WC; ++e) acc[e] = fmaf(wc, part[c][e], acc[e]);
+      }
+    }
+#pragma unroll
+    for (int e = 0; e < WC; ++e) acc[e] *= inv;
+    store_n<WC>(static_cast<float*>(p.out) + q_row(r) * D + WC * lane, acc);
+  }
+  cluster.sync();   // keep this CTA's shared memory alive until the others have read it
+}
+
+template <int D, int RM>
+cudaError_t launch(const CUtensorMap& map_k, const CUtensorMap& map_v, const AttnParams& p, int csize, int m_blocks, cudaStream_t stream) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)((long long)csize * m_blocks * p.hkv * p.batch * p.layers), 1, 1);
+  cfg.blockDim = dim3(kThreads, 1, 1);
+  cfg.dynamicSmemBytes = Layout<D, RM>::kBytes;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)csize;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // placed while the previous kernel drains
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  const cudaError_t e = cudaFuncSetAttribute(tree_attn_simt_kernel<D, RM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)Layout<D, RM>::kBytes);
+  if (e != cudaSuccess) return e;
+  return cudaLaunchKernelEx(&cfg, tree_attn_simt_kernel<D, RM>, map_k, map_v, p, csize, m_blocks,
+                            p.group > 1 ? (uint32_t)((0x100000000ull + p.group - 1) / p.group) : 0u);
+}
+
+template <int D>
+cudaError_t launch_d(const CUtensorMap& map_k, const CUtensorMap& map_v, const AttnParams& p, int max_ctx, int sms, cudaStream_t stream) {
+  const int M = p.max_nodes * p.group;
+  // rows per block: the smallest that holds M, up to 64 (two such CTAs fit an SM's shared memory;
+  // 128-row blocks, one per SM, left a unit's cluster of 8 CTAs short of SMs in some GPCs)
+  int bm = 16;
+  while (bm < 64 && bm < M) bm *= 2;
+  const int m_blocks = (M + bm - 1) / bm;
+  const long long units = (long long)m_blocks * p.hkv * p.batch * p.layers;
+  // CTAs per unit (a cluster): the split whose waves over the SMs take the fewest keys, a CTA's
+  // fixed part (set-up, combination) counted as 48 keys
+  const int keys = max_ctx + p.max_nodes;
+  const long long slots = 2ll * sms;
+  int csize = 1;
+  double best = 1e300;
+  for (int c = 1; c <= kMaxCluster; ++c) {
+    const double waves = (double)((units * c + slots - 1) / slots);
+    const double cost = waves * (((keys + c - 1) / c + 15) / 16 * 16 + 48);
+    if (cost < best) best = cost, csize = c;
+  }
+  if (units * csize > 0x7fffffffll) return cudaErrorInvalidValue;
+  switch (bm) {
+    case 16:
+      return launch<D, 16 / kGroups>(map_k, map_v, p, csize, m_blocks, stream);
+    case 32:
+      return launch<D, 32 / kGroups>(map_k, map_v, p, csize, m_blocks, stream);
+    default:
+      return launch<D, 64 / kGroups>(map_k, map_v, p, csize, m_blocks, stream);
   }
 }
 
 }  // namespace simt
 
-cudaError_t launch_tree_attn_simt(const AttnParams& p, cudaStream_t stream) {
+cudaError_t launch_tree_attn_simt(const CUtensorMap& map_k, const CUtensorMap& map_v, const AttnParams& p, int max_ctx, int sms, cudaStream_t stream) {
   if (p.hq > 65535 || p.n_total > 65535 || p.layers > 65535) return cudaErrorInvalidValue;
-  const dim3 grid((unsigned)p.hq, (unsigned)p.n_total, (unsigned)p.layers);
   switch (p.head_dim) {
     case 32:
-      simt::tree_attn_simt_kernel<32><<<grid, simt::kWarps * 32, 0, stream>>>(p);
-      break;
+      return simt::launch_d<32>(map_k, map_v, p, max_ctx, sms, stream);
     case 64:
-      simt::tree_attn_simt_kernel<64><<<grid, simt::kWarps * 32, 0, stream>>>(p);
-      break;
+      return simt::launch_d<64>(map_k, map_v, p, max_ctx, sms, stream);
     case 128:
-      simt::tree_attn_simt_kernel<128><<<grid, simt::kWarps * 32, 0, stream>>>(p);
-      break;
+      return simt::launch_d<128>(map_k, map_v, p, max_ctx, sms, stream);
     default:
       return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
 }
 
 }  // namespace ptd

@@ -183,6 +183,26 @@ def _check_every_unit(w, got, what, layers=None):
                 _check_attn(got[l][sl][:, hs], ref[:, hs], c.dtype, f"{what} l{l} b{b} kv{kvh}")
 
 
+@pytest.mark.parametrize("hq,hkv,d,nodes,ctx,page,batch,layers", [
+    (1, 1, 32, (1, 1), (0, 0), 0, 1, 1),          # one key, one row
+    (2, 2, 64, (16, 16), (15, 15), 0, 1, 1),      # a full 16-row block, fewer keys than one step of each share
+    (8, 8, 32, (17, 17), (63, 63), 0, 1, 2),      # 32-row block, a tile of 64 keys and 16 more
+    (6, 2, 64, (11, 11), (500, 500), 16, 1, 1),   # 33 rows in a 64-row block, group of 3, pages
+    (8, 2, 128, (32, 32), (1000, 1000), 0, 1, 1),   # 128-row block, full
+    (16, 2, 128, (24, 24), (300, 300), 64, 1, 1),   # 192 rows: three 64-row blocks
+    (28, 4, 128, (128, 128), (70, 70), 0, 1, 1),  # 896 rows: seven 128-row blocks, group of 7
+    (8, 4, 64, (3, 70), (1, 900), 32, 4, 2),      # ragged trees and contexts, most blocks partly empty
+])
+def test_attention_f32_blocks_match_oracle(hq, hkv, d, nodes, ctx, page, batch, layers):
+    """fp32 attention at the edges of its row blocks (16, 32, 64, 128 rows), key tiles and key
+    shares, every unit."""
+    over = dict(hq=hq, hkv=hkv, d=d, nodes=nodes, ctx=ctx, page_size=page, batch=batch, layers=layers, vocab=100,
+                tree="random-depth" if batch > 1 else "chain", branching=(4, 3, 2, 2, 1, 1), depth_range=(3, 6))
+    w = syn.Workload(syn.shrink(syn.CONFIGS["tiny-fp32"], **over), 31)
+    dw, got = _run_attention(w)
+    _check_every_unit(w, got, "f32 blocks")
+
+
 def test_attention_full_size_llama2_layer():
     """The Llama-2-7B-shaped layer at its own size: 32 MHA heads (M = 31 rows per unit, one
     128-row tcgen05 tile mostly padding), context 2048 (17 key tiles), every head."""
