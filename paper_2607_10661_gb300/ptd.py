@@ -2,7 +2,9 @@
 
 Argument marshalling only: every function checks dtype / device / contiguity of the torch
 tensors it is given, passes their data pointers and the current CUDA stream to the C ABI
-function of the same name, and raises PtdError on a non-OK status.  All compute happens
+function of the same name, and raises PtdError on a non-OK status.  The calls of a decoding
+step go through _ptdcall (csrc/pycall.cpp), which makes the same checks natively; whatever it
+does not take (another tensor type, a bad argument) continues on the ctypes path below it.  All compute happens
 in the CUDA kernels; there is no CPU path.  The library is loaded on first use and a
 missing or unloadable libptd.so raises immediately.
 """
@@ -71,6 +73,7 @@ class _HostIO(ctypes.Structure):
 
 
 _lib = None
+_calls = None   # the _ptdcall module, once the library is loaded
 
 
 def lib() -> ctypes.CDLL:
@@ -141,6 +144,26 @@ def lib() -> ctypes.CDLL:
         L.ptd_tree_verify_step_host.argtypes = [P(_Tree), P(_Cache), P(_StepArgs), P(_HostIO), vp]
         _lib = L
     return _lib
+
+
+def _native():
+    """The native call module bound to the loaded library (raises if either was not built)."""
+    global _calls
+    if _calls is None:
+        lib()
+        from . import _ptdcall
+
+        _ptdcall.load(LIB_PATH, torch.Tensor, torch.int32, torch.float32, torch.bfloat16,
+                      torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice)
+        _calls = _ptdcall
+    return _calls
+
+
+def _launched(r: int, where: str) -> int:
+    """A native call's answer: the kernels it launched, or minus its status."""
+    if r < 0:
+        raise PtdError(-r, where)
+    return r
 
 
 def status_string(status: int) -> str:
@@ -266,6 +289,10 @@ def tree_attention(tree: Tree, cache: KVCache, q: torch.Tensor, out: torch.Tenso
                    scale: float = 0.0, workspace: Optional[torch.Tensor] = None, stream=None) -> int:
     """ptd_tree_attention; returns the number of kernels launched."""
     n = cache.num_layers if num_layers is None else num_layers
+    r = (_calls or _native()).tree_attention(tree, cache, layer_begin, n, q, num_q_heads, scale, out, workspace, dev_status,
+                                          stream if stream is None else _stream(stream))
+    if r is not None:
+        return _launched(r, "ptd_tree_attention")
     ws = _dev(workspace, "workspace") if workspace is not None else None
     wsb = workspace.numel() * workspace.element_size() if workspace is not None else 0
     st = lib().ptd_tree_attention(ctypes.byref(tree.c), ctypes.byref(cache.c), layer_begin, n,
@@ -279,6 +306,10 @@ def tree_attention(tree: Tree, cache: KVCache, q: torch.Tensor, out: torch.Tenso
 def topk_draft(logits: torch.Tensor, k: int, out_idx: torch.Tensor, out_val: torch.Tensor,
                vocab: Optional[int] = None, stream=None) -> int:
     """ptd_topk_draft over the rows of a 2-D logits tensor."""
+    r = (_calls or _native()).topk_draft(logits, k, out_idx, out_val, vocab,
+                                      stream if stream is None else _stream(stream))
+    if r is not None:
+        return _launched(r, "ptd_topk_draft")
     rows, stride = logits.shape
     st = lib().ptd_topk_draft(_dev(logits, "logits"), _ptd_dtype(logits.dtype), rows,
                               stride if vocab is None else vocab, stride, k,
@@ -291,6 +322,10 @@ def topk_draft(logits: torch.Tensor, k: int, out_idx: torch.Tensor, out_val: tor
 def verify_greedy(tree: Tree, tokens: torch.Tensor, target: torch.Tensor, target_stride: int,
                   accepted: torch.Tensor, accept_len: torch.Tensor, bonus: torch.Tensor, dev_status: torch.Tensor,
                   stream=None) -> int:
+    r = (_calls or _native()).verify_greedy(tree, tokens, target, target_stride, accepted, accept_len, bonus, dev_status,
+                                         stream if stream is None else _stream(stream))
+    if r is not None:
+        return _launched(r, "ptd_verify_greedy")
     st = lib().ptd_verify_greedy(ctypes.byref(tree.c), _dev(tokens, "tokens", torch.int32),
                                  _dev(target, "target", torch.int32), target_stride,
                                  _dev(accepted, "accepted", torch.int32), _dev(accept_len, "accept_len", torch.int32),
@@ -302,6 +337,10 @@ def verify_greedy(tree: Tree, tokens: torch.Tensor, target: torch.Tensor, target
 
 def kv_compact(tree: Tree, cache: KVCache, accepted: torch.Tensor, accept_len: torch.Tensor,
                new_ctx: torch.Tensor, stream=None) -> int:
+    r = (_calls or _native()).kv_compact(tree, cache, accepted, accept_len, new_ctx,
+                                      stream if stream is None else _stream(stream))
+    if r is not None:
+        return _launched(r, "ptd_kv_compact")
     st = lib().ptd_kv_compact(ctypes.byref(tree.c), ctypes.byref(cache.c), _dev(accepted, "accepted", torch.int32),
                               _dev(accept_len, "accept_len", torch.int32), _dev(new_ctx, "new_ctx", torch.int32),
                               _stream(stream))
@@ -313,6 +352,10 @@ def verify_sampling(tree: Tree, tokens: torch.Tensor, logits: torch.Tensor, temp
                     u_accept: torch.Tensor, u_bonus: torch.Tensor, accepted: torch.Tensor, accept_len: torch.Tensor,
                     bonus: torch.Tensor, dev_status: torch.Tensor, stream=None) -> int:
     """ptd_verify_sampling; logits [N_tot, V] (bf16 or fp32), uniforms fp32."""
+    r = (_calls or _native()).verify_sampling(tree, tokens, logits, temperature, u_accept, u_bonus, accepted, accept_len, bonus,
+                                           dev_status, stream if stream is None else _stream(stream))
+    if r is not None:
+        return _launched(r, "ptd_verify_sampling")
     if logits.dim() != 2 or logits.stride(1) != 1:
         raise ValueError("logits must be [rows, vocab] with unit column stride")
     dt = BF16 if logits.dtype == torch.bfloat16 else F32
@@ -330,6 +373,10 @@ def verify_sampling(tree: Tree, tokens: torch.Tensor, logits: torch.Tensor, temp
 def verify_and_compact(tree: Tree, cache: KVCache, tokens: torch.Tensor, target: torch.Tensor, target_stride: int,
                        accepted: torch.Tensor, accept_len: torch.Tensor, bonus: torch.Tensor, new_ctx: torch.Tensor,
                        dev_status: torch.Tensor, stream=None) -> int:
+    r = (_calls or _native()).verify_and_compact(tree, cache, tokens, target, target_stride, accepted, accept_len, bonus,
+                                              new_ctx, dev_status, stream if stream is None else _stream(stream))
+    if r is not None:
+        return _launched(r, "ptd_verify_and_compact")
     st = lib().ptd_verify_and_compact(ctypes.byref(tree.c), ctypes.byref(cache.c), _dev(tokens, "tokens", torch.int32),
                                       _dev(target, "target", torch.int32), target_stride,
                                       _dev(accepted, "accepted", torch.int32),
@@ -364,6 +411,9 @@ class StepBuffers:
 
 def tree_verify_step(tree: Tree, cache: KVCache, bufs: StepBuffers, stream=None) -> int:
     """ptd_tree_verify_step: attention, top-k, verification and compaction on device buffers."""
+    r = (_calls or _native()).tree_verify_step(tree, cache, bufs, stream if stream is None else _stream(stream))
+    if r is not None:
+        return _launched(r, "ptd_tree_verify_step")
     st = lib().ptd_tree_verify_step(ctypes.byref(tree.c), ctypes.byref(cache.c), ctypes.byref(bufs.c),
                                     _stream(stream))
     _check(st, "ptd_tree_verify_step")
@@ -392,6 +442,11 @@ def draft_tree_update(in_count: torch.Tensor, in_parents: torch.Tensor, in_token
                       out_depths: torch.Tensor, old_to_new: torch.Tensor, dev_status: torch.Tensor, stream=None) -> int:
     """ptd_draft_tree_update.  in_parents / in_tokens / old_to_new: [B, in_stride] int32;
     drafts: [B * in_stride, draft_stride] int32 (a top-k index matrix); out_*: [B, capacity] int32."""
+    r = (_calls or _native()).draft_tree_update(in_count, in_parents, in_tokens, drafts, expand, width, max_depth, capacity,
+                                             out_count, out_parents, out_tokens, out_depths, old_to_new, dev_status,
+                                             stream if stream is None else _stream(stream))
+    if r is not None:
+        return _launched(r, "ptd_draft_tree_update")
     if in_parents.dim() != 2 or in_tokens.shape != in_parents.shape or old_to_new.shape != in_parents.shape:
         raise ValueError("in_parents, in_tokens and old_to_new must be [batch, in_stride]")
     B, stride = in_parents.shape
@@ -428,6 +483,11 @@ class CandidatePool:
 
     def merge(self, step: int, count: torch.Tensor, parents: torch.Tensor, tokens: torch.Tensor,
               dev_status: torch.Tensor, max_load: Optional[int] = None, stream=None) -> int:
+        r = (_calls or _native()).pool_merge(
+            self.buf, self.capacity, self.capacity // 2 if max_load is None else max_load, step, count, parents, tokens,
+            dev_status, stream if stream is None else _stream(stream))
+        if r is not None:
+            return _launched(r, "ptd_pool_merge")
         st = lib().ptd_pool_merge(_dev(self.buf, "pool"), self.capacity,
                                   self.capacity // 2 if max_load is None else int(max_load), int(step),
                                   _dev(count, "count", torch.int32), _dev(parents, "parents", torch.int32),
@@ -438,6 +498,11 @@ class CandidatePool:
 
     def retrieve(self, root_token: torch.Tensor, width: int, max_depth: int, max_nodes: int,
                  out_count: torch.Tensor, out_parents: torch.Tensor, out_tokens: torch.Tensor, stream=None) -> int:
+        r = (_calls or _native()).pool_retrieve(
+            self.buf, self.capacity, root_token, width, max_depth, max_nodes, out_count, out_parents, out_tokens,
+            stream if stream is None else _stream(stream))
+        if r is not None:
+            return _launched(r, "ptd_pool_retrieve")
         if out_parents.numel() < max_nodes or out_tokens.numel() < max_nodes:
             raise ValueError("out_parents / out_tokens need max_nodes entries")
         st = lib().ptd_pool_retrieve(_dev(self.buf, "pool"), self.capacity, _dev(root_token, "root_token", torch.int32),
@@ -455,6 +520,10 @@ def tree_rope_append(tree: Tree, cache: KVCache, layer_begin: int, q: torch.Tens
     into cache layers layer_begin .. layer_begin + L - 1 (a 3-D q, k, v is one layer)."""
     dt = cache.k.dtype
     n_layers = q.shape[0] if q.dim() == 4 else 1
+    r = (_calls or _native()).tree_rope_append(tree, cache, layer_begin, n_layers, q, num_q_heads, k, v, rope_base,
+                                            positions_out, dev_status, stream if stream is None else _stream(stream))
+    if r is not None:
+        return _launched(r, "ptd_tree_rope_append")
     st = lib().ptd_tree_rope_append(ctypes.byref(tree.c), ctypes.byref(cache.c), int(layer_begin), int(n_layers),
                                     _dev(q, "q", dt),
                                     int(num_q_heads), _dev(k, "k", dt), _dev(v, "v", dt), float(rope_base),
@@ -471,6 +540,10 @@ def lm_head_workspace_size(rows: int, vocab: int) -> int:
 def lm_head_topk(hidden: torch.Tensor, weight: torch.Tensor, k: int, out_idx: torch.Tensor, out_val: torch.Tensor,
                  workspace: torch.Tensor, dev_status: torch.Tensor, stream=None) -> int:
     """ptd_lm_head_topk: hidden [rows, d] and weight [vocab, d] bf16 (rows may be strided)."""
+    r = (_calls or _native()).lm_head_topk(hidden, weight, k, out_idx, out_val, workspace, dev_status,
+                                        stream if stream is None else _stream(stream))
+    if r is not None:
+        return _launched(r, "ptd_lm_head_topk")
     if hidden.dim() != 2 or weight.dim() != 2 or hidden.shape[1] != weight.shape[1]:
         raise ValueError("hidden [rows, d] and weight [vocab, d] must share d")
     st = lib().ptd_lm_head_topk(_dev(hidden, "hidden", torch.bfloat16, row_strided=True), hidden.shape[0],

@@ -1,0 +1,87 @@
+"""The native call module (csrc/pycall.cpp): what it does not take goes to the ctypes path, which
+raises the binding's errors; both paths give the same results."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2607_10661_gb300 import ptd
+from paper_2607_10661_gb300 import synthetic as syn
+
+FUNCTIONS = {"tree_attention": 11, "topk_draft": 6, "verify_greedy": 9, "kv_compact": 6, "verify_sampling": 11,
+             "verify_and_compact": 11, "tree_verify_step": 4, "draft_tree_update": 15, "pool_merge": 9,
+             "pool_retrieve": 10, "tree_rope_append": 12, "lm_head_topk": 8}
+
+
+@pytest.fixture(scope="module")
+def calls():
+    import __graft_entry__
+
+    __graft_entry__.build()
+    return ptd._native()
+
+
+@pytest.mark.parametrize("name", list(FUNCTIONS))
+def test_native_calls_leave_other_arguments_alone(calls, name):
+    """Host tensors, plain objects and wrong counts are not taken (None: nothing was enqueued)."""
+    f = getattr(calls, name)
+    host = torch.zeros((2, 4), dtype=torch.int32)
+    for filler in (host, None, 3, [1, 2], 0.5):
+        assert f(*([filler] * FUNCTIONS[name])) is None
+    assert f() is None and f(*([host] * (FUNCTIONS[name] + 1))) is None
+
+
+@pytest.mark.gpu
+def test_native_and_ctypes_paths_agree(calls, monkeypatch):
+    class Refuse:
+        def __getattr__(self, name):
+            return lambda *a: None
+
+    g = torch.Generator(device="cuda").manual_seed(3)
+    x = torch.randn((5, 777), generator=g, device="cuda").to(torch.bfloat16)
+    out = []
+    for native in (True, False):
+        if not native:
+            monkeypatch.setattr(ptd, "_calls", Refuse())
+        idx = torch.zeros((5, 3), dtype=torch.int32, device="cuda")
+        val = torch.zeros((5, 3), device="cuda")
+        assert ptd.topk_draft(x, 3, idx, val) == 1
+        side = torch.cuda.Stream()
+        side.wait_stream(torch.cuda.current_stream())
+        idx2, val2 = torch.zeros_like(idx), torch.zeros_like(val)
+        assert ptd.topk_draft(x, 3, idx2, val2, vocab=np.int64(500), stream=side) == 1
+        torch.cuda.synchronize()
+        out.append((idx, val, idx2, val2))
+        with pytest.raises(TypeError):
+            ptd.topk_draft(x, 3, idx.float(), val)
+        with pytest.raises(ValueError):
+            ptd.topk_draft(x.cpu(), 3, idx, val)
+        with pytest.raises(ValueError):
+            ptd.topk_draft(x[:, ::2], 3, idx, val)
+        with pytest.raises(ptd.PtdError) as e:
+            ptd.topk_draft(x, 17, idx, val)
+        assert e.value.status == ptd.INVALID_ARG
+        with torch.cuda.stream(side):   # the current stream is asked for at every call
+            ptd.topk_draft(x, 3, idx2, val2)
+        side.synchronize()
+        assert torch.equal(idx2, idx) and torch.equal(val2, val)
+    for a, b in zip(*out):
+        assert torch.equal(a, b)
+
+
+@pytest.mark.gpu
+def test_native_step_matches_ctypes_step(calls, monkeypatch):
+    from paper_2607_10661_gb300.harness import DeviceWorkload
+
+    class Refuse:
+        def __getattr__(self, name):
+            return lambda *a: None
+
+    w = syn.Workload(syn.shrink(syn.CONFIGS["llama3-8b-gqa"], layers=2, ctx=(300, 300), vocab=5000), 7)
+    a, b = DeviceWorkload(w), DeviceWorkload(w)
+    na = a.step()
+    monkeypatch.setattr(ptd, "_calls", Refuse())
+    nb = b.step()
+    torch.cuda.synchronize()
+    assert na == nb
+    for name in ("attn_out", "topk_idx", "topk_val", "accepted", "accept_len", "bonus", "new_ctx", "k", "v"):
+        assert torch.equal(getattr(a, name), getattr(b, name)), name
