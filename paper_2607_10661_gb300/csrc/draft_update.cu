@@ -24,6 +24,7 @@
 #include <cstdint>
 
 #include "draft_update.cuh"
+#include "launch.cuh"
 #include "ptd_device.cuh"
 
 namespace ptd {
@@ -55,8 +56,8 @@ __device__ __forceinline__ int block_exclusive_scan(int x, int* warp_s, int* tot
 }
 
 __global__ void __launch_bounds__(kThreads)
-    draft_update_kernel(int in_stride, const int32_t* __restrict__ in_count, const int32_t* __restrict__ in_parents,
-                        const int32_t* __restrict__ in_tokens, const int32_t* __restrict__ drafts, int draft_stride,
+    draft_update_kernel(int in_stride, const int32_t* in_count, const int32_t* in_parents,
+                        const int32_t* in_tokens, const int32_t* drafts, int draft_stride,
                         int expand, int width, int max_depth, int capacity, int32_t* __restrict__ out_count,
                         int32_t* __restrict__ out_parents, int32_t* __restrict__ out_tokens,
                         int32_t* __restrict__ out_depths, int32_t* __restrict__ old_to_new,
@@ -69,6 +70,8 @@ __global__ void __launch_bounds__(kThreads)
   __shared__ int sub_depth_s[kThreads], first_kid_s[kThreads], newidx_s[kThreads];
   __shared__ int warp_s[kWarps];
 
+  if (threadIdx.x == 0) grid_launch_dependents();   // the next grid may be placed now; it waits for this one
+  grid_dependency_wait();   // the forests, the drafts and the outputs belong to the stream's previous work
   const int b = blockIdx.x, i = threadIdx.x;
   const size_t in0 = (size_t)b * in_stride, out0 = (size_t)b * capacity;
 
@@ -223,11 +226,9 @@ cudaError_t launch_draft_update(int batch, int in_stride, const int32_t* in_coun
                                 int width, int max_depth, int capacity, int32_t* out_count, int32_t* out_parents,
                                 int32_t* out_tokens, int32_t* out_depths, int32_t* old_to_new, int32_t* dev_status,
                                 cudaStream_t stream) {
-  du::draft_update_kernel<<<batch, du::kThreads, 0, stream>>>(in_stride, in_count, in_parents, in_tokens, drafts,
-                                                             draft_stride, expand, width, max_depth, capacity,
-                                                             out_count, out_parents, out_tokens, out_depths,
-                                                             old_to_new, dev_status);
-  return cudaGetLastError();
+  return launch_chained(du::draft_update_kernel, dim3(batch), dim3(du::kThreads), 0, stream, 0, in_stride, in_count,
+                        in_parents, in_tokens, drafts, draft_stride, expand, width, max_depth, capacity, out_count,
+                        out_parents, out_tokens, out_depths, old_to_new, dev_status);
 }
 
 }  // namespace ptd

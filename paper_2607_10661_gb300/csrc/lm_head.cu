@@ -22,6 +22,7 @@
 #include <cstdint>
 
 #include "lm_head.cuh"
+#include "launch.cuh"
 #include "ptd_device.cuh"
 
 namespace ptd {
@@ -104,6 +105,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     tmem_relinquish();
     tc_fence_before();
   }
+  // set-up that reads no global memory may overlap the stream's previous grid; the rest waits for it
+  if (threadIdx.x == 0) grid_launch_dependents();
+  grid_dependency_wait();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(smem + kOffTmemPtr);
@@ -244,9 +248,11 @@ __device__ __forceinline__ void warp_top(uint64_t (&top)[KM], uint64_t (&out)[KM
 
 template <int KM>
 __global__ void __launch_bounds__(kMergeThreads)
-    lm_merge_kernel(const uint64_t* __restrict__ partial, int ctas, int rows, int k, int32_t* __restrict__ out_idx,
+    lm_merge_kernel(const uint64_t* partial, int ctas, int rows, int k, int32_t* __restrict__ out_idx,
                     float* __restrict__ out_val) {
   __shared__ uint64_t warp_s[kMergeThreads / 32][KM];
+  if (threadIdx.x == 0) grid_launch_dependents();
+  grid_dependency_wait();   // the candidate lists belong to the product before this grid
   const int r = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   uint64_t top[KM];
 #pragma unroll
@@ -300,11 +306,11 @@ cudaError_t launch_lm_head_topk(const CUtensorMap& map_h, const CUtensorMap& map
     e = cudaFuncSetAttribute(lm::lm_head_topk_kernel<KMV>, cudaFuncAttributeMaxDynamicSharedMemorySize,          \
                              (int)lm::kSmemBytes);                                                                \
     if (e != cudaSuccess) return e;                                                                               \
-    lm::lm_head_topk_kernel<KMV><<<ctas, lm::kThreads, lm::kSmemBytes, stream>>>(                                 \
-        map_h, map_w, rows, d_model, vocab, k, out_idx, out_val, partial, dev_status);                            \
-    e = cudaGetLastError();                                                                                       \
+    e = launch_chained(lm::lm_head_topk_kernel<KMV>, dim3(ctas), dim3(lm::kThreads), lm::kSmemBytes, stream, 0,   \
+                       map_h, map_w, rows, d_model, vocab, k, out_idx, out_val, partial, dev_status);             \
     if (e != cudaSuccess) return e;                                                                               \
-    lm::lm_merge_kernel<KMV><<<rows, lm::kMergeThreads, 0, stream>>>(partial, ctas, rows, k, out_idx, out_val);   \
+    return launch_chained(lm::lm_merge_kernel<KMV>, dim3(rows), dim3(lm::kMergeThreads), 0, stream, 0, partial,   \
+                          ctas, rows, k, out_idx, out_val);                                                       \
   } while (0)
   if (k <= 4)
     PTD_LM_LAUNCH(4);
@@ -313,7 +319,6 @@ cudaError_t launch_lm_head_topk(const CUtensorMap& map_h, const CUtensorMap& map
   else
     PTD_LM_LAUNCH(16);
 #undef PTD_LM_LAUNCH
-  return cudaGetLastError();
 }
 
 }  // namespace ptd

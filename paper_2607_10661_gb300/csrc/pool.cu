@@ -25,6 +25,7 @@
 
 #include <cstdint>
 
+#include "launch.cuh"
 #include "pool.cuh"
 #include "ptd_device.cuh"
 
@@ -125,14 +126,15 @@ __device__ __forceinline__ int block_exclusive_scan(int x, int* warp_s, int* tot
 }
 
 __global__ void __launch_bounds__(kThreads)
-    pool_merge_kernel(void* pool, int cap, int max_load, int step, const int32_t* __restrict__ count,
-                      const int32_t* __restrict__ parents, const int32_t* __restrict__ tokens,
-                      int32_t* __restrict__ dev_status) {
+    pool_merge_kernel(void* pool, int cap, int max_load, int step, const int32_t* count, const int32_t* parents,
+                      const int32_t* tokens, int32_t* dev_status) {
   __shared__ int par_s[kThreads], slot_s[2][kThreads];
   __shared__ int new_parent_s[kThreads], new_slot_s[kThreads];
   __shared__ uint64_t new_key_s[kThreads];
   __shared__ int warp_s[kWarps];
   __shared__ int used_s, fail_s;
+  if (threadIdx.x == 0) grid_launch_dependents();   // the next grid may be placed now; it waits for this one
+  grid_dependency_wait();   // the forest and the pool belong to the stream's previous work
   const View pv = view(pool, cap);
   const int u = threadIdx.x;
   const int T = *count;
@@ -224,11 +226,12 @@ __global__ void __launch_bounds__(kThreads)
 }
 
 __global__ void __launch_bounds__(kThreads)
-    pool_retrieve_kernel(const void* pool, int cap, const int32_t* __restrict__ root_token, int width,
-                         int max_depth, int max_nodes, int32_t* __restrict__ out_count,
-                         int32_t* __restrict__ out_parents, int32_t* __restrict__ out_tokens) {
+    pool_retrieve_kernel(const void* pool, int cap, const int32_t* root_token, int width, int max_depth,
+                         int max_nodes, int32_t* out_count, int32_t* out_parents, int32_t* out_tokens) {
   __shared__ int slot_s[kThreads], par_s[kThreads], tok_s[kThreads];
   __shared__ int warp_s[kWarps];
+  if (threadIdx.x == 0) grid_launch_dependents();   // the next grid may be placed now; it waits for this one
+  grid_dependency_wait();   // the pool, the root token and the outputs belong to the stream's previous work
   const View pv = view(const_cast<void*>(pool), cap);
   const int t = threadIdx.x;
   const int x = *root_token;
@@ -283,17 +286,15 @@ cudaError_t pool_init(void* pool, int capacity, cudaStream_t stream) {
 
 cudaError_t launch_pool_merge(void* pool, int capacity, int max_load, int step, const int32_t* count,
                               const int32_t* parents, const int32_t* tokens, int32_t* dev_status, cudaStream_t stream) {
-  pl::pool_merge_kernel<<<1, pl::kThreads, 0, stream>>>(pool, capacity, max_load, step, count, parents, tokens,
-                                                        dev_status);
-  return cudaGetLastError();
+  return launch_chained(pl::pool_merge_kernel, dim3(1), dim3(pl::kThreads), 0, stream, 0, pool, capacity, max_load, step,
+                        count, parents, tokens, dev_status);
 }
 
 cudaError_t launch_pool_retrieve(const void* pool, int capacity, const int32_t* root_token, int width, int max_depth,
                                  int max_nodes, int32_t* out_count, int32_t* out_parents, int32_t* out_tokens,
                                  cudaStream_t stream) {
-  pl::pool_retrieve_kernel<<<1, pl::kThreads, 0, stream>>>(pool, capacity, root_token, width, max_depth, max_nodes,
-                                                           out_count, out_parents, out_tokens);
-  return cudaGetLastError();
+  return launch_chained(pl::pool_retrieve_kernel, dim3(1), dim3(pl::kThreads), 0, stream, 0, pool, capacity, root_token,
+                        width, max_depth, max_nodes, out_count, out_parents, out_tokens);
 }
 
 }  // namespace ptd

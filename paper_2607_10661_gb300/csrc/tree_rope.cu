@@ -17,6 +17,7 @@
 
 #include <cstdint>
 
+#include "launch.cuh"
 #include "ptd_device.cuh"
 #include "tree_rope.cuh"
 
@@ -85,17 +86,18 @@ __device__ __forceinline__ void st16(T* p, const Vec<T>& r) {
 // D/2 is a multiple of the vector width, so every access is a 16-byte vector.
 template <typename T, bool kVec>
 __global__ void __launch_bounds__(kThreads)
-    tree_rope_kernel(const int32_t* __restrict__ node_offsets, const int32_t* __restrict__ parents,
-                     const int32_t* __restrict__ ctx_lens, int batch, int n_total, int num_layers, int D, int hq,
-                     int hkv, T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v,
-                     T* __restrict__ k_cache, T* __restrict__ v_cache, int layer_begin, int page_size,
-                     int seq_capacity, int num_pages, const int32_t* __restrict__ block_table, int max_pages,
-                     const RopeFreqs freqs, int32_t* __restrict__ positions_out, int32_t* __restrict__ dev_status) {
+    tree_rope_kernel(const int32_t* node_offsets, const int32_t* parents, const int32_t* ctx_lens, int batch,
+                     int n_total, int num_layers, int D, int hq, int hkv, T* __restrict__ q, const T* __restrict__ k,
+                     const T* __restrict__ v, T* __restrict__ k_cache, T* __restrict__ v_cache, int layer_begin,
+                     int page_size, int seq_capacity, int num_pages, const int32_t* block_table, int max_pages,
+                     const __grid_constant__ RopeFreqs freqs, int32_t* positions_out, int32_t* dev_status) {
   __shared__ int par_s[kThreads];
   __shared__ float cos_s[kMaxRopeHalf], sin_s[kMaxRopeHalf];
   __shared__ int pos_s, slot_s, b_s;
   const int n = blockIdx.x, t = threadIdx.x;
   const int l0 = blockIdx.y * kLayersPerCta;   // first layer of this CTA, relative to layer_begin
+  if (t == 0) grid_launch_dependents();   // the next grid may be placed now; it waits for this one
+  grid_dependency_wait();   // the trees, q, k, v and the cache belong to the stream's previous work
   if (t == 0) {   // the tree holding node n (B is small: a linear search)
     int b = 0;
     while (b + 1 < batch && node_offsets[b + 1] <= n) ++b;
@@ -222,8 +224,8 @@ cudaError_t launch_tree_rope(const int32_t* node_offsets, const int32_t* parents
   const auto al16 = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; };
   const bool aligned = al16(q) && al16(k) && al16(v) && al16(k_cache) && al16(v_cache);
 #define PTD_ROPE_LAUNCH(T, VEC)                                                                                    \
-  tr::tree_rope_kernel<T, VEC><<<grid, tr::kThreads, 0, stream>>>(                                                \
-      node_offsets, parents, ctx_lens, batch, n_total, num_layers, head_dim, hq, hkv, static_cast<T*>(q),        \
+  return launch_chained(                                                                                         \
+      tr::tree_rope_kernel<T, VEC>, grid, dim3(tr::kThreads), 0, stream, 0, node_offsets, parents, ctx_lens, batch, n_total, num_layers, head_dim, hq, hkv, static_cast<T*>(q),        \
       static_cast<const T*>(k), static_cast<const T*>(v), static_cast<T*>(k_cache), static_cast<T*>(v_cache),    \
       layer_begin, page_size, seq_capacity, num_pages, block_table, max_pages, freqs, positions_out, dev_status)
   if (bf16) {
@@ -238,7 +240,6 @@ cudaError_t launch_tree_rope(const int32_t* node_offsets, const int32_t* parents
       PTD_ROPE_LAUNCH(float, false);
   }
 #undef PTD_ROPE_LAUNCH
-  return cudaGetLastError();
 }
 
 }  // namespace ptd

@@ -19,6 +19,7 @@
 
 #include <cstdint>
 
+#include "launch.cuh"
 #include "ptd_device.cuh"
 #include "verify_compact.cuh"
 #include "verify_tree.cuh"
@@ -29,8 +30,8 @@ namespace vc {
 constexpr int kVerifyThreads = 128;
 
 __global__ void __launch_bounds__(kVerifyThreads)
-    verify_greedy_kernel(const int32_t* __restrict__ node_offsets, const int32_t* __restrict__ parents,
-                         const int32_t* __restrict__ tokens, const int32_t* __restrict__ target, int target_stride,
+    verify_greedy_kernel(const int32_t* node_offsets, const int32_t* parents, const int32_t* tokens,
+                         const int32_t* target, int target_stride,
                          int n_total, int max_nodes, int32_t* __restrict__ accepted, int32_t* __restrict__ accept_len,
                          int32_t* __restrict__ bonus, int32_t* __restrict__ dev_status) {
   __shared__ int jump_s[kVerifyThreads];
@@ -43,6 +44,8 @@ __global__ void __launch_bounds__(kVerifyThreads)
 
   const int b = blockIdx.x;
   const int i = threadIdx.x;
+  if (i == 0) grid_launch_dependents();   // the next grid may be placed now; it waits for this one
+  grid_dependency_wait();   // the trees, the targets and the outputs belong to the stream's previous work
   const int node0 = node_offsets[b];
   const int T = node_offsets[b + 1] - node0;
   int32_t* acc_row = accepted + (size_t)b * max_nodes;
@@ -269,10 +272,9 @@ cudaError_t launch_verify(const int32_t* node_offsets, const int32_t* parents, c
                           const int32_t* target, int target_stride, int batch, int n_total, int max_nodes,
                           int32_t* accepted, int32_t* accept_len, int32_t* bonus, int32_t* dev_status,
                           cudaStream_t stream) {
-  vc::verify_greedy_kernel<<<batch, vc::kVerifyThreads, 0, stream>>>(node_offsets, parents, tokens, target,
-                                                                     target_stride, n_total, max_nodes, accepted,
-                                                                     accept_len, bonus, dev_status);
-  return cudaGetLastError();
+  return launch_chained(vc::verify_greedy_kernel, dim3(batch), dim3(vc::kVerifyThreads), 0, stream, 0, node_offsets,
+                        parents, tokens, target, target_stride, n_total, max_nodes, accepted, accept_len, bonus,
+                        dev_status);
 }
 
 cudaError_t launch_verify_compact(const int32_t* node_offsets, const int32_t* parents, const int32_t* tokens,

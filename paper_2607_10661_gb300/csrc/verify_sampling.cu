@@ -45,6 +45,7 @@
 #include <cmath>
 #include <cstdint>
 
+#include "launch.cuh"
 #include "ptd_device.cuh"
 #include "verify_sampling.cuh"
 
@@ -181,10 +182,9 @@ __device__ __forceinline__ void load_chunk32(const LT* row, int c0, int c1, floa
 // its chunk of the visited row in registers (the bonus reads no logits again).
 template <typename LT, bool kRegs>
 __global__ void __launch_bounds__(kThreads)
-    verify_sampling_kernel(const int32_t* __restrict__ node_offsets, const int32_t* __restrict__ parents,
-                           const int32_t* __restrict__ tokens, const LT* __restrict__ logits, int vocab,
-                           int64_t row_stride, int vec_ok, float inv_temp, const float* __restrict__ u_accept,
-                           const float* __restrict__ u_bonus, int n_total, int max_nodes,
+    verify_sampling_kernel(const int32_t* node_offsets, const int32_t* parents, const int32_t* tokens,
+                           const LT* __restrict__ logits, int vocab, int64_t row_stride, int vec_ok, float inv_temp,
+                           const float* u_accept, const float* u_bonus, int n_total, int max_nodes,
                            int32_t* __restrict__ accepted, int32_t* __restrict__ accept_len,
                            int32_t* __restrict__ bonus, int32_t* __restrict__ dev_status) {
   cg::cluster_group cluster = cg::this_cluster();
@@ -204,6 +204,8 @@ __global__ void __launch_bounds__(kThreads)
   __shared__ int chosen_s, nrej_s, len_s;
 
   const int b = blockIdx.y, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  if (tid == 0) grid_launch_dependents();   // the next grid may be placed now; it waits for this one
+  grid_dependency_wait();   // the trees, the logits and the outputs belong to the stream's previous work
   const int node0 = node_offsets[b];
   const int T = node_offsets[b + 1] - node0;
   int32_t* acc_row = accepted + (size_t)b * max_nodes;
@@ -532,25 +534,10 @@ cudaError_t launch(const int32_t* node_offsets, const int32_t* parents, const in
                       ((uint64_t)row_stride * sizeof(LT)) % 16 == 0;
   const int G = csize * kThreads;
   const int chunk = (((vocab + G - 1) / G) + 7) & ~7;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)csize, (unsigned)batch, 1);
-  cfg.blockDim = dim3(kThreads, 1, 1);
-  cfg.dynamicSmemBytes = 0;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = (unsigned)csize;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  if (vec_ok && chunk <= 32)
-    return cudaLaunchKernelEx(&cfg, verify_sampling_kernel<LT, true>, node_offsets, parents, tokens, logits, vocab,
-                              row_stride, 1, inv_temp, u_accept, u_bonus, n_total, max_nodes, accepted,
-                              accept_len, bonus, dev_status);
-  return cudaLaunchKernelEx(&cfg, verify_sampling_kernel<LT, false>, node_offsets, parents, tokens, logits, vocab,
-                            row_stride, vec_ok ? 1 : 0, inv_temp, u_accept, u_bonus, n_total, max_nodes, accepted,
-                            accept_len, bonus, dev_status);
+  return launch_chained(vec_ok && chunk <= 32 ? verify_sampling_kernel<LT, true> : verify_sampling_kernel<LT, false>,
+                        dim3((unsigned)csize, (unsigned)batch, 1), dim3(kThreads), 0, stream, (unsigned)csize,
+                        node_offsets, parents, tokens, logits, vocab, row_stride, vec_ok ? 1 : 0, inv_temp, u_accept,
+                        u_bonus, n_total, max_nodes, accepted, accept_len, bonus, dev_status);
 }
 
 }  // namespace vs
