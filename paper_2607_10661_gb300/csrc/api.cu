@@ -374,7 +374,8 @@ static ptd_status topk_draft(const void* logits, ptd_dtype dtype, int64_t rows, 
   ptd_status st0 = check_topk_args(logits, dtype, rows, vocab, row_stride, k, out_idx, out_val);
   if (st0 != PTD_OK) return st0;
   const ptd_status st = cuda_status(ptd::launch_topk(logits, dtype == PTD_BF16, rows, vocab, row_stride, k, out_idx,
-                                                     out_val, nullptr, nullptr, static_cast<cudaStream_t>(stream)));
+                                                     out_val, nullptr, nullptr,
+                                                     static_cast<cudaStream_t>(stream)));
   if (st == PTD_OK) g_last_launches = 1;
   return st;
 }
@@ -630,8 +631,11 @@ constexpr int kTailSeparate = 0, kTailClustered = 1, kTailStreamed = 2;
 // The step's tail for checked arguments.  The streaming top-k needs rows back to back on
 // 16-byte vectors and the whole tail of ptd_step_workspace_size; the clustered one only the
 // per-tree counters; both need the tensor-core attention (which clears the counters) and bf16
-// logits.  With both possible the policy decides (auto: stream when the clustered grid, at
-// three CTAs per SM, would need more than one wave).
+// logits.  With both possible the policy decides.  Auto streams rows of 64K logits and more, k
+// <= 4, when they are more than one wave of 64 KB slices: 640 rows of 128256 k = 1 75.9 -> 67.3
+// us a step, k = 4 79.9 -> 75.2, 266 rows 89.4 / 89.7; elsewhere the clustered form is faster
+// (clustered / streamed: 250 rows k = 8 84.1 / 89.0, 128 rows of 152064 k = 6 150.4 / 153.3, 640
+// rows of 32000 43.5 / 49.4 and of 1000 29.9 / 73.8, one wave of 63 rows 68.5 / 72.4).
 int step_tail(const ptd_tree* tree, const ptd_kv_cache* cache, const ptd_step_args* a, size_t* attn_ws_out,
               int* sms_out) {
   const size_t attn_ws = (ptd_attention_workspace_size(tree, cache, a->num_q_heads, cache->num_layers) + 255) /
@@ -647,9 +651,10 @@ int step_tail(const ptd_tree* tree, const ptd_kv_cache* cache, const ptd_step_ar
                            a->workspace_bytes >= attn_ws + tail_counters_bytes(tree->batch);
   if (can_stream && can_cluster) {
     const int policy = g_step_topk.load();
-    const int64_t cluster_ctas = (int64_t)tree->total_nodes * ptd::topk_cluster_size(a->vocab);
+    const int64_t cluster_ctas = (int64_t)tree->total_nodes * ptd::topk_slices(a->vocab);
     const bool stream = policy == PTD_STEP_TOPK_STREAMED ||
-                        (policy == PTD_STEP_TOPK_AUTO && cluster_ctas > 3 * (int64_t)sms);
+                        (policy == PTD_STEP_TOPK_AUTO && cluster_ctas > 3 * (int64_t)sms && a->k <= 4 &&
+                         a->vocab >= 65536);
     return stream ? kTailStreamed : kTailClustered;
   }
   return can_stream ? kTailStreamed : (can_cluster ? kTailClustered : kTailSeparate);

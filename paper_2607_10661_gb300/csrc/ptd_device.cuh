@@ -76,6 +76,32 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
   }
 }
 
+// As mbar_wait for a barrier that other CTAs of the cluster arrive on: their writes before a
+// releasing arrival are visible after it.  Its limit is four times the others', so that a CTA whose
+// own wait ran out still finds this one there.
+__device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity, volatile int* abort_flag,
+                                                  int* dev_status) {
+  const unsigned long long t0 = globaltimer_ns();
+  for (uint32_t it = 1;; ++it) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    if (ok != 0) return true;
+    if ((it & 63u) == 0) {
+      if (*abort_flag) return false;
+      if (globaltimer_ns() - t0 > 4 * kWaitLimitNs) {
+        *abort_flag = 1;
+        if (dev_status) atomicMax(dev_status, (int)PTD_ERR_TIMEOUT);
+        return false;
+      }
+    }
+  }
+}
+
 // Warp-wide bounded wait: every lane polls, the loop exits for the whole warp at once
 // (so the following .sync.aligned tcgen05 instructions see a converged warp).
 __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag,

@@ -2,11 +2,11 @@
 // each node's draft token d_v and at most k children; Sec. 3.2: the greedy verification
 // token V_n is entry 0).  Pure HBM streaming.
 //
-// One thread-block cluster per logit row.  Every CTA of the cluster scans a contiguous
-// slice of the row with 16-byte vector loads; each thread keeps a sorted list of its KM
-// best (value, index) pairs in registers.  The lists are merged by warp shuffles, then
-// across the 8 warps of the CTA in shared memory, then across the CTAs of the cluster
-// through distributed shared memory (no global scratch, one launch).
+// One thread-block cluster per logit row, each CTA on a contiguous slice of it staged in shared
+// memory (topk_rows_kernel); rows too long for that are scanned with 16-byte vector loads,
+// each thread keeping a sorted list of its KM best (value, index) pairs in registers, the lists
+// merged by warp, CTA and cluster (topk_cluster_kernel).  No global scratch, one launch.  The
+// step's large batches have a streaming form of their own (topk_stream_kernel).
 //
 // Order: a 64-bit key (order-preserving bits of the fp32 value) << 32 | ~index, so a
 // larger key is a larger value or, on equal values, a lower index.  -0.0 is folded into
@@ -17,6 +17,7 @@
 
 #include <cstdint>
 
+#include "launch.cuh"
 #include "ptd_device.cuh"
 #include "topk.cuh"
 #include "verify_tree.cuh"
@@ -272,24 +273,37 @@ __device__ __forceinline__ void verify_and_write_warp(const VerifyArgs& va, int 
   }
 }
 
-// ------------------------------------------------------------------ bf16 fast path
-// Each CTA stages its contiguous slice of the row (up to kSliceVec 16-byte vectors) into
-// shared memory with bulk asynchronous copies, so the row is read from HBM exactly once.
-// Then every warp works on its own share of the slice (vectors lane + 32 w + 256 j) without
-// waiting for the others:
-//   1. every lane's maximum;
-//   2. T_w = the k-th largest lane maximum of the warp (k rounds of "largest wins"): the k
-//      lanes holding those maxima own k distinct elements >= T_w, so the warp's top-k is
-//      among its elements >= T_w;
-//   3. each lane keeps its elements >= T_w in an exact sorted list of KM (value, index)
-//      pairs (elements arrive in increasing index order, so ties keep the lower index), and
-//      the warp selects its top-k from the lists' heads.
-// One CTA barrier, then warp 0 merges the 8 warps' lists and the CTAs of the cluster merge
-// theirs over distributed shared memory.  With verification (the step's tail), the cluster
-// that writes the last row of a tree then verifies that tree (greedy, on one warp), so no
-// separate verification launch follows.
-constexpr int kSliceVec = 4096;            // 64 KB of bf16 logits per CTA
+// ------------------------------------------------------------------ rows in clusters
+// One cluster of CTAs per row (bf16 or fp32 logits).  Each CTA stages its contiguous slice of
+// the row into shared memory with bulk asynchronous copies, so the row is read from HBM exactly
+// once.  Then
+//   1. every lane's maximum (16 KB at a time as the copies land), and of each eight lanes' (32
+//      groups over the CTA);
+//   2. T = the k-th largest of the 32 group maxima: k elements of the slice are >= T, so
+//      nothing below T is among the slice's top-k (about 32 ln(32 / (32 - k)) elements are
+//      >= T: 4 for k = 4, 22 for k = 16);
+//   3. the elements >= T go to a candidate buffer as 64-bit keys in any order; a candidate's
+//      place among the slice's top-k is the number of larger candidates.
+// A slice whose candidates do not fit the buffer (long runs of equal values, or fewer than k
+// groups above -inf) selects by k rounds of "largest key below the last".  Each CTA writes its
+// keys into the shared memory of the cluster's first CTA and leaves; that one places the keys
+// among each other the same way.  With verification (the step's tail), the cluster that writes
+// the last row of a tree then verifies that tree (greedy, on one warp), so no separate
+// verification launch follows.
+//
+// What bounds it: for a few rows the chain copy, pass, selection, merge; for many the time a CTA
+// holds its shared memory (32 KB slices, five CTAs per SM) and its instructions.  Measured
+// (GB300; against the same split with per-thread sorted lists and k rounds of warp maxima at four
+// levels, each thread's list taking every element for fp32), 128256 logits a row: fp32, 63 rows,
+// k = 4 21.1 -> 11.9 us, k = 16 62.6 -> 14.9, 512 rows, k = 16 352 -> 72.5; bf16, 63 rows, k = 4
+// 8.5 -> 7.1, 512 rows 39.6 -> 32.1 (k = 16 102 -> 40.6).  A persistent grid with double-buffered
+// slices took 66 us for those 512 rows (the chain of a row is longer than its copy).
+constexpr int kSliceVec = 4096;            // 64 KB of bf16 logits per CTA at most
+constexpr int kSliceVecF32 = 5120;         // 80 KB of fp32 logits per CTA at most
+constexpr int kTargetVec = 2048;           // 32 KB: the slice that the cluster size aims at
 constexpr uint32_t kChunkBytes = 16384;    // bytes per bulk copy
+constexpr int kMaxK = 16;
+constexpr int kCand = 512;                 // candidate buffer (keys)
 
 __device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }
 __device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w & 0xFFFF0000u); }
@@ -301,242 +315,306 @@ __device__ __forceinline__ uint32_t bf16x2_max(uint32_t a, uint32_t b) {
 }
 constexpr uint32_t kBf16x2NegInf = 0xFF80FF80u;
 
-template <int KM, bool kVerify>
-__global__ void __launch_bounds__(kThreads) topk_bf16_kernel(const __nv_bfloat16* __restrict__ logits,
-                                                             int64_t rows, int vocab, int64_t row_stride, int k,
-                                                             int32_t* __restrict__ out_idx,
-                                                             float* __restrict__ out_val, int32_t* dev_status,
-                                                             const VerifyArgs va) {
+// The largest logit of a 16-byte vector.
+template <typename T>
+__device__ __forceinline__ float vec_max(const uint4& x) {
+  if constexpr (sizeof(T) == 2) {
+    const uint32_t h = bf16x2_max(bf16x2_max(x.x, x.y), bf16x2_max(x.z, x.w));
+    return fmaxf(bf16_lo(h), bf16_hi(h));
+  } else {
+    return fmax3(__uint_as_float(x.x), __uint_as_float(x.y), fmaxf(__uint_as_float(x.z), __uint_as_float(x.w)));
+  }
+}
+
+// The k-th largest of the warp's 32 order-preserving values (0 = a lane without one), or 0 when
+// fewer than k lanes hold one: one warp maximum and one ballot per distinct value, equal values
+// counted together.  Any x with k elements >= x bounds the warp's top-k from below.
+__device__ __forceinline__ uint32_t kth_largest_ord(uint32_t v, int k) {
+  int count = 0;
+  for (int s = 0; s < k; ++s) {
+    const uint32_t m = __reduce_max_sync(0xffffffffu, v);
+    if (m == 0u) return 0u;
+    count += __popc(__ballot_sync(0xffffffffu, v == m));
+    if (count >= k) return m;
+    if (v == m) v = 0u;
+  }
+  return 0u;
+}
+
+// The k-th largest (k <= 32) of 32 shared values, by every warp on its own: a lane's value with
+// k - 1 values before it (larger, or equal at a lower lane).
+__device__ __forceinline__ uint32_t kth_of_32(const uint32_t* v_s, int k) {
+  const int lane = threadIdx.x & 31;
+  const uint32_t mine = v_s[lane];
+  int before = 0;
+#pragma unroll
+  for (int i = 0; i < 32; i += 4) {
+    const uint4 o = *reinterpret_cast<const uint4*>(v_s + i);
+    before += (o.x > mine || (o.x == mine && i < lane)) + (o.y > mine || (o.y == mine && i + 1 < lane)) +
+              (o.z > mine || (o.z == mine && i + 2 < lane)) + (o.w > mine || (o.w == mine && i + 3 < lane));
+  }
+  const uint32_t at = __ballot_sync(0xffffffffu, before == k - 1);
+  return __shfl_sync(0xffffffffu, mine, __ffs(at) - 1);
+}
+
+constexpr int kChunkVec = (int)(kChunkBytes / 16);
+constexpr int kMaxChunks = (kSliceVecF32 + kChunkVec - 1) / kChunkVec;
+static_assert(kChunkVec == 4 * kThreads, "a chunk is four vectors per thread");
+
+template <typename T, bool kVerify>
+__global__ void __launch_bounds__(kThreads) topk_rows_kernel(const T* __restrict__ logits, int64_t rows, int vocab,
+                                                             int64_t row_stride, int k, int per,
+                                                             int32_t* __restrict__ out_idx, float* __restrict__ out_val,
+                                                             int32_t* dev_status, const VerifyArgs va) {
+  constexpr int VN = Vec<T>::kN;
   extern __shared__ __align__(128) uint4 slice[];
-  __shared__ uint64_t warp_keys[kWarps][KM];
-  __shared__ uint64_t cta_keys[KM];
-  __shared__ __align__(8) uint64_t bar_s;
-  __shared__ int abort_s;
+  __shared__ __align__(16) uint64_t cand_s[kCand];
+  __shared__ __align__(16) uint64_t all_keys[kMaxCluster * kMaxK];   // rank 0: every CTA's keys
+  __shared__ __align__(16) uint32_t group_max_s[32];
+  __shared__ __align__(8) uint64_t bars_s[kMaxChunks + 1];
+  __shared__ uint64_t round_s[kWarps];
+  __shared__ int n_cand_s, abort_s;
 
   cg::cluster_group cluster = cg::this_cluster();
-  const int rank = (int)cluster.block_rank();
-  const int csize = (int)cluster.num_blocks();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int tid = threadIdx.x;
-  const uint32_t bar = smem_u32(&bar_s);
+  const int rank = (int)blockIdx.x, csize = (int)gridDim.x;   // the grid's x is one cluster
+  const int64_t r = (int64_t)blockIdx.z * gridDim.y + blockIdx.y;
+  if (r >= rows) return;   // the whole cluster
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const uint32_t bar0 = smem_u32(bars_s), keys_bar = bar0 + 8u * kMaxChunks;
   if (tid == 0) {
-    mbar_init(bar, 1);
+    for (int c = 0; c < kMaxChunks; ++c) mbar_init(bar0 + 8u * (uint32_t)c, 1);
+    mbar_init(keys_bar, (uint32_t)(csize * k));   // one arrival per key (rank 0's is used)
     abort_s = 0;
+    n_cand_s = 0;
     fence_mbar_init();
   }
+  if (rank == 0 && tid < kMaxCluster * kMaxK) all_keys[tid] = 0ull;
   __syncthreads();
   if (tid == 0) grid_launch_dependents();   // the next grid may be placed now; it waits for this one
-  // the tree of a row (rank 0's thread 0 looks it up while the row's copy is in flight)
-  auto tree_of = [&](int64_t r) {
-    int lo = 0, hi = va.batch;
-    while (hi - lo > 1) {
-      const int mid = (lo + hi) >> 1;
-      if (va.node_offsets[mid] <= r) lo = mid; else hi = mid;
-    }
-    return lo;
-  };
+  // the cluster's CTAs are there and rank 0's keys and barrier are set up (waited for before the
+  // first key is sent)
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  // this CTA's slice: the vector body starts at the row's first 16-byte boundary (head and tail
+  // elements outside it go to the first and last CTA one by one)
+  const T* row = logits + r * row_stride;
+  int a0 = (int)(((16 - (reinterpret_cast<uintptr_t>(row) & 15)) & 15) / sizeof(T));
+  if (a0 > vocab) a0 = vocab;
+  const int nvec = (vocab - a0) / VN;
+  const int a1 = a0 + nvec * VN;
+  const int v_begin = min(nvec, rank * per), nv = min(nvec, v_begin + per) - v_begin;
+  const bool own_head = rank == 0 && tid == 0, own_tail = rank == csize - 1 && tid == kThreads - 1;
   int row_tree = 0;
   grid_dependency_wait();   // the logits, the trees and the outputs belong to the stream's previous work
+  if (tid == 0) {
+    const uint8_t* src = reinterpret_cast<const uint8_t*>(row + a0 + (size_t)v_begin * VN);
+    const uint32_t total = (uint32_t)nv * 16u;
+    for (uint32_t off = 0, c = 0; off < total; off += kChunkBytes, ++c) {
+      const uint32_t n = total - off < kChunkBytes ? total - off : kChunkBytes;
+      mbar_arrive_expect_tx(bar0 + 8u * c, n);
+      bulk_load(smem_u32(slice) + off, src + off, n, bar0 + 8u * c);
+    }
+    if constexpr (kVerify) {
+      if (rank == 0) {   // the tree of the row
+        int lo = 0, hi = va.batch;
+        while (hi - lo > 1) {
+          const int mid = (lo + hi) >> 1;
+          if (va.node_offsets[mid] <= r) lo = mid; else hi = mid;
+        }
+        row_tree = lo;
+      }
+    }
+  }
+  // with verification: warp 0 of rank 0 loads its row's tree (parents, tokens) while the copy is
+  // in flight, for the case that this cluster turns out to complete the tree
+  vt::TreeInputs tin;
   if constexpr (kVerify) {
     // Trees that no row completes (an empty or out-of-range node range, or offsets that do not
     // run from 0 to n_total): their outputs and the status are written here, by warp 1 of the
     // first CTA, while its copy is in flight; a tree whose rows all arrive is verified below.
-    if (blockIdx.x == 0 && blockIdx.y == 0 && warp == 1) flag_bad_trees_warp(va);
+    if (r == 0 && rank == 0 && warp == 1) flag_bad_trees_warp(va);
+    if (rank == 0 && warp == 0) {
+      const int b = __shfl_sync(0xffffffffu, row_tree, 0);
+      vt::load_tree_warp(va.node_offsets, va.parents, va.tokens, va.n_total, va.max_nodes, b, tin);
+    }
   }
-  uint32_t phase = 0;
+  // head / tail scalars while the copy is in flight
+  float tmax = -INFINITY;
+  if (own_head)
+    for (int i = 0; i < a0; ++i) tmax = fmaxf(tmax, Vec<T>::scalar(row + i));
+  if (own_tail)
+    for (int i = a1; i < vocab; ++i) tmax = fmaxf(tmax, Vec<T>::scalar(row + i));
 
-  for (int64_t r = blockIdx.y; r < rows; r += gridDim.y, phase ^= 1u) {
-    const __nv_bfloat16* row = logits + r * row_stride;
-    const uintptr_t addr = reinterpret_cast<uintptr_t>(row);
-    int a0 = (int)(((16 - (addr & 15)) & 15) / 2);
-    if (a0 > vocab) a0 = vocab;
-    const int nvec = (vocab - a0) / 8;
-    const int a1 = a0 + nvec * 8;
-    const int per = (nvec + csize - 1) / csize;
-    const int v_begin = min(nvec, rank * per), v_end = min(nvec, v_begin + per);
-    const int nv = v_end - v_begin;
-    const uint4* vrow = reinterpret_cast<const uint4*>(row + a0) + v_begin;
-    const bool own_head = rank == 0 && tid == 0;
-    const bool own_tail = rank == csize - 1 && tid == kThreads - 1;
-
-    if (tid == 0) {
-      fence_proxy_async_smem();   // the previous row's reads of the slice precede this copy
-      const uint32_t total = (uint32_t)nv * 16u;
-      mbar_arrive_expect_tx(bar, total);
-      for (uint32_t off = 0; off < total; off += kChunkBytes) {
-        const uint32_t n = total - off < kChunkBytes ? total - off : kChunkBytes;
-        bulk_load(smem_u32(slice) + off, reinterpret_cast<const uint8_t*>(vrow) + off, n, bar);
-      }
-      if constexpr (kVerify) {
-        if (rank == 0) row_tree = tree_of(r);
-      }
-    }
-    // with verification: warp 0 of rank 0 loads its row's tree (parents, tokens) while the copy is
-    // in flight, for the case that this cluster turns out to complete the tree
-    vt::TreeInputs tin;
-    if constexpr (kVerify) {
-      if (rank == 0 && warp == 0) {
-        const int b = __shfl_sync(0xffffffffu, row_tree, 0);
-        vt::load_tree_warp(va.node_offsets, va.parents, va.tokens, va.n_total, va.max_nodes, b, tin);
-      }
-    }
-    // head / tail scalars while the copy is in flight
-    float tmax = -INFINITY;
-    if (own_head)
-      for (int i = 0; i < a0; ++i) tmax = fmaxf(tmax, Vec<__nv_bfloat16>::scalar(row + i));
-    if (own_tail)
-      for (int i = a1; i < vocab; ++i) tmax = fmaxf(tmax, Vec<__nv_bfloat16>::scalar(row + i));
-    mbar_wait(bar, phase, &abort_s, dev_status);   // bounded: a lost copy only flags PTD_ERR_TIMEOUT
-
-    // 1. lane maximum (four vectors in flight, two chains of packed pair maxima)
-    {
-      uint32_t h0 = kBf16x2NegInf, h1 = kBf16x2NegInf;
-      int v = tid;
-      for (; v + 3 * kThreads < nv; v += 4 * kThreads) {
-        uint4 x[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) x[u] = slice[v + u * kThreads];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          h0 = bf16x2_max(h0, bf16x2_max(x[u].x, x[u].y));
-          h1 = bf16x2_max(h1, bf16x2_max(x[u].z, x[u].w));
-        }
-      }
-      for (; v < nv; v += kThreads) {
-        const uint4 x = slice[v];
+  // 1. lane maxima (four vectors in flight), then of eight lanes
+  {
+    uint32_t h0 = kBf16x2NegInf, h1 = kBf16x2NegInf;
+    float m0 = -INFINITY, m1 = -INFINITY;
+    auto fold = [&](const uint4& x) {
+      if constexpr (VN == 8) {
         h0 = bf16x2_max(h0, bf16x2_max(x.x, x.y));
         h1 = bf16x2_max(h1, bf16x2_max(x.z, x.w));
+      } else {
+        m0 = fmax3(m0, __uint_as_float(x.x), __uint_as_float(x.y));
+        m1 = fmax3(m1, __uint_as_float(x.z), __uint_as_float(x.w));
       }
-      h0 = bf16x2_max(h0, h1);
-      tmax = fmax3(tmax, bf16_lo(h0), bf16_hi(h0));
-    }
-    const bool has_elems = tid < nv || (own_head && a0 > 0) || (own_tail && a1 < vocab);
-
-    // 2. T_w: the k-th largest lane maximum of this warp (-inf when fewer lanes hold elements)
-    float thr;
-    {
-      uint64_t mine = has_elems ? make_key(ordered_bits(tmax), (uint32_t)lane) : 0ull;
-      uint64_t kth = 0ull;
-      for (int s = 0; s < k; ++s) {
-        const uint64_t best = warp_max_u64(mine);
-        if (mine == best) mine = 0ull;
-        kth = best;
-      }
-      thr = kth != 0ull ? from_ordered((uint32_t)(kth >> 32)) : -INFINITY;
-    }
-
-    // 3. every lane's exact list of its elements >= T_w, then the warp's top-k
-    ThreadList<KM> list;
-    list.init();
-    if (own_head)
-      for (int i = 0; i < a0; ++i) {
-        const float f = Vec<__nv_bfloat16>::scalar(row + i);
-        if (f >= thr) list.push(ordered_bits(f), (uint32_t)i);
-      }
-    {
-      auto vec_max = [](const uint4& x) {
-        const uint32_t h = bf16x2_max(bf16x2_max(x.x, x.y), bf16x2_max(x.z, x.w));
-        return fmaxf(bf16_lo(h), bf16_hi(h));
-      };
-      auto push_vec = [&](const uint4& x, int v) {
-        const uint32_t gi = (uint32_t)(a0 + (v_begin + v) * 8);
-        const uint32_t w[4] = {x.x, x.y, x.z, x.w};
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const float f0 = bf16_lo(w[q]), f1 = bf16_hi(w[q]);
-          if (f0 >= thr) list.push(ordered_bits(f0), gi + 2 * q);
-          if (f1 >= thr) list.push(ordered_bits(f1), gi + 2 * q + 1);
-        }
-      };
-      // four vectors in flight; the few that reach T_w are read again and pushed, in index order
-      int v = tid;
-      for (; v + 3 * kThreads < nv; v += 4 * kThreads) {
+    };
+#pragma unroll 1
+    for (int v0 = 0; v0 < nv; v0 += kChunkVec) {
+      // bounded: a lost copy only flags PTD_ERR_TIMEOUT
+      mbar_wait(bar0 + 8u * (uint32_t)(v0 / kChunkVec), 0u, &abort_s, dev_status);
+      const int v = v0 + tid;
+      if (v0 + kChunkVec <= nv) {
         uint4 x[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) x[u] = slice[v + u * kThreads];
-        uint32_t hits = 0u;
 #pragma unroll
-        for (int u = 0; u < 4; ++u) hits |= (vec_max(x[u]) >= thr ? 1u : 0u) << u;
+        for (int u = 0; u < 4; ++u) fold(x[u]);
+      } else {
+        for (int w = v; w < nv; w += kThreads) fold(slice[w]);
+      }
+    }
+    if constexpr (VN == 8) {
+      h0 = bf16x2_max(h0, h1);
+      tmax = fmax3(tmax, bf16_lo(h0), bf16_hi(h0));
+    } else {
+      tmax = fmax3(tmax, m0, m1);
+    }
+    const bool has_elems = tid < nv || (own_head && a0 > 0) || (own_tail && a1 < vocab);
+    uint32_t o = has_elems ? ordered_bits(tmax) : 0u;
+#pragma unroll
+    for (int d = 1; d < 8; d <<= 1) o = max(o, __shfl_xor_sync(0xffffffffu, o, d));
+    if ((lane & 7) == 0) group_max_s[warp * 4 + (lane >> 3)] = o;
+  }
+  __syncthreads();
+
+  // 2. T (0: fewer than k groups hold elements, so every element is a candidate)
+  const uint32_t kth = k <= 8 ? kth_largest_ord(group_max_s[lane], k) : kth_of_32(group_max_s, k);
+  const float thr = kth != 0u ? from_ordered(kth) : -INFINITY;
+
+  // 3. the candidates
+  auto push = [&](float f, uint32_t idx) {
+    const int at = atomicAdd(&n_cand_s, 1);
+    if (at < kCand) cand_s[at] = make_key(ordered_bits(f), idx);
+  };
+  if (own_head)
+    for (int i = 0; i < a0; ++i) {
+      const float f = Vec<T>::scalar(row + i);
+      if (f >= thr) push(f, (uint32_t)i);
+    }
+  if (own_tail)
+    for (int i = a1; i < vocab; ++i) {
+      const float f = Vec<T>::scalar(row + i);
+      if (f >= thr) push(f, (uint32_t)i);
+    }
+  // only lanes whose maximum reaches T (about k of the 256) read their vectors again: four in
+  // flight, and those that reach T once more
 #pragma unroll 1
-        for (; hits != 0u; hits &= hits - 1u) {   // rare: read the vector again
-          const int vu = v + (__ffs(hits) - 1) * kThreads;
-          push_vec(slice[vu], vu);
-        }
-      }
-      for (; v < nv; v += kThreads) {
-        const uint4 x = slice[v];
-        if (vec_max(x) >= thr) push_vec(x, v);
-      }
-    }
-    if (own_tail)
-      for (int i = a1; i < vocab; ++i) {
-        const float f = Vec<__nv_bfloat16>::scalar(row + i);
-        if (f >= thr) list.push(ordered_bits(f), (uint32_t)i);
-      }
-    for (int s = 0; s < k; ++s) {
-      const uint64_t mine = list.head();
-      const uint64_t best = warp_max_u64(mine);
-      if (mine == best) list.pop();
-      if (lane == 0) warp_keys[warp][s] = best;
-    }
-    __syncthreads();   // also: every thread is done reading the slice
-    if (warp == 0) {   // CTA merge across warps (lane w owns warp w's list)
-      int cur = 0;
-      for (int s = 0; s < k; ++s) {
-        const uint64_t mine = (lane < kWarps && cur < k) ? warp_keys[lane][cur] : 0ull;
-        const uint64_t best = warp_max_u64(mine);
-        if (lane < kWarps && mine == best && best != 0ull) ++cur;
-        if (lane == 0) cta_keys[s] = best;
-      }
-    }
-    cluster.sync();
-    // cluster merge: lane c of rank 0's warp 0 reads CTA c's sorted list at once, then k rounds
-    // of "largest head wins"; lane s writes entry s
-    if (rank == 0 && warp == 0) {
-      ThreadList<KM> ml;
-      ml.init();
-      if (lane < csize) {
-        const uint64_t* remote = cluster.map_shared_rank(cta_keys, lane);
-        uint64_t got[KM];
+  for (int v0 = 0; v0 < nv && tmax >= thr; v0 += kChunkVec) {
+    uint32_t hits = 0u;
 #pragma unroll
-        for (int s = 0; s < KM; ++s) got[s] = s < k ? remote[s] : 0ull;
+    for (int u = 0; u < 4; ++u) {
+      const int v = v0 + tid + u * kThreads;
+      if (v < nv && vec_max<T>(slice[v]) >= thr) hits |= 1u << u;
+    }
+#pragma unroll 1
+    for (; hits != 0u; hits &= hits - 1u) {
+      if (*(volatile int*)&n_cand_s > kCand) break;   // the buffer is already lost
+      const int v = v0 + tid + (__ffs(hits) - 1) * kThreads;
+      const uint32_t i0 = (uint32_t)(a0 + (v_begin + v) * VN);
+      float f[8];
+      Vec<T>::unpack(slice[v], f);
 #pragma unroll
-        for (int s = 0; s < KM; ++s)
-          if (got[s] != 0ull) ml.push_key(got[s]);
-      }
-      uint64_t out = 0ull;
-      for (int s = 0; s < k; ++s) {
-        const uint64_t mine = ml.head();
-        const uint64_t best = warp_max_u64(mine);
-        if (mine == best && best != 0ull) ml.pop();
-        if (lane == s) out = best;
-      }
-      if (lane < k) {
-        out_idx[r * k + lane] = (int32_t)(~(uint32_t)(out & 0xFFFFFFFFull));
-        out_val[r * k + lane] = from_ordered((uint32_t)(out >> 32));
-      }
-      if constexpr (kVerify) {
-        // the last row of a tree to be written: this cluster verifies the tree
-        int vb = -1;
-        __syncwarp();   // every lane's entries of this row are written before lane 0 counts the row
-        if (lane == 0) {
-          const int b = row_tree;
-          const int T = tin.T;
-          // release: this row's top-k before its count; acquire: the other rows' top-k (each
-          // written before its own count) before this cluster reads them
-          const int done = (int)atom_add_acq_rel_gpu(va.counters + b, 1u) + 1;
-          if (done == T) vb = b;
-        }
-        vb = __shfl_sync(0xffffffffu, vb, 0);
-        if (vb >= 0) {
-          __shared__ vt::VerifyScratch vsc[1];
-          __shared__ vt::TreeVerdict verdict[1];
-          __syncwarp();   // lane 0's acquire precedes every lane's reads of the tree's rows
-          verify_and_write_warp(va, vb, tin, out_idx, k, vsc[0], verdict[0]);
-        }
+      for (int e = 0; e < VN; ++e)
+        if (f[e] >= thr) push(f[e], i0 + e);
+    }
+  }
+  __syncthreads();
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  // a key's way to rank 0: the store, then an arrival that releases it
+  uint64_t* const dst_keys = cluster.map_shared_rank(all_keys, 0) + rank * kMaxK;
+  uint32_t dst_bar;
+  asm("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(dst_bar) : "r"(keys_bar));
+  auto arrive = [&](int count) {
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0], %1;" ::"r"(dst_bar), "r"(count) : "memory");
+  };
+  const int n = n_cand_s;
+  if (n <= kCand) {
+    for (int i = tid; i < n; i += kThreads) {
+      const uint64_t key = cand_s[i];
+      int before = 0;
+      for (int j = 0; j < n; ++j) before += cand_s[j] > key ? 1 : 0;
+      if (before < k) {
+        dst_keys[before] = key;
+        arrive(1);
       }
     }
-    cluster.sync();   // keep every CTA's shared memory alive until rank 0 has read it
+    if (tid == 0 && n < k) arrive(k - n);   // fewer elements than k in this slice
+  } else {
+    // k rounds over the slice (rare; every thread takes part)
+    uint64_t last = ~0ull;
+    for (int q = 0; q < k; ++q) {
+      uint64_t best = 0ull;
+      auto take = [&](float f, uint32_t idx) {
+        const uint64_t key = make_key(ordered_bits(f), idx);
+        if (key < last && key > best) best = key;
+      };
+      if (own_head)
+        for (int i = 0; i < a0; ++i) take(Vec<T>::scalar(row + i), (uint32_t)i);
+      if (own_tail)
+        for (int i = a1; i < vocab; ++i) take(Vec<T>::scalar(row + i), (uint32_t)i);
+      for (int v = tid; v < nv; v += kThreads) {
+        float f[8];
+        Vec<T>::unpack(slice[v], f);
+#pragma unroll
+        for (int e = 0; e < VN; ++e) take(f[e], (uint32_t)(a0 + (v_begin + v) * VN + e));
+      }
+      best = warp_max_u64(best);
+      if (lane == 0) round_s[warp] = best;
+      __syncthreads();
+      best = round_s[0];
+#pragma unroll
+      for (int w = 1; w < kWarps; ++w) best = best > round_s[w] ? best : round_s[w];
+      if (tid == 0) {
+        dst_keys[q] = best;
+        arrive(1);
+      }
+      last = best;
+      __syncthreads();   // round_s is read
+    }
+  }
+  if (rank != 0) return;
+
+  // ---- rank 0: the row's top-k from the CTAs' keys
+  constexpr int kMergers = kMaxCluster * kMaxK;   // the first four warps
+  if (tid >= kMergers) return;
+  mbar_wait_cluster(keys_bar, 0u, &abort_s, dev_status);
+  const uint64_t key = all_keys[tid];
+  if (key != 0ull) {
+    int before = 0;
+    for (int c = 0; c < csize; ++c)
+      for (int j = 0; j < k; ++j) before += all_keys[c * kMaxK + j] > key ? 1 : 0;
+    if (before < k) {
+      out_idx[r * k + before] = (int32_t)(~(uint32_t)(key & 0xFFFFFFFFull));
+      out_val[r * k + before] = from_ordered((uint32_t)(key >> 32));
+    }
+  }
+  if constexpr (kVerify) {
+    // the last row of a tree to be written: this cluster verifies the tree
+    asm volatile("bar.sync 1, %0;" ::"n"(kMergers) : "memory");   // the row's entries precede its count
+    if (warp == 0) {
+      int vb = -1;
+      if (lane == 0) {
+        // release: this row's top-k before its count; acquire: the other rows' top-k (each
+        // written before its own count) before this cluster reads them
+        if ((int)atom_add_acq_rel_gpu(va.counters + row_tree, 1u) + 1 == tin.T) vb = row_tree;
+      }
+      vb = __shfl_sync(0xffffffffu, vb, 0);
+      if (vb >= 0) {
+        __shared__ vt::VerifyScratch vsc;
+        __shared__ vt::TreeVerdict verdict;
+        __syncwarp();   // lane 0's acquire precedes every lane's reads of the tree's rows
+        verify_and_write_warp(va, vb, tin, out_idx, k, vsc, verdict);
+      }
+    }
   }
 }
 
@@ -560,21 +638,6 @@ __global__ void __launch_bounds__(kThreads) topk_bf16_kernel(const __nv_bfloat16
 // their own, fed through a double buffer of the selection warps' keys, so that the stream
 // never waits for them.  Counters are cleared by the launch before this one (the step's
 // attention); slots are written before they are read within the launch.
-
-// The k-th largest of the warp's 32 order-preserving values (0 = a lane without one), or 0 when
-// fewer than k lanes hold one: one warp maximum and one ballot per distinct value, equal values
-// counted together.  Any x with k elements >= x bounds the warp's top-k from below.
-__device__ __forceinline__ uint32_t kth_largest_ord(uint32_t v, int k) {
-  int count = 0;
-  for (int s = 0; s < k; ++s) {
-    const uint32_t m = __reduce_max_sync(0xffffffffu, v);
-    if (m == 0u) return 0u;
-    count += __popc(__ballot_sync(0xffffffffu, v == m));
-    if (count >= k) return m;
-    if (v == m) v = 0u;
-  }
-  return 0u;
-}
 
 // The k-th largest of the 256 values v[0..7] of the warp's lanes (0 = none), or 0 when fewer
 // than k are nonzero: per distinct value one warp maximum and one warp sum of its copies.
@@ -900,60 +963,48 @@ cudaError_t launch_stream_km(const StreamArgs& a, int grid, const VerifyArgs& va
   return cudaLaunchKernelEx(&cfg, topk_stream_kernel<KM>, a, va);
 }
 
-template <int KM, typename T, bool kFast, bool kVerify>
-cudaError_t launch_km(const T* logits, int64_t rows, int vocab, int64_t row_stride, int k, int32_t* out_idx,
-                      float* out_val, int cluster, int32_t* dev_status, const VerifyArgs& va, cudaStream_t stream) {
-  cudaLaunchConfig_t cfg = {};
+template <int KM, typename T>
+cudaError_t launch_cluster_km(const T* logits, int64_t rows, int vocab, int64_t row_stride, int k, int32_t* out_idx,
+                              float* out_val, cudaStream_t stream) {
+  const int per_cta = (int)(16384 / sizeof(T)) * 2;   // ~32 KB of logits per CTA
+  int cluster = (vocab + per_cta - 1) / per_cta;
+  cluster = cluster < 1 ? 1 : (cluster > kMaxCluster ? kMaxCluster : cluster);
   const int64_t gy = rows < 65535 ? rows : 65535;
-  cfg.gridDim = dim3((unsigned)cluster, (unsigned)gy, 1);
-  cfg.blockDim = dim3(kThreads, 1, 1);
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[2];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = (unsigned)cluster;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // set-up overlaps the previous kernel
-  attr[1].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 2;
-  if constexpr (kFast) {
-    const int nvec = vocab / 8 + 1;
-    const int per = (nvec + cluster - 1) / cluster;
-    cfg.dynamicSmemBytes = (size_t)per * 16;
-    cudaError_t e = cudaFuncSetAttribute(topk_bf16_kernel<KM, kVerify>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         kSliceVec * 16);
-    if (e != cudaSuccess) return e;
-    return cudaLaunchKernelEx(&cfg, topk_bf16_kernel<KM, kVerify>, logits, rows, vocab, row_stride, k, out_idx,
-                              out_val, dev_status, va);
-  } else {
-    cfg.dynamicSmemBytes = 0;
-    return cudaLaunchKernelEx(&cfg, topk_cluster_kernel<KM, T>, logits, rows, vocab, row_stride, k, out_idx,
-                              out_val);
-  }
+  return launch_chained(topk_cluster_kernel<KM, T>, dim3((unsigned)cluster, (unsigned)gy, 1), dim3(kThreads), 0, stream,
+                        (unsigned)cluster, logits, rows, vocab, row_stride, k, out_idx, out_val);
+}
+template <typename T>
+cudaError_t launch_cluster(const T* logits, int64_t rows, int vocab, int64_t row_stride, int k, int32_t* out_idx,
+                           float* out_val, cudaStream_t stream) {
+  if (k <= 4) return launch_cluster_km<4>(logits, rows, vocab, row_stride, k, out_idx, out_val, stream);
+  return launch_cluster_km<16>(logits, rows, vocab, row_stride, k, out_idx, out_val, stream);
 }
 
-template <typename T, bool kFast, bool kVerify>
-cudaError_t launch_t(const T* logits, int64_t rows, int vocab, int64_t row_stride, int k, int32_t* out_idx,
-                     float* out_val, int32_t* dev_status, const VerifyArgs& va, cudaStream_t stream) {
-  int cluster;
-  if (kFast) {
-    const int nvec = vocab / 8 + 1;
-    cluster = (nvec + kSliceVec - 1) / kSliceVec;   // slices of at most 64 KB
-  } else {
-    const int per_cta = (int)(16384 / sizeof(T)) * 2;   // ~32 KB of logits per CTA
-    cluster = (vocab + per_cta - 1) / per_cta;
-  }
-  cluster = cluster < 1 ? 1 : (cluster > kMaxCluster ? kMaxCluster : cluster);
-#define PTD_TOPK_LAUNCH(KMV) \
-  return launch_km<KMV, T, kFast, kVerify>(logits, rows, vocab, row_stride, k, out_idx, out_val, cluster, dev_status, \
-                                           va, stream)
-  if (k <= 1) PTD_TOPK_LAUNCH(1);
-  if (k <= 2) PTD_TOPK_LAUNCH(2);
-  if (k <= 4) PTD_TOPK_LAUNCH(4);
-  if (k <= 8) PTD_TOPK_LAUNCH(8);
-  PTD_TOPK_LAUNCH(16);
-#undef PTD_TOPK_LAUNCH
+// CTAs per row and vectors of the largest slice.
+template <typename T>
+int rows_cluster(int vocab) {
+  const int64_t nvec = (int64_t)vocab / Vec<T>::kN + 1;
+  const int64_t c = (nvec + kTargetVec - 1) / kTargetVec;
+  return c > kMaxCluster ? kMaxCluster : (int)c;
+}
+template <typename T>
+bool rows_fit(int64_t rows, int vocab) {
+  return (int64_t)vocab / Vec<T>::kN + 1 <= (int64_t)kMaxCluster * (sizeof(T) == 2 ? kSliceVec : kSliceVecF32) &&
+         rows <= 32768ll * 65535;
+}
+
+template <typename T, bool kVerify>
+cudaError_t launch_rows(const T* logits, int64_t rows, int vocab, int64_t row_stride, int k, int32_t* out_idx,
+                        float* out_val, int32_t* dev_status, const VerifyArgs& va, cudaStream_t stream) {
+  const int cluster = rows_cluster<T>(vocab);
+  const int per = (vocab / Vec<T>::kN + cluster - 1) / cluster;   // vectors per CTA (rows off 16 bytes have one fewer)
+  const size_t smem = (size_t)(per > 0 ? per : 1) * 16;
+  const unsigned gy = (unsigned)(rows < 32768 ? rows : 32768), gz = (unsigned)((rows + gy - 1) / gy);
+  const cudaError_t e = cudaFuncSetAttribute(topk_rows_kernel<T, kVerify>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             kSliceVecF32 * 16);
+  if (e != cudaSuccess) return e;
+  return launch_chained(topk_rows_kernel<T, kVerify>, dim3((unsigned)cluster, gy, gz), dim3(kThreads), smem, stream,
+                        (unsigned)cluster, logits, rows, vocab, row_stride, k, per, out_idx, out_val, dev_status, va);
 }
 
 }  // namespace topk
@@ -995,36 +1046,31 @@ cudaError_t launch_topk_stream(const void* logits, int64_t rows, int vocab, int 
   return topk::launch_stream_km<16>(a, (int)grid, va, stream);
 }
 
-int topk_cluster_size(int vocab) {
-  const int nvec = vocab / 8 + 1;
-  int cluster = (nvec + topk::kSliceVec - 1) / topk::kSliceVec;
-  return cluster < 1 ? 1 : (cluster > topk::kMaxCluster ? topk::kMaxCluster : cluster);
-}
+int topk_slices(int vocab) { return (int)(((int64_t)vocab / 8 + topk::kSliceVec) / topk::kSliceVec); }
 
-bool topk_can_verify(bool bf16, int vocab) {
-  return bf16 && (int64_t)vocab / 8 + 1 <= (int64_t)topk::kMaxCluster * topk::kSliceVec;
-}
+bool topk_can_verify(bool bf16, int vocab) { return bf16 && topk::rows_fit<__nv_bfloat16>(1, vocab); }
 
 cudaError_t launch_topk(const void* logits, bool bf16, int64_t rows, int vocab, int64_t row_stride, int k,
                         int32_t* out_idx, float* out_val, int32_t* dev_status, const VerifyArgs* va,
                         cudaStream_t stream) {
   const VerifyArgs none = {};
   if (bf16) {
-    // the shared-memory path covers rows up to kMaxCluster slices of kSliceVec vectors
-    if (topk_can_verify(true, vocab)) {
+    const __nv_bfloat16* x = static_cast<const __nv_bfloat16*>(logits);
+    if (topk::rows_fit<__nv_bfloat16>(rows, vocab)) {
       if (va != nullptr)
-        return topk::launch_t<__nv_bfloat16, true, true>(static_cast<const __nv_bfloat16*>(logits), rows, vocab,
-                                                         row_stride, k, out_idx, out_val, dev_status, *va, stream);
-      return topk::launch_t<__nv_bfloat16, true, false>(static_cast<const __nv_bfloat16*>(logits), rows, vocab,
-                                                        row_stride, k, out_idx, out_val, dev_status, none, stream);
+        return topk::launch_rows<__nv_bfloat16, true>(x, rows, vocab, row_stride, k, out_idx, out_val, dev_status, *va,
+                                                      stream);
+      return topk::launch_rows<__nv_bfloat16, false>(x, rows, vocab, row_stride, k, out_idx, out_val, dev_status, none,
+                                                     stream);
     }
     if (va != nullptr) return cudaErrorInvalidValue;
-    return topk::launch_t<__nv_bfloat16, false, false>(static_cast<const __nv_bfloat16*>(logits), rows, vocab,
-                                                       row_stride, k, out_idx, out_val, dev_status, none, stream);
+    return topk::launch_cluster(x, rows, vocab, row_stride, k, out_idx, out_val, stream);
   }
   if (va != nullptr) return cudaErrorInvalidValue;
-  return topk::launch_t<float, false, false>(static_cast<const float*>(logits), rows, vocab, row_stride, k, out_idx,
-                                             out_val, dev_status, none, stream);
+  const float* x = static_cast<const float*>(logits);
+  if (topk::rows_fit<float>(rows, vocab))
+    return topk::launch_rows<float, false>(x, rows, vocab, row_stride, k, out_idx, out_val, dev_status, none, stream);
+  return topk::launch_cluster(x, rows, vocab, row_stride, k, out_idx, out_val, stream);
 }
 
 }  // namespace ptd

@@ -31,8 +31,8 @@ cudaError_t launch_topk_stream(const void* logits, int64_t rows, int vocab, int 
                                int32_t* dev_status, const VerifyArgs& va, unsigned int* row_counters,
                                unsigned long long* part_keys, int sms, cudaStream_t stream);
 
-// CTAs per row of the clustered bf16 top-k (one cluster per row).
-int topk_cluster_size(int vocab);
+// 64 KB slices of a row of bf16 logits.
+int topk_slices(int vocab);
 
 // Whether launch_topk can verify for these logits (bf16 rows within the clustered fast path).
 bool topk_can_verify(bool bf16, int vocab);

@@ -312,6 +312,36 @@ def test_topk_edge_cases(dtype, vocab, k):
     assert np.array_equal(val.cpu().numpy().astype(np.float64), ref_v)
 
 
+@pytest.mark.parametrize("dtype,vocab", [("bf16", 16391), ("bf16", 128256), ("bf16", 262143), ("bf16", 262144),
+                                         ("f32", 8195), ("f32", 128256), ("f32", 163839), ("f32", 163840)])
+@pytest.mark.parametrize("k", [1, 8, 9, 16])
+def test_topk_masked_and_clustered_rows(dtype, vocab, k):
+    """Rows whose best values sit together or are few (masked vocabularies), at the edges of the
+    slices and of the clustered range: every candidate in one lane's vectors, fewer finite values
+    than k, a finite run inside a masked row, the best values at a row's two ends."""
+    g = np.random.default_rng(vocab + k)
+    rows = np.full((6, vocab), -np.inf, np.float32)
+    rows[0] = np.arange(vocab) % 199 - 300.0
+    rows[0, 777:777 + 16] = 1.0 + np.arange(16) / 16.0        # two or four vectors of one lane
+    rows[1, g.integers(0, vocab, 5)] = 2.5                     # at most 5 finite values
+    rows[2, 5000:5700] = np.round(g.standard_normal(700), 2)   # a finite run
+    rows[3] = g.standard_normal(vocab)
+    rows[3, :3], rows[3, -3:] = 9.0, 9.0                       # ties across a row's ends
+    rows[4] = np.finfo(np.float32).min if dtype == "f32" else -3.0e38   # masked with the lowest value
+    rows[4, 4096] = 0.5
+    rows[5, vocab // 2:] = 7.0                                 # half a row of equal values
+    host = syn.bf16_bits(rows) if dtype == "bf16" else rows
+    wide = syn.widen(host, dtype) if dtype == "bf16" else rows.astype(np.float64)
+    t = to_torch(host, dtype).cuda()
+    idx = torch.zeros((6, k), dtype=torch.int32, device="cuda")
+    val = torch.zeros((6, k), dtype=torch.float32, device="cuda")
+    ptd.topk_draft(t, k, idx, val)
+    torch.cuda.synchronize()
+    ref_i, ref_v = oracle.topk_rows(wide, k)
+    assert np.array_equal(idx.cpu().numpy(), ref_i)
+    assert np.array_equal(val.cpu().numpy().astype(np.float64), ref_v)
+
+
 def test_topk_rejects_bad_k():
     t = torch.zeros((2, 10), dtype=torch.bfloat16, device="cuda")
     idx = torch.zeros((2, 17), dtype=torch.int32, device="cuda")
