@@ -45,6 +45,7 @@
 #include <cstdint>
 
 #include "attention.cuh"
+#include "attention_tc.cuh"
 #include "ptd_device.cuh"
 
 namespace ptd {
@@ -52,9 +53,6 @@ namespace tc {
 
 constexpr int kThreads = 320;
 constexpr int kStages = 2;                // K/V stage pairs (K tile then V tile)
-constexpr uint32_t kTileBytes = 32768;   // 128 rows x 128 bf16
-constexpr uint32_t kHalfBytes = 16384;   // 128 rows x 64 bf16 (one 128-byte swizzle column)
-constexpr uint32_t kStageBytes = 2 * kTileBytes;
 constexpr uint32_t kOffQ = 0;
 constexpr uint32_t kOffRing = 2 * kTileBytes;
 constexpr uint32_t kOffBar = kOffRing + kStages * kStageBytes;
@@ -66,26 +64,6 @@ constexpr uint32_t kOffAbort = kOffTmemPtr + 4;
 constexpr uint32_t kOffSched = (kOffAbort + 4 + 15) / 16 * 16;   // schedule constants + one slot per warp
 constexpr uint32_t kSchedBytes = 1024;
 constexpr uint32_t kOffWarp = kOffSched + kSchedBytes;   // one WarpArea per softmax warp (below)
-constexpr uint32_t kTmemCols = 512;
-constexpr float kRescaleLog2 = 8.0f;                // lazy rescale threshold (log2 units)
-
-constexpr uint32_t kIdescS = idesc_bf16_f32(128, 128, 0, 0);    // Q (K-major) x K (K-major)
-constexpr uint32_t kIdescPV = idesc_bf16_f32(128, 128, 0, 1);   // P (K-major) x V (MN-major)
-
-// Bits [a0, a0+32) of "is slot C + a visible": a < 0 is committed context (visible),
-// 0 <= a < 128 reads the node's ancestor mask, a >= 128 is past the tree.
-__device__ __forceinline__ uint32_t vis_word(int a0, uint32_t m0, uint32_t m1, uint32_t m2, uint32_t m3) {
-  if (a0 <= -32) return 0xFFFFFFFFu;
-  if (a0 < 0) {
-    const int sh = -a0;   // 1..31
-    return (m0 << sh) | ((1u << sh) - 1u);
-  }
-  if (a0 >= 128) return 0u;
-  const int w = a0 >> 5, sh = a0 & 31;
-  const uint32_t lo = w == 0 ? m0 : w == 1 ? m1 : w == 2 ? m2 : m3;
-  const uint32_t hi = w == 0 ? m1 : w == 1 ? m2 : w == 2 ? m3 : 0u;
-  return __funnelshift_r(lo, hi, sh);
-}
 
 // One segment of work: key tiles [kt_begin, kt_end) of one unit.
 struct Seg {
@@ -119,6 +97,7 @@ struct WarpArea {
 // global memory each time instead.
 struct TreeInfo {
   int node0, T, C, n_kt, pairs, wb;
+  int start;   // key tiles of the trees before it, in one layer
 };
 constexpr int kMaxCachedTrees = 256;
 constexpr uint32_t kOffTrees = kOffWarp + 8 * sizeof(WarpArea);
@@ -126,9 +105,9 @@ constexpr uint32_t kSmemUsed = kOffTrees + kMaxCachedTrees * sizeof(TreeInfo);
 constexpr uint32_t kSmemBytes = kSmemUsed + 1024;   // slack to align the base to 1024 B
 static_assert(kSmemBytes <= 232448, "shared memory budget");
 
-// Persistent schedule constants: CTA c owns global key tiles [c*W/P, (c+1)*W/P).
+// Persistent schedule constants: CTA c owns global key tiles [c*W/P, (c+1)*W/P); W = q P + rem.
 struct WalkConst {
-  int persistent, W, Wl, P, c, r0, r1;
+  int persistent, W, Wl, P, c, q, rem, r0, r1;
 };
 
 // Tree b: first node, size, context, key tiles and M-tile pairs; returns the key tiles of all
@@ -172,62 +151,115 @@ __device__ __forceinline__ void fill_seg(const AttnParams& p, Seg& s, int b, int
   s.unit = ((s.lq * p.batch + b) * p.hkv + s.hkv) * p.pairs + s.mp;
 }
 
+// floor(c W / P) without a 64-bit division (P is the CTAs of one wave, so c rem fits easily).
 __device__ __forceinline__ int range_start(const WalkConst& wc, int c) {
-  return (int)((long long)c * wc.W / wc.P);
+  return c * wc.q + (int)((unsigned)(c * wc.rem) / (unsigned)wc.P);
 }
+// The CTA whose range holds global tile g: the last c with range_start(c) <= g.
 __device__ __forceinline__ int owner_cta(const WalkConst& wc, int g) {
-  return (int)(((long long)(g + 1) * wc.P - 1) / wc.W);
+  int c = min(wc.P - 1, (int)((float)(g + 1) * (float)wc.P / (float)wc.W));
+  while (c > 0 && range_start(wc, c) > g) --c;
+  while (c + 1 < wc.P && range_start(wc, c + 1) <= g) ++c;
+  return c;
+}
+__device__ __forceinline__ void set_walk(WalkConst& wc, int Wl, int layers, int P, int c) {
+  wc.persistent = 1;
+  wc.Wl = Wl;
+  wc.W = Wl * layers;
+  wc.P = P;
+  wc.c = c;
+  wc.q = (int)((unsigned)wc.W / (unsigned)P);
+  wc.rem = wc.W - wc.q * P;
+  wc.r0 = range_start(wc, c);
+  wc.r1 = range_start(wc, c + 1);
 }
 
+// Global tile g's layer, tree, KV head and pair (warp-collective: the lanes search the trees).
 // Returns false (schedule inconsistent with the tree arrays) if g maps to no tree.
-__device__ __noinline__ bool decode_tile(const AttnParams& p, const TreeInfo* ti, int Wl, int g, Seg& s) {
-  s.lq = g / Wl;
-  int r = g - s.lq * Wl;
-  for (int b = 0; b < p.batch; ++b) {
-    int node0, T, C, n_kt, pairs;
-    const int wb = seq_info(p, ti, b, node0, T, C, n_kt, pairs);
-    if (r < wb) {
-      const int idx = r / n_kt;
-      const int tile = r - idx * n_kt;
-      s.hkv = idx / pairs;
-      s.mp = idx - s.hkv * pairs;
-      fill_seg(p, s, b, node0, T, C, n_kt);
-      s.ug0 = g - tile;
-      return true;
+__device__ __forceinline__ bool decode_tile(const AttnParams& p, const TreeInfo* ti, const WalkConst& wc, int g, Seg& s) {
+  const int lane = threadIdx.x & 31;
+  s.lq = wc.W == wc.Wl ? 0 : (int)((unsigned)g / (unsigned)wc.Wl);
+  const int r = g - s.lq * wc.Wl;
+  int b = -1, start = 0, node0, T, C, n_kt, pairs;
+  if (ti != nullptr) {
+    for (int b0 = 0; b0 < p.batch && b < 0; b0 += 32) {
+      const int q = b0 + lane;
+      const uint32_t hit =
+          __ballot_sync(0xffffffffu, q < p.batch && r >= ti[q].start && r - ti[q].start < ti[q].wb);
+      if (hit != 0u) b = b0 + __ffs(hit) - 1;
     }
-    r -= wb;
+    if (b < 0) return false;
+    start = ti[b].start;
+    seq_info(p, ti, b, node0, T, C, n_kt, pairs);
+  } else {
+    for (int q = 0; q < p.batch; ++q) {
+      const int wb = seq_info(p, nullptr, q, node0, T, C, n_kt, pairs);
+      if (r - start < wb) {
+        b = q;
+        break;
+      }
+      start += wb;
+    }
+    if (b < 0) return false;
   }
-  return false;
+  const int idx = (int)((unsigned)(r - start) / (unsigned)n_kt);
+  const int tile = r - start - idx * n_kt;
+  s.hkv = pairs == 1 ? idx : (int)((unsigned)idx / (unsigned)pairs);
+  s.mp = idx - s.hkv * pairs;
+  fill_seg(p, s, b, node0, T, C, n_kt);
+  s.ug0 = g - tile;
+  return true;
 }
 
-__device__ __noinline__ void make_walk_const(const AttnParams& p, const TreeInfo* ti, WalkConst& wc) {
-  wc.persistent = p.persistent;
-  if (!p.persistent) return;
-  int wl = 0;
-  for (int b = 0; b < p.batch; ++b) {
-    int node0, T, C, n_kt, pairs;
-    const int w = seq_info(p, ti, b, node0, T, C, n_kt, pairs);
-    if (w == 0 && blockIdx.x == 0) atomicMax(p.dev_status, (int)PTD_ERR_INVALID_TREE);   // malformed sizes
-    wl += w;
+// The schedule's constants, by warp 0 (the trees' geometry is in `ti` when there are few enough;
+// their places in the layer are added to it here).
+__device__ __forceinline__ void make_walk_const(const AttnParams& p, TreeInfo* ti, WalkConst& wc) {
+  const int lane = threadIdx.x & 31;
+  if (!p.persistent) {
+    if (lane == 0) wc.persistent = 0;
+    return;
   }
-  wc.Wl = wl;
-  wc.W = wl * p.layers;
-  wc.P = (int)gridDim.x;
-  wc.c = (int)blockIdx.x;
-  wc.r0 = range_start(wc, wc.c);
-  wc.r1 = range_start(wc, wc.c + 1);
+  int wl = 0;
+  for (int b0 = 0; b0 < p.batch; b0 += 32) {
+    const int b = b0 + lane;
+    int w = 0;
+    if (b < p.batch) {
+      int node0, T, C, n_kt, pairs;
+      w = seq_info(p, ti, b, node0, T, C, n_kt, pairs);
+      if (w == 0 && blockIdx.x == 0) atomicMax(p.dev_status, (int)PTD_ERR_INVALID_TREE);   // malformed sizes
+    }
+    int incl = w;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += y;
+    }
+    if (ti != nullptr && b < p.batch) ti[b].start = wl + incl - w;
+    wl += __shfl_sync(0xffffffffu, incl, 31);
+  }
+  if (lane == 0) set_walk(wc, wl, p.layers, (int)gridDim.x, (int)blockIdx.x);
 }
 
 // A walker's cursor before its first step (a walk's cursors lie in [0, W]).
 constexpr int kWalkStart = INT_MIN;
 
 // Next segment of this CTA for one walker (cursor starts at kWalkStart); s.valid = 0 when done.
-__device__ __noinline__ void next_segment(const AttnParams& p, const TreeInfo* ti, const WalkConst& wc, int& cursor,
-                                          Seg& s) {
-  s.valid = 0;
+// Warp-collective: every lane computes the same segment, lane 0 leaves it in *out (shared memory).
+__device__ __noinline__ bool next_segment(const AttnParams& p, const TreeInfo* ti, const WalkConst& wc, int& cursor_io,
+                                          Seg* out) {
+  Seg s;
+  int cursor = cursor_io;
+  auto done = [&](bool valid) {
+    s.valid = valid ? 1 : 0;
+    cursor_io = cursor;
+    if ((threadIdx.x & 31) == 0) {
+      if (valid) *out = s; else out->valid = 0;
+    }
+    return valid;
+  };
   if (!wc.persistent) {
     // grid schedule: CTA u computes unit u whole
-    if (cursor != kWalkStart) return;
+    if (cursor != kWalkStart) return done(false);
     cursor = 0;
     int u = blockIdx.x;
     s.mp = u % p.pairs;
@@ -239,25 +271,24 @@ __device__ __noinline__ void next_segment(const AttnParams& p, const TreeInfo* t
     int node0, T, C, n_kt, pairs;
     if (seq_info(p, ti, b, node0, T, C, n_kt, pairs) == 0) {
       atomicMax(p.dev_status, (int)PTD_ERR_INVALID_TREE);   // malformed sizes
-      return;
+      return done(false);
     }
-    if (s.mp >= pairs) return;
+    if (s.mp >= pairs) return done(false);
     fill_seg(p, s, b, node0, T, C, n_kt);
     s.ug0 = 0;
     s.kt_begin = 0;
     s.kt_end = n_kt;
     s.slot = -1;
-    s.valid = 1;
-    return;
+    return done(true);
   }
-  if (wc.W <= 0) return;
+  if (wc.W <= 0) return done(false);
   if (cursor == kWalkStart) cursor = wc.r0;
-  if (cursor >= wc.r1) return;
+  if (cursor >= wc.r1) return done(false);
   // self-check: every step must decode and move the cursor forward (the walk then ends)
-  if (!decode_tile(p, ti, wc.Wl, cursor, s) || s.ug0 + s.n_kt <= cursor || s.ug0 > cursor) {
+  if (!decode_tile(p, ti, wc, cursor, s) || s.ug0 + s.n_kt <= cursor || s.ug0 > cursor) {
     atomicMax(p.dev_status, (int)PTD_ERR_TIMEOUT);
     cursor = wc.r1;
-    return;
+    return done(false);
   }
   const int g0 = cursor;
   const int g1 = min(s.ug0 + s.n_kt, wc.r1);
@@ -269,36 +300,13 @@ __device__ __noinline__ void next_segment(const AttnParams& p, const TreeInfo* t
   } else {
     s.slot = wc.c * 2 + ((wc.r0 >= s.ug0 && wc.r0 < s.ug0 + s.n_kt) ? 0 : 1);
   }
-  s.valid = 1;
+  return done(true);
 }
 
 // Partial slot of CTA c's piece of the unit starting at global tile ug0 (c owns a piece).
 __device__ __forceinline__ int piece_slot(const WalkConst& wc, int c, int ug0, int ug1) {
   const int rs = range_start(wc, c);
   return c * 2 + ((rs >= ug0 && rs < ug1) ? 0 : 1);
-}
-
-// Rare path of the softmax, kept out of the hot loop: O_t (n_o 16-column groups) and the
-// bf16 P chunks [0, c) of S_t scaled by alpha.  Warp-collective.
-__device__ __noinline__ void rescale_tmem(uint32_t tO, uint32_t tS, int n_o, int c, float alpha) {
-  for (int q = 0; q < n_o; ++q) {
-    uint32_t o16[16];
-    tmem_ld16(tO + (uint32_t)q * 16u, o16);
-    tmem_ld_wait();
-#pragma unroll
-    for (int e = 0; e < 16; ++e) o16[e] = __float_as_uint(__uint_as_float(o16[e]) * alpha);
-    tmem_st16(tO + (uint32_t)q * 16u, o16);
-  }
-  if (c > 0) tmem_st_wait();
-  for (int q = 0; q < c; ++q) {
-    uint32_t p16[16];
-    tmem_ld16(tS + (uint32_t)q * 16u, p16);
-    tmem_ld_wait();
-#pragma unroll
-    for (int e = 0; e < 16; ++e)
-      p16[e] = pack_bf16x2(__uint_as_float(p16[e] << 16) * alpha, __uint_as_float(p16[e] & 0xFFFF0000u) * alpha);
-    tmem_st16(tS + (uint32_t)q * 16u, p16);
-  }
 }
 
 template <bool kPaged, bool kQTma>
@@ -335,9 +343,6 @@ __global__ void __launch_bounds__(kThreads, 1)
   Seg* my_seg = reinterpret_cast<Seg*>(smem + kOffSched + 64) + warp;   // this warp's schedule slot
   static_assert(64 + (kThreads / 32) * sizeof(Seg) <= kSchedBytes, "schedule area");
 
-  // A grid launched after this one with programmatic stream serialization (the step's top-k)
-  // may be scheduled now; its CTAs take the SMs this grid's CTAs leave at its end.
-  if (threadIdx.x == 0) grid_launch_dependents();
   // set-up that reads no global memory: it may overlap the stream's previous grid
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
@@ -360,6 +365,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (warp == 0 && lane == 0) {
     prefetch_tensormap(&map_k);
     prefetch_tensormap(&map_v);
+    if (kQTma) prefetch_tensormap(&map_q);
   }
   if (warp == 1) {
     tmem_alloc(base + kOffTmemPtr, kTmemCols);
@@ -368,6 +374,10 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
   // every input (trees, Q, the cache) and output belongs to the stream's previous work
   grid_dependency_wait();
+  // A grid launched after this one with programmatic stream serialization (the merge, the step's
+  // top-k) may be scheduled from here on; its CTAs take the SMs this grid's CTAs leave at its
+  // end.  (After the wait: the merge reads the trees before its own.)
+  if (threadIdx.x == 0) grid_launch_dependents();
   if (blockIdx.x == 0)   // counters of the work that follows this kernel in the step (see AttnParams)
     for (int i = threadIdx.x; i < p.zero_count; i += kThreads) p.zero_ptr[i] = 0u;
   TreeInfo* const trees_s = reinterpret_cast<TreeInfo*>(smem + kOffTrees);
@@ -375,23 +385,24 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (ti != nullptr) {
     for (int b = threadIdx.x; b < p.batch; b += kThreads) {
       TreeInfo x;
+      x.start = 0;
       x.wb = seq_info(p, nullptr, b, x.node0, x.T, x.C, x.n_kt, x.pairs);
       trees_s[b] = x;
     }
   }
   __syncthreads();
-  if (threadIdx.x == 0) make_walk_const(p, ti, *wc_s);
+  if (warp == 0) make_walk_const(p, p.batch <= kMaxCachedTrees ? trees_s : nullptr, *wc_s);
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(smem + kOffTmemPtr);
   const WalkConst& wc = *wc_s;
-  int cursor = kWalkStart;   // this warp's position in the schedule (lane 0 walks, the warp reads)
+  int cursor = kWalkStart;   // this warp's position in the schedule
   volatile Seg* sgv = my_seg;
   auto advance = [&]() -> bool {
     __syncwarp();
-    if (lane == 0) next_segment(p, ti, wc, cursor, *my_seg);
+    const bool valid = next_segment(p, ti, wc, cursor, my_seg);
     __syncwarp();
-    return sgv->valid != 0;
+    return valid;
   };
 
   if (warp == 0) {
@@ -485,24 +496,11 @@ __global__ void __launch_bounds__(kThreads, 1)
     // ================================================================ MMA issuer (one thread)
     const uint32_t q_base = base + kOffQ, ring = base + kOffRing;
     auto issue_s = [&](int tt, int st) {
-      const uint32_t d = tmem + (uint32_t)tt * 128u;
-#pragma unroll
-      for (int kk = 0; kk < 8; ++kk) {
-        const uint32_t koff = (uint32_t)(kk >> 2) * kHalfBytes + (uint32_t)(kk & 3) * 32u;
-        const uint64_t a = smem_desc_sw128(q_base + (uint32_t)tt * kTileBytes + koff, 16, 1024);
-        const uint64_t bd = smem_desc_sw128(ring + (uint32_t)st * kStageBytes + koff, 16, 1024);
-        mma_bf16_ss(d, a, bd, kIdescS, kk > 0 ? 1u : 0u);
-      }
+      tc::issue_s(tmem + (uint32_t)tt * 128u, q_base + (uint32_t)tt * kTileBytes, ring + (uint32_t)st * kStageBytes);
     };
     auto issue_pv = [&](int tt, int st, bool acc) {
-      const uint32_t d = tmem + 256u + (uint32_t)tt * 128u;
-      const uint32_t a = tmem + (uint32_t)tt * 128u;   // P: 16 keys = 8 packed columns per step
-      const uint32_t vb = ring + (uint32_t)st * kStageBytes + kTileBytes;
-#pragma unroll
-      for (int kk = 0; kk < 8; ++kk) {
-        const uint64_t bd = smem_desc_sw128(vb + (uint32_t)kk * 2048u, kHalfBytes, 1024);
-        mma_bf16_ts(d, a + (uint32_t)kk * 8u, bd, kIdescPV, (acc || kk > 0) ? 1u : 0u);
-      }
+      tc::issue_pv(tmem + 256u + (uint32_t)tt * 128u, tmem + (uint32_t)tt * 128u,
+                   ring + (uint32_t)st * kStageBytes + kTileBytes, acc);
     };
     bool ok = true;
     int gt = 0;
@@ -585,7 +583,6 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
     const uint32_t tS = tmem + lane_base + (uint32_t)t * 128u;
     const uint32_t tO = tmem + lane_base + 256u + (uint32_t)t * 128u;
-    const unsigned long long sl2x2 = f2_pack(sl2, sl2);
     const uint32_t qrow_smem = base + kOffQ + (uint32_t)t * kTileBytes + (uint32_t)row * 128u;
     WarpArea* wa = reinterpret_cast<WarpArea*>(smem + kOffWarp) + (warp - 2);
     volatile WarpArea* wv = wa;
@@ -614,7 +611,16 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int node = grow / G, g = grow - node * G;
       const bool row_valid = node < T;
       const bool has_keys = sgv->kt_end > sgv->kt_begin;
-      // Q rows first: their loads overlap the tree work below (per-thread path only)
+      // Q first: its loads overlap the tree work below
+      if (kQTma && has_keys && (warp & 3) == 0 && lane == 0) {
+        // Q tile of this segment by TMA (every S_t GEMM of the previous segment has
+        // completed): 128 / G nodes x G heads of the pair's M tile, two 64-column halves
+        const int qrow = sgv->lq * p.n_total + node0 + ((2 * mp + t) * 128) / G;
+        const uint32_t dst = base + kOffQ + (uint32_t)t * kTileBytes;
+        mbar_arrive_expect_tx(qready_bar(t), 2 * kHalfBytes);
+        tma_load_3d(dst, &map_q, qready_bar(t), 0, sgv->hkv * G, qrow);
+        tma_load_3d(dst + kHalfBytes, &map_q, qready_bar(t), 64, sgv->hkv * G, qrow);
+      }
       uint4 v[16];
       if constexpr (!kQTma) {
         const size_t orow = (((size_t)sgv->lq * p.n_total + node0 + node) * p.hq + (size_t)sgv->hkv * G + g) * 128;
@@ -662,17 +668,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (lane < kSegWords)
         reinterpret_cast<volatile int*>(&wa->run[k].s)[lane] = reinterpret_cast<const volatile int*>(sgv)[lane];
       if (lane == 0) wa->run[k].invalid = invalid ? 1 : 0;
-      if (kQTma && has_keys) {
-        // Q tile of this segment by TMA (every S_t GEMM of the previous segment has
-        // completed): 128 / G nodes x G heads of the pair's M tile, two 64-column halves
-        if ((warp & 3) == 0 && lane == 0) {
-          const int qrow = sgv->lq * p.n_total + node0 + ((2 * mp + t) * 128) / G;
-          const uint32_t dst = base + kOffQ + (uint32_t)t * kTileBytes;
-          mbar_arrive_expect_tx(qready_bar(t), 2 * kHalfBytes);
-          tma_load_3d(dst, &map_q, qready_bar(t), 0, sgv->hkv * G, qrow);
-          tma_load_3d(dst + kHalfBytes, &map_q, qready_bar(t), 64, sgv->hkv * G, qrow);
-        }
-      } else if (has_keys) {
+      if (!kQTma && has_keys) {
         // Q rows of this segment (every S_t GEMM of the previous segment has completed)
 #pragma unroll
         for (int c = 0; c < 16; ++c) {
@@ -777,75 +773,13 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int kt_begin = cur->s.kt_begin;
       const int C = cur->s.C;
       const int n = cur->s.kt_end - kt_begin;
-      // Reference max m_run (log2 units) against which P = 2^(s*scale*log2e - m_run) is
-      // taken.  It only moves up, and only when a 32-column chunk exceeds it by more than
-      // 2^8; then the row sum, O and the P chunks already written for this tile are rescaled.
       float m_run = -INFINITY, l_run = 0.f;
       for (int jj = 0; jj < n; ++jj, ++tiles) {
         if (!(ok = mbar_wait_warp(sfull_bar(t), (uint32_t)(tiles & 1), abort_flag, p.dev_status))) break;
         tc_fence_after();
         const int t0 = (kt_begin + jj) * 128;
         const bool need_mask = t0 + 128 > C;   // warp-uniform
-        unsigned long long sum = f2_pack(0.f, 0.f);
-#pragma unroll 1
-        for (int c = 0; c < 4; ++c) {
-          tmem_ld32(tS + (uint32_t)c * 32u, r);
-          tmem_ld_wait();
-          if (need_mask) {
-            const uint32_t vw = vis_word(t0 + c * 32 - C, am0, am1, am2, am3);
-#pragma unroll
-            for (int e = 0; e < 32; ++e) r[e] = ((vw >> e) & 1u) ? r[e] : __float_as_uint(-INFINITY);
-          }
-          float cm;
-          {
-            float a0 = -INFINITY, a1 = -INFINITY;
-#pragma unroll
-            for (int e = 0; e < 32; e += 4) {
-              a0 = fmax3(a0, __uint_as_float(r[e]), __uint_as_float(r[e + 1]));
-              a1 = fmax3(a1, __uint_as_float(r[e + 2]), __uint_as_float(r[e + 3]));
-            }
-            cm = fmaxf(a0, a1) * sl2;
-          }
-          // The TMEM accesses of a rescale are warp-collective, so the whole warp takes the
-          // branch when any of its rows needs it; the other rows rescale by exactly 1.  (Rows
-          // differ when a piece starts on a key tile past the committed context: each row
-          // first meets a visible ancestor in whichever chunk holds one.)
-          const bool raise = cm > m_run + kRescaleLog2;
-          if (__any_sync(0xffffffffu, raise)) {
-            // raise the reference: rescale everything taken against the old one
-            float alpha = 1.f;
-            if (raise) {
-              alpha = m_run == -INFINITY ? 0.f : ptx_exp2(m_run - cm);
-              m_run = cm;
-            }
-            float s0, s1;
-            f2_unpack(sum, s0, s1);
-            sum = f2_pack(s0 * alpha, s1 * alpha);
-            l_run *= alpha;
-            rescale_tmem(tO, tS, jj > 0 ? 8 : 0, c, alpha);
-          }
-          const float m_use = m_run == -INFINITY ? 0.f : m_run;   // -inf only while nothing is visible
-          const unsigned long long negm = f2_pack(-m_use, -m_use);
-          uint32_t pk[16];
-#pragma unroll
-          for (int e = 0; e < 32; e += 2) {
-            const unsigned long long x =
-                f2_fma(f2_pack(__uint_as_float(r[e]), __uint_as_float(r[e + 1])), sl2x2, negm);
-            float x0, x1;
-            f2_unpack(x, x0, x1);
-            const float p0 = ptx_exp2(x0), p1 = ptx_exp2(x1);
-            sum = f2_add(sum, f2_pack(p0, p1));
-            pk[e >> 1] = pack_bf16x2(p0, p1);
-          }
-          tmem_st16(tS + (uint32_t)c * 16u, pk);   // P chunk c: columns [16c, 16c+16) of S_t
-        }
-        {
-          float s0, s1;
-          f2_unpack(sum, s0, s1);
-          l_run += s0 + s1;
-        }
-        tmem_st_wait();
-        tc_fence_before();
+        softmax_tile(tS, tO, jj > 0, need_mask, t0 - C, am0, am1, am2, am3, sl2, m_run, l_run);
         __syncwarp();
         if (lane == 0) mbar_arrive(pfull_bar(t));
       }
@@ -980,7 +914,8 @@ constexpr int kMergeMl = 8;      // pieces whose (m, l) stay in registers
 
 __global__ void __launch_bounds__(kMergeThreads, 2) tree_attn_merge_kernel(const AttnParams p, int hsplit) {
   if (threadIdx.x == 0) grid_launch_dependents();   // the next grid may be placed now; it waits for this one
-  grid_dependency_wait();   // the partials and the trees belong to the attention grid before this one
+  // The unit and its pieces, while the attention still runs: the trees were complete before the
+  // attention passed its own dependency wait, after which it let this grid be placed.
   int u = blockIdx.x / hsplit;
   const int hs = blockIdx.x - u * hsplit;
   const int mp = u % p.pairs;
@@ -989,25 +924,31 @@ __global__ void __launch_bounds__(kMergeThreads, 2) tree_attn_merge_kernel(const
   u /= p.hkv;
   const int b = u % p.batch;
   const int lq = u / p.batch;
-  int node0, T, C, n_kt, pairs_b;
-  if (seq_info(p, nullptr, b, node0, T, C, n_kt, pairs_b) == 0 || mp >= pairs_b) return;
   // the flattened (unit, key tile) position of the unit, as the attention's walk decodes it
   int wl = 0, before = 0;
-  for (int bb = 0; bb < p.batch; ++bb) {
+  {
     int n0, tt, cc, nk, pr;
-    const int w = seq_info(p, nullptr, bb, n0, tt, cc, nk, pr);
-    if (bb < b) before += w;
-    wl += w;
+    for (int q = threadIdx.x & 31; q < p.batch; q += 32) {
+      const int w = seq_info(p, nullptr, q, n0, tt, cc, nk, pr);
+      wl += w;
+      before += q < b ? w : 0;
+    }
+    wl = (int)__reduce_add_sync(0xffffffffu, (unsigned)wl);
+    before = (int)__reduce_add_sync(0xffffffffu, (unsigned)before);
   }
+  int node0, T, C, n_kt, pairs_b;
+  const bool none = seq_info(p, nullptr, b, node0, T, C, n_kt, pairs_b) == 0 || mp >= pairs_b;
   WalkConst wc;
-  wc.persistent = 1;
-  wc.Wl = wl;
-  wc.W = wl * p.layers;
-  wc.P = p.ctas;
-  wc.c = 0;
-  wc.r0 = wc.r1 = 0;
-  const int ug0 = lq * wl + before + (hkv * pairs_b + mp) * n_kt, ug1 = ug0 + n_kt;
-  const int first = owner_cta(wc, ug0), last = owner_cta(wc, ug1 - 1);
+  int ug0 = 0, ug1 = 0, first = 0, last = 0;
+  if (!none) {
+    set_walk(wc, wl, p.layers, p.ctas, 0);
+    ug0 = lq * wl + before + (hkv * pairs_b + mp) * n_kt;
+    ug1 = ug0 + n_kt;
+    first = owner_cta(wc, ug0);
+    last = owner_cta(wc, ug1 - 1);
+  }
+  grid_dependency_wait();   // the partials belong to the attention grid before this one
+  if (none) return;
   if (first == last) return;   // whole: written by the attention
   const int t = threadIdx.x >> 7, row = threadIdx.x & 127;
   const int nt = min(2, (T * p.group + 127) / 128 - 2 * mp);
