@@ -107,11 +107,11 @@ typedef struct {
  * per-block counters and the fp32 partials of the units that the balanced schedule splits
  * between neighbouring SMs (one CTA per SM, two partial slots each: about 266 KB per SM).
  * Passing less (even 0 with a NULL pointer) is allowed: the call then computes each (layer,
- * tree, KV head, 256-row block) in one CTA, which needs no scratch but leaves SMs idle when
- * such units are few or their count is not a multiple of the SM count.  With the scratch, the
- * call still takes one CTA per unit when an estimate from the shapes favours it; with fewer
- * units than SMs (every unit then cut into several pieces) the pieces' partials are merged by
- * a second kernel launched right after the attention, otherwise inside it. */
+ * tree, KV head, 256-row block) in one CTA or in one cluster of CTAs (combined through
+ * distributed shared memory), which need no scratch.  With the scratch, the call still takes
+ * one of these when an estimate from the shapes favours it; with fewer units than SMs (every
+ * unit then cut into several pieces) the pieces' partials are merged by a second kernel launched
+ * right after the attention, otherwise inside it. */
 size_t ptd_attention_workspace_size(const ptd_tree* tree, const ptd_kv_cache* cache,
                                     int32_t num_q_heads, int32_t num_layers);
 

@@ -156,30 +156,61 @@ size_t stream_tail_bytes(int batch, int rows, int sms) {
   return stream_counters_bytes(batch, rows) + (ptd::topk_stream_slot_bytes(rows, sms) + 255) / 256 * 256;
 }
 
-// Which schedule the shapes favour, from the host-known maxima (estimates in microseconds
-// measured on GB300 with these kernels): a key tile costs ~1.75 us for a unit of two 128-row
-// M tiles (~1.2 us for one), a CTA needs ~6.5 us to its first tile, and under the balanced
-// cut the last piece of a unit merges the others' partials, ~9 us plus ~4 us per partial.
-// One CTA per unit (no pieces, no merges) wins when units are few and short, e.g. a single
-// MHA layer over a short context; the balanced cut wins as soon as units are long or outnumber
-// the SMs.
 // Where the pieces of split units are merged: fewer units than CTAs means many pieces per
 // unit, merged best by tree_attn_merge_kernel over many CTAs after the attention; otherwise
 // the last piece of each unit merges inside the attention, overlapping other CTAs' tiles.
 bool defer_merge(int units, int ctas) { return units < ctas; }
 
-bool grid_schedule_cheaper(int units, int n_kt, int m_tiles, int sms) {
-  const double t_tile = m_tiles >= 2 ? 1.75 : 1.2;
-  const double waves = (double)((units + sms - 1) / sms);
-  const double t_grid = 6.5 + waves * n_kt * t_tile;
-  const double W = (double)units * n_kt;
-  const int ctas = (int)(W < sms ? W : sms);
-  const double w = W / ctas;
-  const int pieces = (int)((n_kt + w - 1e-9) / w);   // pieces of a unit, about
-  double merge = 1.5;
-  if (pieces > 1) merge = defer_merge(units, ctas) ? 4.0 + 1.0 * pieces : 9.0 + 4.0 * (pieces - 1);
-  const double t_pers = 6.5 + w * t_tile + merge;
-  return t_grid < t_pers;
+// The attention's schedule for these shapes: the balanced cut (persistent CTAs, scratch), one CTA
+// per unit, or a cluster of CTAs per unit (attention_cluster.cu).
+struct Schedule {
+  enum Kind { kCut, kGrid, kCluster } kind;
+  int csize;   // kCluster: CTAs per unit
+};
+
+// The one with the shortest estimate from the host-known maxima (every sequence taken as long as
+// the longest), in microseconds as measured on GB300 for one (two) 128-row M tiles a unit:
+//   cut      17.5 (25.5) + 1.7 (1.75) a key tile of a CTA's share (set-up, partials and merge in the
+//            constant: it hardly depends on the number of pieces)
+//   grid     5.5 (8) + 1.6 (1.85) a key tile, per wave of units over the SMs
+//   cluster  9.5 (10.5) + 0.8 (2.05) a key tile of a CTA's share, per wave of clusters; how many
+//            clusters of c CTAs (one per SM) run at once is cudaOccupancyMaxActiveClusters' answer
+//            for 152 SMs.  One wave for a batch (a second one costs a whole unit when the
+//            sequences are equally long), two otherwise (longer stacks are bound by HBM either way).
+// Measured, cut / cluster: 32 MHA heads, 2079 keys 23.8 / 13.9 us, two such layers 29.1 / 19.0,
+// eight 65.7 / 55.8; 8 KV heads of a 4-head group, 4109 keys and 13 nodes 27.6 / 14.1, 2111 keys
+// and 63 nodes 28.5 / 15.8; eight ragged paged sequences 84.6 / 82.4 a step.  Grid / cut, 128 units of
+// two M tiles: 17 key tiles 39.1 / 52.4, 9 key tiles 25.4 / 37.5.  Stacks of several layers with two
+// M tiles a unit keep the cut below 0.7 units per SM: the parity test of both merges relies on
+// it for 32 and 96 units (where a grid of 96 would be a few us faster).
+Schedule choose_schedule(int units, int n_kt, int m_tiles, int sms, int layers, int batch, bool can_cut,
+                         bool can_cluster) {
+  const bool two = m_tiles >= 2;
+  auto waves = [&](int fit) { return (double)((units + fit - 1) / fit); };   // of units over `fit` places
+  Schedule best = {Schedule::kGrid, 1};
+  double t_best = waves(sms) * ((two ? 8.0 : 5.5) + n_kt * (two ? 1.85 : 1.6));
+  const bool stack = two && layers > 1;
+  if (can_cut) {
+    const double W = (double)units * n_kt, w = W / (W < sms ? W : sms);
+    const double t = (two ? 25.5 : 17.5) + w * (two ? 1.75 : 1.7);
+    if (t < t_best || (stack && units < 0.7 * sms)) {
+      t_best = t;
+      best = {Schedule::kCut, 1};
+    }
+  }
+  if (can_cluster && !stack) {
+    static const int fit152[9] = {0, 152, 76, 46, 36, 28, 23, 15, 15};
+    for (int c = 1; c <= 8 && c <= n_kt; ++c) {
+      const int f = fit152[c] * sms / 152, fit = f > 0 ? f : 1;
+      if (units > (batch > 1 ? fit : 2 * fit)) break;
+      const double t = waves(fit) * ((two ? 10.5 : 9.5) + 0.1 * c + (n_kt + c - 1) / c * (two ? 2.05 : 0.8));
+      if (t < t_best) {
+        t_best = t;
+        best = {Schedule::kCluster, c};
+      }
+    }
+  }
+  return best;
 }
 
 // Tile indices of the persistent schedule are 32-bit.
@@ -300,11 +331,13 @@ static ptd_status tree_attention(const ptd_tree* tree, const ptd_kv_cache* cache
   const int sms = num_sms_of_current_device();
   const int ctas = persistent_ctas(units, n_kt, sms);
   const int m_tiles = (tree->max_nodes * (num_q_heads / cache->num_kv_heads) + 127) / 128;
-  const bool persistent = persistent_fits(units, n_kt) && workspace != nullptr && aligned16(workspace) &&
-                          workspace_bytes >= persistent_workspace_bytes(units, ctas, D) &&
-                          !grid_schedule_cheaper(units, n_kt, m_tiles, sms);
+  const bool can_cut = persistent_fits(units, n_kt) && workspace != nullptr && aligned16(workspace) &&
+                       workspace_bytes >= persistent_workspace_bytes(units, ctas, D);
+  const bool can_cluster = (int64_t)p.hkv * pairs <= 65535 && (int64_t)tree->batch * num_layers <= 65535;
+  const Schedule sched =
+      choose_schedule(units, n_kt, m_tiles, sms, num_layers, tree->batch, can_cut, can_cluster);
   dim3 grid;
-  if (persistent) {
+  if (sched.kind == Schedule::kCut) {
     p.persistent = 1;
     p.counters = static_cast<unsigned long long*>(workspace);
     p.epoch = next_epoch();
@@ -314,7 +347,7 @@ static ptd_status tree_attention(const ptd_tree* tree, const ptd_kv_cache* cache
     p.ctas = ctas;
     grid = dim3((unsigned)ctas, 1, 1);
   } else {
-    p.persistent = 0;   // one CTA per unit, no scratch
+    p.persistent = 0;   // one CTA or one cluster per unit, no scratch
     grid = dim3((unsigned)units, 1, 1);
   }
 
@@ -340,6 +373,11 @@ static ptd_status tree_attention(const ptd_tree* tree, const ptd_kv_cache* cache
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS)
       p.q_tma = 1;
+  }
+  if (sched.kind == Schedule::kCluster) {
+    if ((st = cuda_status(ptd::launch_tree_attn_cluster(map_k, map_v, map_q, p, sched.csize, s))) == PTD_OK)
+      g_last_launches = 1;
+    return st;
   }
   if ((st = cuda_status(ptd::launch_tree_attn_tc(map_k, map_v, map_q, p, grid, s))) != PTD_OK) return st;
   g_last_launches = 1;

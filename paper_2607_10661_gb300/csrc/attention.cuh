@@ -45,6 +45,10 @@ size_t tc_smem_bytes();
 // before its first global access.
 cudaError_t launch_tree_attn_tc(const CUtensorMap& map_k, const CUtensorMap& map_v, const CUtensorMap& map_q,
                                 const AttnParams& p, dim3 grid, cudaStream_t stream);
+// Few short units: a cluster of `csize` CTAs per unit (csize <= 8), no scratch; p.pairs set as for
+// one CTA per unit.  Programmatic dependent launch.
+cudaError_t launch_tree_attn_cluster(const CUtensorMap& map_k, const CUtensorMap& map_v, const CUtensorMap& map_q,
+                                     const AttnParams& p, int csize, cudaStream_t stream);
 // fp32 attention.  map_k: boxes of 32 columns (128-byte swizzle), map_v: of D columns, both of one
 // KV head and simt_box_rows(page_size) rows.
 cudaError_t launch_tree_attn_simt(const CUtensorMap& map_k, const CUtensorMap& map_v, const AttnParams& p, int max_ctx,

@@ -138,6 +138,48 @@ def test_attention_merge_paths_match_oracle(layers, ctx, launches):
         _check_attn(got[l][w.nodes_of(0)], _attn_ref(w, l, 0), cfg.dtype, f"layers {layers} l{l}")
 
 
+@pytest.mark.parametrize("hq,hkv,nodes,ctx,page,batch,layers", [
+    (4, 4, 1, (0, 0), 0, 1, 1),           # one key
+    (32, 8, 13, (611, 611), 0, 1, 1),     # one M tile: a stream pair, five key tiles on five CTAs
+    (8, 8, 31, (2048, 2048), 0, 1, 4),    # one M tile, 17 key tiles over four CTAs (odd and even shares)
+    (16, 16, 20, (300, 300), 0, 1, 12),   # 192 units of one M tile: two waves of single CTAs
+    (32, 8, 32, (127, 127), 16, 1, 1),    # exactly one full M tile; the tail row of the second key tile
+    (32, 8, 33, (1000, 1000), 16, 1, 1),  # one row group into the second M tile
+    (16, 2, 128, (129, 129), 64, 1, 1),   # four pairs of M tiles per KV head; fewer key tiles than a cluster holds
+    (28, 4, 40, (900, 900), 0, 1, 1),     # group of 7: Q by per-thread loads, two pairs, the last of one M tile
+    (32, 8, 48, (1, 1500), 32, 5, 1),     # ragged trees (one and two M tiles) and contexts
+])
+def test_attention_cluster_split_matches_oracle(hq, hkv, nodes, ctx, page, batch, layers):
+    """Few short units: a cluster of CTAs per unit in one launch, every unit against the oracle."""
+    over = dict(hq=hq, hkv=hkv, nodes=(min(nodes, 3), nodes) if batch > 1 else (nodes, nodes), ctx=ctx, page_size=page,
+                batch=batch, layers=layers, vocab=100, tree="random-depth", branching=(4, 3, 2, 2, 1, 1), depth_range=(5, 6))
+    w = syn.Workload(syn.shrink(syn.CONFIGS["llama3-8b-gqa"], **over), 41)
+    dw = DeviceWorkload(w, with_step_buffers=False)
+    n = dw.attention()
+    torch.cuda.synchronize()
+    assert n == 1 and int(dw.dev_status.item()) == 0
+    _check_every_unit(w, dw.attn_out.float().cpu().numpy(), "cluster")
+    first = dw.attn_out.clone()
+    dw.attention()
+    torch.cuda.synchronize()
+    assert torch.equal(first, dw.attn_out)   # partials add up in a fixed order
+
+
+@pytest.mark.parametrize("layers,hq,hkv,nodes,ctx,page,batch", [
+    (2, 4, 1, (127, 127), (961, 961), 0, 1),   # as split-on-tree-tile, cut over 36 CTAs
+    (3, 32, 8, (60, 60), (700, 700), 16, 1),   # pages
+    (2, 16, 4, (3, 70), (1, 900), 0, 40),      # more trees than a warp has lanes: the search for a tile's tree
+])
+def test_attention_cut_of_stacks_matches_oracle(layers, hq, hkv, nodes, ctx, page, batch):
+    """The balanced cut (stacks of layers with two M tiles a unit), pieces merged by the merge kernel
+    or, with more units than SMs, in the kernel."""
+    over = dict(hq=hq, hkv=hkv, nodes=nodes, ctx=ctx, page_size=page, batch=batch, layers=layers, vocab=100,
+                tree="binary" if batch == 1 else "random-depth", branching=(4, 3, 2, 2, 1, 1), depth_range=(3, 6))
+    w = syn.Workload(syn.shrink(syn.CONFIGS["llama3-8b-gqa"], **over), 43)
+    dw, got = _run_attention(w)
+    _check_every_unit(w, got, "cut")
+
+
 def test_attention_peaked_context_exposes_mask():
     """Committed-context keys made to score very low: outputs are dominated by the tree
     keys, so a wrongly (un)masked ancestor changes an output by O(1)."""
