@@ -121,10 +121,10 @@ size_t ptd_attention_workspace_size(const ptd_tree* tree, const ptd_kv_cache* ca
  * counter per tree and one per node row (together rounded up to 256 bytes), then one slot of
  * 16 eight-byte keys per node row and two per SM of the current device (rounded up to 256
  * bytes).  With that much (and a bf16 cache and bf16 logits whose rows start on 16 bytes,
- * vocab a multiple of 8), a persistent top-k streams the rows back to back, one equal share
- * per CTA, and also verifies every tree (the CTA that completes a tree's last row does it);
- * a copy kernel compacts.  With the tree counters alone the clustered top-k (one cluster per
- * row) verifies instead; with less, the top-k is followed by ptd_verify_and_compact, every
+ * vocab a multiple of 8), the top-k can stream the rows' parts through single CTAs
+ * (ptd_step_topk_policy) and verifies every tree (the CTA that completes a tree's last row does
+ * it); a copy kernel compacts.  With the tree counters alone the clustered top-k (one cluster per
+ * row) verifies; with less, the top-k is followed by ptd_verify_and_compact, every
  * CTA of which verifies its tree before copying.  The scratch needs no clearing: the
  * attention kernel clears the tail's counters and tags its own with the launch.  0 for
  * invalid arguments. */
@@ -351,17 +351,19 @@ ptd_status ptd_lm_head_topk(const void* hidden, int32_t rows, int64_t hidden_str
 
 /* One whole tree-verify step on device buffers: attention over all cache layers,
  * top-k of the logits, greedy verification on top-k column 0, KV compaction.
- * Equivalent to ptd_tree_attention, ptd_topk_draft and ptd_verify_and_compact in that
- * order on `stream` (three launches, or four with the attention's merge kernel); when the
- * workspace holds ptd_step_workspace_size
- * bytes and the logits are bf16 (vocab a multiple of 8, or vocab <= 262143), the top-k's
- * CTAs verify the trees instead and the third launch only copies the accepted rows (node_offsets must then run
+ * Equivalent to ptd_tree_attention, ptd_topk_draft and ptd_verify_and_compact on `stream` (three
+ * launches, or four with the attention's merge kernel); the top-k runs beside the attention, so
+ * topk_idx, topk_val and the verification's outputs are written while that still reads its inputs
+ * and must not overlap them.  When the workspace holds the tail's counters
+ * (ptd_step_workspace_size) and the logits are bf16, the top-k's CTAs verify the trees as well and
+ * the last launch only copies the accepted rows (node_offsets must then run
  * from 0 to total_nodes without decreasing, as ptd_tree states; a tree with an empty or
  * out-of-range node range is reported as PTD_ERR_INVALID_TREE with accept_len 0, and when
  * the offsets decrease the outputs of the other trees are unspecified).  Each launch may be
- * placed on the SMs while the one before it drains (programmatic dependent launch); it reads
- * its inputs only after that one has completed, so every kernel sees the previous one's
- * writes, as stream order would give. */
+ * placed on the SMs while the one before it drains (programmatic dependent launch); the first
+ * reads its inputs only after the stream's previous work has completed, the top-k once the
+ * attention has done so, the others after the launch before them, so every kernel sees the writes
+ * it depends on, as stream order would give. */
 typedef struct {
   const void* q;               /* [L][N_tot][Hq][D]                                    */
   int32_t num_q_heads;
@@ -387,12 +389,13 @@ ptd_status ptd_tree_verify_step(const ptd_tree* tree, const ptd_kv_cache* cache,
                                 const ptd_step_args* args, void* stream);
 
 /* Which top-k the one-call step (and the steps built on it) uses when its workspace allows
- * both: AUTO streams the rows back to back for k <= 4, vocab >= 65536 and more than one wave of
+ * both: CLUSTERED gives a row to a cluster of CTAs, STREAMED gives its parts to single CTAs that
+ * merge through the workspace; AUTO streams for k <= 4, vocab >= 65536 and more than one wave of
  * 64 KB row slices (three per SM), and clusters otherwise (measured on GB300: 640 rows of 128256
- * logits stream faster; fewer rows, larger k and shorter rows run faster clustered); CLUSTERED
- * and STREAMED force one where it applies (streaming needs vocab a multiple of 8 and 16-byte
- * aligned rows; clustering needs vocab <= 262143).  Process-wide; returns the previous policy,
- * or -1 (nothing changed) for an unknown value.  Results are identical either way. */
+ * logits stream faster, 128 rows of 152064 with k = 6 run faster clustered).  CLUSTERED and
+ * STREAMED force one where it applies (streaming needs vocab a multiple of 8 and 16-byte
+ * aligned rows).  Process-wide; returns the previous policy, or -1 (nothing changed) for an
+ * unknown value.  Results are identical either way. */
 typedef enum { PTD_STEP_TOPK_AUTO = 0, PTD_STEP_TOPK_CLUSTERED = 1, PTD_STEP_TOPK_STREAMED = 2 } ptd_step_topk;
 int32_t ptd_step_topk_policy(int32_t policy);
 

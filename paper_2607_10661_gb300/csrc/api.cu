@@ -266,11 +266,14 @@ size_t ptd_step_workspace_size(const ptd_tree* tree, const ptd_kv_cache* cache, 
 }
 
 // ptd_tree_attention, and besides: the tensor-core kernel's CTA 0 clears zero_count words at
-// zero_ptr after its dependency wait (the step's tail counters).
+// zero_ptr after its dependency wait (the step's tail counters), and `beside` launches what runs
+// beside the attention kernel (after it in the stream, before its merge kernel).
+extern "C++" {
+template <typename F>
 static ptd_status tree_attention(const ptd_tree* tree, const ptd_kv_cache* cache, int32_t layer_begin,
                                  int32_t num_layers, const void* q, int32_t num_q_heads, float scale, void* out,
                                  void* workspace, size_t workspace_bytes, int32_t* dev_status, unsigned int* zero_ptr,
-                                 int zero_count, void* stream) {
+                                 int zero_count, void* stream, F&& beside) {
   g_last_launches = 0;
   ptd_status st = check_tree(tree);
   if (st != PTD_OK) return st;
@@ -319,6 +322,7 @@ static ptd_status tree_attention(const ptd_tree* tree, const ptd_kv_cache* cache
       return PTD_ERR_CUDA;
     st = cuda_status(
         ptd::launch_tree_attn_simt(map_k, map_v, p, tree->max_ctx, num_sms_of_current_device(), s));
+    if (st == PTD_OK) st = beside();
     if (st == PTD_OK) g_last_launches = 1;
     return st;
   }
@@ -375,11 +379,13 @@ static ptd_status tree_attention(const ptd_tree* tree, const ptd_kv_cache* cache
       p.q_tma = 1;
   }
   if (sched.kind == Schedule::kCluster) {
-    if ((st = cuda_status(ptd::launch_tree_attn_cluster(map_k, map_v, map_q, p, sched.csize, s))) == PTD_OK)
-      g_last_launches = 1;
+    st = cuda_status(ptd::launch_tree_attn_cluster(map_k, map_v, map_q, p, sched.csize, s));
+    if (st == PTD_OK) st = beside();
+    if (st == PTD_OK) g_last_launches = 1;
     return st;
   }
   if ((st = cuda_status(ptd::launch_tree_attn_tc(map_k, map_v, map_q, p, grid, s))) != PTD_OK) return st;
+  if ((st = beside()) != PTD_OK) return st;
   g_last_launches = 1;
   if (p.persistent && p.defer_merge) {
     if ((st = cuda_status(ptd::launch_tree_attn_merge(p, units, sms, s))) != PTD_OK) return st;
@@ -387,12 +393,13 @@ static ptd_status tree_attention(const ptd_tree* tree, const ptd_kv_cache* cache
   }
   return PTD_OK;
 }
+}  // extern "C++"
 
 ptd_status ptd_tree_attention(const ptd_tree* tree, const ptd_kv_cache* cache, int32_t layer_begin,
                               int32_t num_layers, const void* q, int32_t num_q_heads, float scale, void* out,
                               void* workspace, size_t workspace_bytes, int32_t* dev_status, void* stream) {
   return tree_attention(tree, cache, layer_begin, num_layers, q, num_q_heads, scale, out, workspace, workspace_bytes,
-                        dev_status, nullptr, 0, stream);
+                        dev_status, nullptr, 0, stream, [] { return PTD_OK; });
 }
 
 // Host checks of ptd_topk_draft's arguments (no launch).
@@ -407,20 +414,20 @@ static ptd_status check_topk_args(const void* logits, ptd_dtype dtype, int64_t r
 }
 
 static ptd_status topk_draft(const void* logits, ptd_dtype dtype, int64_t rows, int32_t vocab, int64_t row_stride,
-                             int32_t k, int32_t* out_idx, float* out_val, void* stream) {
+                             int32_t k, bool beside, int32_t* out_idx, float* out_val, void* stream) {
   g_last_launches = 0;
   ptd_status st0 = check_topk_args(logits, dtype, rows, vocab, row_stride, k, out_idx, out_val);
   if (st0 != PTD_OK) return st0;
-  const ptd_status st = cuda_status(ptd::launch_topk(logits, dtype == PTD_BF16, rows, vocab, row_stride, k, out_idx,
-                                                     out_val, nullptr, nullptr,
-                                                     static_cast<cudaStream_t>(stream)));
+  const ptd_status st =
+      cuda_status(ptd::launch_topk(logits, dtype == PTD_BF16, rows, vocab, row_stride, k, beside, out_idx, out_val,
+                                   nullptr, nullptr, num_sms_of_current_device(), static_cast<cudaStream_t>(stream)));
   if (st == PTD_OK) g_last_launches = 1;
   return st;
 }
 
 ptd_status ptd_topk_draft(const void* logits, ptd_dtype dtype, int64_t rows, int32_t vocab, int64_t row_stride,
                           int32_t k, int32_t* out_idx, float* out_val, void* stream) {
-  return topk_draft(logits, dtype, rows, vocab, row_stride, k, out_idx, out_val, stream);
+  return topk_draft(logits, dtype, rows, vocab, row_stride, k, false, out_idx, out_val, stream);
 }
 
 ptd_status ptd_verify_greedy(const ptd_tree* tree, const int32_t* tokens, const int32_t* target,
@@ -670,10 +677,10 @@ constexpr int kTailSeparate = 0, kTailClustered = 1, kTailStreamed = 2;
 // 16-byte vectors and the whole tail of ptd_step_workspace_size; the clustered one only the
 // per-tree counters; both need the tensor-core attention (which clears the counters) and bf16
 // logits.  With both possible the policy decides.  Auto streams rows of 64K logits and more, k
-// <= 4, when they are more than one wave of 64 KB slices: 640 rows of 128256 k = 1 75.9 -> 67.3
-// us a step, k = 4 79.9 -> 75.2, 266 rows 89.4 / 89.7; elsewhere the clustered form is faster
-// (clustered / streamed: 250 rows k = 8 84.1 / 89.0, 128 rows of 152064 k = 6 150.4 / 153.3, 640
-// rows of 32000 43.5 / 49.4 and of 1000 29.9 / 73.8, one wave of 63 rows 68.5 / 72.4).
+// <= 4 (a row's slots then hold four parts), when they are more than one wave of 64 KB slices
+// (clustered / streamed, us a step: 640 rows of 128256, k = 4 69.0 / 65.1, 322 rows 57.1 / 56.2);
+// with fewer parts a row streaming loses (128 rows of 152064, k = 6 142.3 / 149.9), elsewhere the
+// two are about even (640 rows of 32000 38.6 / 37.3, of 1000 24.5 / 24.6; 63 rows of 128256 31.0 / 30.0).
 int step_tail(const ptd_tree* tree, const ptd_kv_cache* cache, const ptd_step_args* a, size_t* attn_ws_out,
               int* sms_out) {
   const size_t attn_ws = (ptd_attention_workspace_size(tree, cache, a->num_q_heads, cache->num_layers) + 255) /
@@ -685,8 +692,7 @@ int step_tail(const ptd_tree* tree, const ptd_kv_cache* cache, const ptd_step_ar
                        aligned16(a->workspace);
   const bool can_stream = tail_ok && ptd::topk_stream_ok(a->logits, a->vocab) &&
                           a->workspace_bytes >= attn_ws + stream_tail_bytes(tree->batch, tree->total_nodes, sms);
-  const bool can_cluster = tail_ok && ptd::topk_can_verify(true, a->vocab) &&
-                           a->workspace_bytes >= attn_ws + tail_counters_bytes(tree->batch);
+  const bool can_cluster = tail_ok && a->workspace_bytes >= attn_ws + tail_counters_bytes(tree->batch);
   if (can_stream && can_cluster) {
     const int policy = g_step_topk.load();
     const int64_t cluster_ctas = (int64_t)tree->total_nodes * ptd::topk_slices(a->vocab);
@@ -724,13 +730,14 @@ ptd_status ptd_tree_verify_step(const ptd_tree* tree, const ptd_kv_cache* cache,
   if ((st = check_topk_args(a->logits, a->logits_dtype, tree->total_nodes, a->vocab, a->vocab, a->k, a->topk_idx,
                             a->topk_val)) != PTD_OK)
     return st;
-  // The tail: with room for its counters after the attention's scratch (the size given by
-  // ptd_step_workspace_size), the tensor-core attention (which clears those counters) and bf16
-  // logits on the clustered path, the top-k kernel also verifies every tree (the cluster that
-  // writes a tree's last row does it) and a copy kernel compacts.  Otherwise the top-k, then
-  // verification + compaction in one launch.  Each launch may be placed while the previous one
-  // drains; it reads its inputs only after that one has completed (the top-k's logits come from
-  // the step's forward pass).
+  // The top-k is launched right behind the attention kernel and runs beside it: its logits come
+  // from the step's forward pass, so it starts on them as soon as the attention lets it be
+  // placed, in what the attention leaves free of each SM.  With room for the tail's counters
+  // after the attention's scratch (the size given by ptd_step_workspace_size), the tensor-core
+  // attention (which clears those counters) and bf16 logits, the top-k also verifies every tree
+  // (whoever writes a tree's last row does it) and a copy kernel compacts.  Otherwise verification +
+  // compaction in one launch.  The top-k completes after the attention, and each later launch
+  // waits for the one before it, so the kernels after it see everything.
   size_t attn_ws = 0;
   int sms = 0;
   const int tail = step_tail(tree, cache, a, &attn_ws, &sms);
@@ -739,54 +746,49 @@ ptd_status ptd_tree_verify_step(const ptd_tree* tree, const ptd_kv_cache* cache,
   unsigned int* tail_counters =
       fused ? reinterpret_cast<unsigned int*>(static_cast<uint8_t*>(a->workspace) + attn_ws) : nullptr;
   const int zero_count = streamed ? tree->batch + tree->total_nodes : tree->batch;
-  int total = 0;
-  st = tree_attention(tree, cache, 0, cache->num_layers, a->q, a->num_q_heads, a->scale, a->attn_out, a->workspace,
-                      a->workspace_bytes, a->dev_status, tail_counters, zero_count, stream);
-  if (st != PTD_OK) return st;
-  total += g_last_launches;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  if (fused) {
-    ptd::VerifyArgs va = {};
-    va.node_offsets = tree->node_offsets;
-    va.parents = tree->parents;
-    va.tokens = a->tokens;
-    va.ctx_lens = tree->ctx_lens;
-    va.counters = tail_counters;
-    va.batch = tree->batch;
-    va.n_total = tree->total_nodes;
-    va.max_nodes = tree->max_nodes;
-    va.accepted = a->accepted_nodes;
-    va.accept_len = a->accept_len;
-    va.bonus = a->bonus_token;
-    va.dev_status = a->dev_status;
+  ptd::VerifyArgs va = {};
+  va.node_offsets = tree->node_offsets;
+  va.parents = tree->parents;
+  va.tokens = a->tokens;
+  va.ctx_lens = tree->ctx_lens;
+  va.counters = tail_counters;
+  va.batch = tree->batch;
+  va.n_total = tree->total_nodes;
+  va.max_nodes = tree->max_nodes;
+  va.accepted = a->accepted_nodes;
+  va.accept_len = a->accept_len;
+  va.bonus = a->bonus_token;
+  va.dev_status = a->dev_status;
+  auto launch_beside = [&]() -> ptd_status {
     if (streamed) {
       unsigned long long* slots = reinterpret_cast<unsigned long long*>(
           static_cast<uint8_t*>(a->workspace) + attn_ws + stream_counters_bytes(tree->batch, tree->total_nodes));
-      st = cuda_status(ptd::launch_topk_stream(a->logits, tree->total_nodes, a->vocab, a->k, a->topk_idx, a->topk_val,
-                                               a->dev_status, va, tail_counters + tree->batch, slots, sms, s));
-    } else {
-      st = cuda_status(ptd::launch_topk(a->logits, true, tree->total_nodes, a->vocab, a->vocab, a->k, a->topk_idx,
-                                        a->topk_val, a->dev_status, &va, s));
+      return cuda_status(ptd::launch_topk_stream(a->logits, tree->total_nodes, a->vocab, a->k, true, a->topk_idx,
+                                                 a->topk_val, a->dev_status, va, tail_counters + tree->batch, slots, s));
     }
-    if (st != PTD_OK) return st;
+    if (fused)
+      return cuda_status(ptd::launch_topk(a->logits, true, tree->total_nodes, a->vocab, a->vocab, a->k, true, a->topk_idx,
+                                          a->topk_val, a->dev_status, &va, sms, s));
+    return topk_draft(a->logits, a->logits_dtype, tree->total_nodes, a->vocab, a->vocab, a->k, true, a->topk_idx,
+                      a->topk_val, stream);
+  };
+  st = tree_attention(tree, cache, 0, cache->num_layers, a->q, a->num_q_heads, a->scale, a->attn_out, a->workspace,
+                      a->workspace_bytes, a->dev_status, tail_counters, zero_count, stream, launch_beside);
+  if (st != PTD_OK) return st;
+  const int total = g_last_launches + 1;   // the attention's and the top-k
+  if (fused) {
     const int row_bytes = cache->num_kv_heads * cache->head_dim * (int)dtype_size(cache->dtype);
-    if ((st = cuda_status(ptd::launch_compact(cache->k, cache->v, row_bytes, cache->num_layers, tree->batch,
-                                              cache->page_size, cache->seq_capacity, cache->num_pages,
-                                              cache->block_table, cache->max_pages, tree->ctx_lens, a->accepted_nodes,
-                                              a->accept_len, tree->max_nodes, a->new_ctx_lens, s))) != PTD_OK)
-      return st;
-    g_last_launches = total + 2;
-    return PTD_OK;
+    st = cuda_status(ptd::launch_compact(cache->k, cache->v, row_bytes, cache->num_layers, tree->batch, cache->page_size,
+                                         cache->seq_capacity, cache->num_pages, cache->block_table, cache->max_pages,
+                                         tree->ctx_lens, a->accepted_nodes, a->accept_len, tree->max_nodes,
+                                         a->new_ctx_lens, s));
+  } else {
+    st = verify_and_compact(tree, cache, a->tokens, a->topk_idx, a->k, a->accepted_nodes, a->accept_len, a->bonus_token,
+                            a->new_ctx_lens, a->dev_status, stream);
   }
-  st = topk_draft(a->logits, a->logits_dtype, tree->total_nodes, a->vocab, a->vocab, a->k, a->topk_idx,
-                  a->topk_val, stream);
   if (st != PTD_OK) return st;
-  total += g_last_launches;
-  st = verify_and_compact(tree, cache, a->tokens, a->topk_idx, a->k, a->accepted_nodes, a->accept_len,
-                          a->bonus_token, a->new_ctx_lens, a->dev_status, stream);
-  if (st != PTD_OK) return st;
-  total += g_last_launches;
-  g_last_launches = total;
+  g_last_launches = total + 1;
   return PTD_OK;
 }
 

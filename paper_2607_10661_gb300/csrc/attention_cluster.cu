@@ -109,9 +109,10 @@ __global__ void __launch_bounds__(kThreads, 1)
   tc_fence_after();
   const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(smem + kOffTmemPtr);
   grid_dependency_wait();   // every input (trees, Q, the cache) and output belongs to the stream's previous work
-  if (tid == 0) grid_launch_dependents();   // the next grid may be placed as this one's CTAs leave; it waits for all
-  if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0)   // counters of the step's tail (see AttnParams)
+  if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0) {   // counters of the step's tail (see AttnParams)
     for (int i = tid; i < p.zero_count; i += kThreads) p.zero_ptr[i] = 0u;
+    __threadfence();
+  }
 
   // ---- this CTA's share (every CTA of the cluster decides alike on its unit)
   const int rank = (int)blockIdx.x, csize = (int)gridDim.x;
@@ -197,6 +198,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     bad_par = tid == 0 ? (pp != -1) : (pp < 0 || pp >= tid);
   }
   const bool invalid = __syncthreads_or(bad_par) != 0;
+  // the grids after this one may be placed from here on (as in attention_tc.cu)
+  if (tid == 0) grid_launch_dependents();
   if (invalid && rank == 0 && tid == 0) atomicMax(p.dev_status, (int)PTD_ERR_INVALID_TREE);
 
   float m_run = -INFINITY, l_run = 0.f;

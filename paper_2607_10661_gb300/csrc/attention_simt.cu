@@ -193,9 +193,11 @@ __global__ void __launch_bounds__(kThreads, 2)
     fence_mbar_init();
     prefetch_tensormap(&map_k);
     prefetch_tensormap(&map_v);
-    grid_launch_dependents();   // the next grid may be placed now; it waits for this one
   }
   grid_dependency_wait();   // the trees, Q, the cache and the output belong to the stream's previous work
+  // the next grid may be placed now (not before the wait: the step's top-k starts on its logits
+  // beside this kernel)
+  if (tid == 0) grid_launch_dependents();
   // ---- the tree (every CTA of the cluster decides alike, so all of them leave here or none)
   const int node0 = p.node_offsets[b];
   const int T = p.node_offsets[b + 1] - node0;

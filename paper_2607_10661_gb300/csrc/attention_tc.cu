@@ -374,12 +374,10 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
   // every input (trees, Q, the cache) and output belongs to the stream's previous work
   grid_dependency_wait();
-  // A grid launched after this one with programmatic stream serialization (the merge, the step's
-  // top-k) may be scheduled from here on; its CTAs take the SMs this grid's CTAs leave at its
-  // end.  (After the wait: the merge reads the trees before its own.)
-  if (threadIdx.x == 0) grid_launch_dependents();
-  if (blockIdx.x == 0)   // counters of the work that follows this kernel in the step (see AttnParams)
+  if (blockIdx.x == 0) {   // counters of the work beside and after this kernel in the step (see AttnParams)
     for (int i = threadIdx.x; i < p.zero_count; i += kThreads) p.zero_ptr[i] = 0u;
+    __threadfence();
+  }
   TreeInfo* const trees_s = reinterpret_cast<TreeInfo*>(smem + kOffTrees);
   const TreeInfo* const ti = p.batch <= kMaxCachedTrees ? trees_s : nullptr;
   if (ti != nullptr) {
@@ -391,6 +389,11 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
   }
   __syncthreads();
+  // Grids launched after this one with programmatic stream serialization may be placed from here
+  // on: the step's top-k runs beside this kernel (after the clearing above), the merge finds its
+  // units, others take the SMs this grid's CTAs leave.  (Not before the wait: both read the
+  // trees, the top-k the logits, before any wait of their own.)
+  if (threadIdx.x == 0) grid_launch_dependents();
   if (warp == 0) make_walk_const(p, p.batch <= kMaxCachedTrees ? trees_s : nullptr, *wc_s);
   __syncthreads();
   tc_fence_after();

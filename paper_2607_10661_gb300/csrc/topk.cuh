@@ -21,28 +21,30 @@ struct VerifyArgs {
   int32_t* dev_status;
 };
 
-// The step's streaming top-k with verification (bf16 rows back to back, vocab a multiple of 8,
-// logits 16-byte aligned): a persistent grid of at most 2 * sms CTAs, each over an equal share
-// of the rows' bytes.  row_counters [rows] (and va.counters) must be zero before the launch;
-// part_keys holds topk_stream_slot_bytes(rows, sms) bytes of scratch (no clearing needed).
+// `beside` (below): the kernel's CTAs start on the logits at once, beside the stream's previous grid,
+// instead of waiting for it.  For a previous grid that lets its successors be placed only after
+// its own dependency wait, and inputs that were complete before that grid began; the outputs are
+// written while it runs.  The kernel completes after that grid has.
+
+// The step's streamed top-k with verification (bf16 rows back to back, vocab a multiple of 8,
+// logits 16-byte aligned): parts of the rows without clusters, merged through scratch.
+// row_counters [rows] (and va.counters) must be zero before the launch; slots holds
+// topk_stream_slot_bytes(rows, sms) bytes of scratch (no clearing needed).
 bool topk_stream_ok(const void* logits, int vocab);
 size_t topk_stream_slot_bytes(int64_t rows, int sms);
-cudaError_t launch_topk_stream(const void* logits, int64_t rows, int vocab, int k, int32_t* out_idx, float* out_val,
-                               int32_t* dev_status, const VerifyArgs& va, unsigned int* row_counters,
-                               unsigned long long* part_keys, int sms, cudaStream_t stream);
+cudaError_t launch_topk_stream(const void* logits, int64_t rows, int vocab, int k, bool beside, int32_t* out_idx,
+                               float* out_val, int32_t* dev_status, const VerifyArgs& va, unsigned int* row_counters,
+                               unsigned long long* slots, cudaStream_t stream);
 
 // 64 KB slices of a row of bf16 logits.
 int topk_slices(int vocab);
 
-// Whether launch_topk can verify for these logits (bf16 rows within the clustered fast path).
-bool topk_can_verify(bool bf16, int vocab);
-
-// Launched with programmatic stream serialization: the kernel waits for the stream's previous
-// grid before its first global access and lets the next grid be placed early.  With `va`
-// (bf16 fast path only) it also verifies every tree, as ptd_verify_greedy on its column 0 would;
-// the node_offsets / parents / tokens it reads must have been complete before the stream's
-// previous grid began.
-cudaError_t launch_topk(const void* logits, bool bf16, int64_t rows, int vocab, int64_t row_stride, int k,
-                        int32_t* out_idx, float* out_val, int32_t* dev_status, const VerifyArgs* va,
+// Launched with programmatic stream serialization; without `beside` the kernel waits for the
+// stream's previous grid before its first global access, and it lets the next grid be placed
+// early.  With `va` (bf16 only) it also verifies every tree, as ptd_verify_greedy on its column 0
+// would; the node_offsets / parents / tokens it reads must have been complete before the
+// stream's previous grid began.
+cudaError_t launch_topk(const void* logits, bool bf16, int64_t rows, int vocab, int64_t row_stride, int k, bool beside,
+                        int32_t* out_idx, float* out_val, int32_t* dev_status, const VerifyArgs* va, int sms,
                         cudaStream_t stream);
 }  // namespace ptd
