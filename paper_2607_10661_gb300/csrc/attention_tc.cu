@@ -859,6 +859,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (done) {
           __threadfence();
           merge(cur, true, have_o ? m_run : -INFINITY, have_o ? l_run : 0.f);
+          // the unit's pieces have all counted: back to zero, for a replay of this launch (a captured
+          // graph) carries the same epoch
+          if (lane == 0) *counter = 0ull;
         } else {
           float4* po = reinterpret_cast<float4*>(p.part_o + ((size_t)slot * 2 + t) * (128 * 128)) + row;
 #pragma unroll 1
@@ -888,6 +891,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           if (is_last) {
             __threadfence();
             merge(cur, false, 0.f, 0.f);
+            if (lane == 0) *counter = 0ull;
           }
         }
       }

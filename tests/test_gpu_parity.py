@@ -278,6 +278,62 @@ def test_attention_full_size_batched_paged_every_unit():
     _check_every_unit(w, got, "paged")
 
 
+def test_attention_graph_replay_with_new_inputs():
+    """One captured attention launch replayed on changed inputs: the in-kernel merge of split units
+    (more units than SMs) must not take the counts that the previous replay left for its own."""
+    w = syn.Workload(syn.shrink(syn.CONFIGS["llama3-8b-gqa"], layers=20, ctx=(1000, 1000), vocab=100), 29)
+    dw = DeviceWorkload(w, with_step_buffers=False)
+    dw.attention()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        dw.attention(stream=torch.cuda.current_stream())
+    for _ in range(4):
+        for _ in range(3):   # replay after replay: the counts between them are the graph's own
+            dw.v.copy_(dw.v.roll(1, 0))
+            dw.q.copy_(dw.q.roll(1, 1))
+            dw.attn_out.zero_()
+            graph.replay()
+        got = dw.attn_out.clone()
+        dw.attention()
+        torch.cuda.synchronize()
+        assert torch.equal(got, dw.attn_out)
+    assert int(dw.dev_status.item()) == 0
+
+
+def test_step_graph_replay_with_new_inputs():
+    """One captured step replayed on changed inputs equals the step called directly (its top-k runs
+    beside the attention and counts rows in the step's scratch)."""
+    for over in (dict(layers=20, ctx=(700, 700), vocab=3000), dict(layers=1, ctx=(900, 900), vocab=70000, batch=6)):
+        cfg = syn.shrink(syn.CONFIGS["llama3-8b-gqa"], **over)
+        w = syn.Workload(cfg, 33)
+        dw = DeviceWorkload(w)
+        dw.step()
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            ptd.tree_verify_step(dw.tree, dw.cache, dw.bufs, torch.cuda.current_stream())
+        names = ("attn_out", "topk_idx", "topk_val", "accepted", "accept_len", "bonus", "new_ctx")
+        for i in range(3):
+            dw.logits.copy_(dw.logits.roll(i + 1, 1))
+            dw.tokens.add_(i + 1).remainder_(cfg.vocab)
+            dw.q.copy_(dw.q.flip(1))
+            k0, v0 = dw.k.clone(), dw.v.clone()
+            for _ in range(2):   # replay after replay
+                dw.k.copy_(k0), dw.v.copy_(v0)
+                for n in names:
+                    getattr(dw, n).fill_(0)
+                graph.replay()
+            got = {n: getattr(dw, n).clone() for n in names}
+            got["k"], got["v"] = dw.k.clone(), dw.v.clone()
+            dw.k.copy_(k0), dw.v.copy_(v0)
+            dw.step()
+            torch.cuda.synchronize()
+            for n, x in got.items():
+                assert torch.equal(x, getattr(dw, n)), (over, i, n)
+        assert int(dw.dev_status.item()) == 0
+
+
 def test_attention_is_bit_reproducible():
     """Two launches on the same inputs write the same bits: the merge of a unit's pieces runs
     in a fixed order whatever piece finishes last."""
