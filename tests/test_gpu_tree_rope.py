@@ -112,3 +112,38 @@ def test_layer_range_in_one_launch():
     torch.cuda.synchronize()
     assert torch.equal(qa, qb) and torch.equal(dws[0].k, dws[1].k) and torch.equal(dws[0].v, dws[1].v)
     assert int(dws[0].dev_status.item()) == 0 and int(dws[1].dev_status.item()) == 0
+
+
+@pytest.mark.parametrize("dtype,hq,hkv,d,layers,nodes,batch", [
+    ("f32", 64, 16, 128, 2, 5, 1),     # more items a layer than a CTA takes at once
+    ("bf16", 4, 1, 32, 7, 3, 1),       # all layers in one CTA, a remainder of its items
+    ("bf16", 8, 2, 48, 5, 31, 1),      # three vectors a half row
+    ("bf16", 6, 2, 40, 3, 9, 1),       # rows that are no 16-byte vectors: element by element
+    ("bf16", 32, 8, 128, 3, 20, 40),   # more trees than a warp has lanes
+])
+def test_rope_items_match_oracle(dtype, hq, hkv, d, layers, nodes, batch):
+    """The items of a CTA at their edges, every layer of one call, against the oracle."""
+    over = dict(dtype=dtype, hq=hq, hkv=hkv, d=d, layers=layers, nodes=(min(2, nodes), nodes) if batch > 1 else (nodes, nodes),
+                batch=batch, ctx=(17, 60), vocab=50, tree="random-depth", branching=(3, 2, 2, 1), depth_range=(2, 4))
+    w = syn.Workload(syn.shrink(syn.CONFIGS["llama3-8b-gqa"], **over), 71)
+    dw = DeviceWorkload(w, with_step_buffers=False)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(72)
+    q, k, v = (torch.randn((layers, w.n_total, h, d), generator=g, device="cuda").to(dw.tdtype) for h in (hq, hkv, hkv))
+    q0, kb, vb = q.float().cpu().numpy(), dw.k.cpu(), dw.v.cpu()
+    assert ptd.tree_rope_append(dw.tree, dw.cache, 0, q, hq, k, v, 10000.0, dw.dev_status) == 1
+    torch.cuda.synchronize()
+    assert int(dw.dev_status.item()) == 0
+    pos = np.concatenate([oracle.tree_positions(w.trees[b], int(w.ctx_lens[b])) for b in range(batch)])
+    kc, vc = dw.k.cpu(), dw.v.cpu()
+    written = torch.zeros(kc.shape[:-2], dtype=torch.bool)
+    for l in range(layers):
+        _close(q[l].float().cpu().numpy(), oracle.rope(q0[l], pos, 10000.0), dtype)
+        k_rot = oracle.rope(k[l].float().cpu().numpy(), pos, 10000.0)
+        for b in range(batch):
+            sl, C = w.nodes_of(b), int(w.ctx_lens[b])
+            o, i = (x[C:] for x in w.slot_rows(b))
+            _close(kc[l, o, i].float().numpy(), k_rot[sl], dtype)
+            assert torch.equal(vc[l, o, i], v[l, sl].cpu())
+            written[l, o, i] = True
+    assert torch.equal(kc[~written], kb[~written]) and torch.equal(vc[~written], vb[~written])
