@@ -7,7 +7,9 @@
 // merge them: for a layer of a few us of work these took most of the time (32 MHA heads, 2048 + 31
 // keys: of 25 us, 5.5 us were key tiles; 26.9 -> 14.0 us here).  Here a CTA's work follows from its block index, the
 // first copies start as soon as the tree's sizes are read, and the merge is two cluster
-// barriers and one pass over shared memory (no scratch).
+// barriers and one pass over shared memory (no scratch): the partials go to shared memory as they are,
+// and a warp per row weighs and adds them (with the weights applied before, three barriers and 1-2
+// us more).
 //
 // Units of one M tile run their key tiles as two streams: softmax warps 2-5 take the even tiles
 // and warps 6-9 the odd ones, each with S, O, maximum and sum of its own (the TMEM that a second M
@@ -24,6 +26,7 @@
 
 #include <cmath>
 #include <cstdint>
+#include <type_traits>
 
 #include "attention.cuh"
 #include "attention_tc.cuh"
@@ -54,8 +57,10 @@ constexpr uint32_t kOffAbort = kOffTmemPtr + 4;
 constexpr uint32_t kSmemBytes = kOffAbort + 16 + 1024;   // slack to align the base to 1024 B
 static_assert(kSmemBytes <= 232448 && kStages * kStageBytes >= 2 * 128 * 128 * 4, "shared memory");
 
+// (A bound of 512 threads keeps the kernel at 128 registers: two CTAs of the step's top-k then fit
+// beside each of its CTAs.)
 template <bool kPaged, bool kQTma>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(512, 1)
     tree_attn_cluster_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
                              const __grid_constant__ CUtensorMap map_q, const __grid_constant__ AttnParams p) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -375,84 +380,93 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     if (todo > 0 && ok) ok = mbar_wait_warp(ofull_bar(t), 0u, abort_flag, p.dev_status);
     tc_fence_after();
-    if (!ok) l_run = 0.f;   // (the status says so)
-    ml_s[t * 128 + row] = make_float2(m_run, l_run);
-  }
-
-  // ---- combine: every partial (CTA, and stream where there are two) scaled to the row's maximum and
-  // sum over all of them, then added up in a fixed order
-  cluster.sync();   // maxima and sums are published; this CTA's GEMMs are done, so the ring is free
-  float* const o_s = reinterpret_cast<float*>(smem + kOffRing);   // [2][128][128], chunk c of row r at c ^ (r & 31)
-  if (warp >= 2 && warp != kVWarp) {
-    float M = -INFINITY, L = 0.f;
-    float2 ml[8][2];
-#pragma unroll
-    for (int c = 0; c < 8; ++c) {
-      const float2* src = cluster.map_shared_rank(ml_s, c < csize ? c : 0);
-      ml[c][0] = c < csize ? src[(dual ? 0 : t * 128) + row] : make_float2(-INFINITY, 0.f);
-      ml[c][1] = c < csize && dual ? src[128 + row] : make_float2(-INFINITY, 0.f);
-    }
-#pragma unroll
-    for (int c = 0; c < 8; ++c)
-#pragma unroll
-      for (int h = 0; h < 2; ++h)
-        if (ml[c][h].y > 0.f) M = fmaxf(M, ml[c][h].x);
-#pragma unroll
-    for (int c = 0; c < 8; ++c)
-#pragma unroll
-      for (int h = 0; h < 2; ++h)
-        if (ml[c][h].y > 0.f) L += ml[c][h].y * ptx_exp2(ml[c][h].x - M);
-    const float scale = l_run > 0.f && L > 0.f ? ptx_exp2(m_run - M) / L : 0.f;
-    float4* dst = reinterpret_cast<float4*>(o_s) + (size_t)(t * 128 + row) * 32;
+    // ---- this thread's partial row, as it is, into shared memory: the ring is free once both halves of
+    // the softmax warps have seen their last P V
+    asm volatile("bar.sync 1, 256;" ::: "memory");
+    ml_s[t * 128 + row] = make_float2(m_run, ok ? l_run : 0.f);   // (a failed wait: the status says so)
+    if (todo > 0) {   // (else O was not written; its weight is 0)
+      float4* dst = reinterpret_cast<float4*>(smem + kOffRing) + (size_t)(t * 128 + row) * 32;
 #pragma unroll 1
-    for (int c = 0; c < 4; ++c) {
-      uint32_t r[32];
-      tmem_ld32(tO + (uint32_t)c * 32u, r);
-      tmem_ld_wait();
+      for (int c = 0; c < 4; ++c) {
+        uint32_t r[32];
+        tmem_ld32(tO + (uint32_t)c * 32u, r);
+        tmem_ld_wait();
 #pragma unroll
-      for (int g = 0; g < 8; ++g) {
-        float4 o;
-        o.x = scale > 0.f ? __uint_as_float(r[4 * g]) * scale : 0.f;   // (no key seen: O was not written)
-        o.y = scale > 0.f ? __uint_as_float(r[4 * g + 1]) * scale : 0.f;
-        o.z = scale > 0.f ? __uint_as_float(r[4 * g + 2]) * scale : 0.f;
-        o.w = scale > 0.f ? __uint_as_float(r[4 * g + 3]) * scale : 0.f;
-        dst[(c * 8 + g) ^ lane] = o;   // (row & 31 = lane)
+        for (int g = 0; g < 8; ++g)   // chunk c of row r at c ^ (r & 31), and r & 31 = lane
+          dst[(c * 8 + g) ^ lane] = make_float4(__uint_as_float(r[4 * g]), __uint_as_float(r[4 * g + 1]),
+                                                __uint_as_float(r[4 * g + 2]), __uint_as_float(r[4 * g + 3]));
       }
     }
     tc_fence_before();
   }
+
+  // ---- combine: a warp per row of this CTA's share, over the row's partials (CTA, and stream where
+  // there are two) in a fixed order: O = sum_c 2^(m_c - M) O_c / sum_c 2^(m_c - M) l_c
   cluster.sync();
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc(tmem, kTmemCols);
   }
   {
+    const float4* const o_s = reinterpret_cast<const float4*>(smem + kOffRing);
     const int rows = min(nt * 128, T * G - 256 * mp);
     const int r_lo = rank * rows / csize, r_hi = (rank + 1) * rows / csize;
+    const int np = dual ? 2 * csize : csize;   // partial i: CTA i / 2, stream i % 2, or CTA i
+    auto cta_of = [&](int i) { return dual ? i >> 1 : i; };
+    auto row_of = [&](int r, int i) { return r + (dual ? (i & 1) * 128 : 0); };
+    // rows of at most NP partials each, eight partials in flight per lane (16 with NP = 16)
+    auto reduce = [&](auto np_max) {
+      constexpr int NP = decltype(np_max)::value, R = NP < 8 ? 8 / NP : 1;
 #pragma unroll 1
-    for (int r = r_lo + warp; r < r_hi; r += kWarps) {
-      float4 part[8][2];
+      for (int r0 = r_lo + warp * R; r0 < r_hi; r0 += kWarps * R) {
+        float2 ml = make_float2(-INFINITY, 0.f);   // lane: row r0 + lane / NP, partial lane % NP
+        const int li = lane % NP, lr = r0 + lane / NP;
+        if (lane < R * NP && li < np && lr < r_hi) ml = *(cluster.map_shared_rank(ml_s, cta_of(li)) + row_of(lr, li));
+        float4 part[R][NP];
 #pragma unroll
-      for (int c = 0; c < 8; ++c) {
-        const float4* src = reinterpret_cast<const float4*>(cluster.map_shared_rank(o_s, c < csize ? c : 0)) + (size_t)r * 32 + lane;
-        part[c][0] = c < csize ? src[0] : make_float4(0.f, 0.f, 0.f, 0.f);
-        part[c][1] = c < csize && dual ? src[128 * 32] : make_float4(0.f, 0.f, 0.f, 0.f);
-      }
-      float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int q = 0; q < R; ++q)
 #pragma unroll
-      for (int c = 0; c < 8; ++c)
+          for (int i = 0; i < NP; ++i)
+            if (i < np && r0 + q < r_hi)
+              part[q][i] = *(cluster.map_shared_rank(o_s, cta_of(i)) + (size_t)row_of(r0 + q, i) * 32 + lane);
+        float M = ml.y > 0.f ? ml.x : -INFINITY;
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          acc.x += part[c][h].x;
-          acc.y += part[c][h].y;
-          acc.z += part[c][h].z;
-          acc.w += part[c][h].w;
+        for (int o = NP / 2; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+        const float w = ml.y > 0.f ? ptx_exp2(ml.x - M) : 0.f;
+#pragma unroll
+        for (int q = 0; q < R; ++q) {
+          const int r = r0 + q;
+          float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+          float L = 0.f;
+#pragma unroll
+          for (int i = 0; i < NP; ++i) {
+            const float wi = __shfl_sync(0xffffffffu, w, q * NP + i), l = __shfl_sync(0xffffffffu, ml.y, q * NP + i);
+            if (wi > 0.f) {
+              L = fmaf(wi, l, L);
+              acc.x = fmaf(wi, part[q][i].x, acc.x);
+              acc.y = fmaf(wi, part[q][i].y, acc.y);
+              acc.z = fmaf(wi, part[q][i].z, acc.z);
+              acc.w = fmaf(wi, part[q][i].w, acc.w);
+            }
+          }
+          const float inv = L > 0.f ? 1.f / L : 0.f;
+          if (r < r_hi) {
+            const int grow = 256 * mp + r, node = grow / G;
+            uint2* dst = reinterpret_cast<uint2*>(p.out) + (out_row0 + (size_t)node * p.hq + (grow - node * G)) * 32;
+            const uint2 v = make_uint2(pack_bf16x2(acc.x * inv, acc.y * inv), pack_bf16x2(acc.z * inv, acc.w * inv));
+            dst[lane ^ (r & 31)] = invalid ? make_uint2(0u, 0u) : v;
+          }
         }
-      if (invalid) acc = make_float4(0.f, 0.f, 0.f, 0.f);
-      const int grow = 256 * mp + r, node = grow / G;
-      uint2* dst = reinterpret_cast<uint2*>(p.out) + (out_row0 + (size_t)node * p.hq + (grow - node * G)) * 32;
-      dst[lane ^ (r & 31)] = make_uint2(pack_bf16x2(acc.x, acc.y), pack_bf16x2(acc.z, acc.w));
-    }
+      }
+    };
+    if (np <= 2)
+      reduce(std::integral_constant<int, 2>{});
+    else if (np <= 4)
+      reduce(std::integral_constant<int, 4>{});
+    else if (np <= 8)
+      reduce(std::integral_constant<int, 8>{});
+    else
+      reduce(std::integral_constant<int, 16>{});
   }
   cluster.sync();   // keep this CTA's shared memory alive until the others have read it
 }
