@@ -144,17 +144,16 @@ __device__ __forceinline__ void verify_and_write_warp(const VerifyArgs& va, int 
 // the tiny fp32 step 13.4 -> 10.8, the 32-layer step ~240 -> ~236.
 //
 // What bounds it alone: for a few rows the chain of two reads, selection and merge; for many the
-// reads in flight (four 16-byte loads a thread, six CTAs per SM).  Measured (GB300; at first with
+// reads in flight (four or eight 16-byte loads a thread, six or four CTAs per SM).  Measured (GB300; at first with
 // per-thread sorted lists and k rounds of warp maxima at four levels, each thread's list taking
-// every element for fp32), 128256 logits a row: fp32, 63 rows, k = 4 21.1 -> 11.2 us, k = 16
-// 62.6 -> 14.0, 512 rows, k = 16 352 -> 59.2; bf16, 63 rows, k = 4 8.5 -> 7.3, 512 rows 39.6 -> 34.3
+// every element for fp32), 128256 logits a row: fp32, 63 rows, k = 4 21.1 -> 7.8 us, k = 16
+// 62.6 -> 10.2, 512 rows, k = 16 352 -> 61.4; bf16, 63 rows, k = 4 8.5 -> 7.3, 512 rows 39.6 -> 34.3
 // (k = 16 102 -> 44.3).  Parts staged in shared memory by bulk copies took 32.1 us for the 512 bf16
 // rows and 72.5 for the fp32 ones, but left no room beside the attention; a persistent grid
 // with double-buffered parts took 66 (the chain of a row is longer than its copy).
 constexpr int kTargetVec = 2048;   // 32 KB: the part that the cluster size aims at
 constexpr int kMaxK = 16;
 constexpr int kCand = 256;         // candidate buffer (keys)
-constexpr int kLoads = 4;          // vectors in flight per thread
 constexpr int kCluster = 0, kClusterVerify = 1, kSlotsVerify = 2;
 
 __device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }
@@ -213,12 +212,22 @@ __device__ __forceinline__ uint32_t kth_of_32(const uint32_t* v_s, int k) {
 // be placed, so the CTAs start on them at once, beside that grid; the outputs and counters
 // belong to no grid still running.  One CTA waits for the previous grid before it leaves, so
 // that this grid's completion implies that one's.
+// Vectors in flight per thread and CTAs per SM (registers).  Kernels that run beside the tensor-core
+// attention keep to four and 40 registers, and bf16 rows do best so (eight: 512 rows of 128256
+// 34.3 -> 43.8 us); a part of fp32 logits is twice as many vectors (four -> eight: 63 rows 11.2 -> 7.8
+// us, 512 rows with k = 16 59.2 -> 61.4).
 template <typename T, int kMode>
-__global__ void __launch_bounds__(kThreads, 6)
+struct Depth {
+  static constexpr bool kDeep = kMode == kCluster && sizeof(T) == 4;
+  static constexpr int kLoads = kDeep ? 8 : 4, kCtas = kDeep ? 4 : 6;
+};
+
+template <typename T, int kMode>
+__global__ void __launch_bounds__(kThreads, Depth<T, kMode>::kCtas)
     topk_rows_kernel(const T* __restrict__ logits, int64_t rows, int vocab, int64_t row_stride, int k, int per, int beside,
                      int32_t* __restrict__ out_idx, float* __restrict__ out_val, int32_t* dev_status,
                      unsigned int* row_counters, unsigned long long* slots, const __grid_constant__ VerifyArgs va) {
-  constexpr int VN = Vec<T>::kN;
+  constexpr int VN = Vec<T>::kN, kLoads = Depth<T, kMode>::kLoads;
   __shared__ __align__(16) uint64_t cand_s[kCand];
   __shared__ __align__(16) uint64_t all_keys[kMaxCluster * kMaxK];   // the row's parts' keys, at its last merger
   __shared__ __align__(16) uint32_t group_max_s[32];
