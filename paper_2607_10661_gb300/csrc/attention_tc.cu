@@ -910,13 +910,22 @@ __global__ void __launch_bounds__(kThreads, 1)
 
 // ------------------------------------------------------------------- merge of split units
 // CTA (unit, column part) of the persistent cut, 256 threads = (M tile t, row); the unit's
-// 128 output columns are cut into `hsplit` parts (1, 2 or 4) of 128 / hsplit columns.  A unit
+// 128 output columns are cut into `hsplit` parts (1, 2, 4 or 8) of 128 / hsplit columns.  A unit
 // whose key tiles fall in one CTA's range was written whole by the attention; otherwise
 // every piece left a partial and the rows are
 //   O = sum_c 2^(m_c - M) O_c / sum_c 2^(m_c - M) l_c   over the pieces in CTA order
 // (M the maximum over the pieces; a piece that saw no key has l_c = 0 and weight 0).
+// Bound by L2 latency: the pieces of a row are read in batches, so what counts is how few round
+// trips a thread makes.  16 columns of four pieces at a time, the first batch beside the (m, l)
+// loads and up to eight column parts a unit (32 columns of two pieces after the (m, l), up to four
+// parts): 32768 keys under 128 nodes of 64 heads 118.4 -> 117.6 us for attention and merge, 20000
+// keys, 100 nodes, 40 heads 65.1 -> 64.1, four paged trees of 16000 keys 69.4 -> 68.1.  8 columns
+// (four CTAs per SM) are slower, 120.1, 68.7 and 71.6: more CTAs hold the SMs that the attention
+// still needs.
 constexpr int kMergeThreads = 256;
-constexpr int kMergeBatch = 2;   // pieces whose partial columns are in flight at a time
+constexpr int kMergeBatch = 4;   // pieces whose partial columns are in flight at a time
+constexpr int kMergeCols = 16;   // output columns a thread takes at a time
+constexpr int kMergeParts = 128 / kMergeCols;   // most column parts per unit
 constexpr int kMergeMl = 8;      // pieces whose (m, l) stay in registers
 
 __global__ void __launch_bounds__(kMergeThreads, 2) tree_attn_merge_kernel(const AttnParams p, int hsplit) {
@@ -969,6 +978,21 @@ __global__ void __launch_bounds__(kMergeThreads, 2) tree_attn_merge_kernel(const
   auto piece_ml = [&](int c) -> float2 {
     return has_piece(c) ? __ldcg(pml + (size_t)piece_slot(wc, c, ug0, ug1) * 256) : make_float2(-INFINITY, 0.f);
   };
+  constexpr int kVec = kMergeCols / 4;
+  const int h_per = kMergeParts / hsplit;
+  float4 o[kMergeBatch][kVec];
+  auto load_batch = [&](int h, int c0) {
+#pragma unroll
+    for (int q = 0; q < kMergeBatch; ++q) {
+      if (has_piece(c0 + q)) {
+        const float4* po = reinterpret_cast<const float4*>(p.part_o) +
+                           (((size_t)piece_slot(wc, c0 + q, ug0, ug1) * 2 + t) * 32 + h * kVec) * 128 + row;
+#pragma unroll
+        for (int g4 = 0; g4 < kVec; ++g4) o[q][g4] = __ldcg(po + (size_t)g4 * 128);
+      }
+    }
+  };
+  load_batch(hs * h_per, first);   // beside the (m, l) loads, not after them
   float2 mlc[kMergeMl];
 #pragma unroll
   for (int q = 0; q < kMergeMl; ++q) mlc[q] = piece_ml(first + q);
@@ -990,49 +1014,39 @@ __global__ void __launch_bounds__(kMergeThreads, 2) tree_attn_merge_kernel(const
   const float inv = L > 0.f ? 1.f / L : 0.f;
   const size_t orow = (((size_t)lq * p.n_total + node0 + node) * p.hq + (size_t)hkv * G + g) * 128;
   uint4* dst = reinterpret_cast<uint4*>(p.out) + orow / 8;
-  const int h_per = 4 / hsplit;
 #pragma unroll 1
-  for (int h = hs * h_per; h < (hs + 1) * h_per; ++h) {   // 32 output columns at a time
-    float acc[32];
+  for (int h = hs * h_per; h < (hs + 1) * h_per; ++h) {
+    float acc[kMergeCols];
 #pragma unroll
-    for (int d = 0; d < 32; ++d) acc[d] = 0.f;
+    for (int d = 0; d < kMergeCols; ++d) acc[d] = 0.f;
     for (int c0 = first; c0 <= last; c0 += kMergeBatch) {
-      float4 o[kMergeBatch][8];
+      if (h > hs * h_per || c0 > first) load_batch(h, c0);
+      // rows of a piece that saw no key were not written: weight 0 and never taken into acc
       float wgt[kMergeBatch];
 #pragma unroll
       for (int q = 0; q < kMergeBatch; ++q) {
-        const int c = c0 + q;
-        wgt[q] = 0.f;
-        if (has_piece(c)) {
-          const size_t sl = (size_t)piece_slot(wc, c, ug0, ug1);
-          const float2 ml = __ldcg(pml + sl * 256);
-          const float4* po = reinterpret_cast<const float4*>(p.part_o + (sl * 2 + t) * (128 * 128)) +
-                             (size_t)(h * 8) * 128 + row;
-#pragma unroll
-          for (int gg = 0; gg < 8; ++gg) o[q][gg] = __ldcg(po + (size_t)gg * 128);
-          // rows of a piece that saw no key were not written: weight 0 and never read into acc
-          wgt[q] = ml.y > 0.f ? ptx_exp2(ml.x - M) : 0.f;
-        }
+        const float2 ml = piece_ml(c0 + q);
+        wgt[q] = ml.y > 0.f ? ptx_exp2(ml.x - M) : 0.f;
       }
 #pragma unroll
       for (int q = 0; q < kMergeBatch; ++q) {
         if (wgt[q] > 0.f) {
 #pragma unroll
-          for (int gg = 0; gg < 8; ++gg) {
-            acc[4 * gg] = fmaf(wgt[q], o[q][gg].x, acc[4 * gg]);
-            acc[4 * gg + 1] = fmaf(wgt[q], o[q][gg].y, acc[4 * gg + 1]);
-            acc[4 * gg + 2] = fmaf(wgt[q], o[q][gg].z, acc[4 * gg + 2]);
-            acc[4 * gg + 3] = fmaf(wgt[q], o[q][gg].w, acc[4 * gg + 3]);
+          for (int g4 = 0; g4 < kVec; ++g4) {
+            acc[4 * g4] = fmaf(wgt[q], o[q][g4].x, acc[4 * g4]);
+            acc[4 * g4 + 1] = fmaf(wgt[q], o[q][g4].y, acc[4 * g4 + 1]);
+            acc[4 * g4 + 2] = fmaf(wgt[q], o[q][g4].z, acc[4 * g4 + 2]);
+            acc[4 * g4 + 3] = fmaf(wgt[q], o[q][g4].w, acc[4 * g4 + 3]);
           }
         }
       }
     }
 #pragma unroll
-    for (int c8 = 0; c8 < 4; ++c8) {
+    for (int c8 = 0; c8 < kMergeCols / 8; ++c8) {
       uint32_t w[4];
 #pragma unroll
       for (int e = 0; e < 4; ++e) w[e] = pack_bf16x2(acc[c8 * 8 + 2 * e] * inv, acc[c8 * 8 + 2 * e + 1] * inv);
-      dst[h * 4 + c8] = make_uint4(w[0], w[1], w[2], w[3]);
+      dst[h * (kMergeCols / 8) + c8] = make_uint4(w[0], w[1], w[2], w[3]);
     }
   }
 }
@@ -1043,9 +1057,9 @@ __global__ void __launch_bounds__(kMergeThreads, 2) tree_attn_merge_kernel(const
 size_t tc_smem_bytes() { return tc::kSmemBytes; }
 
 cudaError_t launch_tree_attn_merge(const AttnParams& p, int units, int sms, cudaStream_t stream) {
-  // column parts per unit: about two CTAs per SM over the grid (1, 2 or 4)
-  const int want = units > 0 ? 2 * sms / units : 1;
-  const int hsplit = want >= 4 ? 4 : (want >= 2 ? 2 : 1);
+  // column parts per unit: at most two CTAs per SM over the grid (1, 2, 4 or 8)
+  int hsplit = 1;
+  while (hsplit < tc::kMergeParts && units * hsplit * 2 <= 2 * sms) hsplit *= 2;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(units * hsplit), 1, 1);
   cfg.blockDim = dim3(tc::kMergeThreads, 1, 1);

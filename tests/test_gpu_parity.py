@@ -119,12 +119,12 @@ def test_attention_without_workspace_matches_oracle(case):
 
 @pytest.mark.parametrize("layers,ctx,launches", [
     (12, 2000, 2),   # 96 units on 152 CTAs: pieces merged by the merge kernel, two column parts per unit
-    (4, 2000, 2),    # 32 units: four column parts per unit
+    (4, 2000, 2),    # 32 units: eight column parts per unit
     (20, 1000, 1),   # 160 units: the last piece of each split unit merges inside the attention
 ])
 def test_attention_merge_paths_match_oracle(layers, ctx, launches):
     """Both merges of split units (in the attention kernel, or by the merge kernel with two or
-    four column parts per unit), every unit against the oracle."""
+    eight column parts per unit), every unit against the oracle."""
     cfg = syn.shrink(syn.CONFIGS["llama3-8b-gqa"], layers=layers, ctx=(ctx, ctx), vocab=100)
     w = syn.Workload(cfg, 23)
     dw = DeviceWorkload(w, with_step_buffers=False)
@@ -178,6 +178,26 @@ def test_attention_cut_of_stacks_matches_oracle(layers, hq, hkv, nodes, ctx, pag
     w = syn.Workload(syn.shrink(syn.CONFIGS["llama3-8b-gqa"], **over), 43)
     dw, got = _run_attention(w)
     _check_every_unit(w, got, "cut")
+
+
+@pytest.mark.parametrize("layers,hq,hkv,nodes,ctx", [
+    (1, 4, 1, 20, 20000),    # one unit in a piece on every CTA; half an M tile
+    (1, 8, 2, 128, 9000),    # four units of ~36 pieces, eight column parts
+    (1, 28, 4, 63, 12000),   # group of 7: the second pair of each KV head has one M tile, partly filled
+    (6, 32, 8, 63, 2000),    # 48 units of ~3 pieces, four column parts
+])
+def test_attention_merge_of_many_pieces_matches_oracle(layers, hq, hkv, nodes, ctx):
+    """The merge kernel over more pieces than it takes at a time, and its column parts."""
+    over = dict(hq=hq, hkv=hkv, nodes=(nodes, nodes), ctx=(ctx, ctx), layers=layers, vocab=100, tree="random-depth",
+                branching=(4, 3, 2, 2, 1, 1), depth_range=(5, 6))
+    w = syn.Workload(syn.shrink(syn.CONFIGS["llama3-8b-gqa"], **over), 47)
+    dw = DeviceWorkload(w, with_step_buffers=False)
+    n = dw.attention()
+    torch.cuda.synchronize()
+    assert int(dw.dev_status.item()) == 0
+    if torch.cuda.get_device_properties(0).multi_processor_count == 152:
+        assert n == 2
+    _check_every_unit(w, dw.attn_out.float().cpu().numpy(), "merge")
 
 
 def test_attention_peaked_context_exposes_mask():
