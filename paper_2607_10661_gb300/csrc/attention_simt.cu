@@ -1,5 +1,5 @@
-// Tree-masked attention in fp32 on the CUDA cores (the fp32 path; no tensor cores, so
-// the result keeps full fp32 accuracy).
+// Tree-masked attention in fp32 on the CUDA cores, and the choice between it and the kernel that
+// splits fp32 operands for the tensor cores (D = 128, many rows and keys).
 //
 // Same operation as the tensor-core kernel (Sec. 3.1 ancestor-only visibility over the
 // committed prefix plus the tree, Sec. 3.2), and the same dense view of it: the T nodes times
@@ -21,7 +21,7 @@
 // per 32 FMAs, an 8 x 8 tile of O 16 per 64; the pipe gives ~110 FMA per cycle and SM) for many
 // rows, the latency of a tile's chain and the K/V stream for few.  Measured (GB300, one layer,
 // against one CTA per (node, head) over all keys, which read every K/V row T * G times): 32 query
-// / 8 KV heads, D 128, 2048 + 63 keys, 63 nodes 628 -> 69.5 us (31 TFLOP/s); the same with one
+// / 8 KV heads, D 128, 2048 + 63 keys, 63 nodes 628 -> 69.5 us (31 TFLOP/s; the tensor-core kernel 30.8); the same with one
 // node 86 -> 26 us; 8 heads, D 64, 256 + 15 keys, 15 nodes 14.5 -> 6.6 us.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
@@ -524,6 +524,35 @@ cudaError_t launch_d(const CUtensorMap& map_k, const CUtensorMap& map_v, const A
     if (cost < best) best = cost, csize = c;
   }
   if (units * csize > 0x7fffffffll) return cudaErrorInvalidValue;
+  if constexpr (D == 128) {
+    // The tensor-core kernel where it is estimated to be faster (us, fitted to measurements of 65
+    // shapes on 152 SMs; of the ones it sends there none is more than 2 % slower for it): here a fixed
+    // part and a time per key of a CTA's share that depends on the rows of a block and on whether
+    // two CTAs share an SM; there a fixed part and a time per tile of 64 keys.  Tensor cores / CUDA
+    // cores, 32 query and 8 KV heads: 63 nodes 64 keys 16.6 / 16.1, 300 keys 15.4 / 21.7, 1000 keys 21.5 /
+    // 43.0, 4000 keys 48.7 / 115.5; 8 heads of one row group: 32 nodes 1000 keys 18.4 / 17.3, 4000 keys
+    // 35.1 / 41.9, 8 nodes 4000 keys 34.7 / 33.2.
+    const double share = ((keys + csize - 1) / csize + 15) / 16 * 16;
+    const double waves = (double)((units * csize + slots - 1) / slots);
+    // clusters of c CTAs at one CTA per SM that fit at once, measured on 152 SMs
+    static const int fit152[kMaxCluster + 1] = {0, 152, 76, 46, 36, 28, 23, 15, 15};
+    auto fit = [&](int c) { return fit152[c] * sms / 152 > 0 ? fit152[c] * sms / 152 : 1; };
+    const bool shared_sm = units > fit(csize);
+    const double fixed = bm == 16 ? 5.5 : bm == 32 ? 7.3 : 11.;
+    const double per_key = bm == 16 ? (shared_sm ? 0.085 : 0.054) : bm == 32 ? (shared_sm ? 0.117 : 0.069)
+                                                                            : (shared_sm ? 0.205 : 0.112);
+    const double t_here = waves * (fixed + per_key * share);
+    const int split_blocks = (M + 127) / 128;
+    const long long split_units = (long long)split_blocks * p.hkv * p.batch * p.layers;
+    int split_csize = 0;
+    double t_split = t_here;
+    for (int c = 1; c <= kMaxCluster; ++c) {
+      const int tiles = (((keys + c - 1) / c + 15) / 16 * 16 + 63) / 64;
+      const double t = (double)((split_units + fit(c) - 1) / fit(c)) * (12. + 3.35 * tiles);
+      if (t < t_split) t_split = t, split_csize = c;
+    }
+    if (split_csize > 0) return launch_tree_attn_split(p, split_csize, split_blocks, stream);
+  }
   switch (bm) {
     case 16:
       return launch<D, 16 / kGroups>(map_k, map_v, p, csize, m_blocks, stream);

@@ -265,6 +265,57 @@ def test_attention_f32_blocks_match_oracle(hq, hkv, d, nodes, ctx, page, batch, 
     _check_every_unit(w, got, "f32 blocks")
 
 
+@pytest.mark.parametrize("hq,hkv,nodes,ctx,page,batch,layers", [
+    (8, 8, 128, (4000, 4000), 0, 1, 1),     # 128 rows exactly; tree keys over three tiles; eight CTAs a unit
+    (32, 8, 33, (1000, 1000), 0, 1, 1),     # 132 rows: the second block has four
+    (28, 4, 65, (777, 777), 16, 1, 1),      # group of 7, 455 rows in four blocks, pages
+    (16, 16, 127, (1023, 1023), 64, 1, 1),  # the context ends one short of a tile
+    (32, 8, 24, (300, 300), 0, 1, 1),       # 96 rows, one tile a CTA
+    (32, 8, 70, (1, 2000), 32, 3, 2),       # ragged trees and contexts, two layers: CTAs without keys
+    (8, 2, 128, (3000, 3000), 0, 4, 8),     # 256 units: several waves, whole units
+])
+def test_attention_f32_split_matches_oracle(hq, hkv, nodes, ctx, page, batch, layers):
+    """fp32 attention on the tensor cores (D = 128, many rows and keys), every unit."""
+    over = dict(hq=hq, hkv=hkv, d=128, nodes=(min(nodes, 20), nodes) if batch == 3 else (nodes, nodes), ctx=ctx,
+                page_size=page, batch=batch, layers=layers, vocab=100, tree="random-depth",
+                branching=(4, 3, 2, 2, 1, 1), depth_range=(5, 6))
+    w = syn.Workload(syn.shrink(syn.CONFIGS["tiny-fp32"], **over), 37)
+    dw, got = _run_attention(w)
+    _check_every_unit(w, got, "f32 split")
+
+
+def test_attention_f32_split_extreme_values():
+    """Values whose nearest bf16 is infinite, infinities and NaN: the affected columns and rows only."""
+    over = dict(hq=32, hkv=8, d=128, nodes=(63, 63), ctx=(1500, 1500), layers=1, vocab=100, tree="binary")
+    w = syn.Workload(syn.shrink(syn.CONFIGS["tiny-fp32"], **over), 53)
+    dw = DeviceWorkload(w, with_step_buffers=False)
+    dw.attention()
+    torch.cuda.synchronize()
+    ref = dw.attn_out.float().clone()
+    k, v = dw.k[0], dw.v[0]                  # [batch][slots][KV heads][D]
+    v[0, 700, 1, 5] = 3.4e38                 # finite, but not as a bf16
+    v[0, 40, 2, 9] = float("inf")
+    v[0, 1200, 3, 11] = float("nan")
+    dw.q[0, 7, 16] = float("inf")            # a row of KV head 4
+    k[0, 900, 5, 3] = float("nan")           # a key of KV head 5: all its rows
+    dw.attention()
+    torch.cuda.synchronize()
+    got = dw.attn_out.float()
+    assert int(dw.dev_status.item()) == 0
+    touched = torch.zeros_like(ref, dtype=torch.bool)
+    touched[0, :, 4:8, 5] = True
+    touched[0, :, 8:12, 9] = True
+    touched[0, :, 12:16, 11] = True
+    touched[0, 7, 16] = True
+    touched[0, :, 20:24] = True
+    # the share with the value goes through fp32 loops: a sum in another order (2 x 1563 roundings of
+    # terms below max |V| = 6, against 1e-5)
+    assert torch.allclose(got[~touched], ref[~touched], rtol=0.0, atol=1e-5)
+    big = got[0, :, 4:8, 5]
+    assert torch.isfinite(big).all() and (big > 1e30).all()
+    assert (got[0, :, 8:12, 9] == float("inf")).all()
+
+
 def test_attention_full_size_llama2_layer():
     """The Llama-2-7B-shaped layer at its own size: 32 MHA heads (M = 31 rows per unit, one
     128-row tcgen05 tile mostly padding), context 2048 (17 key tiles), every head."""
