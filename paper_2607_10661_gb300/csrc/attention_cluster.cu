@@ -69,7 +69,8 @@ __global__ void __launch_bounds__(512, 1)
   uint8_t* smem = smem_raw + pad;
   base += pad;
   cg::cluster_group cluster = cg::this_cluster();
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // known to be uniform, for the GEMM issue
   auto bar = [&](int i) { return base + kOffBar + 8u * (uint32_t)i; };
   auto fullk_bar = [&](int s) { return bar(s); };
   auto fullv_bar = [&](int s) { return bar(2 + s); };
@@ -258,18 +259,22 @@ __global__ void __launch_bounds__(512, 1)
       }
     }
   } else if (warp == 1) {
-    // ================================================================ MMA issuer (one thread)
-    if (lane == 0 && n > 0) {
-      const uint32_t q_base = base + kOffQ, ring = base + kOffRing;
-      auto wait = [&](uint32_t bar_, uint32_t parity) { return mbar_wait(bar_, parity, abort_flag, p.dev_status); };
+    // ================================================================ MMA issuer
+    if (n > 0) {
+      const uint32_t dq = (uint32_t)smem_desc_sw128(base + kOffQ, 16, 1024), dk = (uint32_t)smem_desc_sw128(base + kOffRing, 16, 1024),
+                     dv = (uint32_t)smem_desc_sw128(base + kOffRing + kTileBytes, kHalfBytes, 1024);
+      const uint32_t leader = lane == 0 ? 1u : 0u;
+      auto commit = [&](uint32_t b) {
+        if (leader) mma_commit(b);
+      };
+      auto wait = [&](uint32_t bar_, uint32_t parity) { return mbar_wait_warp(bar_, parity, abort_flag, p.dev_status); };
       auto s_gemm = [&](int tt, int j) {   // S_tt of tile j
-        issue_s(tmem + (uint32_t)tt * 128u, q_base + (dual ? 0u : (uint32_t)tt * kTileBytes),
-                ring + (uint32_t)(j & 1) * kStageBytes);
-        mma_commit(sfull_bar(tt));
+        issue_s(leader, tmem + (uint32_t)tt * 128u, dq + (dual ? 0u : (uint32_t)tt * (kTileBytes >> 4)),
+                dk + (uint32_t)(j & 1) * (kStageBytes >> 4));
+        commit(sfull_bar(tt));
       };
       auto pv_gemm = [&](int tt, int j, bool acc) {
-        issue_pv(tmem + 256u + (uint32_t)tt * 128u, tmem + (uint32_t)tt * 128u,
-                 ring + (uint32_t)(j & 1) * kStageBytes + kTileBytes, acc);
+        issue_pv(leader, tmem + (uint32_t)tt * 128u, dv + (uint32_t)(j & 1) * (kStageBytes >> 4), acc);
       };
       bool ok = true;
       for (int tt = 0; tt < nt && ok; ++tt) ok = wait(qready_bar(tt), 0u);
@@ -279,7 +284,7 @@ __global__ void __launch_bounds__(512, 1)
           if (!(ok = wait(fullk_bar(j), 0u))) break;
           tc_fence_after();
           s_gemm(j, j);
-          mma_commit(emptyk_bar(j));
+          commit(emptyk_bar(j));
         }
         for (int j = 0; j < n && ok; ++j) {
           const int tt = j & 1;
@@ -288,14 +293,14 @@ __global__ void __launch_bounds__(512, 1)
           if (!(ok = wait(pfull_bar(tt), ph))) break;
           tc_fence_after();
           pv_gemm(tt, j, j >= 2);
-          mma_commit(emptyv_bar(tt));
+          commit(emptyv_bar(tt));
           if (j + 2 >= n) {
-            mma_commit(ofull_bar(tt));
+            commit(ofull_bar(tt));
           } else {
             if (!(ok = wait(fullk_bar(tt), ph ^ 1u))) break;
             tc_fence_after();
             s_gemm(tt, j + 2);
-            mma_commit(emptyk_bar(tt));
+            commit(emptyk_bar(tt));
           }
         }
       } else {
@@ -304,7 +309,7 @@ __global__ void __launch_bounds__(512, 1)
           tc_fence_after();
           s_gemm(0, 0);
           s_gemm(1, 0);
-          mma_commit(emptyk_bar(0));
+          commit(emptyk_bar(0));
         }
         for (int j = 0; j < n && ok; ++j) {
           const int st = j & 1, st1 = st ^ 1;
@@ -318,21 +323,21 @@ __global__ void __launch_bounds__(512, 1)
             tc_fence_after();
             s_gemm(0, j + 1);
           } else {
-            mma_commit(ofull_bar(0));
+            commit(ofull_bar(0));
           }
           if (!(ok = wait(pfull_bar(1), (uint32_t)(j & 1)))) break;
           tc_fence_after();
           pv_gemm(1, j, j > 0);
-          mma_commit(emptyv_bar(st));
+          commit(emptyv_bar(st));
           if (more) {
             s_gemm(1, j + 1);
-            mma_commit(emptyk_bar(st1));
+            commit(emptyk_bar(st1));
           } else {
-            mma_commit(ofull_bar(1));
+            commit(ofull_bar(1));
           }
         }
       }
-      if (!ok) {   // error path: let the tensor core finish what was issued before TMEM is freed
+      if (!ok && leader) {   // error path: let the tensor core finish what was issued before TMEM is freed
         mma_commit(drain_bar);
         mbar_drain(drain_bar, 0, 100000000ull);
       }

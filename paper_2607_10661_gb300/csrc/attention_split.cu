@@ -107,27 +107,6 @@ __device__ __forceinline__ void store_split(uint32_t dst, uint32_t part, int r, 
   asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(at + 2 * part), "r"(l0), "r"(l1) : "memory");
 }
 
-// tcgen05.mma (kind::f16, A from shared memory / from tensor memory) issued where `go` is not 0.  A
-// descriptor comes as its low word; the high one (strides, version, swizzle) is the same for all.
-__device__ __forceinline__ void mma_ss_if(uint32_t go, uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t hi,
-                                          uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p, g;\n\t.reg .b64 a, b;\n\tmov.b64 a, {%1, %3};\n\tmov.b64 b, {%2, %3};\n\t"
-      "setp.ne.b32 p, %5, 0;\n\tsetp.ne.b32 g, %6, 0;\n\t"
-      "@g tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %4, p;\n\t}" ::"r"(d_tmem),
-      "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate), "r"(go)
-      : "memory");
-}
-__device__ __forceinline__ void mma_ts_if(uint32_t go, uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t hi,
-                                          uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p, g;\n\t.reg .b64 b;\n\tmov.b64 b, {%2, %3};\n\t"
-      "setp.ne.b32 p, %5, 0;\n\tsetp.ne.b32 g, %6, 0;\n\t"
-      "@g tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], b, %4, p;\n\t}" ::"r"(d_tmem),
-      "r"(a_tmem), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate), "r"(go)
-      : "memory");
-}
-
 // Four floats, or zeros where `there` is false, as one predicated load: nothing waits for it before its use.
 __device__ __forceinline__ float4 load_or_zero(const float* src, bool there) {
   float4 x;
@@ -209,7 +188,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   base += pad;
   cg::cluster_group cluster = cg::this_cluster();
   const int tid = threadIdx.x, lane = tid & 31;
-  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // uniform, so that warp branches are
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // known to be uniform, for the GEMM issue
   const int rank = blockIdx.x % csize;
   int u = blockIdx.x / csize;
   const int mb = u % m_blocks;
@@ -329,14 +308,13 @@ __global__ void __launch_bounds__(kThreads, 1)
     asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
     if (warp == kRowWarps) {
       // ================================================================ GEMM issue
-      // The warp walks together and one lane issues by predication, descriptors broadcast (issued
-      // inside a one-lane branch a GEMM instruction took 95-110 cycles, so 80-100; 54 alone).
+      // The warp walks together and one lane issues by predication (see tc::issue_s): a GEMM
+      // instruction takes 80-100 cycles instead of 95-110 (54 in a kernel that does nothing else).
       const uint32_t leader = lane == 0 ? 1u : 0u;
       // descriptors of the first part's first 16 columns (Q, K) or keys (V); the address field counts
       // 16-byte units, so the others are sums
       const uint32_t dq = (uint32_t)smem_desc_sw128(base, 16, 1024), dk = (uint32_t)smem_desc_sw128(base + kOffK, 16, 1024),
                      dv = (uint32_t)smem_desc_sw128(base + kOffV, kKvHalf, 1024);
-      const uint32_t hi = (uint32_t)(smem_desc_sw128(0, 16, 1024) >> 32);
       // the products, the smallest first: parts of the two operands, four bits each (a loop over
       // them: unrolled, the descriptors would be kept over the tiles and spill)
       constexpr uint32_t kPartA = 0x010120u, kPartB = 0x001102u;
@@ -354,7 +332,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
           for (int kk = 0; kk < 8; ++kk)
             mma_ss_if(leader, kk < 4 ? d0 : d1, a + (uint32_t)((kk >> 2) * (int)(kQHalf / 16) + (kk & 3) * 2),
-                      c + (uint32_t)((kk >> 2) * (int)(kKvHalf / 16) + (kk & 3) * 2), hi, kIdescS,
+                      c + (uint32_t)((kk >> 2) * (int)(kKvHalf / 16) + (kk & 3) * 2), tc::kDescHi, kIdescS,
                       kk == 0 ? (i > 0 && !hh ? 1u : 0u) : kk == 4 ? (hh ? 0u : 1u) : 1u);
         }
         if (leader) mma_commit(s_full(t));
@@ -369,7 +347,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           const uint32_t c = dvt + ((kPartB >> (4 * i)) & 3u) * (kKvPart / 16);
 #pragma unroll
           for (int kk = 0; kk < kBN / 16; ++kk)
-            mma_ts_if(leader, tm + kColO, a + (uint32_t)kk * 8u, c + (uint32_t)(kk * 128), hi, kIdescPV,
+            mma_ts_if(leader, tm + kColO, a + (uint32_t)kk * 8u, c + (uint32_t)(kk * 128), tc::kDescHi, kIdescPV,
                       i > 0 || kk > 0 ? 1u : 0u);
         }
         if (leader) mma_commit(o_full);
