@@ -158,6 +158,58 @@ __device__ __forceinline__ void load_tile(const AttnParams& p, const CUtensorMap
   }
 }
 
+// Rare path, one warp: a row over the visible keys of [k_lo, k_hi) alone, in order (the tiles multiply the
+// P = 0 of hidden nodes into their V, which must not be infinite or NaN).  O (unnormalised) to dst;
+// returns the running maximum (log2 units) and the row sum.
+template <int D>
+__device__ __noinline__ float2 visible_row(const AttnParams& p, const float* q, int layer, int b, int hkv, int k_lo, int k_hi,
+                                           int C, const int* parents, int node, float* dst) {
+  constexpr int WC = D / 32;
+  const int lane = threadIdx.x & 31;
+  uint32_t am[4] = {0, 0, 0, 0};
+  for (int a = node; a >= 0; a = parents[a])
+#pragma unroll
+    for (int w = 0; w < 4; ++w) am[w] |= (a >> 5) == w ? 1u << (a & 31) : 0u;
+  float qv[WC], o[WC], m = -INFINITY, l = 0.f;
+  load_n<WC>(q + WC * lane, qv);
+#pragma unroll
+  for (int c = 0; c < WC; ++c) o[c] = 0.f;
+#pragma unroll 1
+  for (int key = k_lo; key < k_hi; ++key) {
+    const int a = key - C;
+    if (a >= 0 && !((a < 32 ? am[0] : a < 64 ? am[1] : a < 96 ? am[2] : am[3]) >> (a & 31) & 1u)) continue;
+    long long row;
+    bool there = true;
+    if (p.page_size > 0) {
+      const int page = p.block_table[(size_t)b * p.max_pages + key / p.page_size];
+      there = (unsigned)page < (unsigned)p.num_pages;
+      row = ((long long)layer * p.num_pages + page) * p.page_size + key % p.page_size;
+    } else {
+      row = ((long long)layer * p.batch + b) * p.seq_capacity + key;
+    }
+    const long long at = (row * p.hkv + hkv) * D + WC * lane;
+    float kv[WC], vv[WC], x = 0.f;
+#pragma unroll
+    for (int c = 0; c < WC; ++c) kv[c] = vv[c] = 0.f;
+    if (there) {
+      load_n<WC>(static_cast<const float*>(p.k) + at, kv);
+      load_n<WC>(static_cast<const float*>(p.v) + at, vv);
+    }
+#pragma unroll
+    for (int c = 0; c < WC; ++c) x = fmaf(qv[c], kv[c], x);
+    x = warp_sum(x);
+    const float m_new = fmaxf(m, x * p.scale_log2);
+    const float m_use = m_new == -INFINITY ? 0.f : m_new;
+    const float alpha = exp2f(m - m_use), w = exp2f(fmaf(x, p.scale_log2, -m_use));
+    m = m_new;
+    l = fmaf(l, alpha, w);
+#pragma unroll
+    for (int c = 0; c < WC; ++c) o[c] = fmaf(o[c], alpha, w * vv[c]);
+  }
+  store_n<WC>(dst + WC * lane, o);
+  return make_float2(m, l);
+}
+
 template <int D, int RM>
 __global__ void __launch_bounds__(kThreads, 2)
     tree_attn_simt_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
@@ -420,7 +472,19 @@ __global__ void __launch_bounds__(kThreads, 2)
     }
   }
   // ---- this CTA's partial rows into shared memory (over V and P)
-  __syncthreads();
+  bool wild = false;   // a row of this thread is not finite
+#pragma unroll
+  for (int i = 0; i < RM; ++i) {
+    bool x = !(fabsf(l_run[i]) < INFINITY);
+#pragma unroll
+    for (int c = 0; c < DC; ++c) {
+      float lo, hi;
+      f2_unpack(o[c][i / 2], lo, hi);
+      x = x || !(fabsf(i & 1 ? hi : lo) < INFINITY);
+    }
+    wild = wild || (x && rg * RM + i < rows);
+  }
+  wild = __syncthreads_or(wild) && ok;
 #pragma unroll
   for (int i = 0; i < RM; ++i) {
     const float l = group_sum(l_run[i]);
@@ -443,9 +507,25 @@ __global__ void __launch_bounds__(kThreads, 2)
       store_n<DC>(dst + DC * g, x);
     }
   }
+  constexpr int WC = D / 32;   // columns per lane of a whole warp
+  if (wild) {
+    __syncthreads();
+#pragma unroll 1
+    for (int r = warp; r < rows; r += kWarps) {
+      float* const row = sm + L::kO + r * D;
+      float2* const ml = reinterpret_cast<float2*>(sm + L::kMl + 2 * r);
+      bool x = !(fabsf(ml->y) < INFINITY);
+#pragma unroll
+      for (int c = 0; c < WC; ++c) x = x || !(fabsf(row[WC * lane + c]) < INFINITY);
+      if (!__any_sync(0xffffffffu, x)) continue;
+      const float2 y = visible_row<D>(p, static_cast<const float*>(p.q) + q_row(r) * D, layer, b, hkv, k_lo, k_hi, C,
+                                      p.parents + node0, node_of(row0 + r), row);
+      __syncwarp();
+      if (lane == 0) *ml = y;
+    }
+  }
   cluster.sync();
   // ---- combine: CTA r writes the r-th share of the rows, one row per warp at a time
-  constexpr int WC = D / 32;   // columns per lane of a whole warp
   const int r_lo = rank * rows / csize, r_hi = (rank + 1) * rows / csize;
 #pragma unroll 1
   for (int r = r_lo + warp; r < r_hi; r += kWarps) {

@@ -316,6 +316,42 @@ def test_attention_f32_split_extreme_values():
     assert (got[0, :, 8:12, 9] == float("inf")).all()
 
 
+@pytest.mark.parametrize("hq,hkv,d,nodes,ctx,page", [
+    (8, 8, 64, 15, 40, 0),       # CUDA cores, one column run a lane
+    (8, 8, 32, 31, 100, 16),
+    (32, 8, 128, 31, 60, 0),     # CUDA cores, two blocks of 64 rows
+    (32, 8, 128, 63, 1500, 0),   # tensor cores
+])
+@pytest.mark.parametrize("value", [float("inf"), float("nan")])
+def test_attention_f32_hidden_values_stay_hidden(hq, hkv, d, nodes, ctx, page, value):
+    """An infinity or NaN in a tree node's V reaches the node and its descendants only."""
+    over = dict(hq=hq, hkv=hkv, d=d, nodes=(nodes, nodes), ctx=(ctx, ctx), page_size=page, layers=1, vocab=100, tree="binary")
+    w = syn.Workload(syn.shrink(syn.CONFIGS["tiny-fp32"], **over), 59)
+    dw = DeviceWorkload(w, with_step_buffers=False)
+    dw.attention()
+    torch.cuda.synchronize()
+    ref = dw.attn_out.float().clone()
+    bad = 2
+    sees = torch.zeros(nodes, dtype=torch.bool, device=ref.device)
+    for i in range(nodes):
+        a = i
+        while a >= 0 and a != bad:
+            a = int(w.trees[0][a])
+        sees[i] = a == bad
+    slot = ctx + bad
+    if page:
+        dw.v[0][int(dw.block_table[0, slot // page]), slot % page] = value
+    else:
+        dw.v[0][0, slot] = value
+    dw.attention()
+    torch.cuda.synchronize()
+    got = dw.attn_out.float()
+    assert int(dw.dev_status.item()) == 0
+    # (a redone row sums in another order: 2 x (ctx + nodes) roundings of terms below max |V| = 6)
+    assert torch.allclose(got[0][~sees], ref[0][~sees], rtol=0.0, atol=1e-5)
+    assert not torch.isfinite(got[0][sees]).any()
+
+
 def test_attention_full_size_llama2_layer():
     """The Llama-2-7B-shaped layer at its own size: 32 MHA heads (M = 31 rows per unit, one
     128-row tcgen05 tile mostly padding), context 2048 (17 key tiles), every head."""
