@@ -58,7 +58,7 @@ MEASURED_PEAKS = os.path.join(ROOT, "MEASURED_PEAKS.json")
 # the tail of the one-call step (ptd_step_tail)
 STEP_TAILS = {0: "top-k, then verification + compaction in one launch",
               1: "clustered top-k (one cluster per row) verifying the trees, then a compaction kernel",
-              2: "streamed top-k (rows back to back, one share per CTA) verifying the trees, then a compaction kernel"}
+              2: "streamed top-k (a row's parts in single CTAs that merge through scratch) verifying the trees, then a compaction kernel"}
 FALLBACK_HBM_GBS = 6800.0
 FALLBACK_BF16_TFLOPS_SUSTAINED = 1700.0
 NOMINAL_HBM_GBS = 8000.0
@@ -564,7 +564,7 @@ def run_gpu(args, rank: int, world: int, dist):
         roof = {"bound": "hbm", "achieved": round(achieved_gbs, 1), "peak": hbm_peak, "unit": "GB/s",
                 "frac": round(achieved_gbs / hbm_peak, 4), "peak_kind": peak_kind,
                 "tensor_tflops": round(achieved_tf, 1), "tensor_frac": round(achieved_tf / tf_peak, 4)}
-    kernel = "tree_attn_tc_kernel" if cfg.dtype == "bf16" else "tree_attn_simt_kernel"
+    kernel = "tree_attn_tc_kernel or tree_attn_cluster_kernel" if cfg.dtype == "bf16" else "tree_attn_simt_kernel"
     if attn_kernels[0] == 2:   # timed from the attention's start to the end of the merge of split units
         kernel += " + tree_attn_merge_kernel"
     roof.update({"kernel": kernel, "traffic": _profiled_traffic(PROFILED_ATTENTION_TRAFFIC, "attention_tc.cu",

@@ -173,7 +173,7 @@ struct Schedule {
 //   cut      17.5 (25.5) + 1.7 (1.75) a key tile of a CTA's share (set-up, partials and merge in the
 //            constant: it hardly depends on the number of pieces)
 //   grid     5.5 (8) + 1.6 (1.85) a key tile, per wave of units over the SMs
-//   cluster  9.5 (10.5) + 0.8 (2.05) a key tile of a CTA's share, per wave of clusters; how many
+//   cluster  9.5 (10.5) + 0.1 a CTA of the cluster + 0.8 (2.05) a key tile of a CTA's share, per wave of clusters; how many
 //            clusters of c CTAs (one per SM) run at once is cudaOccupancyMaxActiveClusters' answer
 //            for 152 SMs.  One wave for a batch (a second one costs a whole unit when the
 //            sequences are equally long), two otherwise (longer stacks are bound by HBM either way).

@@ -5,7 +5,7 @@
 // Same operation, tiles, GEMMs and softmax as attention_tc.cu.  That kernel's balanced cut needs
 // a schedule walk before the first copy, fp32 partials in global memory and a second kernel to
 // merge them: for a layer of a few us of work these took most of the time (32 MHA heads, 2048 + 31
-// keys: of 25 us, 5.5 us were key tiles; 26.9 -> 14.0 us here).  Here a CTA's work follows from its block index, the
+// keys: of 25 us, 5.5 us were key tiles; 26.9 -> 12.6 us here).  Here a CTA's work follows from its block index, the
 // first copies start as soon as the tree's sizes are read, and the merge is two cluster
 // barriers and one pass over shared memory (no scratch): the partials go to shared memory as they are,
 // and a warp per row weighs and adds them (with the weights applied before, three barriers and 1-2
@@ -15,7 +15,7 @@
 // and warps 6-9 the odd ones, each with S, O, maximum and sum of its own (the TMEM that a second M
 // tile would use), so that a tile's chain (S GEMM, softmax, P V) overlaps the next tile's; the
 // streams are two more partials of the merge.  A key tile takes ~0.8 us this way against ~1.5 us as
-// one stream: 32 MHA heads, 32768 keys 105.7 -> 82.6 us (6.5 TB/s, 0.95 of the HBM copy rate).
+// one stream: 32 MHA heads, 32768 keys 105.7 -> 82.6 us (79.4 with the GEMMs issued as now: 6.6 TB/s).
 //
 // Warp roles (352 threads): warp 0 K producer (and Q), warp 10 V producer (their copies of a paged
 // tile are 16 each: one thread issuing both took longer than a tile's GEMMs), warp 1 TMEM and

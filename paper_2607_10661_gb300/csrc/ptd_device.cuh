@@ -277,9 +277,9 @@ __device__ __forceinline__ void mma_commit(uint32_t bar) {
                : "memory");
 }
 
-// The same issued where `go` is not 0, with A from shared memory or from tensor memory (M x 16, bf16
-// packed two per column).  A
-// descriptor comes as its low word; the high one (strides, version, swizzle) is the same for all.
+// tcgen05.mma as above where `go` is not 0, with A from shared memory or from tensor memory (M x 16,
+// bf16 packed two per column).  A descriptor comes as its low word; the high one (strides, version,
+// swizzle) is the same for all.
 __device__ __forceinline__ void mma_ss_if(uint32_t go, uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t hi,
                                           uint32_t idesc, uint32_t accumulate) {
   asm volatile(

@@ -140,7 +140,7 @@ __device__ __forceinline__ void verify_and_write_warp(const VerifyArgs& va, int 
 //
 // The kernel holds little (40 registers a thread, ~8 KB of shared memory a CTA) so that in the
 // step its CTAs fit beside the attention's and run while that does (`beside`, see below): a
-// batched paged step 82.4 -> 56.2 us, one 8-head layer with 63 rows of 128256 logits 68.5 -> 30,
+// batched paged step 82.4 -> 55 us, one 8-head layer with 63 rows of 128256 logits 68.5 -> 30,
 // the tiny fp32 step 13.4 -> 10.8, the 32-layer step ~240 -> ~236.
 //
 // What bounds it alone: for a few rows the chain of two reads, selection and merge; for many the
