@@ -21,7 +21,7 @@
 // per 32 FMAs, an 8 x 8 tile of O 16 per 64; the pipe gives ~110 FMA per cycle and SM) for many
 // rows, the latency of a tile's chain and the K/V stream for few.  Measured (GB300, one layer,
 // against one CTA per (node, head) over all keys, which read every K/V row T * G times): 32 query
-// / 8 KV heads, D 128, 2048 + 63 keys, 63 nodes 628 -> 69.5 us (31 TFLOP/s; the tensor-core kernel 30.8); the same with one
+// / 8 KV heads, D 128, 2048 + 63 keys, 63 nodes 628 -> 69.5 us (31 TFLOP/s; the tensor-core kernel 29.1); the same with one
 // node 86 -> 26 us; 8 heads, D 64, 256 + 15 keys, 15 nodes 14.5 -> 6.6 us.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
@@ -606,12 +606,12 @@ cudaError_t launch_d(const CUtensorMap& map_k, const CUtensorMap& map_v, const A
   if (units * csize > 0x7fffffffll) return cudaErrorInvalidValue;
   if constexpr (D == 128) {
     // The tensor-core kernel where it is estimated to be faster (us, fitted to measurements of 65
-    // shapes on 152 SMs; of the ones it sends there none is more than 2 % slower for it): here a fixed
+    // shapes on 152 SMs; none of them runs more than 4 % slower than on the other kernel): here a fixed
     // part and a time per key of a CTA's share that depends on the rows of a block and on whether
     // two CTAs share an SM; there a fixed part and a time per tile of 64 keys.  Tensor cores / CUDA
-    // cores, 32 query and 8 KV heads: 63 nodes 64 keys 16.6 / 16.1, 300 keys 15.4 / 21.7, 1000 keys 21.5 /
-    // 43.0, 4000 keys 48.7 / 115.5; 8 heads of one row group: 32 nodes 1000 keys 18.4 / 17.3, 4000 keys
-    // 35.1 / 41.9, 8 nodes 4000 keys 34.7 / 33.2.
+    // cores, 32 query and 8 KV heads: 63 nodes 64 keys 14.1 / 16.4, 300 keys 13.9 / 21.7, 1000 keys 20.0 /
+    // 43.0, 4000 keys 46.4 / 115.5; 8 heads of one row group: 32 nodes 1000 keys 18.4 / 17.2, 4000 keys
+    // 33.9 / 41.9, 8 nodes 4000 keys 34.7 / 33.2.
     const double share = ((keys + csize - 1) / csize + 15) / 16 * 16;
     const double waves = (double)((units * csize + slots - 1) / slots);
     // clusters of c CTAs at one CTA per SM that fit at once, measured on 152 SMs
@@ -628,7 +628,7 @@ cudaError_t launch_d(const CUtensorMap& map_k, const CUtensorMap& map_v, const A
     double t_split = t_here;
     for (int c = 1; c <= kMaxCluster; ++c) {
       const int tiles = (((keys + c - 1) / c + 15) / 16 * 16 + 63) / 64;
-      const double t = (double)((split_units + fit(c) - 1) / fit(c)) * (12. + 3.35 * tiles);
+      const double t = (double)((split_units + fit(c) - 1) / fit(c)) * (11. + 3.25 * tiles);
       if (t < t_split) t_split = t, split_csize = c;
     }
     if (split_csize > 0) return launch_tree_attn_split(p, split_csize, split_blocks, stream);

@@ -23,11 +23,12 @@
 // products), P over the first 96 columns of its set, the P V tile.
 //
 // What bounds it: per tile the GEMMs, 48 instructions of S and 24 of P V in series (~7,400 cycles; the
-// conversions and the softmax run beside them), and about 10 us of set-up (Q and the first tiles
+// conversions and the softmax run beside them), and about 9 us of set-up (Q and the first tiles
 // are read, converted and the code is fetched) and combination.  The tile is 64 keys because the three
 // parts of 128 rows of Q (96 KB) and of K and V (48 KB each) fill shared memory.  Measured (GB300,
 // one layer, against the CUDA-core kernel): 32 query / 8 KV heads, 2048 + 63 keys, 63 nodes 69.2 ->
-// 30.9 us (70 TFLOP/s); 4000 keys 115.5 -> 48.7; 128 nodes, 4000 keys 229 -> 68.
+// 29.1 us (75 TFLOP/s); 4000 keys 115.5 -> 46.4; 128 nodes, 4000 keys 229 -> 64.7.  (Set-up written out
+// per piece, with divisions by the group, and the combination one row after the other: 30.8.)
 //
 // Precision: relative error against 64 bits over 14 shapes drawn for it, at scores of deviation 1/4,
 // 1 and 4: 1.0e-7 .. 1.3e-7, 1.5e-7 .. 1.9e-7, 2.5e-7 .. 4.2e-7; the CUDA-core kernel's, whose chains of
@@ -180,7 +181,7 @@ __device__ __noinline__ float2 plain_row(const AttnParams& p, const float* q, in
 }
 
 __global__ void __launch_bounds__(kThreads, 1)
-    tree_attn_split_kernel(const __grid_constant__ AttnParams p, int csize, int m_blocks) {
+    tree_attn_split_kernel(const __grid_constant__ AttnParams p, int csize, int m_blocks, uint32_t inv_group) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint32_t base = smem_u32(smem_raw);
   const uint32_t pad = (1024u - (base & 1023u)) & 1023u;   // the same in every CTA of the launch
@@ -238,8 +239,10 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (row0 >= M) return;
   const int rows = min(kBM, M - row0);
   const size_t out_row0 = ((size_t)lq * p.n_total + node0) * p.hq + (size_t)hkv * G;   // + node * hq + head
+  // row m's node: m / G by a multiplication (m < 2^16; inv_group = ceil(2^32 / G), 0 for G = 1)
+  auto node_of = [&](int m) { return inv_group != 0u ? (int)__umulhi((uint32_t)m, inv_group) : m; };
   auto q_row = [&](int r) {   // row r of the block in q and out
-    const int m = row0 + r, node = m / G;
+    const int m = row0 + r, node = node_of(m);
     return out_row0 + (size_t)node * p.hq + (m - node * G);
   };
   // this CTA's keys: the rank-th of csize shares, in steps of 16
@@ -385,21 +388,23 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (int i = 0; i < kRowsPerWarp; ++i) store_split(base + off, kKvPart, warp + kRowWarps * i, lane, y[i]);
       fence_proxy_async_smem();
     };
-    // Q in two halves, then the first tile's K: one loop, so that little code is fetched cold
+    // Q in two halves, then the first tile's K, each stored while the next (V last) is on its way: one
+    // loop with one copy of each piece of code, as it is fetched cold
     float4 kx[kRowsPerWarp], vx[kRowsPerWarp];
     if (n_tiles > 0) {
-      load_q(kx, 0);
 #pragma unroll 1
-      for (int j = 0; j < 3; ++j) {
-        if (j == 0)
-          load_q(vx, 1);
+      for (int j = 0; j < 4; ++j) {
+        if (j < 2)
+          load_q(vx, j);
         else
-          load(vx, j == 1 ? kg : vg, 0);
-        const uint32_t part = j < 2 ? kQPart : kKvPart, off = j < 2 ? 0u : kOffK;
+          load(vx, j == 2 ? kg : vg, 0);
+        if (j > 0) {
+          const uint32_t part = j < 3 ? kQPart : kKvPart, off = j < 3 ? 0u : kOffK;
 #pragma unroll
-        for (int i = 0; i < kRowsPerWarp; ++i)
-          store_split(base + off, part, warp + kRowWarps * i + (j == 1 ? kBN : 0), lane, kx[i]);
-        if (j < 2) {
+          for (int i = 0; i < kRowsPerWarp; ++i)
+            store_split(base + off, part, warp + kRowWarps * i + (j == 2 ? kBN : 0), lane, kx[i]);
+        }
+        if (j < 3) {
 #pragma unroll
           for (int i = 0; i < kRowsPerWarp; ++i) kx[i] = vx[i];
         }
@@ -411,7 +416,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     // the row's ancestor mask (walk up the strictly decreasing parents), for keys past the context
     if (k_hi > C && row < rows)
-      for (int a = (row0 + row) / G; a >= 0; a = par_s[a]) {
+      for (int a = node_of(row0 + row); a >= 0; a = par_s[a]) {
         const uint32_t bit = 1u << (a & 31);
 #pragma unroll
         for (int w = 0; w < 4; ++w) am[w] |= (a >> 5) == w ? bit : 0u;
@@ -539,41 +544,46 @@ __global__ void __launch_bounds__(kThreads, 1)
     cluster.sync();
     // ---- combine: CTA r writes the r-th share of the rows, one row per warp at a time
     const int r_lo = rank * rows / csize, r_hi = (rank + 1) * rows / csize;
+    float4 part[kMaxCluster], next[kMaxCluster];
+    float2 ml = make_float2(-INFINITY, 0.f), ml_next = ml;
 #pragma unroll 1
-    for (int r = r_lo + warp; r < r_hi; r += kRowWarps) {
-      float4 part[kMaxCluster];
+    for (int r = r_lo + warp - kRowWarps; r < r_hi; r += kRowWarps) {   // (a row's reads are issued one row ahead)
+      const int rn = r + kRowWarps;
+      if (rn < r_hi) {
+        if (lane < csize) ml_next = *reinterpret_cast<const float2*>(cluster.map_shared_rank(ml_s, lane) + 2 * rn);
 #pragma unroll
-      for (int c = 0; c < kMaxCluster; ++c)
-        if (c < csize)
-          part[c] = *reinterpret_cast<const float4*>(cluster.map_shared_rank(reinterpret_cast<float*>(smem), c) + r * kD +
-                                                     ((lane ^ (r & 7)) << 2));
-      float m = -INFINITY, l = 0.f;
-      if (lane < csize) {
-        const float2 ml = *reinterpret_cast<const float2*>(cluster.map_shared_rank(ml_s, lane) + 2 * r);
-        m = ml.x, l = ml.y;
+        for (int c = 0; c < kMaxCluster; ++c)
+          if (c < csize)
+            next[c] = *reinterpret_cast<const float4*>(cluster.map_shared_rank(reinterpret_cast<float*>(smem), c) +
+                                                       rn * kD + ((lane ^ (rn & 7)) << 2));
       }
-      float mm = m;
+      if (r >= r_lo) {
+        float mm = ml.x;
 #pragma unroll
-      for (int d = 4; d > 0; d >>= 1) mm = fmaxf(mm, __shfl_xor_sync(0xffffffffu, mm, d));
-      const float w = l > 0.f ? exp2f(m - mm) : 0.f;
-      float lw = l * w;
+        for (int d = 4; d > 0; d >>= 1) mm = fmaxf(mm, __shfl_xor_sync(0xffffffffu, mm, d));
+        const float w = ml.y > 0.f ? exp2f(ml.x - mm) : 0.f;
+        float lw = ml.y * w;
 #pragma unroll
-      for (int d = 4; d > 0; d >>= 1) lw += __shfl_xor_sync(0xffffffffu, lw, d);
-      lw = __shfl_sync(0xffffffffu, lw, 0);
-      const float inv = lw > 0.f ? 1.f / lw : 0.f;
-      float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int d = 4; d > 0; d >>= 1) lw += __shfl_xor_sync(0xffffffffu, lw, d);
+        lw = __shfl_sync(0xffffffffu, lw, 0);
+        const float inv = lw > 0.f ? 1.f / lw : 0.f;
+        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-      for (int c = 0; c < kMaxCluster; ++c) {
-        const float wc = __shfl_sync(0xffffffffu, w, c);
-        if (c < csize) {
-          acc.x = fmaf(wc, part[c].x, acc.x);
-          acc.y = fmaf(wc, part[c].y, acc.y);
-          acc.z = fmaf(wc, part[c].z, acc.z);
-          acc.w = fmaf(wc, part[c].w, acc.w);
+        for (int c = 0; c < kMaxCluster; ++c) {
+          const float wc = __shfl_sync(0xffffffffu, w, c);
+          if (c < csize) {
+            acc.x = fmaf(wc, part[c].x, acc.x);
+            acc.y = fmaf(wc, part[c].y, acc.y);
+            acc.z = fmaf(wc, part[c].z, acc.z);
+            acc.w = fmaf(wc, part[c].w, acc.w);
+          }
         }
+        reinterpret_cast<float4*>(static_cast<float*>(p.out) + q_row(r) * kD)[lane] =
+            make_float4(acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv);
       }
-      reinterpret_cast<float4*>(static_cast<float*>(p.out) + q_row(r) * kD)[lane] =
-          make_float4(acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv);
+#pragma unroll
+      for (int c = 0; c < kMaxCluster; ++c) part[c] = next[c];
+      ml = ml_next;
     }
   }
   cluster.sync();   // keep this CTA's shared memory alive until the others have read it
@@ -588,7 +598,8 @@ cudaError_t launch_tree_attn_split(const AttnParams& p, int csize, int m_blocks,
                                              (int)split::kSmemBytes);
   if (e != cudaSuccess) return e;
   return launch_chained(split::tree_attn_split_kernel, dim3((unsigned)grid), dim3(split::kThreads), split::kSmemBytes, stream,
-                        (unsigned)csize, p, csize, m_blocks);
+                        (unsigned)csize, p, csize, m_blocks,
+                        p.group > 1 ? (uint32_t)((0x100000000ull + p.group - 1) / p.group) : 0u);
 }
 
 }  // namespace ptd
