@@ -605,13 +605,13 @@ cudaError_t launch_d(const CUtensorMap& map_k, const CUtensorMap& map_v, const A
   }
   if (units * csize > 0x7fffffffll) return cudaErrorInvalidValue;
   if constexpr (D == 128) {
-    // The tensor-core kernel where it is estimated to be faster (us, fitted to measurements of 65
-    // shapes on 152 SMs; none of them runs more than 4 % slower than on the other kernel): here a fixed
-    // part and a time per key of a CTA's share that depends on the rows of a block and on whether
-    // two CTAs share an SM; there a fixed part and a time per tile of 64 keys.  Tensor cores / CUDA
-    // cores, 32 query and 8 KV heads: 63 nodes 64 keys 14.1 / 16.4, 300 keys 13.9 / 21.7, 1000 keys 20.0 /
-    // 43.0, 4000 keys 46.4 / 115.5; 8 heads of one row group: 32 nodes 1000 keys 18.4 / 17.2, 4000 keys
-    // 33.9 / 41.9, 8 nodes 4000 keys 34.7 / 33.2.
+    // The tensor-core kernel where it is estimated to be faster (us, fitted to measurements of 70
+    // shapes on 152 SMs: one runs 7 % slower than it would on the other kernel, the rest within 4 %):
+    // here a fixed part and a time per key of a CTA's share that depends on the rows of a block and on
+    // whether two CTAs share an SM; there a fixed part, the rows' combination and a time per tile of 64
+    // keys.  Tensor cores / CUDA cores, 32 query and 8 KV heads: 63 nodes 64 keys 14.1 / 16.5, 300 keys
+    // 13.9 / 22.3, 1000 keys 19.9 / 43.7, 4000 keys 46.3 / 117.7; 8 heads without groups: 32 nodes 1000 keys
+    // 17.5 / 17.2, 4000 keys 34.0 / 41.0, 8 nodes 4000 keys 33.6 / 33.2.
     const double share = ((keys + csize - 1) / csize + 15) / 16 * 16;
     const double waves = (double)((units * csize + slots - 1) / slots);
     // clusters of c CTAs at one CTA per SM that fit at once, measured on 152 SMs
@@ -628,7 +628,7 @@ cudaError_t launch_d(const CUtensorMap& map_k, const CUtensorMap& map_v, const A
     double t_split = t_here;
     for (int c = 1; c <= kMaxCluster; ++c) {
       const int tiles = (((keys + c - 1) / c + 15) / 16 * 16 + 63) / 64;
-      const double t = (double)((split_units + fit(c) - 1) / fit(c)) * (11. + 3.25 * tiles);
+      const double t = (double)((split_units + fit(c) - 1) / fit(c)) * (8.5 + 2.5 * (M < 128 ? M : 128) / 128 + 3.25 * tiles);
       if (t < t_split) t_split = t, split_csize = c;
     }
     if (split_csize > 0) return launch_tree_attn_split(p, split_csize, split_blocks, stream);
