@@ -151,6 +151,31 @@ ptd_status ptd_tree_attention(const ptd_tree* tree, const ptd_kv_cache* cache,
                               void* workspace, size_t workspace_bytes,
                               int32_t* dev_status, void* stream);
 
+/* The kernels of ptd_tree_attention.  AUTO is the one with the shortest estimate for the shapes. */
+typedef enum {
+  PTD_ATTN_AUTO = 0,
+  PTD_ATTN_UNIT = 1,         /* bf16: one CTA per (layer, tree, KV head, 256-row block)                  */
+  PTD_ATTN_CUT = 2,          /* bf16: persistent CTAs over equal shares of the key tiles (takes scratch) */
+  PTD_ATTN_CLUSTER = 3,      /* bf16: a cluster of CTAs per (layer, tree, KV head, 256-row block)        */
+  PTD_ATTN_F32_CORES = 4,    /* fp32 on the CUDA cores, a cluster per block of up to 64 rows             */
+  PTD_ATTN_F32_TENSOR = 5    /* fp32, D = 128: operands in three bf16 parts on the tensor cores          */
+} ptd_attn_kernel;
+
+/* The kernel that ptd_tree_attention takes for these shapes with `workspace_bytes` of 16-byte
+ * aligned scratch, and its cluster size (1 for UNIT and CUT).  Host-side only.
+ * PTD_ERR_INVALID_ARG or PTD_ERR_UNSUPPORTED as ptd_tree_attention would return. */
+ptd_status ptd_attention_plan(const ptd_tree* tree, const ptd_kv_cache* cache, int32_t num_q_heads,
+                              int32_t num_layers, size_t workspace_bytes, int32_t* kernel, int32_t* cluster_size);
+
+/* ptd_tree_attention by a named kernel (for tests and measurements): cluster_size 1 .. 8 for CLUSTER
+ * and both F32 kernels, 0 for the others; AUTO with 0 is ptd_tree_attention.  PTD_ERR_UNSUPPORTED where
+ * that kernel does not take the call (dtype, head_dim, missing scratch, grid limits). */
+ptd_status ptd_tree_attention_as(const ptd_tree* tree, const ptd_kv_cache* cache,
+                                 int32_t layer_begin, int32_t num_layers,
+                                 const void* q, int32_t num_q_heads, float scale, void* out,
+                                 void* workspace, size_t workspace_bytes, int32_t* dev_status,
+                                 int32_t kernel, int32_t cluster_size, void* stream);
+
 /* Tree-masked attention for callers that cannot allocate device memory.  Some embedders
  * hand this library only their input and output buffers: a plugin running inside another
  * runtime's engine may have no allocator of its own to ask, and a latency-critical decode

@@ -218,6 +218,56 @@ bool persistent_fits(int units, int n_kt) { return (long long)units * n_kt < (1l
 
 ptd_status cuda_status(cudaError_t e) { return e == cudaSuccess ? PTD_OK : PTD_ERR_CUDA; }
 
+// The kernel that a call with checked arguments takes (ptd_attn_kernel), and its cluster size.
+struct AttnPlan {
+  int kernel, csize;
+};
+
+// `want` / `want_csize`: the caller's (PTD_ATTN_AUTO, 0: the one with the shortest estimate).
+ptd_status plan_attention(const ptd_tree* tree, const ptd_kv_cache* cache, int hq, int layers, size_t scratch_bytes,
+                          int want, int want_csize, AttnPlan* out) {
+  if (want < PTD_ATTN_AUTO || want > PTD_ATTN_F32_TENSOR) return PTD_ERR_INVALID_ARG;
+  const bool clustered = want == PTD_ATTN_CLUSTER || want == PTD_ATTN_F32_CORES || want == PTD_ATTN_F32_TENSOR;
+  if (clustered ? want_csize < 1 || want_csize > 8 : want_csize != 0) return PTD_ERR_INVALID_ARG;
+  const int D = cache->head_dim, sms = num_sms_of_current_device();
+  *out = {want, clustered ? want_csize : 1};
+  if (cache->dtype == PTD_F32) {
+    if (D != 32 && D != 64 && D != 128) return PTD_ERR_UNSUPPORTED;
+    if (want == PTD_ATTN_AUTO) {
+      ptd::AttnParams p = {};
+      p.batch = tree->batch;
+      p.hkv = cache->num_kv_heads;
+      p.group = hq / cache->num_kv_heads;
+      p.head_dim = D;
+      p.layers = layers;
+      p.max_nodes = tree->max_nodes;
+      const ptd::F32Plan f = ptd::choose_tree_attn_f32(p, tree->max_ctx, sms);
+      *out = {f.tensor ? PTD_ATTN_F32_TENSOR : PTD_ATTN_F32_CORES, f.csize};
+      return PTD_OK;
+    }
+    const bool takes = want == PTD_ATTN_F32_CORES || (want == PTD_ATTN_F32_TENSOR && D == 128);
+    return takes ? PTD_OK : PTD_ERR_UNSUPPORTED;
+  }
+  if (!use_tensor_cores(cache)) return PTD_ERR_UNSUPPORTED;
+  int pairs, units, n_kt;
+  tc_geometry(tree, cache, hq, layers, &pairs, &units, &n_kt);
+  if (units <= 0 || n_kt <= 0) return PTD_ERR_INVALID_ARG;
+  const int m_tiles = (tree->max_nodes * (hq / cache->num_kv_heads) + 127) / 128;
+  const bool can_cut = persistent_fits(units, n_kt) &&
+                       scratch_bytes >= persistent_workspace_bytes(units, persistent_ctas(units, n_kt, sms), D);
+  const bool can_cluster =
+      (int64_t)cache->num_kv_heads * pairs <= 65535 && (int64_t)tree->batch * layers <= 65535;
+  if (want == PTD_ATTN_AUTO) {
+    const Schedule s = choose_schedule(units, n_kt, m_tiles, sms, layers, tree->batch, can_cut, can_cluster);
+    *out = {s.kind == Schedule::kCut ? PTD_ATTN_CUT : s.kind == Schedule::kCluster ? PTD_ATTN_CLUSTER : PTD_ATTN_UNIT,
+            s.csize};
+    return PTD_OK;
+  }
+  const bool takes =
+      want == PTD_ATTN_UNIT || (want == PTD_ATTN_CUT && can_cut) || (want == PTD_ATTN_CLUSTER && can_cluster);
+  return takes ? PTD_OK : PTD_ERR_UNSUPPORTED;
+}
+
 }  // namespace
 
 extern "C" {
@@ -267,13 +317,14 @@ size_t ptd_step_workspace_size(const ptd_tree* tree, const ptd_kv_cache* cache, 
 
 // ptd_tree_attention, and besides: the tensor-core kernel's CTA 0 clears zero_count words at
 // zero_ptr after its dependency wait (the step's tail counters), and `beside` launches what runs
-// beside the attention kernel (after it in the stream, before its merge kernel).
+// beside the attention kernel (after it in the stream, before its merge kernel).  kernel, csize: as
+// ptd_tree_attention_as takes them.
 extern "C++" {
 template <typename F>
 static ptd_status tree_attention(const ptd_tree* tree, const ptd_kv_cache* cache, int32_t layer_begin,
                                  int32_t num_layers, const void* q, int32_t num_q_heads, float scale, void* out,
-                                 void* workspace, size_t workspace_bytes, int32_t* dev_status, unsigned int* zero_ptr,
-                                 int zero_count, void* stream, F&& beside) {
+                                 void* workspace, size_t workspace_bytes, int32_t* dev_status, int kernel, int csize,
+                                 unsigned int* zero_ptr, int zero_count, void* stream, F&& beside) {
   g_last_launches = 0;
   ptd_status st = check_tree(tree);
   if (st != PTD_OK) return st;
@@ -283,6 +334,11 @@ static ptd_status tree_attention(const ptd_tree* tree, const ptd_kv_cache* cache
     return PTD_ERR_INVALID_ARG;
   if (!aligned16(q) || !aligned16(out)) return PTD_ERR_INVALID_ARG;
   const int D = cache->head_dim;
+  AttnPlan plan;
+  if ((st = plan_attention(tree, cache, num_q_heads, num_layers,
+                           workspace != nullptr && aligned16(workspace) ? workspace_bytes : 0, kernel, csize, &plan)) !=
+      PTD_OK)
+    return st;
   ptd::AttnParams p = {};
   p.q = q;
   p.out = out;
@@ -314,34 +370,28 @@ static ptd_status tree_attention(const ptd_tree* tree, const ptd_kv_cache* cache
   cudaStream_t s = static_cast<cudaStream_t>(stream);
 
   if (cache->dtype == PTD_F32) {
-    if (D != 32 && D != 64 && D != 128) return PTD_ERR_UNSUPPORTED;
-    CUtensorMap map_k, map_v;
-    const uint32_t rows = (uint32_t)ptd::simt_box_rows(cache->page_size);
-    if (!encode_cache(&map_k, cache, tree->batch, cache->k, 32, rows, true) ||
-        !encode_cache(&map_v, cache, tree->batch, cache->v, (uint32_t)D, rows, false))
-      return PTD_ERR_CUDA;
-    st = cuda_status(
-        ptd::launch_tree_attn_simt(map_k, map_v, p, tree->max_ctx, num_sms_of_current_device(), s));
+    if (plan.kernel == PTD_ATTN_F32_TENSOR) {
+      st = cuda_status(ptd::launch_tree_attn_split(p, plan.csize, s));
+    } else {
+      CUtensorMap map_k, map_v;
+      const uint32_t rows = (uint32_t)ptd::simt_box_rows(cache->page_size);
+      if (!encode_cache(&map_k, cache, tree->batch, cache->k, 32, rows, true) ||
+          !encode_cache(&map_v, cache, tree->batch, cache->v, (uint32_t)D, rows, false))
+        return PTD_ERR_CUDA;
+      st = cuda_status(ptd::launch_tree_attn_simt(map_k, map_v, p, plan.csize, s));
+    }
     if (st == PTD_OK) st = beside();
     if (st == PTD_OK) g_last_launches = 1;
     return st;
   }
-  if (!use_tensor_cores(cache)) return PTD_ERR_UNSUPPORTED;
 
   int pairs, units, n_kt;
   tc_geometry(tree, cache, num_q_heads, num_layers, &pairs, &units, &n_kt);
-  if (units <= 0 || n_kt <= 0) return PTD_ERR_INVALID_ARG;
   p.pairs = pairs;
   const int sms = num_sms_of_current_device();
   const int ctas = persistent_ctas(units, n_kt, sms);
-  const int m_tiles = (tree->max_nodes * (num_q_heads / cache->num_kv_heads) + 127) / 128;
-  const bool can_cut = persistent_fits(units, n_kt) && workspace != nullptr && aligned16(workspace) &&
-                       workspace_bytes >= persistent_workspace_bytes(units, ctas, D);
-  const bool can_cluster = (int64_t)p.hkv * pairs <= 65535 && (int64_t)tree->batch * num_layers <= 65535;
-  const Schedule sched =
-      choose_schedule(units, n_kt, m_tiles, sms, num_layers, tree->batch, can_cut, can_cluster);
   dim3 grid;
-  if (sched.kind == Schedule::kCut) {
+  if (plan.kernel == PTD_ATTN_CUT) {
     p.persistent = 1;
     p.counters = static_cast<unsigned long long*>(workspace);
     p.epoch = next_epoch();
@@ -378,8 +428,8 @@ static ptd_status tree_attention(const ptd_tree* tree, const ptd_kv_cache* cache
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS)
       p.q_tma = 1;
   }
-  if (sched.kind == Schedule::kCluster) {
-    st = cuda_status(ptd::launch_tree_attn_cluster(map_k, map_v, map_q, p, sched.csize, s));
+  if (plan.kernel == PTD_ATTN_CLUSTER) {
+    st = cuda_status(ptd::launch_tree_attn_cluster(map_k, map_v, map_q, p, plan.csize, s));
     if (st == PTD_OK) st = beside();
     if (st == PTD_OK) g_last_launches = 1;
     return st;
@@ -399,7 +449,31 @@ ptd_status ptd_tree_attention(const ptd_tree* tree, const ptd_kv_cache* cache, i
                               int32_t num_layers, const void* q, int32_t num_q_heads, float scale, void* out,
                               void* workspace, size_t workspace_bytes, int32_t* dev_status, void* stream) {
   return tree_attention(tree, cache, layer_begin, num_layers, q, num_q_heads, scale, out, workspace, workspace_bytes,
-                        dev_status, nullptr, 0, stream, [] { return PTD_OK; });
+                        dev_status, PTD_ATTN_AUTO, 0, nullptr, 0, stream, [] { return PTD_OK; });
+}
+
+ptd_status ptd_tree_attention_as(const ptd_tree* tree, const ptd_kv_cache* cache, int32_t layer_begin,
+                                 int32_t num_layers, const void* q, int32_t num_q_heads, float scale, void* out,
+                                 void* workspace, size_t workspace_bytes, int32_t* dev_status, int32_t kernel,
+                                 int32_t cluster_size, void* stream) {
+  return tree_attention(tree, cache, layer_begin, num_layers, q, num_q_heads, scale, out, workspace, workspace_bytes,
+                        dev_status, kernel, cluster_size, nullptr, 0, stream, [] { return PTD_OK; });
+}
+
+ptd_status ptd_attention_plan(const ptd_tree* tree, const ptd_kv_cache* cache, int32_t num_q_heads,
+                              int32_t num_layers, size_t workspace_bytes, int32_t* kernel, int32_t* cluster_size) {
+  ptd_status st = check_tree(tree);
+  if (st != PTD_OK) return st;
+  if ((st = check_cache(cache)) != PTD_OK) return st;
+  if (!kernel || !cluster_size || num_q_heads < 1 || num_layers < 1 || num_layers > cache->num_layers ||
+      num_q_heads % cache->num_kv_heads != 0)
+    return PTD_ERR_INVALID_ARG;
+  AttnPlan plan;
+  if ((st = plan_attention(tree, cache, num_q_heads, num_layers, workspace_bytes, PTD_ATTN_AUTO, 0, &plan)) != PTD_OK)
+    return st;
+  *kernel = plan.kernel;
+  *cluster_size = plan.csize;
+  return PTD_OK;
 }
 
 // Host checks of ptd_topk_draft's arguments (no launch).
@@ -774,7 +848,8 @@ ptd_status ptd_tree_verify_step(const ptd_tree* tree, const ptd_kv_cache* cache,
                       a->topk_val, stream);
   };
   st = tree_attention(tree, cache, 0, cache->num_layers, a->q, a->num_q_heads, a->scale, a->attn_out, a->workspace,
-                      a->workspace_bytes, a->dev_status, tail_counters, zero_count, stream, launch_beside);
+                      a->workspace_bytes, a->dev_status, PTD_ATTN_AUTO, 0, tail_counters, zero_count, stream,
+                      launch_beside);
   if (st != PTD_OK) return st;
   const int total = g_last_launches + 1;   // the attention's and the top-k
   if (fused) {

@@ -49,13 +49,20 @@ cudaError_t launch_tree_attn_tc(const CUtensorMap& map_k, const CUtensorMap& map
 // one CTA per unit.  Programmatic dependent launch.
 cudaError_t launch_tree_attn_cluster(const CUtensorMap& map_k, const CUtensorMap& map_v, const CUtensorMap& map_q,
                                      const AttnParams& p, int csize, cudaStream_t stream);
-// fp32 attention.  map_k: boxes of 32 columns (128-byte swizzle), map_v: of D columns, both of one
-// KV head and simt_box_rows(page_size) rows.
-cudaError_t launch_tree_attn_simt(const CUtensorMap& map_k, const CUtensorMap& map_v, const AttnParams& p, int max_ctx,
-                                  int sms, cudaStream_t stream);
-// fp32 attention on the tensor cores, D = 128: a cluster of `csize` CTAs (csize <= 8) per unit of
-// `m_blocks` blocks of 128 rows.  Programmatic dependent launch.
-cudaError_t launch_tree_attn_split(const AttnParams& p, int csize, int m_blocks, cudaStream_t stream);
+// fp32 attention on the CUDA cores, a cluster of `csize` CTAs (csize <= 8) per block of rows.  map_k:
+// boxes of 32 columns (128-byte swizzle), map_v: of D columns, both of one KV head and
+// simt_box_rows(page_size) rows.
+cudaError_t launch_tree_attn_simt(const CUtensorMap& map_k, const CUtensorMap& map_v, const AttnParams& p, int csize,
+                                  cudaStream_t stream);
+// fp32 attention on the tensor cores, D = 128: a cluster of `csize` CTAs (csize <= 8) per block of 128
+// rows.  Programmatic dependent launch.
+cudaError_t launch_tree_attn_split(const AttnParams& p, int csize, cudaStream_t stream);
+// Which of the two, and the cluster size, from the shapes (batch, hkv, group, head_dim, layers, max_nodes).
+struct F32Plan {
+  bool tensor;
+  int csize;
+};
+F32Plan choose_tree_attn_f32(const AttnParams& p, int max_ctx, int sms);
 inline int simt_box_rows(int page_size) { return page_size > 0 ? 16 : 64; }
 // The merge of the units the persistent cut split, after the attention kernel (programmatic
 // dependent launch): one CTA per unit, the pieces' partials combined in CTA order.

@@ -583,56 +583,18 @@ cudaError_t launch(const CUtensorMap& map_k, const CUtensorMap& map_v, const Att
                             p.group > 1 ? (uint32_t)((0x100000000ull + p.group - 1) / p.group) : 0u);
 }
 
-template <int D>
-cudaError_t launch_d(const CUtensorMap& map_k, const CUtensorMap& map_v, const AttnParams& p, int max_ctx, int sms, cudaStream_t stream) {
-  const int M = p.max_nodes * p.group;
-  // rows per block: the smallest that holds M, up to 64 (two such CTAs fit an SM's shared memory;
-  // 128-row blocks, one per SM, left a unit's cluster of 8 CTAs short of SMs in some GPCs)
+// Rows per block: the smallest that holds M, up to 64 (two such CTAs fit an SM's shared memory;
+// 128-row blocks, one per SM, left a unit's cluster of 8 CTAs short of SMs in some GPCs).
+int block_rows(int M) {
   int bm = 16;
   while (bm < 64 && bm < M) bm *= 2;
-  const int m_blocks = (M + bm - 1) / bm;
-  const long long units = (long long)m_blocks * p.hkv * p.batch * p.layers;
-  // CTAs per unit (a cluster): the split whose waves over the SMs take the fewest keys, a CTA's
-  // fixed part (set-up, combination) counted as 48 keys
-  const int keys = max_ctx + p.max_nodes;
-  const long long slots = 2ll * sms;
-  int csize = 1;
-  double best = 1e300;
-  for (int c = 1; c <= kMaxCluster; ++c) {
-    const double waves = (double)((units * c + slots - 1) / slots);
-    const double cost = waves * (((keys + c - 1) / c + 15) / 16 * 16 + 48);
-    if (cost < best) best = cost, csize = c;
-  }
-  if (units * csize > 0x7fffffffll) return cudaErrorInvalidValue;
-  if constexpr (D == 128) {
-    // The tensor-core kernel where it is estimated to be faster (us, fitted to measurements of 70
-    // shapes on 152 SMs: one runs 7 % slower than it would on the other kernel, the rest within 4 %):
-    // here a fixed part and a time per key of a CTA's share that depends on the rows of a block and on
-    // whether two CTAs share an SM; there a fixed part, the rows' combination and a time per tile of 64
-    // keys.  Tensor cores / CUDA cores, 32 query and 8 KV heads: 63 nodes 64 keys 14.1 / 16.5, 300 keys
-    // 13.9 / 22.3, 1000 keys 19.9 / 43.7, 4000 keys 46.3 / 117.7; 8 heads without groups: 32 nodes 1000 keys
-    // 17.5 / 17.2, 4000 keys 34.0 / 41.0, 8 nodes 4000 keys 33.6 / 33.2.
-    const double share = ((keys + csize - 1) / csize + 15) / 16 * 16;
-    const double waves = (double)((units * csize + slots - 1) / slots);
-    // clusters of c CTAs at one CTA per SM that fit at once, measured on 152 SMs
-    static const int fit152[kMaxCluster + 1] = {0, 152, 76, 46, 36, 28, 23, 15, 15};
-    auto fit = [&](int c) { return fit152[c] * sms / 152 > 0 ? fit152[c] * sms / 152 : 1; };
-    const bool shared_sm = units > fit(csize);
-    const double fixed = bm == 16 ? 5.5 : bm == 32 ? 7.3 : 11.;
-    const double per_key = bm == 16 ? (shared_sm ? 0.085 : 0.054) : bm == 32 ? (shared_sm ? 0.117 : 0.069)
-                                                                            : (shared_sm ? 0.205 : 0.112);
-    const double t_here = waves * (fixed + per_key * share);
-    const int split_blocks = (M + 127) / 128;
-    const long long split_units = (long long)split_blocks * p.hkv * p.batch * p.layers;
-    int split_csize = 0;
-    double t_split = t_here;
-    for (int c = 1; c <= kMaxCluster; ++c) {
-      const int tiles = (((keys + c - 1) / c + 15) / 16 * 16 + 63) / 64;
-      const double t = (double)((split_units + fit(c) - 1) / fit(c)) * (8.5 + 2.5 * (M < 128 ? M : 128) / 128 + 3.25 * tiles);
-      if (t < t_split) t_split = t, split_csize = c;
-    }
-    if (split_csize > 0) return launch_tree_attn_split(p, split_csize, split_blocks, stream);
-  }
+  return bm;
+}
+
+template <int D>
+cudaError_t launch_d(const CUtensorMap& map_k, const CUtensorMap& map_v, const AttnParams& p, int csize, cudaStream_t stream) {
+  const int M = p.max_nodes * p.group, bm = block_rows(M), m_blocks = (M + bm - 1) / bm;
+  if ((long long)m_blocks * p.hkv * p.batch * p.layers * csize > 0x7fffffffll) return cudaErrorInvalidValue;
   switch (bm) {
     case 16:
       return launch<D, 16 / kGroups>(map_k, map_v, p, csize, m_blocks, stream);
@@ -645,15 +607,60 @@ cudaError_t launch_d(const CUtensorMap& map_k, const CUtensorMap& map_v, const A
 
 }  // namespace simt
 
-cudaError_t launch_tree_attn_simt(const CUtensorMap& map_k, const CUtensorMap& map_v, const AttnParams& p, int max_ctx, int sms, cudaStream_t stream) {
+F32Plan choose_tree_attn_f32(const AttnParams& p, int max_ctx, int sms) {
+  using simt::kMaxCluster;
+  const int M = p.max_nodes * p.group, bm = simt::block_rows(M);
+  const long long units = (long long)((M + bm - 1) / bm) * p.hkv * p.batch * p.layers;
+  // CTAs per unit (a cluster): the split whose waves over the SMs take the fewest keys, a CTA's
+  // fixed part (set-up, combination) counted as 48 keys
+  const int keys = max_ctx + p.max_nodes;
+  const long long slots = 2ll * sms;
+  int csize = 1;
+  double best = 1e300;
+  for (int c = 1; c <= kMaxCluster; ++c) {
+    const double waves = (double)((units * c + slots - 1) / slots);
+    const double cost = waves * (((keys + c - 1) / c + 15) / 16 * 16 + 48);
+    if (cost < best) best = cost, csize = c;
+  }
+  if (p.head_dim != 128) return {false, csize};
+  // The tensor-core kernel where it is estimated to be faster (us, fitted to measurements of 70
+  // shapes on 152 SMs: one runs 7 % slower than it would on the other kernel, the rest within 4 %):
+  // on the cores a fixed part and a time per key of a CTA's share that depends on the rows of a block and
+  // on whether two CTAs share an SM; on the tensor cores a fixed part, the rows' combination and a time per tile of 64
+  // keys.  Tensor cores / CUDA cores, 32 query and 8 KV heads: 63 nodes 64 keys 14.1 / 16.5, 300 keys
+  // 13.9 / 22.3, 1000 keys 19.9 / 43.7, 4000 keys 46.3 / 117.7; 8 heads without groups: 32 nodes 1000 keys
+  // 17.5 / 17.2, 4000 keys 34.0 / 41.0, 8 nodes 4000 keys 33.6 / 33.2.
+  const double share = ((keys + csize - 1) / csize + 15) / 16 * 16;
+  const double waves = (double)((units * csize + slots - 1) / slots);
+  // clusters of c CTAs at one CTA per SM that fit at once, measured on 152 SMs
+  static const int fit152[kMaxCluster + 1] = {0, 152, 76, 46, 36, 28, 23, 15, 15};
+  auto fit = [&](int c) { return fit152[c] * sms / 152 > 0 ? fit152[c] * sms / 152 : 1; };
+  const bool shared_sm = units > fit(csize);
+  const double fixed = bm == 16 ? 5.5 : bm == 32 ? 7.3 : 11.;
+  const double per_key = bm == 16 ? (shared_sm ? 0.085 : 0.054) : bm == 32 ? (shared_sm ? 0.117 : 0.069)
+                                                                          : (shared_sm ? 0.205 : 0.112);
+  const double t_here = waves * (fixed + per_key * share);
+  const int split_blocks = (M + 127) / 128;
+  const long long split_units = (long long)split_blocks * p.hkv * p.batch * p.layers;
+  int split_csize = 0;
+  double t_split = t_here;
+  for (int c = 1; c <= kMaxCluster; ++c) {
+    const int tiles = (((keys + c - 1) / c + 15) / 16 * 16 + 63) / 64;
+    const double t = (double)((split_units + fit(c) - 1) / fit(c)) * (8.5 + 2.5 * (M < 128 ? M : 128) / 128 + 3.25 * tiles);
+    if (t < t_split) t_split = t, split_csize = c;
+  }
+  return split_csize > 0 ? F32Plan{true, split_csize} : F32Plan{false, csize};
+}
+
+cudaError_t launch_tree_attn_simt(const CUtensorMap& map_k, const CUtensorMap& map_v, const AttnParams& p, int csize, cudaStream_t stream) {
   if (p.hq > 65535 || p.n_total > 65535 || p.layers > 65535) return cudaErrorInvalidValue;
   switch (p.head_dim) {
     case 32:
-      return simt::launch_d<32>(map_k, map_v, p, max_ctx, sms, stream);
+      return simt::launch_d<32>(map_k, map_v, p, csize, stream);
     case 64:
-      return simt::launch_d<64>(map_k, map_v, p, max_ctx, sms, stream);
+      return simt::launch_d<64>(map_k, map_v, p, csize, stream);
     case 128:
-      return simt::launch_d<128>(map_k, map_v, p, max_ctx, sms, stream);
+      return simt::launch_d<128>(map_k, map_v, p, csize, stream);
     default:
       return cudaErrorInvalidValue;
   }

@@ -591,7 +591,9 @@ __global__ void __launch_bounds__(kThreads, 1)
 
 }  // namespace split
 
-cudaError_t launch_tree_attn_split(const AttnParams& p, int csize, int m_blocks, cudaStream_t stream) {
+cudaError_t launch_tree_attn_split(const AttnParams& p, int csize, cudaStream_t stream) {
+  if (p.hq > 65535 || p.n_total > 65535 || p.layers > 65535) return cudaErrorInvalidValue;
+  const int m_blocks = (p.max_nodes * p.group + split::kBM - 1) / split::kBM;
   const long long grid = (long long)csize * m_blocks * p.hkv * p.batch * p.layers;
   if (grid > 0x7fffffffll) return cudaErrorInvalidValue;
   const cudaError_t e = cudaFuncSetAttribute(split::tree_attn_split_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,

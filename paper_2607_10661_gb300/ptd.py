@@ -33,8 +33,10 @@ EXPORTED = (
     "ptd_draft_tree_update", "ptd_pool_bytes", "ptd_pool_init", "ptd_pool_merge", "ptd_pool_retrieve",
     "ptd_tree_rope_append", "ptd_lm_head_topk_workspace_size", "ptd_lm_head_topk", "ptd_pipeline_create",
     "ptd_pipeline_submit", "ptd_pipeline_wait", "ptd_pipeline_destroy", "ptd_check_bounded_wait",
-    "ptd_step_workspace_size", "ptd_step_topk_policy", "ptd_step_tail",
+    "ptd_step_workspace_size", "ptd_step_topk_policy", "ptd_step_tail", "ptd_attention_plan",
+    "ptd_tree_attention_as",
 )
+ATTN_AUTO, ATTN_UNIT, ATTN_CUT, ATTN_CLUSTER, ATTN_F32_CORES, ATTN_F32_TENSOR = range(6)
 
 
 class PtdError(RuntimeError):
@@ -101,6 +103,10 @@ def lib() -> ctypes.CDLL:
         L.ptd_tree_attention.argtypes = [P(_Tree), P(_Cache), i32, i32, vp, i32, f32, vp, vp, sz, vp, vp]
         L.ptd_tree_attention_noalloc.restype = ctypes.c_int
         L.ptd_tree_attention_noalloc.argtypes = [P(_Tree), P(_Cache), i32, i32, vp, i32, f32, vp, vp, vp]
+        L.ptd_tree_attention_as.restype = ctypes.c_int
+        L.ptd_tree_attention_as.argtypes = [P(_Tree), P(_Cache), i32, i32, vp, i32, f32, vp, vp, sz, vp, i32, i32, vp]
+        L.ptd_attention_plan.restype = ctypes.c_int
+        L.ptd_attention_plan.argtypes = [P(_Tree), P(_Cache), i32, i32, sz, P(i32), P(i32)]
         L.ptd_topk_draft.restype = ctypes.c_int
         L.ptd_topk_draft.argtypes = [vp, ctypes.c_int, i64, i32, i64, i32, vp, vp, vp]
         L.ptd_verify_greedy.restype = ctypes.c_int
@@ -301,6 +307,33 @@ def tree_attention(tree: Tree, cache: KVCache, q: torch.Tensor, out: torch.Tenso
                                   _stream(stream))
     _check(st, "ptd_tree_attention")
     return last_launch_count()
+
+
+def attention_plan(tree: Tree, cache: KVCache, num_q_heads: int, num_layers: Optional[int] = None,
+                   workspace_bytes: int = 0):
+    """ptd_attention_plan: (kernel, cluster size) that tree_attention takes with that much scratch."""
+    n = cache.num_layers if num_layers is None else num_layers
+    kernel, csize = ctypes.c_int32(), ctypes.c_int32()
+    st = lib().ptd_attention_plan(ctypes.byref(tree.c), ctypes.byref(cache.c), num_q_heads, n, workspace_bytes,
+                                  ctypes.byref(kernel), ctypes.byref(csize))
+    _check(st, "ptd_attention_plan")
+    return kernel.value, csize.value
+
+
+def tree_attention_as(kernel: int, cluster_size: int, tree: Tree, cache: KVCache, q: torch.Tensor, out: torch.Tensor,
+                      num_q_heads: int, dev_status: torch.Tensor, layer_begin: int = 0,
+                      num_layers: Optional[int] = None, scale: float = 0.0,
+                      workspace: Optional[torch.Tensor] = None, stream=None) -> int:
+    """ptd_tree_attention_as: tree_attention by a named kernel (ATTN_*)."""
+    n = cache.num_layers if num_layers is None else num_layers
+    st = lib().ptd_tree_attention_as(ctypes.byref(tree.c), ctypes.byref(cache.c), layer_begin, n,
+                                     _dev(q, "q", cache.k.dtype), num_q_heads, float(scale),
+                                     _dev(out, "out", cache.k.dtype),
+                                     None if workspace is None else _dev(workspace, "workspace"),
+                                     0 if workspace is None else workspace.numel() * workspace.element_size(),
+                                     _dev(dev_status, "dev_status", torch.int32), kernel, cluster_size, _stream(stream))
+    _check(st, "ptd_tree_attention_as")
+    return int(lib().ptd_last_launch_count())
 
 
 def topk_draft(logits: torch.Tensor, k: int, out_idx: torch.Tensor, out_val: torch.Tensor,

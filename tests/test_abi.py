@@ -105,6 +105,38 @@ def test_host_checks_reject_without_gpu(lib):
     assert lib.ptd_attention_workspace_size(ctypes.byref(t), ctypes.byref(c), 32, 1) == 0
 
 
+def test_attention_plan_and_named_kernels_check_their_arguments(lib):
+    """The plan needs no GPU; a kernel that does not take a call, and a cluster size out of range, are
+    refused before anything is enqueued."""
+    from paper_2607_10661_gb300 import ptd
+
+    def plan(tree, cache, hq, layers, nbytes):
+        k, c = ctypes.c_int32(), ctypes.c_int32()
+        st = lib.ptd_attention_plan(ctypes.byref(tree), ctypes.byref(cache), hq, layers, nbytes, ctypes.byref(k),
+                                    ctypes.byref(c))
+        return (k.value, c.value) if st == ptd.OK else -st
+
+    t = ptd._Tree(1, 63, 63, 8192, 16, 16, 16)
+    bf, f32 = (ptd._Cache(16, 16, dt, 32, 8, 128, 0, 8300, 0, None, 0) for dt in (ptd.BF16, ptd.F32))
+    need = lib.ptd_attention_workspace_size(ctypes.byref(t), ctypes.byref(bf), 32, 32)
+    assert plan(t, bf, 32, 32, need) == (ptd.ATTN_CUT, 1)
+    assert plan(t, bf, 32, 32, need - 1)[0] == ptd.ATTN_UNIT      # no scratch for the cut
+    assert plan(t, bf, 32, 1, 0)[0] == ptd.ATTN_CLUSTER
+    assert plan(t, f32, 32, 1, 0)[0] == ptd.ATTN_F32_TENSOR
+    assert plan(ptd._Tree(1, 15, 15, 256, 16, 16, 16), ptd._Cache(16, 16, ptd.F32, 1, 8, 64, 0, 300, 0, None, 0), 8, 1,
+                0)[0] == ptd.ATTN_F32_CORES
+    assert plan(t, bf, 30, 1, 0) == -ptd.INVALID_ARG and plan(t, bf, 32, 33, 0) == -ptd.INVALID_ARG
+    named = lambda cache, kernel, csize: lib.ptd_tree_attention_as(
+        ctypes.byref(t), ctypes.byref(cache), 0, 1, 16, 32, 0.0, 16, None, 0, 16, kernel, csize, None)
+    for kernel, csize in ((ptd.ATTN_CLUSTER, 0), (ptd.ATTN_CLUSTER, 9), (ptd.ATTN_UNIT, 1), (6, 0), (-1, 0)):
+        assert named(bf, kernel, csize) == ptd.INVALID_ARG
+    assert named(bf, ptd.ATTN_CUT, 0) == ptd.UNSUPPORTED             # no scratch
+    assert named(bf, ptd.ATTN_F32_CORES, 1) == ptd.UNSUPPORTED
+    assert named(f32, ptd.ATTN_UNIT, 0) == ptd.UNSUPPORTED
+    f32.head_dim = 64
+    assert named(f32, ptd.ATTN_F32_TENSOR, 1) == ptd.UNSUPPORTED
+
+
 def test_binding_rejects_host_tensors_and_bad_dtypes(lib):
     """The Python binding checks device, layout and dtype before any call into the library:
     there is no host fallback, a CPU tensor is an error."""

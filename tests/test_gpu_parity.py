@@ -53,6 +53,29 @@ def _check_attn(got, ref, dtype, what=""):
     assert rel <= REL_RMS, (what, rel)
 
 
+def _run_as(dw, kernel, csize=0):
+    """The attention by a named kernel, into a cleared output; its host copy and the launches."""
+    dw.attn_out.zero_()
+    n = ptd.tree_attention_as(kernel, csize, dw.tree, dw.cache, dw.q, dw.attn_out, dw.w.cfg.hq, dw.dev_status,
+                              workspace=dw.workspace)
+    torch.cuda.synchronize()
+    assert int(dw.dev_status.item()) == 0
+    return dw.attn_out.float().cpu().numpy(), n
+
+
+def _check_auto(dw, *kernels):
+    """The plain call takes one of `kernels`: the same bits as that kernel by name."""
+    nbytes = 0 if dw.workspace is None else dw.workspace.numel()
+    kernel, csize = ptd.attention_plan(dw.tree, dw.cache, dw.w.cfg.hq, workspace_bytes=nbytes)
+    if kernels:
+        assert kernel in kernels
+    _run_as(dw, kernel, csize if kernel not in (ptd.ATTN_UNIT, ptd.ATTN_CUT) else 0)
+    named = dw.attn_out.clone()
+    dw.attention()
+    torch.cuda.synchronize()
+    assert torch.equal(named, dw.attn_out)
+
+
 def _run_attention(w):
     dw = DeviceWorkload(w, with_step_buffers=False)
     dw.attention()
@@ -128,12 +151,9 @@ def test_attention_merge_paths_match_oracle(layers, ctx, launches):
     cfg = syn.shrink(syn.CONFIGS["llama3-8b-gqa"], layers=layers, ctx=(ctx, ctx), vocab=100)
     w = syn.Workload(cfg, 23)
     dw = DeviceWorkload(w, with_step_buffers=False)
-    n = dw.attention()
-    torch.cuda.synchronize()
-    assert int(dw.dev_status.item()) == 0
+    got, n = _run_as(dw, ptd.ATTN_CUT)
     if torch.cuda.get_device_properties(0).multi_processor_count == 152:
         assert n == launches
-    got = dw.attn_out.float().cpu().numpy()
     for l in range(layers):
         _check_attn(got[l][w.nodes_of(0)], _attn_ref(w, l, 0), cfg.dtype, f"layers {layers} l{l}")
 
@@ -150,19 +170,23 @@ def test_attention_merge_paths_match_oracle(layers, ctx, launches):
     (32, 8, 48, (1, 1500), 32, 5, 1),     # ragged trees (one and two M tiles) and contexts
 ])
 def test_attention_cluster_split_matches_oracle(hq, hkv, nodes, ctx, page, batch, layers):
-    """Few short units: a cluster of CTAs per unit in one launch, every unit against the oracle."""
+    """Units by every bf16 kernel, clusters of every size among them (some with CTAs that get no key),
+    every unit against the oracle."""
     over = dict(hq=hq, hkv=hkv, nodes=(min(nodes, 3), nodes) if batch > 1 else (nodes, nodes), ctx=ctx, page_size=page,
                 batch=batch, layers=layers, vocab=100, tree="random-depth", branching=(4, 3, 2, 2, 1, 1), depth_range=(5, 6))
     w = syn.Workload(syn.shrink(syn.CONFIGS["llama3-8b-gqa"], **over), 41)
     dw = DeviceWorkload(w, with_step_buffers=False)
-    n = dw.attention()
-    torch.cuda.synchronize()
-    assert n == 1 and int(dw.dev_status.item()) == 0
-    _check_every_unit(w, dw.attn_out.float().cpu().numpy(), "cluster")
-    first = dw.attn_out.clone()
-    dw.attention()
-    torch.cuda.synchronize()
-    assert torch.equal(first, dw.attn_out)   # partials add up in a fixed order
+    refs = list(_unit_refs(w))
+    for csize in range(1, 9):
+        got, n = _run_as(dw, ptd.ATTN_CLUSTER, csize)
+        assert n == 1
+        _check_units(w, got, f"cluster {csize}", refs)
+        first = dw.attn_out.clone()
+        _run_as(dw, ptd.ATTN_CLUSTER, csize)
+        assert torch.equal(first, dw.attn_out)   # partials add up in a fixed order
+    for kernel in (ptd.ATTN_UNIT, ptd.ATTN_CUT):
+        _check_units(w, _run_as(dw, kernel)[0], f"kernel {kernel}", refs)
+    _check_auto(dw)
 
 
 @pytest.mark.parametrize("layers,hq,hkv,nodes,ctx,page,batch", [
@@ -176,8 +200,8 @@ def test_attention_cut_of_stacks_matches_oracle(layers, hq, hkv, nodes, ctx, pag
     over = dict(hq=hq, hkv=hkv, nodes=nodes, ctx=ctx, page_size=page, batch=batch, layers=layers, vocab=100,
                 tree="binary" if batch == 1 else "random-depth", branching=(4, 3, 2, 2, 1, 1), depth_range=(3, 6))
     w = syn.Workload(syn.shrink(syn.CONFIGS["llama3-8b-gqa"], **over), 43)
-    dw, got = _run_attention(w)
-    _check_every_unit(w, got, "cut")
+    dw = DeviceWorkload(w, with_step_buffers=False)
+    _check_every_unit(w, _run_as(dw, ptd.ATTN_CUT)[0], "cut")
 
 
 @pytest.mark.parametrize("layers,hq,hkv,nodes,ctx", [
@@ -192,12 +216,10 @@ def test_attention_merge_of_many_pieces_matches_oracle(layers, hq, hkv, nodes, c
                 branching=(4, 3, 2, 2, 1, 1), depth_range=(5, 6))
     w = syn.Workload(syn.shrink(syn.CONFIGS["llama3-8b-gqa"], **over), 47)
     dw = DeviceWorkload(w, with_step_buffers=False)
-    n = dw.attention()
-    torch.cuda.synchronize()
-    assert int(dw.dev_status.item()) == 0
+    got, n = _run_as(dw, ptd.ATTN_CUT)
     if torch.cuda.get_device_properties(0).multi_processor_count == 152:
         assert n == 2
-    _check_every_unit(w, dw.attn_out.float().cpu().numpy(), "merge")
+    _check_every_unit(w, got, "merge")
 
 
 def test_attention_peaked_context_exposes_mask():
@@ -231,18 +253,26 @@ def _check_every_unit(w, got, what, layers=None):
     """Oracle attention of every (layer, tree, KV head) unit of a workload, each unit checked
     on its own (a per-unit tolerance, so that one wrong unit cannot hide in a mean over the
     others).  `got` is the kernel's [L][N_tot][Hq][D] output."""
+    _check_units(w, got, what, _unit_refs(w, layers))
+
+
+def _unit_refs(w, layers=None):
+    """((layer, tree), oracle attention) of a workload, one at a time."""
     c = w.cfg
-    G = c.hq // c.hkv
     for l in (range(c.layers) if layers is None else layers):
         q_all = syn.widen(w.q_layer(l), c.dtype)
         kc, vc = (syn.widen(x, c.dtype) for x in w.kv_layer(l))
         for b in range(c.batch):
-            sl = w.nodes_of(b)
-            ref = oracle.tree_attention(q_all[sl], w.seq_view(kc, b), w.seq_view(vc, b), w.trees[b],
-                                        int(w.ctx_lens[b]))
-            for kvh in range(c.hkv):
-                hs = slice(kvh * G, (kvh + 1) * G)
-                _check_attn(got[l][sl][:, hs], ref[:, hs], c.dtype, f"{what} l{l} b{b} kv{kvh}")
+            yield (l, b), oracle.tree_attention(q_all[w.nodes_of(b)], w.seq_view(kc, b), w.seq_view(vc, b), w.trees[b],
+                                                int(w.ctx_lens[b]))
+
+
+def _check_units(w, got, what, refs):
+    G = w.cfg.hq // w.cfg.hkv
+    for (l, b), ref in refs:
+        for kvh in range(w.cfg.hkv):
+            hs = slice(kvh * G, (kvh + 1) * G)
+            _check_attn(got[l][w.nodes_of(b)][:, hs], ref[:, hs], w.cfg.dtype, f"{what} l{l} b{b} kv{kvh}")
 
 
 @pytest.mark.parametrize("hq,hkv,d,nodes,ctx,page,batch,layers", [
@@ -250,19 +280,26 @@ def _check_every_unit(w, got, what, layers=None):
     (2, 2, 64, (16, 16), (15, 15), 0, 1, 1),      # a full 16-row block, fewer keys than one step of each share
     (8, 8, 32, (17, 17), (63, 63), 0, 1, 2),      # 32-row block, a tile of 64 keys and 16 more
     (6, 2, 64, (11, 11), (500, 500), 16, 1, 1),   # 33 rows in a 64-row block, group of 3, pages
-    (8, 2, 128, (32, 32), (1000, 1000), 0, 1, 1),   # 128-row block, full
+    (8, 2, 128, (32, 32), (1000, 1000), 0, 1, 1),   # 128 rows: two full 64-row blocks
     (16, 2, 128, (24, 24), (300, 300), 64, 1, 1),   # 192 rows: three 64-row blocks
-    (28, 4, 128, (128, 128), (70, 70), 0, 1, 1),  # 896 rows: seven 128-row blocks, group of 7
+    (28, 4, 128, (128, 128), (70, 70), 0, 1, 1),  # 896 rows: fourteen 64-row blocks, group of 7
     (8, 4, 64, (3, 70), (1, 900), 32, 4, 2),      # ragged trees and contexts, most blocks partly empty
+    (4, 4, 128, (16, 16), (129, 129), 16, 1, 1),  # D = 128: a full 16-row block, pages, a tile and one key more
+    (6, 2, 128, (10, 10), (260, 260), 0, 1, 1),   # 30 rows in a 32-row block
+    (8, 4, 128, (3, 70), (1, 900), 32, 4, 2),     # 64-row blocks, ragged, pages
 ])
 def test_attention_f32_blocks_match_oracle(hq, hkv, d, nodes, ctx, page, batch, layers):
-    """fp32 attention at the edges of its row blocks (16, 32, 64, 128 rows), key tiles and key
-    shares, every unit."""
+    """fp32 attention on the CUDA cores at the edges of its row blocks (16, 32, 64 rows), key tiles and
+    key shares, and the same shapes on the tensor cores where D = 128; every unit."""
     over = dict(hq=hq, hkv=hkv, d=d, nodes=nodes, ctx=ctx, page_size=page, batch=batch, layers=layers, vocab=100,
                 tree="random-depth" if batch > 1 else "chain", branching=(4, 3, 2, 2, 1, 1), depth_range=(3, 6))
     w = syn.Workload(syn.shrink(syn.CONFIGS["tiny-fp32"], **over), 31)
-    dw, got = _run_attention(w)
-    _check_every_unit(w, got, "f32 blocks")
+    dw = DeviceWorkload(w, with_step_buffers=False)
+    refs = list(_unit_refs(w))
+    for kernel in (ptd.ATTN_F32_CORES, ptd.ATTN_F32_TENSOR) if d == 128 else (ptd.ATTN_F32_CORES,):
+        for csize in (1, 3, 8):
+            _check_units(w, _run_as(dw, kernel, csize)[0], f"f32 kernel {kernel} cluster {csize}", refs)
+    _check_auto(dw)
 
 
 @pytest.mark.parametrize("hq,hkv,nodes,ctx,page,batch,layers", [
@@ -280,8 +317,11 @@ def test_attention_f32_split_matches_oracle(hq, hkv, nodes, ctx, page, batch, la
                 page_size=page, batch=batch, layers=layers, vocab=100, tree="random-depth",
                 branching=(4, 3, 2, 2, 1, 1), depth_range=(5, 6))
     w = syn.Workload(syn.shrink(syn.CONFIGS["tiny-fp32"], **over), 37)
-    dw, got = _run_attention(w)
-    _check_every_unit(w, got, "f32 split")
+    dw = DeviceWorkload(w, with_step_buffers=False)
+    refs = list(_unit_refs(w))
+    for csize in (1, 2, 5, 8):
+        _check_units(w, _run_as(dw, ptd.ATTN_F32_TENSOR, csize)[0], f"f32 split {csize}", refs)
+    _check_auto(dw, ptd.ATTN_F32_TENSOR)
 
 
 def test_attention_f32_split_extreme_values():
@@ -289,8 +329,7 @@ def test_attention_f32_split_extreme_values():
     over = dict(hq=32, hkv=8, d=128, nodes=(63, 63), ctx=(1500, 1500), layers=1, vocab=100, tree="binary")
     w = syn.Workload(syn.shrink(syn.CONFIGS["tiny-fp32"], **over), 53)
     dw = DeviceWorkload(w, with_step_buffers=False)
-    dw.attention()
-    torch.cuda.synchronize()
+    _run_as(dw, ptd.ATTN_F32_TENSOR, 4)
     ref = dw.attn_out.float().clone()
     k, v = dw.k[0], dw.v[0]                  # [batch][slots][KV heads][D]
     v[0, 700, 1, 5] = 3.4e38                 # finite, but not as a bf16
@@ -298,10 +337,8 @@ def test_attention_f32_split_extreme_values():
     v[0, 1200, 3, 11] = float("nan")
     dw.q[0, 7, 16] = float("inf")            # a row of KV head 4
     k[0, 900, 5, 3] = float("nan")           # a key of KV head 5: all its rows
-    dw.attention()
-    torch.cuda.synchronize()
+    _run_as(dw, ptd.ATTN_F32_TENSOR, 4)
     got = dw.attn_out.float()
-    assert int(dw.dev_status.item()) == 0
     touched = torch.zeros_like(ref, dtype=torch.bool)
     touched[0, :, 4:8, 5] = True
     touched[0, :, 8:12, 9] = True
@@ -316,20 +353,20 @@ def test_attention_f32_split_extreme_values():
     assert (got[0, :, 8:12, 9] == float("inf")).all()
 
 
-@pytest.mark.parametrize("hq,hkv,d,nodes,ctx,page", [
-    (8, 8, 64, 15, 40, 0),       # CUDA cores, one column run a lane
-    (8, 8, 32, 31, 100, 16),
-    (32, 8, 128, 31, 60, 0),     # CUDA cores, two blocks of 64 rows
-    (32, 8, 128, 63, 1500, 0),   # tensor cores
+@pytest.mark.parametrize("hq,hkv,d,nodes,ctx,page,kernel", [
+    (8, 8, 64, 15, 40, 0, ptd.ATTN_F32_CORES),       # one column run a lane
+    (8, 8, 32, 31, 100, 16, ptd.ATTN_F32_CORES),
+    (32, 8, 128, 31, 60, 0, ptd.ATTN_F32_CORES),     # two blocks of 64 rows
+    (32, 8, 128, 31, 60, 0, ptd.ATTN_F32_TENSOR),
+    (32, 8, 128, 63, 1500, 0, ptd.ATTN_F32_TENSOR),
 ])
 @pytest.mark.parametrize("value", [float("inf"), float("nan")])
-def test_attention_f32_hidden_values_stay_hidden(hq, hkv, d, nodes, ctx, page, value):
+def test_attention_f32_hidden_values_stay_hidden(hq, hkv, d, nodes, ctx, page, kernel, value):
     """An infinity or NaN in a tree node's V reaches the node and its descendants only."""
     over = dict(hq=hq, hkv=hkv, d=d, nodes=(nodes, nodes), ctx=(ctx, ctx), page_size=page, layers=1, vocab=100, tree="binary")
     w = syn.Workload(syn.shrink(syn.CONFIGS["tiny-fp32"], **over), 59)
     dw = DeviceWorkload(w, with_step_buffers=False)
-    dw.attention()
-    torch.cuda.synchronize()
+    _run_as(dw, kernel, 2)
     ref = dw.attn_out.float().clone()
     bad = 2
     sees = torch.zeros(nodes, dtype=torch.bool, device=ref.device)
@@ -343,10 +380,8 @@ def test_attention_f32_hidden_values_stay_hidden(hq, hkv, d, nodes, ctx, page, v
         dw.v[0][int(dw.block_table[0, slot // page]), slot % page] = value
     else:
         dw.v[0][0, slot] = value
-    dw.attention()
-    torch.cuda.synchronize()
+    _run_as(dw, kernel, 2)
     got = dw.attn_out.float()
-    assert int(dw.dev_status.item()) == 0
     # (a redone row sums in another order: 2 x (ctx + nodes) roundings of terms below max |V| = 6)
     assert torch.allclose(got[0][~sees], ref[0][~sees], rtol=0.0, atol=1e-5)
     assert not torch.isfinite(got[0][sees]).any()
