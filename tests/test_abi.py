@@ -125,6 +125,12 @@ def test_attention_plan_and_named_kernels_check_their_arguments(lib):
     assert plan(t, f32, 32, 1, 0)[0] == ptd.ATTN_F32_TENSOR
     assert plan(ptd._Tree(1, 15, 15, 256, 16, 16, 16), ptd._Cache(16, 16, ptd.F32, 1, 8, 64, 0, 300, 0, None, 0), 8, 1,
                 0)[0] == ptd.ATTN_F32_CORES
+    # stacks of short layers with two M tiles a unit: no cut into pieces of a few key tiles
+    for layers, keys, kinds in ((12, 300, (ptd.ATTN_UNIT,)), (8, 96, (ptd.ATTN_UNIT, ptd.ATTN_CLUSTER)),
+                                (2, 96, (ptd.ATTN_UNIT, ptd.ATTN_CLUSTER)), (4, 2000, (ptd.ATTN_CLUSTER,))):
+        s = ptd._Tree(1, 63, 63, keys, 16, 16, 16)
+        assert plan(s, bf, 32, layers, lib.ptd_attention_workspace_size(ctypes.byref(s), ctypes.byref(bf), 32,
+                                                                        layers))[0] in kinds, (layers, keys)
     assert plan(t, bf, 30, 1, 0) == -ptd.INVALID_ARG and plan(t, bf, 32, 33, 0) == -ptd.INVALID_ARG
     named = lambda cache, kernel, csize: lib.ptd_tree_attention_as(
         ctypes.byref(t), ctypes.byref(cache), 0, 1, 16, 32, 0.0, 16, None, 0, 16, kernel, csize, None)

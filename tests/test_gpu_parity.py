@@ -168,6 +168,7 @@ def test_attention_merge_paths_match_oracle(layers, ctx, launches):
     (16, 2, 128, (129, 129), 64, 1, 1),   # four pairs of M tiles per KV head; fewer key tiles than a cluster holds
     (28, 4, 40, (900, 900), 0, 1, 1),     # group of 7: Q by per-thread loads, two pairs, the last of one M tile
     (32, 8, 48, (1, 1500), 32, 5, 1),     # ragged trees (one and two M tiles) and contexts
+    (32, 8, 63, (1000, 1000), 0, 1, 3),   # a stack of layers, two M tiles a unit
 ])
 def test_attention_cluster_split_matches_oracle(hq, hkv, nodes, ctx, page, batch, layers):
     """Units by every bf16 kernel, clusters of every size among them (some with CTAs that get no key),
