@@ -434,10 +434,10 @@ __global__ void __launch_bounds__(512, 1)
           for (int i = 0; i < NP; ++i)
             if (i < np && r0 + q < r_hi)
               part[q][i] = *(cluster.map_shared_rank(o_s, cta_of(i)) + (size_t)row_of(r0 + q, i) * 32 + lane);
-        float M = ml.y > 0.f ? ml.x : -INFINITY;
+        float M = partial_counts(ml.y) ? ml.x : -INFINITY;
 #pragma unroll
         for (int o = NP / 2; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
-        const float w = ml.y > 0.f ? ptx_exp2(ml.x - M) : 0.f;
+        const float w = partial_counts(ml.y) ? ptx_exp2(ml.x - M) : 0.f;
 #pragma unroll
         for (int q = 0; q < R; ++q) {
           const int r = r0 + q;
@@ -446,7 +446,7 @@ __global__ void __launch_bounds__(512, 1)
 #pragma unroll
           for (int i = 0; i < NP; ++i) {
             const float wi = __shfl_sync(0xffffffffu, w, q * NP + i), l = __shfl_sync(0xffffffffu, ml.y, q * NP + i);
-            if (wi > 0.f) {
+            if (partial_counts(l)) {
               L = fmaf(wi, l, L);
               acc.x = fmaf(wi, part[q][i].x, acc.x);
               acc.y = fmaf(wi, part[q][i].y, acc.y);

@@ -716,14 +716,15 @@ __global__ void __launch_bounds__(kThreads, 1)
       float M = -INFINITY, L = 0.f;
       for (int c = first; c <= last; ++c) {
         const float2 ml = piece_ml(c);
-        if (ml.y > 0.f) M = fmaxf(M, ml.x);
+        if (partial_counts(ml.y)) M = fmaxf(M, ml.x);
       }
       for (int c = first; c <= last; ++c) {
         const float2 ml = piece_ml(c);
-        if (ml.y > 0.f) L += ml.y * ptx_exp2(ml.x - M);
+        if (partial_counts(ml.y)) L += ml.y * ptx_exp2(ml.x - M);
       }
       const float inv = (L > 0.f && !invalid) ? 1.f / L : 0.f;
-      const float w_own = (own && l_own > 0.f) ? ptx_exp2(m_own - M) : 0.f;
+      const bool own_counts = own && partial_counts(l_own);
+      const float w_own = own_counts ? ptx_exp2(m_own - M) : 0.f;
       const size_t orow = (((size_t)rec->s.lq * p.n_total + rec->s.node0 + node) * p.hq + (size_t)rec->s.hkv * G + g) * 128;
       uint4* dst = reinterpret_cast<uint4*>(p.out) + (row_valid ? orow : 0) / 8;
 #pragma unroll 1
@@ -736,7 +737,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             tmem_ld32(tO + (uint32_t)h * 32u, r);
             tmem_ld_wait();
 #pragma unroll
-            for (int d = 0; d < 32; ++d) acc[d] = w_own > 0.f ? fmaf(w_own, __uint_as_float(r[d]), acc[d]) : acc[d];
+            for (int d = 0; d < 32; ++d) acc[d] = own_counts ? fmaf(w_own, __uint_as_float(r[d]), acc[d]) : acc[d];
             continue;
           }
           if (!partial_of(c)) continue;
@@ -754,10 +755,11 @@ __global__ void __launch_bounds__(kThreads, 1)
             o[4 * g + 2] = v4.z;
             o[4 * g + 3] = v4.w;
           }
-          // rows of a piece that saw no key were not written: weight 0 and never read into acc
-          const float wgt = ml.y > 0.f ? ptx_exp2(ml.x - M) : 0.f;
+          // rows of a piece that saw no key were not written: never taken into acc
+          const bool counts = partial_counts(ml.y);
+          const float wgt = counts ? ptx_exp2(ml.x - M) : 0.f;
 #pragma unroll
-          for (int d = 0; d < 32; ++d) acc[d] = wgt > 0.f ? fmaf(wgt, o[d], acc[d]) : acc[d];
+          for (int d = 0; d < 32; ++d) acc[d] = counts ? fmaf(wgt, o[d], acc[d]) : acc[d];
         }
         if (row_valid) {
 #pragma unroll
@@ -1002,17 +1004,17 @@ __global__ void __launch_bounds__(kMergeThreads, 2) tree_attn_merge_kernel(const
   float M = -INFINITY, L = 0.f;
 #pragma unroll
   for (int q = 0; q < kMergeMl; ++q)
-    if (mlc[q].y > 0.f) M = fmaxf(M, mlc[q].x);
+    if (partial_counts(mlc[q].y)) M = fmaxf(M, mlc[q].x);
   for (int c = first + kMergeMl; c <= last; ++c) {
     const float2 ml = piece_ml(c);
-    if (ml.y > 0.f) M = fmaxf(M, ml.x);
+    if (partial_counts(ml.y)) M = fmaxf(M, ml.x);
   }
 #pragma unroll
   for (int q = 0; q < kMergeMl; ++q)
-    if (mlc[q].y > 0.f) L += mlc[q].y * ptx_exp2(mlc[q].x - M);
+    if (partial_counts(mlc[q].y)) L += mlc[q].y * ptx_exp2(mlc[q].x - M);
   for (int c = first + kMergeMl; c <= last; ++c) {
     const float2 ml = piece_ml(c);
-    if (ml.y > 0.f) L += ml.y * ptx_exp2(ml.x - M);
+    if (partial_counts(ml.y)) L += ml.y * ptx_exp2(ml.x - M);
   }
   const float inv = L > 0.f ? 1.f / L : 0.f;
   const size_t orow = (((size_t)lq * p.n_total + node0 + node) * p.hq + (size_t)hkv * G + g) * 128;
@@ -1024,16 +1026,18 @@ __global__ void __launch_bounds__(kMergeThreads, 2) tree_attn_merge_kernel(const
     for (int d = 0; d < kMergeCols; ++d) acc[d] = 0.f;
     for (int c0 = first; c0 <= last; c0 += kMergeBatch) {
       if (h > hs * h_per || c0 > first) load_batch(h, c0);
-      // rows of a piece that saw no key were not written: weight 0 and never taken into acc
+      // rows of a piece that saw no key were not written: never taken into acc
       float wgt[kMergeBatch];
+      bool counts[kMergeBatch];
 #pragma unroll
       for (int q = 0; q < kMergeBatch; ++q) {
         const float2 ml = piece_ml(c0 + q);
-        wgt[q] = ml.y > 0.f ? ptx_exp2(ml.x - M) : 0.f;
+        counts[q] = partial_counts(ml.y);
+        wgt[q] = counts[q] ? ptx_exp2(ml.x - M) : 0.f;
       }
 #pragma unroll
       for (int q = 0; q < kMergeBatch; ++q) {
-        if (wgt[q] > 0.f) {
+        if (counts[q]) {
 #pragma unroll
           for (int g4 = 0; g4 < kVec; ++g4) {
             acc[4 * g4] = fmaf(wgt[q], o[q][g4].x, acc[4 * g4]);

@@ -84,6 +84,10 @@ __device__ __forceinline__ void issue_pv(uint32_t leader, uint32_t s_tmem, uint3
               (acc || kk > 0) ? 1u : 0u);
 }
 
+// A partial (m, l, O) of a row counts unless the row saw no key in it: then l is exactly 0, m = -inf and O
+// was not written.  (Not l > 0: a NaN among the scores makes l NaN, and has to reach the output.)
+__device__ __forceinline__ bool partial_counts(float l) { return !(l == 0.f); }
+
 // Softmax of one key tile of this thread's row: S (TMEM at tS) becomes the bf16 P over its first
 // 64 columns, against the reference maximum m_run (log2 units), which only moves up, and only
 // when a 32-column chunk exceeds it by more than 2^8; then the row sum, O (TMEM at tO, if `has_o`)

@@ -388,6 +388,40 @@ def test_attention_f32_hidden_values_stay_hidden(hq, hkv, d, nodes, ctx, page, k
     assert not torch.isfinite(got[0][sees]).any()
 
 
+@pytest.mark.parametrize("hq,hkv,nodes,ctx,layers,kernel,csize", [
+    (8, 8, 31, 1000, 1, ptd.ATTN_UNIT, 0),
+    (8, 8, 31, 1000, 1, ptd.ATTN_CLUSTER, 1),      # two streams of one CTA
+    (8, 8, 31, 1000, 1, ptd.ATTN_CLUSTER, 3),
+    (32, 8, 63, 1000, 1, ptd.ATTN_CLUSTER, 1),
+    (32, 8, 63, 1000, 1, ptd.ATTN_CLUSTER, 8),
+    (32, 8, 63, 1000, 1, ptd.ATTN_CUT, 0),         # merge kernel, a tile or so a piece
+    (4, 1, 31, 20000, 1, ptd.ATTN_CUT, 0),         # merge kernel, more pieces than it keeps the sums of
+    (32, 8, 63, 1000, 20, ptd.ATTN_CUT, 0),        # pieces merged inside the attention
+])
+def test_attention_bf16_nan_reaches_its_rows(hq, hkv, nodes, ctx, layers, kernel, csize):
+    """A NaN in a committed key makes all rows of its KV head NaN, one in a query row that row, whichever
+    kernel takes the call; every other output keeps its bits."""
+    over = dict(hq=hq, hkv=hkv, nodes=(nodes, nodes), ctx=(ctx, ctx), layers=layers, vocab=100, tree="binary")
+    w = syn.Workload(syn.shrink(syn.CONFIGS["llama3-8b-gqa"], **over), 61)
+    dw = DeviceWorkload(w, with_step_buffers=False)
+    _run_as(dw, kernel, csize)
+    ref = dw.attn_out.clone()
+    assert torch.isfinite(ref).all()
+    G = hq // hkv
+    nan = torch.zeros(ref.shape[:3], dtype=torch.bool, device=ref.device)
+    for layer in {0, layers // 2, layers - 1}:
+        dw.q[layer, nodes // 2, 0, 17] = float("nan")
+        nan[layer, nodes // 2, 0] = True
+        for head, key in ((hkv - 1, ctx - 130 - layer), (hkv // 2, 5)):
+            if hkv > 1:
+                dw.k[layer, 0, key, head, 3] = float("nan")
+                nan[layer, :, head * G:(head + 1) * G] = True
+    _run_as(dw, kernel, csize)
+    got = dw.attn_out
+    assert torch.isnan(got[nan]).all()
+    assert torch.equal(got[~nan], ref[~nan])
+
+
 def test_attention_full_size_llama2_layer():
     """The Llama-2-7B-shaped layer at its own size: 32 MHA heads (M = 31 rows per unit, one
     128-row tcgen05 tile mostly padding), context 2048 (17 key tiles), every head."""
