@@ -209,7 +209,7 @@ ptd_status ptd_tree_attention_noalloc(const ptd_tree* tree, const ptd_kv_cache* 
  *   logits: [rows][row_stride] of `dtype`, the first `vocab` entries of a row are used.
  *   out_idx: [rows][k] int32, out_val: [rows][k] fp32 (exact value of the logit).
  *   Order: value descending; equal values by lower index first; -0.0 equals +0.0.
- *   NaN logits are not supported (their placement is unspecified).
+ *   NaN logits come after every number, lower index first (value: NaN).
  *   1 <= k <= min(PTD_MAX_TOPK, vocab). */
 ptd_status ptd_topk_draft(const void* logits, ptd_dtype dtype, int64_t rows, int32_t vocab,
                           int64_t row_stride, int32_t k, int32_t* out_idx, float* out_val,

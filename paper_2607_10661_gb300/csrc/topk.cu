@@ -7,7 +7,7 @@
 //
 // Order: a 64-bit key (order-preserving bits of the fp32 value) << 32 | ~index, so a
 // larger key is a larger value or, on equal values, a lower index.  -0.0 is folded into
-// +0.0 before the key is formed.
+// +0.0 before the key is formed.  NaN come after every number, in the order of their indices.
 #include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -128,7 +128,8 @@ __device__ __forceinline__ void verify_and_write_warp(const VerifyArgs& va, int 
 //      >= T into a candidate buffer as 64-bit keys, in any order; a candidate's place among
 //      the part's top-k is the number of larger candidates.
 // A part whose candidates do not fit the buffer (long runs of equal values, or fewer than k
-// groups above -inf) selects by k rounds of "largest key below the last".  The parts' keys are
+// groups above -inf), or that has NaN and fewer than k numbers (NaN is never >= T), selects by k
+// rounds of "largest key below the last", so that every entry is written.  The parts' keys are
 // placed among each other the same way:
 //   kCluster, kClusterVerify  in the shared memory of the first CTA of the row's cluster, which
 //       the others write to before they leave;
@@ -378,7 +379,8 @@ __global__ void __launch_bounds__(kThreads, Depth<T, kMode>::kCtas)
                    : "memory");
   };
   const int n = n_cand_s;
-  if (n <= kCand) {
+  const int n_elems = nv * VN + (rank == 0 ? a0 : 0) + (rank == parts - 1 ? vocab - a1 : 0);
+  if (n <= kCand && n >= min(k, n_elems)) {
     for (int i = tid; i < n; i += kThreads) {
       const uint64_t key = cand_s[i];
       int before = 0;
@@ -396,12 +398,12 @@ __global__ void __launch_bounds__(kThreads, Depth<T, kMode>::kCtas)
       }
     }
   } else {
-    // k rounds over the part (rare; every thread takes part)
+    // k rounds over the part (rare; every thread takes part); 0 is below every number's order
     uint64_t last = ~0ull;
     for (int q = 0; q < k; ++q) {
       uint64_t best = 0ull;
       auto take = [&](float f, uint32_t idx) {
-        const uint64_t key = make_key(ordered_bits(f), idx);
+        const uint64_t key = make_key(f == f ? ordered_bits(f) : 0u, idx);
         if (key < last && key > best) best = key;
       };
       if (own_head)

@@ -388,6 +388,58 @@ def test_attention_f32_hidden_values_stay_hidden(hq, hkv, d, nodes, ctx, page, k
     assert not torch.isfinite(got[0][sees]).any()
 
 
+def _nan_rows(vocab, g):
+    """Rows with 0, 1, 3, 17 numbers among NaN of both signs, and one with a few NaN among numbers."""
+    x = np.full((5, vocab), np.nan, np.float32)
+    x[1::2] = np.copysign(x[1::2], -1.0)
+    for r, n in enumerate((0, 1, 3, 17)):
+        at = g.permutation(vocab)[:min(n, vocab)]
+        x[r, at] = g.integers(-4, 5, size=len(at))
+    x[4] = g.integers(-1000, 1000, size=vocab)
+    x[4, g.permutation(vocab)[:3]] = np.nan
+    x[3, 0] = -np.inf
+    return x
+
+
+def _nan_topk(x, k):
+    """Numbers by value and index, then NaN by index."""
+    return np.lexsort((np.broadcast_to(np.arange(x.shape[1]), x.shape), np.where(np.isnan(x), 0, -x), np.isnan(x)),
+                      axis=1)[:, :k]
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("vocab,k", [(3, 3), (16, 16), (35, 16), (1000, 4), (32003, 8), (128256, 4), (128256, 16)])
+def test_topk_rows_of_nan_write_every_entry(vocab, k, dtype):
+    """With fewer than k numbers in a row the rest of its entries are NaN logits, lowest index first."""
+    x = torch.tensor(_nan_rows(vocab, np.random.default_rng([vocab, k])), device="cuda").to(
+        torch.bfloat16 if dtype == "bf16" else torch.float32)
+    idx = torch.full((5, k), -7, dtype=torch.int32, device="cuda")
+    val = torch.full((5, k), -7.0, device="cuda")
+    ptd.topk_draft(x, k, idx, val)
+    torch.cuda.synchronize()
+    ref = _nan_topk(x.float().cpu().numpy(), k)
+    assert np.array_equal(idx.cpu().numpy(), ref)
+    want = np.take_along_axis(x.float().cpu().numpy(), ref, axis=1)
+    assert np.array_equal(val.cpu().numpy(), want, equal_nan=True)
+
+
+@pytest.mark.parametrize("policy", [1, 2])
+def test_step_topk_rows_of_nan_write_every_entry(policy):
+    """The same in the one-call step, clustered and streamed: no token of an earlier step is verified."""
+    w = syn.Workload(syn.shrink(syn.CONFIGS["llama3-8b-gqa"], layers=1, ctx=(300, 300), vocab=70000), 67)
+    dw = DeviceWorkload(w)
+    k = w.cfg.k
+    dw.logits[:5] = torch.tensor(_nan_rows(70000, np.random.default_rng(67)), device="cuda").to(torch.bfloat16)
+    before = ptd.step_topk_policy(policy)
+    try:
+        dw.topk_idx.fill_(-7)
+        dw.step()
+        torch.cuda.synchronize()
+    finally:
+        ptd.step_topk_policy(before)
+    assert np.array_equal(dw.topk_idx.cpu().numpy(), _nan_topk(dw.logits.float().cpu().numpy(), k))
+
+
 @pytest.mark.parametrize("hq,hkv,nodes,ctx,layers,kernel,csize", [
     (8, 8, 31, 1000, 1, ptd.ATTN_UNIT, 0),
     (8, 8, 31, 1000, 1, ptd.ATTN_CLUSTER, 1),      # two streams of one CTA
