@@ -32,6 +32,7 @@
 
 #include "attention.cuh"
 #include "ptd_device.cuh"
+#include "row_division.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -213,7 +214,7 @@ __device__ __noinline__ float2 visible_row(const AttnParams& p, const float* q, 
 template <int D, int RM>
 __global__ void __launch_bounds__(kThreads, 2)
     tree_attn_simt_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
-                          const __grid_constant__ AttnParams p, int csize, int m_blocks, uint32_t inv_group) {
+                          const __grid_constant__ AttnParams p, int csize, int m_blocks, GroupDivisor by_group) {
   using L = Layout<D, RM>;
   constexpr int BM = L::BM;
   constexpr int DC = D / kLanes;            // output columns per thread
@@ -232,8 +233,7 @@ __global__ void __launch_bounds__(kThreads, 2)
   const int lq = u / p.batch;
   const int layer = p.layer_begin + lq;
   const int G = p.group;
-  // row m's node: m / G by a multiplication (m < 2^16; inv_group = ceil(2^32 / G), 0 for G = 1)
-  auto node_of = [&](int m) { return inv_group != 0u ? (int)__umulhi((uint32_t)m, inv_group) : m; };
+  auto node_of = [&](int m) { return divide_by_group(m, by_group); };   // row m's node
   const uint32_t bar_q = smem_u32(sm + L::kBar), bar_k = bar_q + 8, bar_v = bar_q + 16;
   volatile int* abort_flag = reinterpret_cast<volatile int*>(sm + L::kBar + 6);
 
@@ -580,7 +580,7 @@ cudaError_t launch(const CUtensorMap& map_k, const CUtensorMap& map_v, const Att
                                              (int)Layout<D, RM>::kBytes);
   if (e != cudaSuccess) return e;
   return cudaLaunchKernelEx(&cfg, tree_attn_simt_kernel<D, RM>, map_k, map_v, p, csize, m_blocks,
-                            p.group > 1 ? (uint32_t)((0x100000000ull + p.group - 1) / p.group) : 0u);
+                            group_divisor(p.group));
 }
 
 // Rows per block: the smallest that holds M, up to 64 (two such CTAs fit an SM's shared memory;

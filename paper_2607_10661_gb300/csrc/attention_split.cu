@@ -49,6 +49,7 @@
 #include "attention_tc.cuh"
 #include "launch.cuh"
 #include "ptd_device.cuh"
+#include "row_division.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -181,7 +182,7 @@ __device__ __noinline__ float2 plain_row(const AttnParams& p, const float* q, in
 }
 
 __global__ void __launch_bounds__(kThreads, 1)
-    tree_attn_split_kernel(const __grid_constant__ AttnParams p, int csize, int m_blocks, uint32_t inv_group) {
+    tree_attn_split_kernel(const __grid_constant__ AttnParams p, int csize, int m_blocks, GroupDivisor by_group) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint32_t base = smem_u32(smem_raw);
   const uint32_t pad = (1024u - (base & 1023u)) & 1023u;   // the same in every CTA of the launch
@@ -239,8 +240,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (row0 >= M) return;
   const int rows = min(kBM, M - row0);
   const size_t out_row0 = ((size_t)lq * p.n_total + node0) * p.hq + (size_t)hkv * G;   // + node * hq + head
-  // row m's node: m / G by a multiplication (m < 2^16; inv_group = ceil(2^32 / G), 0 for G = 1)
-  auto node_of = [&](int m) { return inv_group != 0u ? (int)__umulhi((uint32_t)m, inv_group) : m; };
+  auto node_of = [&](int m) { return divide_by_group(m, by_group); };   // row m's node
   auto q_row = [&](int r) {   // row r of the block in q and out
     const int m = row0 + r, node = node_of(m);
     return out_row0 + (size_t)node * p.hq + (m - node * G);
@@ -601,7 +601,7 @@ cudaError_t launch_tree_attn_split(const AttnParams& p, int csize, cudaStream_t 
   if (e != cudaSuccess) return e;
   return launch_chained(split::tree_attn_split_kernel, dim3((unsigned)grid), dim3(split::kThreads), split::kSmemBytes, stream,
                         (unsigned)csize, p, csize, m_blocks,
-                        p.group > 1 ? (uint32_t)((0x100000000ull + p.group - 1) / p.group) : 0u);
+                        group_divisor(p.group));
 }
 
 }  // namespace ptd

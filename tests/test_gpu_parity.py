@@ -325,6 +325,32 @@ def test_attention_f32_split_matches_oracle(hq, hkv, nodes, ctx, page, batch, la
     _check_auto(dw, ptd.ATTN_F32_TENSOR)
 
 
+@pytest.mark.parametrize("d,kernel,csize", [(32, ptd.ATTN_F32_CORES, 1), (128, ptd.ATTN_F32_CORES, 2),
+                                            (128, ptd.ATTN_F32_TENSOR, 1)])
+def test_attention_f32_thousands_of_query_heads(d, kernel, csize):
+    """5843 query heads of one KV head, a group size at which m ceil(2^32 / group) / 2^32 takes the last row of
+    128 nodes for one of a node past the tree."""
+    hq, T, C = 5843, 128, 16
+    g = torch.Generator(device="cuda").manual_seed(71)
+    i32 = dict(dtype=torch.int32, device="cuda")
+    q = torch.randn((1, T, hq, d), generator=g, device="cuda")
+    k, v = (torch.randn((1, 1, C + T, 1, d), generator=g, device="cuda") for _ in range(2))
+    # a chain, but node 127 hangs on the root: its row of visible slots differs from its neighbours'
+    offsets, parents = torch.tensor([0, T], **i32), torch.arange(-1, T - 1, **i32)
+    parents[T - 1] = 0
+    ctx, status = torch.tensor([C], **i32), torch.zeros(1, **i32)
+    tree, cache, out = ptd.Tree(offsets, parents, ctx, T, C), ptd.KVCache(k, v, 1, d), torch.zeros_like(q)
+    ptd.tree_attention_as(kernel, csize, tree, cache, q, out, hq, status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    see = torch.ones((T, C + T), dtype=torch.bool, device="cuda").tril(C)
+    see[T - 1, C + 1:C + T - 1] = False
+    for n in (0, 1, 63, 126, 127):
+        s = (q[0, n].double() @ k[0, 0, :, 0].double().T) * d ** -0.5
+        p = torch.softmax(s.masked_fill_(~see[n], float("-inf")), dim=1)
+        assert (out[0, n].double() - p @ v[0, 0, :, 0].double()).abs().max() <= F32_MAX, n
+
+
 def test_attention_f32_split_extreme_values():
     """Values whose nearest bf16 is infinite, infinities and NaN: the affected columns and rows only."""
     over = dict(hq=32, hkv=8, d=128, nodes=(63, 63), ctx=(1500, 1500), layers=1, vocab=100, tree="binary")
