@@ -484,7 +484,7 @@ __global__ void __launch_bounds__(kThreads, 2)
     }
     wild = wild || (x && rg * RM + i < rows);
   }
-  wild = __syncthreads_or(wild) && ok;
+  wild = cta_any_unless_aborted(wild, abort_flag);
 #pragma unroll
   for (int i = 0; i < RM; ++i) {
     const float l = group_sum(l_run[i]);

@@ -102,6 +102,14 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity,
   }
 }
 
+// Whether any thread of the CTA has `any` set and none of its bounded waits gave up (a barrier; every
+// wait of the CTA comes before it).  One answer for all threads, so that they may branch to further
+// barriers on it: their own waits may have ended differently, where what one of them gave up on
+// arrived just before another looked.
+__device__ __forceinline__ bool cta_any_unless_aborted(bool any, volatile int* abort_flag) {
+  return __syncthreads_or(any ? 1 : 0) != 0 && *abort_flag == 0;
+}
+
 // Warp-wide bounded wait: every lane polls, the loop exits for the whole warp at once
 // (so the following .sync.aligned tcgen05 instructions see a converged warp).
 __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag,
