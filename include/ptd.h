@@ -377,9 +377,8 @@ ptd_status ptd_lm_head_topk(const void* hidden, int32_t rows, int64_t hidden_str
 /* One whole tree-verify step on device buffers: attention over all cache layers,
  * top-k of the logits, greedy verification on top-k column 0, KV compaction.
  * Equivalent to ptd_tree_attention, ptd_topk_draft and ptd_verify_and_compact on `stream` (three
- * launches, or four with the attention's merge kernel); the top-k runs beside the attention, so
- * topk_idx, topk_val and the verification's outputs are written while that still reads its inputs
- * and must not overlap them.  When the workspace holds the tail's counters
+ * launches, or four with the attention's merge kernel); the top-k runs beside the attention where
+ * no buffer of the one overlaps what the other writes, else after it.  When the workspace holds the tail's counters
  * (ptd_step_workspace_size) and the logits are bf16, the top-k's CTAs verify the trees as well and
  * the last launch only copies the accepted rows (node_offsets must then run
  * from 0 to total_nodes without decreasing, as ptd_tree states; a tree with an empty or

@@ -792,6 +792,44 @@ int32_t ptd_step_topk_policy(int32_t policy) {
   return g_step_topk.exchange(policy);
 }
 
+// Whether the step's top-k may run beside its attention: nothing that it writes is read or written
+// there, nothing that it reads is written there (`verifies`: it also verifies the trees).
+static bool topk_may_run_beside(const ptd_tree* tree, const ptd_kv_cache* cache, const ptd_step_args* a, bool verifies) {
+  struct Span {
+    const void* p;
+    size_t n;
+  };
+  auto meet = [](const Span& x, const Span& y) {
+    const uintptr_t a0 = reinterpret_cast<uintptr_t>(x.p), b0 = reinterpret_cast<uintptr_t>(y.p);
+    return x.p != nullptr && y.p != nullptr && a0 < b0 + y.n && b0 < a0 + x.n;
+  };
+  const size_t B = (size_t)tree->batch, N = (size_t)tree->total_nodes, es = dtype_size(cache->dtype);
+  const size_t q_bytes = (size_t)cache->num_layers * N * a->num_q_heads * cache->head_dim * es;
+  const size_t kv_bytes = (size_t)cache_rows_per_layer(cache, tree->batch) * cache->num_layers * cache->num_kv_heads *
+                          cache->head_dim * es;
+  const Span attention[9] = {{a->attn_out, q_bytes},   // it writes the first two
+                             {a->workspace, a->workspace_bytes},
+                             {a->q, q_bytes},
+                             {cache->k, kv_bytes},
+                             {cache->v, kv_bytes},
+                             {cache->page_size > 0 ? cache->block_table : nullptr, B * cache->max_pages * 4},
+                             {tree->node_offsets, (B + 1) * 4},
+                             {tree->parents, N * 4},
+                             {tree->ctx_lens, B * 4}};
+  const Span written[5] = {{a->topk_idx, N * a->k * 4},
+                           {a->topk_val, N * a->k * 4},
+                           {a->accepted_nodes, B * tree->max_nodes * 4},
+                           {a->accept_len, B * 4},
+                           {a->bonus_token, B * 4}};
+  const Span read[2] = {{a->logits, N * a->vocab * dtype_size(a->logits_dtype)}, {a->tokens, N * 4}};
+  for (int i = 0; i < (verifies ? 5 : 2); ++i)
+    for (const Span& x : attention)
+      if (meet(written[i], x)) return false;
+  for (const Span& r : read)
+    if (meet(r, attention[0]) || meet(r, attention[1])) return false;
+  return true;
+}
+
 ptd_status ptd_tree_verify_step(const ptd_tree* tree, const ptd_kv_cache* cache, const ptd_step_args* a,
                                 void* stream) {
   g_last_launches = 0;
@@ -806,7 +844,8 @@ ptd_status ptd_tree_verify_step(const ptd_tree* tree, const ptd_kv_cache* cache,
     return st;
   // The top-k is launched right behind the attention kernel and runs beside it: its logits come
   // from the step's forward pass, so it starts on them as soon as the attention lets it be
-  // placed, in what the attention leaves free of each SM.  With room for the tail's counters
+  // placed, in what the attention leaves free of each SM (with buffers that overlap the attention's
+  // it comes after the attention and its merge).  With room for the tail's counters
   // after the attention's scratch (the size given by ptd_step_workspace_size), the tensor-core
   // attention (which clears those counters) and bf16 logits, the top-k also verifies every tree
   // (whoever writes a tree's last row does it) and a copy kernel compacts.  Otherwise verification +
@@ -834,24 +873,26 @@ ptd_status ptd_tree_verify_step(const ptd_tree* tree, const ptd_kv_cache* cache,
   va.accept_len = a->accept_len;
   va.bonus = a->bonus_token;
   va.dev_status = a->dev_status;
-  auto launch_beside = [&]() -> ptd_status {
+  const bool beside = topk_may_run_beside(tree, cache, a, fused);
+  auto launch_tail_topk = [&]() -> ptd_status {
     if (streamed) {
       unsigned long long* slots = reinterpret_cast<unsigned long long*>(
           static_cast<uint8_t*>(a->workspace) + attn_ws + stream_counters_bytes(tree->batch, tree->total_nodes));
-      return cuda_status(ptd::launch_topk_stream(a->logits, tree->total_nodes, a->vocab, a->k, true, a->topk_idx,
+      return cuda_status(ptd::launch_topk_stream(a->logits, tree->total_nodes, a->vocab, a->k, beside, a->topk_idx,
                                                  a->topk_val, a->dev_status, va, tail_counters + tree->batch, slots, s));
     }
     if (fused)
-      return cuda_status(ptd::launch_topk(a->logits, true, tree->total_nodes, a->vocab, a->vocab, a->k, true, a->topk_idx,
-                                          a->topk_val, a->dev_status, &va, sms, s));
-    return topk_draft(a->logits, a->logits_dtype, tree->total_nodes, a->vocab, a->vocab, a->k, true, a->topk_idx,
+      return cuda_status(ptd::launch_topk(a->logits, true, tree->total_nodes, a->vocab, a->vocab, a->k, beside,
+                                          a->topk_idx, a->topk_val, a->dev_status, &va, sms, s));
+    return topk_draft(a->logits, a->logits_dtype, tree->total_nodes, a->vocab, a->vocab, a->k, beside, a->topk_idx,
                       a->topk_val, stream);
   };
   st = tree_attention(tree, cache, 0, cache->num_layers, a->q, a->num_q_heads, a->scale, a->attn_out, a->workspace,
                       a->workspace_bytes, a->dev_status, PTD_ATTN_AUTO, 0, tail_counters, zero_count, stream,
-                      launch_beside);
+                      [&] { return beside ? launch_tail_topk() : PTD_OK; });
   if (st != PTD_OK) return st;
   const int total = g_last_launches + 1;   // the attention's and the top-k
+  if (!beside && (st = launch_tail_topk()) != PTD_OK) return st;
   if (fused) {
     const int row_bytes = cache->num_kv_heads * cache->head_dim * (int)dtype_size(cache->dtype);
     st = cuda_status(ptd::launch_compact(cache->k, cache->v, row_bytes, cache->num_layers, tree->batch, cache->page_size,

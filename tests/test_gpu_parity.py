@@ -449,6 +449,34 @@ def test_topk_rows_of_nan_write_every_entry(vocab, k, dtype):
     assert np.array_equal(val.cpu().numpy(), want, equal_nan=True)
 
 
+@pytest.mark.parametrize("base,over", [
+    ("llama3-8b-gqa", dict(layers=12, ctx=(6000, 6000), vocab=4096)),    # cut and merge kernel
+    ("llama3-8b-gqa", dict(layers=1, ctx=(3000, 3000), vocab=4096)),     # clusters
+    ("tiny-fp32", dict(hq=32, hkv=8, d=128, nodes=(63, 63), ctx=(3000, 3000), tree="binary")),   # verification apart
+])
+def test_step_outputs_over_the_attention_inputs(base, over):
+    """Outputs that lie over the attention's last rows of Q are written after these are read, as the
+    three calls in order would."""
+    w = syn.Workload(syn.shrink(syn.CONFIGS[base], **over), 73)
+    a, b = DeviceWorkload(w), DeviceWorkload(w)
+    a.step()
+    ints = b.q.view(-1).view(torch.int32)
+    n, k, end = w.n_total, w.cfg.k, ints.numel()
+    B, most = w.cfg.batch, w.max_nodes
+    parts = []
+    for shape, dtype in (((n, k), torch.int32), ((n, k), torch.float32), ((B, most), torch.int32), ((B,), torch.int32),
+                         ((B,), torch.int32)):
+        size = int(np.prod(shape))
+        parts.append(ints[end - size:end].view(dtype).view(shape))
+        end -= size
+    b.topk_idx, b.topk_val, b.accepted, b.accept_len, b.bonus = parts
+    b.bufs = ptd.StepBuffers(b.q, w.cfg.hq, b.attn_out, b.logits, k, b.tokens, *parts, b.new_ctx, b.dev_status, b.workspace)
+    b.step()
+    torch.cuda.synchronize()
+    for name in ("attn_out", "topk_idx", "topk_val", "accepted", "accept_len", "bonus", "new_ctx", "k", "v", "dev_status"):
+        assert torch.equal(getattr(a, name), getattr(b, name)), name
+
+
 @pytest.mark.parametrize("policy", [1, 2])
 def test_step_topk_rows_of_nan_write_every_entry(policy):
     """The same in the one-call step, clustered and streamed: no token of an earlier step is verified."""
