@@ -1,6 +1,7 @@
 // Tree-masked attention in fp32 on the tensor cores (tcgen05), D = 128: every fp32 operand is split
-// exactly into three bf16 parts, x = h + m + l (each the nearest bf16 to what is left), and a product
-// x y is taken as the six partial products
+// into three bf16 parts, x = h + m + l (each the nearest bf16 to what is left; exact from 2^-110 up, below
+// that off by at most 2^-134, half of bf16's smallest subnormal), and a product x y is taken as the six
+// partial products
 //   h l' + l h' + m m' + h m' + m h' + h h'
 // (exact in fp32, summed in fp32; what is left out is below 2^-26 of x y).  The small ones are
 // summed first and apart from h h'.
@@ -36,8 +37,12 @@
 // truncates its fp32 sums, so few h h' are chained: four instructions per accumulator of S, four per
 // tile of O.
 //
-// A row that comes out infinite or NaN (an input that is, or whose nearest bf16 is, or an overflow) is
-// taken again, over its CTA's share of the keys, by plain fp32 loops.
+// A row is taken again, over its CTA's share of the keys, by plain fp32 loops where the parts do not
+// carry it: one that comes out infinite or NaN (an input that is, or whose nearest bf16 is, or an
+// overflow); one with a column below 2^-88 (the 2^-134 then count: V of 2^-120 was off by 4e-5); and all
+// rows of a CTA that meets an operand of 2^90 or more (which the 2^-134 of its partner, or of a
+// probability, may stand against: Q of 2^120 on K of 2^-120 was off by 4e-5).  Such inputs run at a
+// fraction of the speed.
 #include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -75,10 +80,13 @@ constexpr uint32_t kOffPar = kOffMl + kBM * 8;     // the tree's parents
 constexpr uint32_t kOffBar = kOffPar + kMaxNodes * 4;   // k and p ready, o full, drain, s full[2]
 constexpr uint32_t kOffTmem = kOffBar + 6 * 8;
 constexpr uint32_t kOffAbort = kOffTmem + 4;
-constexpr uint32_t kSmemBytes = kOffAbort + 4 + 1024;   // slack to align the base to 1024 B
+constexpr uint32_t kOffHuge = kOffAbort + 4;
+constexpr uint32_t kSmemBytes = kOffHuge + 4 + 1024;   // slack to align the base to 1024 B
 static_assert(kSmemBytes <= 232448, "shared memory budget");
 // O of the block, fp32 [kBM][kD], over Q at the end: 16-byte chunk c of row r at c ^ (r & 7)
 static_assert(kBM * kD * 4 <= 3 * kQPart, "O lies over Q");
+
+constexpr float kHuge = 0x1p90f, kTiny = 0x1p-88f;   // operands from which, columns of O up to which plain loops run
 
 constexpr uint32_t kTmemCols = 512;
 constexpr uint32_t kSetCols = 192;             // S set: h h' (columns 0-63) | h h' (64-127) | the rest
@@ -205,6 +213,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   // one per S set: a set is written again only after the row warps have passed its last S
   auto s_full = [&](int t) { return k_ready + 32 + 8u * (uint32_t)(t & 1); };
   volatile int* const abort_flag = reinterpret_cast<volatile int*>(smem + kOffAbort);
+  volatile int* const huge_s = reinterpret_cast<volatile int*>(smem + kOffHuge);   // an operand reached kHuge
   float* const x_s = reinterpret_cast<float*>(smem + kOffX);
   float* const ml_s = reinterpret_cast<float*>(smem + kOffMl);
   int* const par_s = reinterpret_cast<int*>(smem + kOffPar);
@@ -217,6 +226,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     mbar_init(o_full, 1);
     mbar_init(drain, 1);
     *abort_flag = 0;
+    *huge_s = 0;
     fence_mbar_init();
   }
   grid_dependency_wait();   // the trees, Q, the cache and the output belong to the stream's previous work
@@ -383,6 +393,17 @@ __global__ void __launch_bounds__(kThreads, 1)
     float m_run = -INFINITY, l_run = 0.f;   // running maximum (log2 units), this thread's share of the row sum
     float o[64];                            // columns [64 half, 64 half + 64) of the row
     uint32_t am[4] = {0, 0, 0, 0};
+    auto note = [&](const float4(&y)[kRowsPerWarp]) {
+      float m[4] = {0.f, 0.f, 0.f, 0.f};   // (four chains: one of sixteen maxima takes 29.55 us instead of 29.41, 63 nodes over 2048 keys)
+#pragma unroll
+      for (int i = 0; i < kRowsPerWarp; i += 2) {
+        m[0] = fmax3(fabsf(y[i].x), fabsf(y[i].y), m[0]);
+        m[1] = fmax3(fabsf(y[i].z), fabsf(y[i].w), m[1]);
+        m[2] = fmax3(fabsf(y[i + 1].x), fabsf(y[i + 1].y), m[2]);
+        m[3] = fmax3(fabsf(y[i + 1].z), fabsf(y[i + 1].w), m[3]);
+      }
+      if (fmaxf(fmax3(m[0], m[1], m[2]), m[3]) >= kHuge) *huge_s = 1;
+    };
     auto store = [&](uint32_t off, const float4(&y)[kRowsPerWarp]) {
 #pragma unroll
       for (int i = 0; i < kRowsPerWarp; ++i) store_split(base + off, kKvPart, warp + kRowWarps * i, lane, y[i]);
@@ -403,6 +424,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
           for (int i = 0; i < kRowsPerWarp; ++i)
             store_split(base + off, part, warp + kRowWarps * i + (j == 2 ? kBN : 0), lane, kx[i]);
+          note(kx);
         }
         if (j < 3) {
 #pragma unroll
@@ -448,6 +470,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         store(kOffK, kx);
         __syncwarp();
         if (lane == 0) mbar_arrive(k_ready);
+        note(kx);
         if (t + 2 < n_tiles) load(kx, kg, t + 2);
       }
       // ---- S, mask, row maximum, P
@@ -509,18 +532,25 @@ __global__ void __launch_bounds__(kThreads, 1)
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(p_ready);
+      note(vx);
       if (t + 1 < n_tiles) load(vx, vg, t + 1);
     }
     if (n_tiles > 0) add_tile(n_tiles - 1);
-    // ---- a row that is not finite: the share again, in plain fp32
+    // ---- a row that the parts do not carry (see above): the share again, in plain fp32
     bool redo = !(fabsf(l_run) < INFINITY);
+    uint32_t least = 0xFFFFFFFFu, most = 0u;   // magnitudes as integers, less one: 0 is the largest of all
 #pragma unroll
-    for (int c = 0; c < 64; ++c) redo = redo || !(fabsf(o[c]) < INFINITY);
+    for (int c = 0; c < 64; ++c) {
+      const uint32_t a = 2u * __float_as_uint(o[c]);
+      least = min(least, a - 1u);
+      most = max(most, a);
+    }
+    redo = redo || most >= 2u * 0x7F800000u || least < 2u * __float_as_uint(kTiny) - 1u;
     {   // for both halves of the row
       float* const xt = x_s + (n_tiles & 1) * 2 * kBM;
       xt[half * kBM + row] = redo ? 1.f : 0.f;
-      asm volatile("bar.sync %0, 64;" ::"r"(1 + (warp & 3)) : "memory");
-      redo = redo || xt[(half ^ 1) * kBM + row] != 0.f;
+      asm volatile("bar.sync 5, 256;" ::: "memory");   // the row warps
+      redo = redo || xt[(half ^ 1) * kBM + row] != 0.f || *huge_s != 0;
     }
     // ---- this CTA's partial rows into shared memory (over Q: the last P V followed every S)
     float* const dst = reinterpret_cast<float*>(smem) + row * kD;

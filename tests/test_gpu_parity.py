@@ -351,6 +351,38 @@ def test_attention_f32_thousands_of_query_heads(d, kernel, csize):
         assert (out[0, n].double() - p @ v[0, 0, :, 0].double()).abs().max() <= F32_MAX, n
 
 
+@pytest.mark.parametrize("kernel", [ptd.ATTN_F32_CORES, ptd.ATTN_F32_TENSOR])
+@pytest.mark.parametrize("q_exp,k_exp,v_exp", [
+    (0, 0, 0), (0, 0, -90), (0, 0, -105), (0, 0, -114), (0, 0, -120),   # V down to where its third bf16 part is 0
+    (0, 0, 80), (0, 0, 120), (120, -120, 0), (-121, 121, 0), (60, -60, -60)])
+def test_attention_f32_scales(q_exp, k_exp, v_exp, kernel):
+    """fp32 accuracy over the range of fp32: Q, K and V scaled by powers of two, V up on one key only, whose
+    probability is below 2^-100 in some rows."""
+    hq, hkv, T, C, d = 32, 8, 40, 600, 128
+    g = torch.Generator(device="cuda").manual_seed(79)
+    i32 = dict(dtype=torch.int32, device="cuda")
+    q = torch.randn((1, T, hq, d), generator=g, device="cuda")
+    k, v = (torch.randn((1, 1, C + T, hkv, d), generator=g, device="cuda") for _ in range(2))
+    if v_exp > 0:
+        v[0, 0, 300] *= 2.0 ** v_exp
+        k[0, 0, 300] *= 30.0
+    q, k, v = q * 2.0 ** q_exp, k * 2.0 ** k_exp, v * 2.0 ** min(v_exp, 0)
+    tree = ptd.Tree(torch.tensor([0, T], **i32), torch.arange(-1, T - 1, **i32), torch.tensor([C], **i32), T, C)
+    out, status = torch.zeros_like(q), torch.zeros(1, **i32)
+    ptd.tree_attention_as(kernel, 2, tree, ptd.KVCache(k, v, hkv, d), q, out, hq, status)
+    torch.cuda.synchronize()
+    assert int(status.item()) == 0
+    see = torch.ones((T, C + T), dtype=torch.bool, device="cuda").tril(C)
+    kd, vd = (x[0, 0].double().repeat_interleave(hq // hkv, 1).transpose(0, 1) for x in (k, v))
+    p = torch.softmax((q[0].double().transpose(0, 1) @ kd.mT * d ** -0.5).masked_fill(~see, float("-inf")), dim=2)
+    ref = (p @ vd).transpose(0, 1)
+    err = out[0].double() - ref
+    # row by row too, as the large V makes rows of very different size; a row's worst: its scores, of up to
+    # 120 there, are rounded at 2^-24 of that and more than once
+    rows, total = (err.norm(dim=2) / ref.norm(dim=2)).max(), err.norm() / ref.norm()
+    assert rows <= 4e-5 and total <= 2e-6, (rows, total)
+
+
 def test_attention_f32_split_extreme_values():
     """Values whose nearest bf16 is infinite, infinities and NaN: the affected columns and rows only."""
     over = dict(hq=32, hkv=8, d=128, nodes=(63, 63), ctx=(1500, 1500), layers=1, vocab=100, tree="binary")
