@@ -32,9 +32,16 @@ struct Args {
   PyObject* const* a;
   Py_ssize_t n, i = 0;
   bool ok = true;
+  PyObject* kept[3] = {};   // the structures read, held until the call has returned
+  int n_kept = 0;
   Args(PyObject* const* args, Py_ssize_t count, Py_ssize_t want) : a(args), n(count) {
     ok = count == want && g_tensor != nullptr;
   }
+  ~Args() {
+    while (n_kept > 0) Py_DECREF(kept[--n_kept]);
+  }
+  Args(const Args&) = delete;
+  Args& operator=(const Args&) = delete;
   void fail() {
     ok = false;
     PyErr_Clear();
@@ -156,7 +163,8 @@ struct Args {
     if (PyErr_Occurred()) fail();
     return (float)v;
   }
-  // the ctypes structure in the attribute `c` of a Tree, KVCache or StepBuffers
+  // the ctypes structure in the attribute `c` of a Tree, KVCache or StepBuffers (the attribute may be
+  // a new object at each read, or be replaced by another thread while the call runs without the lock)
   template <typename S>
   S* structure() {
     PyObject* o = next();
@@ -165,11 +173,15 @@ struct Args {
     Py_buffer v;
     S* p = nullptr;
     if (c != nullptr && PyObject_GetBuffer(c, &v, PyBUF_SIMPLE) == 0) {
-      if ((size_t)v.len == sizeof(S)) p = static_cast<S*>(v.buf);   // kept by `o`, which the caller holds
+      if ((size_t)v.len == sizeof(S) && n_kept < 3) p = static_cast<S*>(v.buf);
       PyBuffer_Release(&v);
     }
-    Py_XDECREF(c);
-    if (p == nullptr) fail();
+    if (p == nullptr) {
+      Py_XDECREF(c);
+      fail();
+      return nullptr;
+    }
+    kept[n_kept++] = c;
     return p;
   }
   // None (the current stream of the current device) or the stream's address

@@ -1,5 +1,7 @@
 """The native call module (csrc/pycall.cpp): what it does not take goes to the ctypes path, which
 raises the binding's errors; both paths give the same results."""
+import weakref
+
 import numpy as np
 import pytest
 import torch
@@ -28,6 +30,45 @@ def test_native_calls_leave_other_arguments_alone(calls, name):
     for filler in (host, None, 3, [1, 2], 0.5):
         assert f(*([filler] * FUNCTIONS[name])) is None
     assert f() is None and f(*([host] * (FUNCTIONS[name] + 1))) is None
+
+
+def test_native_call_keeps_its_structures(calls):
+    """The ctypes structures of a call live until it returns, also where `c` is made anew at each read
+    (the call is refused by the library's checks: no batch)."""
+    alive = []
+
+    class Holder:
+        def __init__(self, cls):
+            self.cls, self.refs = cls, []
+
+        @property
+        def c(self):
+            s = self.cls()
+            self.refs.append(weakref.ref(s))
+            return s
+
+    tree, cache = Holder(type("T", (ptd._Tree,), {})), Holder(type("C", (ptd._Cache,), {}))
+
+    class FakeTensor:
+        is_cuda, dtype = True, torch.int32
+
+        def is_contiguous(self):
+            return True
+
+        def data_ptr(self):
+            alive.extend(r() is not None for r in tree.refs + cache.refs)
+            return 16
+
+    args = (ptd.LIB_PATH, FakeTensor, torch.int32, torch.float32, torch.bfloat16, lambda d: 0, lambda: 0)
+    try:
+        calls.load(*args)
+        x = FakeTensor()
+        assert calls.kv_compact(tree, cache, x, x, x, 0) == -ptd.INVALID_ARG
+    finally:
+        ptd._calls = None
+        ptd._native()
+    assert len(alive) == 6 and all(alive)
+    assert all(r() is None for r in tree.refs + cache.refs)   # and no longer
 
 
 @pytest.mark.gpu
