@@ -152,6 +152,13 @@ def lib() -> ctypes.CDLL:
     return _lib
 
 
+def _stream_getters():
+    """(address of a device's current stream, current device): torch's raw functions, or the public ones
+    where a torch build has no such names."""
+    return (getattr(torch._C, "_cuda_getCurrentRawStream", None) or (lambda d: torch.cuda.current_stream(d).cuda_stream),
+            getattr(torch._C, "_cuda_getDevice", None) or torch.cuda.current_device)
+
+
 def _native():
     """The native call module bound to the loaded library (raises if either was not built)."""
     global _calls
@@ -159,8 +166,7 @@ def _native():
         lib()
         from . import _ptdcall
 
-        _ptdcall.load(LIB_PATH, torch.Tensor, torch.int32, torch.float32, torch.bfloat16,
-                      torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice)
+        _ptdcall.load(LIB_PATH, torch.Tensor, torch.int32, torch.float32, torch.bfloat16, *_stream_getters())
         _calls = _ptdcall
     return _calls
 

@@ -32,6 +32,23 @@ def test_native_calls_leave_other_arguments_alone(calls, name):
     assert f() is None and f(*([host] * (FUNCTIONS[name] + 1))) is None
 
 
+def test_native_calls_bind_without_the_private_stream_functions(calls, monkeypatch):
+    """A torch without its raw stream and device functions (private names): the public ones are taken."""
+    monkeypatch.delattr(torch._C, "_cuda_getCurrentRawStream", raising=False)
+    monkeypatch.delattr(torch._C, "_cuda_getDevice", raising=False)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda device=None: type("S", (), {"cuda_stream": 4096 + device})())
+    monkeypatch.setattr(torch.cuda, "current_device", lambda: 3)
+    monkeypatch.setattr(ptd, "_calls", None)
+    try:
+        assert ptd._native() is calls
+        stream, device = ptd._stream_getters()
+        assert stream(device()) == 4099
+    finally:
+        monkeypatch.undo()
+        ptd._calls = None
+        ptd._native()
+
+
 def test_native_call_keeps_its_structures(calls):
     """The ctypes structures of a call live until it returns, also where `c` is made anew at each read
     (the call is refused by the library's checks: no batch)."""
