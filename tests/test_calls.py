@@ -143,3 +143,69 @@ def test_native_step_matches_ctypes_step(calls, monkeypatch):
     assert na == nb
     for name in ("attn_out", "topk_idx", "topk_val", "accepted", "accept_len", "bonus", "new_ctx", "k", "v"):
         assert torch.equal(getattr(a, name), getattr(b, name)), name
+
+
+@pytest.mark.gpu
+def test_every_native_call_is_taken_and_matches_ctypes(calls, monkeypatch):
+    """Each function of the module takes its plain arguments (kernels launched, not None) and gives what the
+    ctypes path gives."""
+    from paper_2607_10661_gb300.harness import DeviceWorkload
+
+    taken = {}
+
+    class Record:
+        def __getattr__(self, name):
+            def call(*a):
+                r = getattr(calls, name)(*a)
+                taken[name] = r
+                return r
+
+            return call
+
+    class Refuse:
+        def __getattr__(self, name):
+            return lambda *a: None
+
+    cfg = syn.shrink(syn.CONFIGS["llama3-8b-gqa"], layers=2, ctx=(300, 300), vocab=5000)
+
+    def run_all():
+        """Every call of the binding once; their launches and outputs."""
+        g = torch.Generator(device="cuda").manual_seed(11)
+        i32 = dict(dtype=torch.int32, device="cuda")
+        zeros = lambda *shape: torch.zeros(shape, **i32)
+        dw = DeviceWorkload(syn.Workload(cfg, 7))
+        n, B, k = dw.w.n_total, cfg.batch, cfg.k
+        kv = [torch.randn((2, n, cfg.hkv, cfg.d), generator=g, device="cuda").to(torch.bfloat16) for _ in range(2)]
+        pos = zeros(n)
+        launches = [ptd.tree_rope_append(dw.tree, dw.cache, 0, dw.q, cfg.hq, *kv, 1e4, dw.dev_status, positions_out=pos),
+                    dw.attention(), dw.topk(), dw.verify(), dw.compact()]
+        out = [x.clone() for x in (pos, dw.attn_out, dw.topk_idx, dw.topk_val, dw.accepted, dw.accept_len, dw.bonus,
+                                   dw.new_ctx, dw.k, dw.v)]
+        launches += [dw.verify_and_compact(), dw.step()]
+        out += [x.clone() for x in (dw.accepted, dw.accept_len, dw.bonus, dw.new_ctx, dw.k, dw.v, dw.attn_out)]
+        u, ub = (torch.rand(m, generator=g, device="cuda") for m in (n, B))
+        sampled = zeros(B, dw.w.max_nodes), zeros(B), zeros(B)
+        launches.append(ptd.verify_sampling(dw.tree, dw.tokens, dw.logits, 0.8, u, ub, *sampled, dw.dev_status))
+        hidden, weight = (torch.randn((m, 256), generator=g, device="cuda").to(torch.bfloat16) for m in (n, 3000))
+        idx, val = zeros(n, k), torch.zeros((n, k), device="cuda")
+        ws = torch.empty(ptd.lm_head_workspace_size(n, 3000), dtype=torch.uint8, device="cuda")
+        launches.append(ptd.lm_head_topk(hidden, weight, k, idx, val, ws, dw.dev_status))
+        forest = zeros(1), zeros(1, 128), zeros(1, 128), zeros(1, 128), zeros(1, n)
+        count, parents, tokens = torch.full((1,), n, **i32), dw.parents.view(1, -1), dw.tokens.view(1, -1)
+        launches.append(ptd.draft_tree_update(count, parents, tokens, dw.topk_idx, 2, 4, 6, 128, *forest, dw.dev_status))
+        pool = ptd.CandidatePool(4096, "cuda")
+        launches.append(pool.merge(0, *forest[:3], dw.dev_status))
+        got = zeros(1), zeros(64), zeros(64)
+        launches.append(pool.retrieve(forest[2][0, :1].clone(), 4, 6, 64, *got))
+        torch.cuda.synchronize()
+        assert int(dw.dev_status.item()) == 0
+        return launches, out + [idx, val, *sampled, *forest, *got]
+
+    monkeypatch.setattr(ptd, "_calls", Record())
+    native = run_all()
+    assert set(taken) == set(FUNCTIONS) and all(isinstance(r, int) and r > 0 for r in taken.values()), taken
+    monkeypatch.setattr(ptd, "_calls", Refuse())
+    plain = run_all()
+    assert native[0] == plain[0]
+    for i, (a, b) in enumerate(zip(native[1], plain[1])):
+        assert torch.equal(a, b), i
