@@ -119,8 +119,7 @@ size_t ptd_attention_workspace_size(const ptd_tree* tree, const ptd_kv_cache* ca
  * steps built on it) wants as ptd_step_args.workspace: the attention's scratch
  * (ptd_attention_workspace_size, rounded up to 256 bytes) followed by the tail's: one 4-byte
  * counter per tree and one per node row (together rounded up to 256 bytes), then one slot of
- * 16 eight-byte keys per node row and two per SM of the current device (rounded up to 256
- * bytes).  With that much (and a bf16 cache and bf16 logits whose rows start on 16 bytes,
+ * 16 eight-byte keys per node row (rounded up to 256 bytes).  With that much (and a bf16 cache and bf16 logits whose rows start on 16 bytes,
  * vocab a multiple of 8), the top-k can stream the rows' parts through single CTAs
  * (ptd_step_topk_policy) and verifies every tree (the CTA that completes a tree's last row does
  * it); a copy kernel compacts.  With the tree counters alone the clustered top-k (one cluster per

@@ -152,8 +152,8 @@ size_t tail_counters_bytes(int batch) { return ((size_t)batch * sizeof(unsigned 
 size_t stream_counters_bytes(int batch, int rows) {
   return (((size_t)batch + (size_t)rows) * sizeof(unsigned int) + 255) / 256 * 256;
 }
-size_t stream_tail_bytes(int batch, int rows, int sms) {
-  return stream_counters_bytes(batch, rows) + (ptd::topk_stream_slot_bytes(rows, sms) + 255) / 256 * 256;
+size_t stream_tail_bytes(int batch, int rows) {
+  return stream_counters_bytes(batch, rows) + (ptd::topk_stream_slot_bytes(rows) + 255) / 256 * 256;
 }
 
 // Where the pieces of split units are merged: fewer units than CTAs means many pieces per
@@ -312,7 +312,7 @@ size_t ptd_attention_workspace_size(const ptd_tree* tree, const ptd_kv_cache* ca
 size_t ptd_step_workspace_size(const ptd_tree* tree, const ptd_kv_cache* cache, int32_t num_q_heads) {
   if (check_tree(tree) != PTD_OK || check_cache(cache) != PTD_OK) return 0;
   const size_t attn = ptd_attention_workspace_size(tree, cache, num_q_heads, cache->num_layers);
-  return (attn + 255) / 256 * 256 + stream_tail_bytes(tree->batch, tree->total_nodes, num_sms_of_current_device());
+  return (attn + 255) / 256 * 256 + stream_tail_bytes(tree->batch, tree->total_nodes);
 }
 
 // ptd_tree_attention, and besides: the tensor-core kernel's CTA 0 clears zero_count words at
@@ -765,7 +765,7 @@ int step_tail(const ptd_tree* tree, const ptd_kv_cache* cache, const ptd_step_ar
   const bool tail_ok = use_tensor_cores(cache) && a->logits_dtype == PTD_BF16 && a->workspace &&
                        aligned16(a->workspace);
   const bool can_stream = tail_ok && ptd::topk_stream_ok(a->logits, a->vocab) &&
-                          a->workspace_bytes >= attn_ws + stream_tail_bytes(tree->batch, tree->total_nodes, sms);
+                          a->workspace_bytes >= attn_ws + stream_tail_bytes(tree->batch, tree->total_nodes);
   const bool can_cluster = tail_ok && a->workspace_bytes >= attn_ws + tail_counters_bytes(tree->batch);
   if (can_stream && can_cluster) {
     const int policy = g_step_topk.load();

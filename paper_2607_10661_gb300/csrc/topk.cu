@@ -527,8 +527,8 @@ bool topk_stream_ok(const void* logits, int vocab) {
   return vocab >= 8 && vocab % 8 == 0 && (reinterpret_cast<uintptr_t>(logits) & 15u) == 0;
 }
 
-size_t topk_stream_slot_bytes(int64_t rows, int sms) {
-  return (size_t)(rows + 2 * (int64_t)sms) * topk::kMaxK * sizeof(unsigned long long);
+size_t topk_stream_slot_bytes(int64_t rows) {
+  return (size_t)rows * topk::kMaxK * sizeof(unsigned long long);
 }
 
 cudaError_t launch_topk_stream(const void* logits, int64_t rows, int vocab, int k, bool beside, int32_t* out_idx,

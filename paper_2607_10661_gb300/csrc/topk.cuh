@@ -29,9 +29,9 @@ struct VerifyArgs {
 // The step's streamed top-k with verification (bf16 rows back to back, vocab a multiple of 8,
 // logits 16-byte aligned): parts of the rows without clusters, merged through scratch.
 // row_counters [rows] (and va.counters) must be zero before the launch; slots holds
-// topk_stream_slot_bytes(rows, sms) bytes of scratch (no clearing needed).
+// topk_stream_slot_bytes(rows) bytes of scratch (no clearing needed).
 bool topk_stream_ok(const void* logits, int vocab);
-size_t topk_stream_slot_bytes(int64_t rows, int sms);
+size_t topk_stream_slot_bytes(int64_t rows);
 cudaError_t launch_topk_stream(const void* logits, int64_t rows, int vocab, int k, bool beside, int32_t* out_idx,
                                float* out_val, int32_t* dev_status, const VerifyArgs& va, unsigned int* row_counters,
                                unsigned long long* slots, cudaStream_t stream);

@@ -340,6 +340,11 @@ def test_step_tail_choice(lib):
         assert tail(**ws)[0] == ptd.STEP_TAIL_STREAMED
         assert tail(vocab=128250, **ws)[0] == ptd.STEP_TAIL_CLUSTERED
         assert tail(logits=A * 32 + 8, **ws)[0] == ptd.STEP_TAIL_CLUSTERED
+        # counters of the tree and of 63 rows, then 16 keys a row: enough for the stream, and what the size asks
+        slots_end = (attn + 255) // 256 * 256 + 256 + (63 * 16 * 8 + 255) // 256 * 256
+        assert tail(workspace=A * 64, workspace_bytes=slots_end)[0] == ptd.STEP_TAIL_STREAMED
+        assert tail(workspace=A * 64, workspace_bytes=slots_end - 1)[0] == ptd.STEP_TAIL_CLUSTERED
+        assert full == slots_end
         counters_only = (attn + 255) // 256 * 256 + 256
         assert tail(workspace=A * 64, workspace_bytes=counters_only)[0] == ptd.STEP_TAIL_CLUSTERED
         ptd.step_topk_policy(ptd.STEP_TOPK_CLUSTERED)
