@@ -59,6 +59,9 @@ MEASURED_PEAKS = os.path.join(ROOT, "MEASURED_PEAKS.json")
 STEP_TAILS = {0: "top-k, then verification + compaction in one launch",
               1: "clustered top-k (one cluster per row) verifying the trees, then a compaction kernel",
               2: "streamed top-k (a row's parts in single CTAs that merge through scratch) verifying the trees, then a compaction kernel"}
+# the attention's kernel (ptd_attention_plan)
+ATTENTION_KERNELS = {1: "tree_attn_tc_kernel", 2: "tree_attn_tc_kernel", 3: "tree_attn_cluster_kernel",
+                     4: "tree_attn_simt_kernel", 5: "tree_attn_split_kernel"}
 FALLBACK_HBM_GBS = 6800.0
 FALLBACK_BF16_TFLOPS_SUSTAINED = 1700.0
 NOMINAL_HBM_GBS = 8000.0
@@ -564,7 +567,8 @@ def run_gpu(args, rank: int, world: int, dist):
         roof = {"bound": "hbm", "achieved": round(achieved_gbs, 1), "peak": hbm_peak, "unit": "GB/s",
                 "frac": round(achieved_gbs / hbm_peak, 4), "peak_kind": peak_kind,
                 "tensor_tflops": round(achieved_tf, 1), "tensor_frac": round(achieved_tf / tf_peak, 4)}
-    kernel = "tree_attn_tc_kernel or tree_attn_cluster_kernel" if cfg.dtype == "bf16" else "tree_attn_simt_kernel"
+    kernel = ATTENTION_KERNELS[ptd.attention_plan(dw.tree, dw.cache, cfg.hq, workspace_bytes=(
+        0 if dw.workspace is None else dw.workspace.numel()))[0]]
     if attn_kernels[0] == 2:   # timed from the attention's start to the end of the merge of split units
         kernel += " + tree_attn_merge_kernel"
     roof.update({"kernel": kernel, "traffic": _profiled_traffic(PROFILED_ATTENTION_TRAFFIC, "attention_tc.cu",

@@ -173,9 +173,8 @@ struct Schedule {
 //   cut      17.5 (25.5) + 1.7 (1.75) a key tile of a CTA's share (set-up, partials and merge in the
 //            constant: it hardly depends on the number of pieces)
 //   grid     5.5 (8) + 1.6 (1.85) a key tile, per wave of units over the SMs
-//   cluster  9.5 (10.5) + 0.1 a CTA of the cluster + 0.8 (2.05) a key tile of a CTA's share, per wave of clusters; how many
-//            clusters of c CTAs (one per SM) run at once is cudaOccupancyMaxActiveClusters' answer
-//            for 152 SMs.  One wave for a batch (a second one costs a whole unit when the
+//   cluster  9.5 (10.5) + 0.1 a CTA of the cluster + 0.8 (2.05) a key tile of a CTA's share, per wave of
+//            clusters (clusters_at_once).  One wave for a batch (a second one costs a whole unit when the
 //            sequences are equally long), two otherwise (longer stacks are bound by HBM either way).
 // Measured, cut / cluster: 32 MHA heads, 2079 keys 23.8 / 13.9 us, two such layers 29.1 / 19.0,
 // eight 65.7 / 55.8; 8 KV heads of a 4-head group, 4109 keys and 13 nodes 27.6 / 14.1, 2111 keys
@@ -199,9 +198,8 @@ Schedule choose_schedule(int units, int n_kt, int m_tiles, int sms, int batch, b
     }
   }
   if (can_cluster) {
-    static const int fit152[9] = {0, 152, 76, 46, 36, 28, 23, 15, 15};
     for (int c = 1; c <= 8 && c <= n_kt; ++c) {
-      const int f = fit152[c] * sms / 152, fit = f > 0 ? f : 1;
+      const int fit = ptd::clusters_at_once(c, sms);
       if (units > (batch > 1 ? fit : 2 * fit)) break;
       const double t = waves(fit) * ((two ? 10.5 : 9.5) + 0.1 * c + (n_kt + c - 1) / c * (two ? 2.05 : 0.8));
       if (t < t_best) {
@@ -363,7 +361,6 @@ static ptd_status tree_attention(const ptd_tree* tree, const ptd_kv_cache* cache
   p.num_pages = cache->num_pages;
   p.max_pages = cache->max_pages;
   const float sc = scale > 0.f ? scale : 1.0f / std::sqrt((float)D);
-  p.scale = sc;
   p.scale_log2 = sc * 1.4426950408889634f;
   p.zero_ptr = zero_ptr;
   p.zero_count = zero_ptr != nullptr ? zero_count : 0;
@@ -864,7 +861,6 @@ ptd_status ptd_tree_verify_step(const ptd_tree* tree, const ptd_kv_cache* cache,
   va.node_offsets = tree->node_offsets;
   va.parents = tree->parents;
   va.tokens = a->tokens;
-  va.ctx_lens = tree->ctx_lens;
   va.counters = tail_counters;
   va.batch = tree->batch;
   va.n_total = tree->total_nodes;

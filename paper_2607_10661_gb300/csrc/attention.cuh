@@ -36,7 +36,6 @@ struct AttnParams {
   int q_tma;                   // 1: Q tiles arrive by TMA (map_q), else by per-thread loads
   int page_size, seq_capacity, num_pages, max_pages;
   float scale_log2;            // scale * log2(e)
-  float scale;
 };
 
 size_t tc_smem_bytes();
@@ -45,6 +44,15 @@ size_t tc_smem_bytes();
 // before its first global access.
 cudaError_t launch_tree_attn_tc(const CUtensorMap& map_k, const CUtensorMap& map_v, const CUtensorMap& map_q,
                                 const AttnParams& p, dim3 grid, cudaStream_t stream);
+// How many clusters of c CTAs (1 to 8), each filling an SM, run at once: cudaOccupancyMaxActiveClusters'
+// answers on the 152 SMs of a GB300, whose clusters lie within a GPC; by proportion for another number
+// of SMs (an estimate only, for the choice between kernels).
+inline int clusters_at_once(int c, int sms) {
+  constexpr int fit152[9] = {0, 152, 76, 46, 36, 28, 23, 15, 15};
+  const int f = fit152[c] * sms / 152;
+  return f > 0 ? f : 1;
+}
+
 // Few short units: a cluster of `csize` CTAs per unit (csize <= 8), no scratch; p.pairs set as for
 // one CTA per unit.  Programmatic dependent launch.
 cudaError_t launch_tree_attn_cluster(const CUtensorMap& map_k, const CUtensorMap& map_v, const CUtensorMap& map_q,

@@ -632,9 +632,7 @@ F32Plan choose_tree_attn_f32(const AttnParams& p, int max_ctx, int sms) {
   // 17.5 / 17.2, 4000 keys 34.0 / 41.0, 8 nodes 4000 keys 33.6 / 33.2.
   const double share = ((keys + csize - 1) / csize + 15) / 16 * 16;
   const double waves = (double)((units * csize + slots - 1) / slots);
-  // clusters of c CTAs at one CTA per SM that fit at once, measured on 152 SMs
-  static const int fit152[kMaxCluster + 1] = {0, 152, 76, 46, 36, 28, 23, 15, 15};
-  auto fit = [&](int c) { return fit152[c] * sms / 152 > 0 ? fit152[c] * sms / 152 : 1; };
+  auto fit = [&](int c) { return clusters_at_once(c, sms); };
   const bool shared_sm = units > fit(csize);
   const double fixed = bm == 16 ? 5.5 : bm == 32 ? 7.3 : 11.;
   const double per_key = bm == 16 ? (shared_sm ? 0.085 : 0.054) : bm == 32 ? (shared_sm ? 0.117 : 0.069)

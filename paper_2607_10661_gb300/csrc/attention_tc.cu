@@ -11,7 +11,7 @@
 // nodes x 4 heads = 252 rows, and its keys are cut into 128-key tiles.  Each K/V tile is
 // loaded from HBM once by TMA and used by both M tiles.
 //
-// Schedules.  Persistent (the default when the caller's scratch allows it): the flattened
+// Schedules, one per call (choose_schedule in api.cu).  Persistent (needs the caller's scratch): the flattened
 // (unit, key tile) space is cut into one equal contiguous range per CTA, one CTA per SM, so
 // every SM gets the same number of key tiles whatever the unit count.  Each warp walks its
 // CTA's range as segments (whole units, or a piece of a unit at either end of the range).
@@ -19,7 +19,7 @@
 // last leave an fp32 partial (O unnormalised, running max, row sum); the warp that finishes
 // the last one merges those partials with its own O, still in TMEM.  The softmax warps load
 // the next segment's Q before the epilogue of the current one, so the tensor core does not
-// wait on it.  Grid (fallback without scratch): one CTA per unit.
+// wait on it.  Grid: one CTA per unit.  (The third, a cluster of CTAs per unit, is attention_cluster.cu.)
 //
 // Warp roles (320 threads):
 //   warp 0      TMA producer: K and V tiles into two stage pairs (K_j, V_j | K_j+1, V_j+1).

@@ -12,7 +12,6 @@ struct VerifyArgs {
   const int32_t* node_offsets;   // [batch + 1]
   const int32_t* parents;        // [n_total]
   const int32_t* tokens;         // [n_total]
-  const int32_t* ctx_lens;       // [batch]
   unsigned int* counters;        // [batch] rows done per tree, zero before the launch
   int batch, n_total, max_nodes;
   int32_t* accepted;             // [batch][max_nodes]
