@@ -106,7 +106,6 @@ __global__ void __launch_bounds__(kThreads, 1)
     tc_fence_before();
   }
   // set-up that reads no global memory may overlap the stream's previous grid; the rest waits for it
-  if (threadIdx.x == 0) grid_launch_dependents();
   grid_dependency_wait();
   __syncthreads();
   tc_fence_after();
@@ -210,6 +209,11 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
   }
   __syncthreads();
+  // The merge may be placed now, not at the start: where its CTAs had waited beside this kernel a call took
+  // 10-14 us longer with k > 4 and 3 us with k <= 4 (4096 columns, 63 rows; 32000 tokens, k = 8 81.9 -> 63.4,
+  // k = 4 59.6 -> 56.0; 128256 tokens, k = 8 189.5 -> 170.9, k = 4 170.9 -> 167.4; a plain launch of the merge
+  // 66.0, 58.2, 173.1, 169.8).
+  if (threadIdx.x == 0) grid_launch_dependents();
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc(tmem, kTmemCols);
@@ -258,7 +262,10 @@ __global__ void __launch_bounds__(kMergeThreads)
 #pragma unroll
   for (int j = 0; j < KM; ++j) top[j] = 0ull;
   for (int c = threadIdx.x; c < ctas; c += kMergeThreads) {
-    const uint64_t* lst = partial + ((size_t)c * rows + r) * KM;
+    const uint64_t* src = partial + ((size_t)c * rows + r) * KM;
+    uint64_t lst[KM];   // read together: an insertion may end early, and the next load would wait for it
+#pragma unroll
+    for (int j = 0; j < KM; ++j) lst[j] = src[j];
 #pragma unroll
     for (int j = 0; j < KM; ++j) insert<KM>(top, lst[j]);
   }
