@@ -685,7 +685,8 @@ ptd_status ptd_tree_rope_append(const ptd_tree* tree, const ptd_kv_cache* cache,
                                          cache->k, cache->v, layer_begin, num_layers, cache->page_size,
                                          cache->seq_capacity,
                                          cache->num_pages, cache->block_table, cache->max_pages, f, positions_out,
-                                         dev_status, static_cast<cudaStream_t>(stream)));
+                                         dev_status, num_sms_of_current_device(),
+                                         static_cast<cudaStream_t>(stream)));
   if (st == PTD_OK) g_last_launches = 1;
   return st;
 }

@@ -15,8 +15,10 @@
 // What bounds it: the reads and writes (49.5 MB for 32 layers of 63 nodes, 32 query / 8 KV heads)
 // and, for few layers, the chain tree, parents, slot, angles.  Measured (GB300; at first with
 // that chain before the first read of a row, one thread walking, four layers one after the other):
-// 32 layers 14.2 -> 11.3 us (4.4 TB/s), one layer 6.2 -> 3.7, eight fp32 layers 10.4 -> 5.6.  Three
-// items a thread at four CTAs per SM: two items 14.1, four 11.7, six 13.3 us.
+// 32 layers 14.2 -> 10.4 us (4.8 TB/s), one layer 6.2 -> 3.7, eight fp32 layers 10.4 -> 5.6.  Three
+// items a thread at four CTAs per SM: two items 14.1, four 11.7, six 13.3 us.  An item's layer and head by
+// multiplications: by division, six a thread and round, batches of some hundred nodes were slower than
+// they had been with one item at a time (8 layers of ~345 nodes, 64 / 8 heads 15.9 us, then 21.7, now 17.3).
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -24,6 +26,7 @@
 
 #include "launch.cuh"
 #include "ptd_device.cuh"
+#include "row_division.cuh"
 #include "tree_rope.cuh"
 
 namespace ptd {
@@ -157,15 +160,14 @@ __device__ __forceinline__ void make_table(const RopeFreqs& freqs, int pos_i, in
 // j + D/2; a CTA takes all items of one node in `layers_per_cta` layers, kItems per thread at a
 // time, and asks for the first kItems before it looks the node up, so that the reads (which
 // depend on no position) overlap the chain tree, parents, slot, angles.
-constexpr int kItems = 3;
-
-template <typename T>
-__global__ void __launch_bounds__(kThreads, 4)
+// kItems = 3 at four CTAs per SM; two at five where that saves a wave (see launch_tree_rope).
+template <typename T, int kItems>
+__global__ void __launch_bounds__(kThreads, kItems == 3 ? 4 : 5)
     tree_rope_kernel(const int32_t* node_offsets, const int32_t* parents, const int32_t* ctx_lens, int batch,
                      int n_total, int num_layers, int layers_per_cta, int D, int hq, int hkv, T* q, const T* k, const T* v,
                      T* k_cache, T* v_cache, int layer_begin, int page_size, int seq_capacity, int num_pages,
                      const int32_t* block_table, int max_pages, const __grid_constant__ RopeFreqs freqs,
-                     int32_t* positions_out, int32_t* dev_status) {
+                     int32_t* positions_out, int32_t* dev_status, GroupDivisor by_layer, GroupDivisor by_chunks) {
   __shared__ int par_s[kThreads];
   __shared__ float cos_s[kMaxRopeHalf], sin_s[kMaxRopeHalf];
   const int n = blockIdx.x, t = threadIdx.x;
@@ -178,9 +180,9 @@ __global__ void __launch_bounds__(kThreads, 4)
   const int heads = hq + 2 * hkv, per_layer = heads * chunks, items = layers * per_layer;
   // item e: its layer (relative), head (q heads, then k heads, then v heads) and first column
   auto place_of = [&](int e, int& lq, int& h, int& j) {
-    lq = (int)((unsigned)e / (unsigned)per_layer);
+    lq = layers > 1 ? divide_by_group(e, by_layer) : 0;
     const int r = e - lq * per_layer;
-    h = (int)((unsigned)r / (unsigned)chunks);
+    h = divide_by_group(r, by_chunks);
     j = (r - h * chunks) * V;
   };
   auto src_of = [&](int e) -> const T* {
@@ -293,25 +295,41 @@ cudaError_t launch_tree_rope(const int32_t* node_offsets, const int32_t* parents
                              int batch, int n_total, bool bf16, int head_dim, int hq, int hkv, void* q, const void* k,
                              const void* v, void* k_cache, void* v_cache, int layer_begin, int num_layers,
                              int page_size, int seq_capacity, int num_pages, const int32_t* block_table, int max_pages,
-                             const RopeFreqs& freqs, int32_t* positions_out, int32_t* dev_status,
+                             const RopeFreqs& freqs, int32_t* positions_out, int32_t* dev_status, int sms,
                              cudaStream_t stream) {
   const auto al16 = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; };
   const bool aligned = al16(q) && al16(k) && al16(v) && al16(k_cache) && al16(v_cache);
   const int vec = bf16 ? 8 : 4;
-  if (aligned && (head_dim / 2) % vec == 0) {
-    // as many layers a CTA as fill kItems items of its threads
-    const int per_layer = (hq + 2 * hkv) * (head_dim / 2 / vec);
-    int layers = tr::kItems * tr::kThreads / per_layer;
-    layers = layers < 1 ? 1 : (layers > num_layers ? num_layers : layers);
+  // (2^26 items a layer: the bound of the kernel's quotients)
+  if (aligned && (head_dim / 2) % vec == 0 && ((int64_t)hq + 2 * (int64_t)hkv) * (head_dim / 2 / vec) < (1 << 26)) {
+    // As many layers a CTA as fill three items of its threads; twice that over more than two waves of CTAs
+    // (few heads' remainders, and half the look-ups: 32 layers of 128 nodes, 64 / 8 heads, bf16 31.1 -> 26.9
+    // us, 8 layers of ~345 nodes 19.3 -> 17.3).  A grid just above one wave of four CTAs per SM runs with
+    // five (~650 nodes, one layer, 32 / 8 heads 6.1 -> 4.7 us, 64 / 8 heads 7.2 -> 6.5); with five everywhere
+    // the others lose 5 % (geometric mean over 249 sizes).
+    const int chunks = head_dim / 2 / vec, per_layer = (hq + 2 * hkv) * chunks;
+    auto layers_of = [&](int items) {
+      const int l = items * tr::kThreads / per_layer;
+      return l < 1 ? 1 : (l > num_layers ? num_layers : l);
+    };
+    int layers = layers_of(3);
+    const int64_t ctas = (int64_t)n_total * ((num_layers + layers - 1) / layers), slots = 4 * (int64_t)sms;
+    const bool five = ctas > slots && ctas <= 5 * (int64_t)sms;
+    if (five) layers = layers_of(2);
+    if (ctas > 2 * slots) layers = layers_of(6);
     const dim3 grid(n_total, (num_layers + layers - 1) / layers);
-#define PTD_ROPE_LAUNCH(T)                                                                                          \
-  return launch_chained(tr::tree_rope_kernel<T>, grid, dim3(tr::kThreads), 0, stream, 0, node_offsets, parents,     \
+#define PTD_ROPE_LAUNCH(T, ITEMS)                                                                                   \
+  return launch_chained(tr::tree_rope_kernel<T, ITEMS>, grid, dim3(tr::kThreads), 0, stream, 0, node_offsets, parents,     \
                         ctx_lens, batch, n_total, num_layers, layers, head_dim, hq, hkv, static_cast<T*>(q),        \
                         static_cast<const T*>(k), static_cast<const T*>(v), static_cast<T*>(k_cache),               \
                         static_cast<T*>(v_cache), layer_begin, page_size, seq_capacity, num_pages, block_table,     \
-                        max_pages, freqs, positions_out, dev_status)
-    if (bf16) PTD_ROPE_LAUNCH(__nv_bfloat16);
-    PTD_ROPE_LAUNCH(float);
+                        max_pages, freqs, positions_out, dev_status, group_divisor(per_layer), group_divisor(chunks))
+    if (bf16) {
+      if (five) PTD_ROPE_LAUNCH(__nv_bfloat16, 2);
+      PTD_ROPE_LAUNCH(__nv_bfloat16, 3);
+    }
+    if (five) PTD_ROPE_LAUNCH(float, 2);
+    PTD_ROPE_LAUNCH(float, 3);
 #undef PTD_ROPE_LAUNCH
   }
   const dim3 grid(n_total, num_layers);

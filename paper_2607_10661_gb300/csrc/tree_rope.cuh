@@ -15,5 +15,5 @@ cudaError_t launch_tree_rope(const int32_t* node_offsets, const int32_t* parents
                              const void* v, void* k_cache, void* v_cache, int layer_begin, int num_layers,
                              int page_size, int seq_capacity,
                              int num_pages, const int32_t* block_table, int max_pages, const RopeFreqs& freqs,
-                             int32_t* positions_out, int32_t* dev_status, cudaStream_t stream);
+                             int32_t* positions_out, int32_t* dev_status, int sms, cudaStream_t stream);
 }  // namespace ptd

@@ -120,6 +120,10 @@ def test_layer_range_in_one_launch():
     ("bf16", 8, 2, 48, 5, 31, 1),      # three vectors a half row
     ("bf16", 6, 2, 40, 3, 9, 1),       # rows that are no 16-byte vectors: element by element
     ("bf16", 32, 8, 128, 3, 20, 40),   # more trees than a warp has lanes
+    # 31 nodes and 80 heads a layer, one layer a CTA: 651 CTAs (five per SM on 152), then 1271 (two layers a CTA)
+    ("bf16", 64, 8, 128, 21, 31, 1),
+    ("f32", 64, 8, 128, 21, 31, 1),
+    ("bf16", 64, 8, 128, 41, 31, 1),
 ])
 def test_rope_items_match_oracle(dtype, hq, hkv, d, layers, nodes, batch):
     """The items of a CTA at their edges, every layer of one call, against the oracle."""
