@@ -133,6 +133,8 @@ __device__ __forceinline__ void verify_and_write_warp(const VerifyArgs& va, int 
 // placed among each other the same way:
 //   kCluster, kClusterVerify  in the shared memory of the first CTA of the row's cluster, which
 //       the others write to before they leave;
+//   kWhole  (a row in one part) not at all: they are the row's entries (15 fp32 rows of 1000, k = 2: 3.0 us
+//       with the merge, 2.4 without; 1500 rows 10.7 / 7.0);
 //   kSlotsVerify  (the step's "streamed" form) by the CTA that counts in the row's last part,
 //       from slots in global scratch: parts of all rows run one by one wherever an SM has
 //       room, with no cluster to place, and a CTA leaves as soon as its part is done.
@@ -155,7 +157,7 @@ __device__ __forceinline__ void verify_and_write_warp(const VerifyArgs& va, int 
 constexpr int kTargetVec = 2048;   // 32 KB: the part that the cluster size aims at
 constexpr int kMaxK = 16;
 constexpr int kCand = 256;         // candidate buffer (keys)
-constexpr int kCluster = 0, kClusterVerify = 1, kSlotsVerify = 2;
+constexpr int kCluster = 0, kClusterVerify = 1, kSlotsVerify = 2, kWhole = 3;
 
 __device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }
 __device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w & 0xFFFF0000u); }
@@ -219,7 +221,7 @@ __device__ __forceinline__ uint32_t kth_of_32(const uint32_t* v_s, int k) {
 // us, 512 rows with k = 16 59.2 -> 61.4).
 template <typename T, int kMode>
 struct Depth {
-  static constexpr bool kDeep = kMode == kCluster && sizeof(T) == 4;
+  static constexpr bool kDeep = (kMode == kCluster || kMode == kWhole) && sizeof(T) == 4;
   static constexpr int kLoads = kDeep ? 8 : 4, kCtas = kDeep ? 4 : 6;
 };
 
@@ -229,6 +231,7 @@ __global__ void __launch_bounds__(kThreads, Depth<T, kMode>::kCtas)
                      int32_t* __restrict__ out_idx, float* __restrict__ out_val, int32_t* dev_status,
                      unsigned int* row_counters, unsigned long long* slots, const __grid_constant__ VerifyArgs va) {
   constexpr int VN = Vec<T>::kN, kLoads = Depth<T, kMode>::kLoads;
+  constexpr bool kClustered = kMode == kCluster || kMode == kClusterVerify;
   __shared__ __align__(16) uint64_t cand_s[kCand];
   __shared__ __align__(16) uint64_t all_keys[kMaxCluster * kMaxK];   // the row's parts' keys, at its last merger
   __shared__ __align__(16) uint32_t group_max_s[32];
@@ -244,19 +247,19 @@ __global__ void __launch_bounds__(kThreads, Depth<T, kMode>::kCtas)
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint32_t keys_bar = smem_u32(&keys_bar_s);
   if (tid == 0) {
-    if (kMode != kSlotsVerify) {
+    if (kClustered) {
       mbar_init(keys_bar, (uint32_t)(parts * k));   // one arrival per key (rank 0's is used)
       fence_mbar_init();
     }
     abort_s = 0;
     n_cand_s = 0;
   }
-  if (rank == 0 && tid < kMaxCluster * kMaxK) all_keys[tid] = 0ull;
+  if (kMode != kWhole && rank == 0 && tid < kMaxCluster * kMaxK) all_keys[tid] = 0ull;
   __syncthreads();
   if (tid == 0) grid_launch_dependents();   // the next grid may be placed now; it waits for this one
   // the cluster's CTAs are there and rank 0's keys and barrier are set up (waited for before the
   // first key is sent)
-  if (kMode != kSlotsVerify) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  if (kClustered) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
   if (!beside) grid_dependency_wait();   // the logits, the trees and the outputs belong to the stream's previous work
   // this CTA's part: the vector body starts at the row's first 16-byte boundary (head and tail
   // elements outside it go to the first and last CTA one by one)
@@ -268,7 +271,7 @@ __global__ void __launch_bounds__(kThreads, Depth<T, kMode>::kCtas)
   const int v_begin = min(nvec, rank * per), nv = min(nvec, v_begin + per) - v_begin;
   const uint4* vrow = reinterpret_cast<const uint4*>(row + a0) + v_begin;
   const bool own_head = rank == 0 && tid == 0, own_tail = rank == parts - 1 && tid == kThreads - 1;
-  if constexpr (kMode != kCluster) {
+  if constexpr (kMode == kClusterVerify || kMode == kSlotsVerify) {
     // Trees that no row completes (an empty or out-of-range node range, or offsets that do not
     // run from 0 to n_total): their outputs and the status are written here, by warp 1 of the
     // first CTA; a tree whose rows all arrive is verified below.
@@ -362,19 +365,23 @@ __global__ void __launch_bounds__(kThreads, Depth<T, kMode>::kCtas)
     }
   }
   __syncthreads();
-  if (kMode != kSlotsVerify) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  if (kClustered) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
   // where a key of this part goes: rank 0's shared memory, with an arrival that releases it, or the
   // part's slot
-  uint64_t* dst_keys;
+  uint64_t* dst_keys = nullptr;
   uint32_t dst_bar = 0;
-  if constexpr (kMode != kSlotsVerify) {
+  if constexpr (kClustered) {
     dst_keys = cluster.map_shared_rank(all_keys, 0) + rank * kMaxK;
     asm("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(dst_bar) : "r"(keys_bar));
-  } else {
+  } else if constexpr (kMode == kSlotsVerify) {
     dst_keys = reinterpret_cast<uint64_t*>(slots) + (r * parts + rank) * k;
   }
+  auto write_entry = [&](int at, uint64_t key) {   // entry `at` of the row
+    out_idx[r * k + at] = (int32_t)(~(uint32_t)(key & 0xFFFFFFFFull));
+    out_val[r * k + at] = from_ordered((uint32_t)(key >> 32));
+  };
   auto arrive = [&](int count) {
-    if constexpr (kMode != kSlotsVerify)
+    if constexpr (kClustered)
       asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0], %1;" ::"r"(dst_bar), "r"(count)
                    : "memory");
   };
@@ -386,11 +393,15 @@ __global__ void __launch_bounds__(kThreads, Depth<T, kMode>::kCtas)
       int before = 0;
       for (int j = 0; j < n; ++j) before += cand_s[j] > key ? 1 : 0;
       if (before < k) {
-        dst_keys[before] = key;
-        arrive(1);
+        if constexpr (kMode == kWhole) {
+          write_entry(before, key);
+        } else {
+          dst_keys[before] = key;
+          arrive(1);
+        }
       }
     }
-    if (n < k) {   // fewer elements than k in this part
+    if (kMode != kWhole && n < k) {   // fewer elements than k in this part
       if (kMode == kSlotsVerify) {
         if (tid >= n && tid < k) dst_keys[tid] = 0ull;
       } else if (tid == 0) {
@@ -423,8 +434,12 @@ __global__ void __launch_bounds__(kThreads, Depth<T, kMode>::kCtas)
 #pragma unroll
       for (int w = 1; w < kWarps; ++w) best = best > round_s[w] ? best : round_s[w];
       if (tid == 0) {
-        dst_keys[q] = best;
-        arrive(1);
+        if constexpr (kMode == kWhole) {
+          write_entry(q, best);
+        } else {
+          dst_keys[q] = best;
+          arrive(1);
+        }
       }
       last = best;
       __syncthreads();   // round_s is read
@@ -433,7 +448,7 @@ __global__ void __launch_bounds__(kThreads, Depth<T, kMode>::kCtas)
 
   // ---- the row's top-k from its parts' keys
   constexpr int kMergers = kMaxCluster * kMaxK;   // the first four warps
-  bool merger = rank == 0;
+  bool merger = kMode != kWhole && rank == 0;
   if constexpr (kMode == kSlotsVerify) {
     __syncthreads();   // the part's keys are written before it is counted
     if (tid == 0) last_s = (int)atom_add_acq_rel_gpu(row_counters + r, 1u) + 1 == parts ? 1 : 0;
@@ -455,12 +470,9 @@ __global__ void __launch_bounds__(kThreads, Depth<T, kMode>::kCtas)
       int before = 0;
       for (int c = 0; c < parts; ++c)
         for (int j = 0; j < k; ++j) before += all_keys[c * kMaxK + j] > key ? 1 : 0;
-      if (before < k) {
-        out_idx[r * k + before] = (int32_t)(~(uint32_t)(key & 0xFFFFFFFFull));
-        out_val[r * k + before] = from_ordered((uint32_t)(key >> 32));
-      }
+      if (before < k) write_entry(before, key);
     }
-    if constexpr (kMode != kCluster) {
+    if constexpr (kMode == kClusterVerify || kMode == kSlotsVerify) {
       // the last row of a tree to be written: its tree is verified
       asm volatile("bar.sync 1, %0;" ::"n"(kMergers) : "memory");   // the row's entries precede its count
       if (warp == 0) {
@@ -504,18 +516,34 @@ cudaError_t launch_rows(const T* logits, int64_t rows, int vocab, int64_t row_st
   const int per = (vocab / Vec<T>::kN + parts - 1) / parts;   // vectors per CTA (rows off 16 bytes have one fewer)
   const unsigned gy = (unsigned)(rows < 32768 ? rows : 32768), gz = (unsigned)((rows + gy - 1) / gy);
   return launch_chained(topk_rows_kernel<T, kMode>, dim3((unsigned)parts, gy, gz), dim3(kThreads), 0, stream,
-                        kMode == kSlotsVerify ? 0u : (unsigned)parts, logits, rows, vocab, row_stride, k, per, beside,
+                        kMode == kSlotsVerify || kMode == kWhole ? 0u : (unsigned)parts, logits, rows, vocab, row_stride, k, per, beside,
                         out_idx, out_val, dev_status, row_counters, slots, va);
+}
+
+// Parts of each of many rows: where 32 KB parts are more CTAs than run at once, the next power of two
+// below that fits, while a part stays under 128 KB.  GB300, us, 32 KB parts -> these: 300 bf16 rows of 50257,
+// k = 1 9.0 -> 7.4, 700 rows 17.2 -> 11.3; fp32, 300 rows of 50257 15.0 -> 8.3, 512 rows of 32000 13.7 -> 7.7;
+// over 600 sizes 8 % less on average, none more than 2 % slower.
+template <typename T>
+int row_parts_of_many(int vocab, int64_t rows, int sms) {
+  const int most = row_parts<T>(vocab);
+  const int64_t slots = (int64_t)Depth<T, kCluster>::kCtas * sms, bytes = (int64_t)vocab * (int64_t)sizeof(T);
+  if (rows * most <= slots) return most;
+  int parts = kMaxCluster;
+  while (parts > 1 && (parts >= most || rows * parts > slots) && bytes / (parts / 2) <= 128000) parts /= 2;
+  return parts < most ? parts : most;
 }
 
 template <typename T>
 cudaError_t launch_plain(const T* logits, int64_t rows, int vocab, int64_t row_stride, int k, int beside,
-                         int32_t* out_idx, float* out_val, int32_t* dev_status, cudaStream_t stream) {
+                         int32_t* out_idx, float* out_val, int32_t* dev_status, int sms, cudaStream_t stream) {
   constexpr int64_t kMost = 32768ll * 32768;   // rows of one grid
+  const int parts = beside ? row_parts<T>(vocab) : row_parts_of_many<T>(vocab, rows, sms);
   for (int64_t r = 0; r < rows; r += kMost) {
-    const cudaError_t e = launch_rows<T, kCluster>(logits + r * row_stride, rows - r < kMost ? rows - r : kMost, vocab,
-                                                   row_stride, k, row_parts<T>(vocab), beside, out_idx + r * k,
-                                                   out_val + r * k, dev_status, nullptr, nullptr, VerifyArgs{}, stream);
+    auto* const launch = parts == 1 ? launch_rows<T, kWhole> : launch_rows<T, kCluster>;
+    const cudaError_t e = launch(logits + r * row_stride, rows - r < kMost ? rows - r : kMost, vocab, row_stride, k, parts,
+                                 beside, out_idx + r * k, out_val + r * k, dev_status, nullptr, nullptr, VerifyArgs{},
+                                 stream);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -561,9 +589,9 @@ cudaError_t launch_topk(const void* logits, bool bf16, int64_t rows, int vocab, 
   }
   if (bf16)
     return topk::launch_plain(static_cast<const __nv_bfloat16*>(logits), rows, vocab, row_stride, k, beside ? 1 : 0,
-                              out_idx, out_val, dev_status, stream);
+                              out_idx, out_val, dev_status, sms, stream);
   return topk::launch_plain(static_cast<const float*>(logits), rows, vocab, row_stride, k, beside ? 1 : 0, out_idx,
-                            out_val, dev_status, stream);
+                            out_val, dev_status, sms, stream);
 }
 
 }  // namespace ptd

@@ -481,6 +481,23 @@ def test_topk_rows_of_nan_write_every_entry(vocab, k, dtype):
     assert np.array_equal(val.cpu().numpy(), want, equal_nan=True)
 
 
+@pytest.mark.parametrize("dtype,rows,vocab,k", [
+    ("bf16", 228, 50257, 4), ("bf16", 229, 50257, 4),     # the most rows of four parts, then two parts (152 SMs)
+    ("bf16", 457, 50257, 16), ("f32", 100, 50257, 8),     # one part; fp32: four of seven
+    ("f32", 305, 32000, 1), ("f32", 609, 128256, 4),      # one part; parts of at most 128 KB
+    ("f32", 1500, 1001, 2), ("bf16", 1, 16376, 16),       # whole rows off 16 bytes; the longest bf16 row in one part
+])
+def test_topk_parts_of_many_rows(dtype, rows, vocab, k):
+    """Rows in fewer and larger parts when there are many, and rows of one part."""
+    g = torch.Generator(device="cuda").manual_seed(83)
+    x = torch.randn((rows, vocab), generator=g, device="cuda").to(torch.bfloat16 if dtype == "bf16" else torch.float32)
+    idx = torch.full((rows, k), -7, dtype=torch.int32, device="cuda")
+    val = torch.full((rows, k), -7.0, device="cuda")
+    ptd.topk_draft(x, k, idx, val)
+    v, i = torch.sort(x, dim=1, descending=True, stable=True)   # ties by lower index
+    assert torch.equal(idx.long(), i[:, :k]) and torch.equal(val, v[:, :k].float())
+
+
 @pytest.mark.parametrize("base,over", [
     ("llama3-8b-gqa", dict(layers=12, ctx=(6000, 6000), vocab=4096)),    # cut and merge kernel
     ("llama3-8b-gqa", dict(layers=1, ctx=(3000, 3000), vocab=4096)),     # clusters
