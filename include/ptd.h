@@ -347,7 +347,7 @@ ptd_status ptd_pool_retrieve(const void* pool, int32_t capacity, const int32_t* 
  * relative).  positions_out [N_tot] (device, may be NULL)
  * receives p.  A tree that is not one, or a slot outside the cache (or a page outside the
  * pool), sets PTD_ERR_INVALID_TREE in dev_status; that node writes nothing.  q must not
- * alias k or v.  One launch, one CTA per (node, layer).  This is what puts the tree's K/V
+ * alias k or v.  One launch, one CTA per node and group of layers.  This is what puts the tree's K/V
  * where ptd_tree_attention expects them. */
 ptd_status ptd_tree_rope_append(const ptd_tree* tree, const ptd_kv_cache* cache, int32_t layer_begin,
                                 int32_t num_layers, void* q, int32_t num_q_heads, const void* k, const void* v,

@@ -21,7 +21,7 @@
 // per 32 FMAs, an 8 x 8 tile of O 16 per 64; the pipe gives ~110 FMA per cycle and SM) for many
 // rows, the latency of a tile's chain and the K/V stream for few.  Measured (GB300, one layer,
 // against one CTA per (node, head) over all keys, which read every K/V row T * G times): 32 query
-// / 8 KV heads, D 128, 2048 + 63 keys, 63 nodes 628 -> 69.5 us (31 TFLOP/s; the tensor-core kernel 29.1); the same with one
+// / 8 KV heads, D 128, 2048 + 63 keys, 63 nodes 628 -> 69.5 us (31 TFLOP/s; the tensor-core kernel 29.4); the same with one
 // node 86 -> 26 us; 8 heads, D 64, 256 + 15 keys, 15 nodes 14.5 -> 6.6 us.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>

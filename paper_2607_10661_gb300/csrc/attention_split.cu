@@ -28,8 +28,9 @@
 // are read, converted and the code is fetched) and combination.  The tile is 64 keys because the three
 // parts of 128 rows of Q (96 KB) and of K and V (48 KB each) fill shared memory.  Measured (GB300,
 // one layer, against the CUDA-core kernel): 32 query / 8 KV heads, 2048 + 63 keys, 63 nodes 69.2 ->
-// 29.1 us (75 TFLOP/s); 4000 keys 115.5 -> 46.4; 128 nodes, 4000 keys 229 -> 64.7.  (Set-up written out
-// per piece, with divisions by the group, and the combination one row after the other: 30.8.)
+// 29.4 us (74 TFLOP/s); 4000 keys 115.5 -> 46.4; 128 nodes, 4000 keys 229 -> 64.7.  (Set-up written out
+// per piece, with divisions by the group, and the combination one row after the other: 30.8; without the
+// checks for tiny results and huge operands 29.1.)
 //
 // Precision: relative error against 64 bits over 14 shapes drawn for it, at scores of deviation 1/4,
 // 1 and 4: 1.0e-7 .. 1.3e-7, 1.5e-7 .. 1.9e-7, 2.5e-7 .. 4.2e-7; the CUDA-core kernel's, whose chains of

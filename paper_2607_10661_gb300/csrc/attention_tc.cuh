@@ -63,9 +63,9 @@ static __device__ __noinline__ void rescale_tmem(uint32_t tO, uint32_t tS, int n
 // GEMM issue.  The whole warp calls, in a branch on a broadcast warp number (so that the compiler
 // knows it uniform), and the lane with `leader` != 0 issues, by predication: descriptors and TMEM
 // addresses then lie in uniform registers, where the instruction takes them.  Against one thread
-// issuing in a branch of its own: 32768 keys under 128 nodes of 64 heads 117.1 -> 113.8 us, 32 layers of
-// 8192 keys under 63 nodes with the step's tail 233 -> 227, a 32-head MHA layer 13.3 -> 12.5, 611 keys
-// 8.6 -> 8.25.  Descriptors come as their low words; the high word is the same for all.
+// issuing in a branch of its own (back to back): 32768 keys under 128 nodes of 64 heads 117.4 -> 112.4 us, 32
+// layers of 8192 keys under 63 nodes with the step's tail 234.7 -> 225.8, a 32-head MHA layer 13.4 -> 12.6, 611
+// keys 8.5 -> 8.25.  Descriptors come as their low words; the high word is the same for all.
 constexpr uint32_t kDescHi = (1u << 14) | (1024u >> 4) | (2u << 29);   // stride 1024, version 1, 128-byte swizzle
 // S_t (TMEM, 128 columns at s_tmem) = Q K^T: descriptor words of the Q tile and the K tile.
 __device__ __forceinline__ void issue_s(uint32_t leader, uint32_t s_tmem, uint32_t q_desc, uint32_t k_desc) {

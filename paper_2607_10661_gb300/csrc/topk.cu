@@ -215,6 +215,12 @@ __device__ __forceinline__ uint32_t kth_of_32(const uint32_t* v_s, int k) {
 // be placed, so the CTAs start on them at once, beside that grid; the outputs and counters
 // belong to no grid still running.  One CTA waits for the previous grid before it leaves, so
 // that this grid's completion implies that one's.
+// The counters that this kernel adds to (rows done per tree, parts done per row) were cleared by CTA 0 of that
+// grid, and being placed makes nothing visible by itself.  What orders the two: CTA 0 stores the zeros, then
+// fences device-wide, then (after a barrier) gives its permission, and this grid has no CTA before every CTA
+// there has given it or left; the stores are then performed in L2, where the counts, atomics all of them, are
+// made.  A plain load of a counter would have to wait for that grid.
+//
 // Vectors in flight per thread and CTAs per SM (registers).  Kernels that run beside the tensor-core
 // attention keep to four and 40 registers, and bf16 rows do best so (eight: 512 rows of 128256
 // 34.3 -> 43.8 us); a part of fp32 logits is twice as many vectors (four -> eight: 63 rows 11.2 -> 7.8
