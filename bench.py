@@ -52,8 +52,8 @@ METRIC = "tree-verify steps/sec (HBM GB/s and fraction of ~8 TB/s alongside)"
 # dram__bytes_read.sum + dram__bytes_write.sum per attention launch from one ncu capture,
 # keyed by (workload, the kernel source's sha256 prefix): a changed kernel reports null
 # until it is captured again
-PROFILED_ATTENTION_TRAFFIC = {(("llama3-8b-gqa", 32), "766310cc72ef5798"): 1112748032}
-PROFILED_LM_HEAD_TRAFFIC = {"c177b463ccbf468a": 1056910592}
+PROFILED_ATTENTION_TRAFFIC = {(("llama3-8b-gqa", 32), "87509defc54fcb45"): 1112503808}
+PROFILED_LM_HEAD_TRAFFIC = {"2e9ecc48401405b8": 1056829952}
 MEASURED_PEAKS = os.path.join(ROOT, "MEASURED_PEAKS.json")
 # the tail of the one-call step (ptd_step_tail)
 STEP_TAILS = {0: "top-k, then verification + compaction in one launch",
