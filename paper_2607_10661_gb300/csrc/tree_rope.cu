@@ -312,9 +312,10 @@ cudaError_t launch_tree_rope(const int32_t* node_offsets, const int32_t* parents
       const int l = items * tr::kThreads / per_layer;
       return l < 1 ? 1 : (l > num_layers ? num_layers : l);
     };
+    auto ctas_of = [&](int l) { return (int64_t)n_total * ((num_layers + l - 1) / l); };
     int layers = layers_of(3);
-    const int64_t ctas = (int64_t)n_total * ((num_layers + layers - 1) / layers), slots = 4 * (int64_t)sms;
-    const bool five = ctas > slots && ctas <= 5 * (int64_t)sms;
+    const int64_t ctas = ctas_of(layers), slots = 4 * (int64_t)sms;
+    const bool five = ctas > slots && ctas_of(layers_of(2)) <= 5 * (int64_t)sms;
     if (five) layers = layers_of(2);
     if (ctas > 2 * slots) layers = layers_of(6);
     const dim3 grid(n_total, (num_layers + layers - 1) / layers);

@@ -65,7 +65,7 @@ def test_single_process_reduction_is_identity():
 
 
 def test_reference_arm_under_torchrun_prints_once():
-    """`bench.py --impl reference` launched as the driver launches it for N = 2: rank 0 runs the
+    """`bench.py --impl reference` launched by torchrun for N = 2: rank 0 runs the
     oracle and prints one JSON line, the other rank exits 0 without work."""
     port = _free_port()
     cmd = [sys.executable, "-m", "torch.distributed.run", "--nnodes=1", "--nproc-per-node", "2", "--master-addr",
@@ -81,7 +81,7 @@ def test_reference_arm_under_torchrun_prints_once():
     cb = d["cpu_baseline"]
     assert cb["kind"] == "oracle" and cb["cores"] >= 1 and cb["value"] == d["value"]
     assert d["e2e"] == {"value": d["value"], "unit": "steps/s", "h2d_bytes_per_step": 0, "d2h_bytes_per_step": 0}
-    # the steps and warm-up the driver asked for, whole steps, and the GPU arm's config
+    # the steps and warm-up asked for, whole steps, and the GPU arm's config
     assert d["steps"] == 4 and d["warmup"] == 3 and cb["steps"] == 4 and cb["unit_sample_fraction"] == 1.0
     assert d["ms_per_step"] == pytest.approx(1e3 / d["value"])
     sys.path.insert(0, ROOT)
