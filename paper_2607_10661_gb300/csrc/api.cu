@@ -171,7 +171,9 @@ struct Schedule {
 // The one with the shortest estimate from the host-known maxima (every sequence taken as long as
 // the longest), in microseconds as measured on GB300 for one (two) 128-row M tiles a unit:
 //   cut      17.5 (25.5) + 1.7 (1.75) a key tile of a CTA's share (set-up, partials and merge in the
-//            constant: it hardly depends on the number of pieces)
+//            constant: it hardly depends on the number of pieces); for at least as many units as SMs of at most
+//            12 key tiles 18.4 (27.6) + 1.67 (1.95) a key tile + 1.1 (1.55) a unit of a CTA's share (its Q, its
+//            output, the merges at both ends)
 //   grid     5.5 (8) + 1.6 (1.85) a key tile, per wave of units over the SMs
 //   cluster  9.5 (10.5) + 0.1 a CTA of the cluster + 0.8 (2.05) a key tile of a CTA's share, per wave of
 //            clusters (clusters_at_once).  One wave for a batch (a second one costs a whole unit when the
@@ -181,9 +183,11 @@ struct Schedule {
 // and 63 nodes 28.5 / 15.8; eight ragged paged sequences 84.6 / 82.4 a step.  Grid / cut, 128 units of
 // two M tiles: 17 key tiles 39.1 / 52.4, 9 key tiles 25.4 / 37.5.  Stacks of several layers of 8 KV
 // heads, 63 nodes, cut / grid / best cluster: 12 layers 300 keys 29.0 / 14.2 / 18.2, 2000 keys 46.5 / 36.0 / 41.2;
-// 4 layers 300 keys 17.8 / 13.4 / 11.9, 2000 keys 28.4 / 35.0 / 19.6.  Over 810 shapes (1 to 32 layers, 60 to 8000
-// keys, one to four M tiles, batches of up to 8) the choice is 1.1 % slower than the best kernel on average,
-// 19 % at most.
+// 4 layers 300 keys 17.8 / 13.4 / 11.9, 2000 keys 28.4 / 35.0 / 19.6; 432 units of 3 key tiles 46.5 / 39.4 / -, 720 of
+// 3 66.2 / 64.0 / -.  Over 810 shapes (1 to 32 layers, 60 to 8000 keys, one to four M tiles, batches of up to 8) the
+// choice is 1.0 % slower than the best kernel on average, 19 % at most; over 865 batches of up to 16 equally
+// long sequences 2.4 %, 35 % at most; of ragged ones (a quarter to all of the longest) 6.3 %; over 1672 calls of
+// 152 to 4500 short units 0.9 % (equally long) and 1.8 %.
 Schedule choose_schedule(int units, int n_kt, int m_tiles, int sms, int batch, bool can_cut, bool can_cluster) {
   const bool two = m_tiles >= 2;
   auto waves = [&](int fit) { return (double)((units + fit - 1) / fit); };   // of units over `fit` places
@@ -191,7 +195,10 @@ Schedule choose_schedule(int units, int n_kt, int m_tiles, int sms, int batch, b
   double t_best = waves(sms) * ((two ? 8.0 : 5.5) + n_kt * (two ? 1.85 : 1.6));
   if (can_cut) {
     const double W = (double)units * n_kt, w = W / (W < sms ? W : sms);
-    const double t = (two ? 25.5 : 17.5) + w * (two ? 1.75 : 1.7);
+    const double share = (double)units / sms;   // units of a CTA's share
+    const double t = units < sms || n_kt > 12
+                         ? (two ? 25.5 + 1.75 * w : 17.5 + 1.7 * w)
+                         : (two ? 27.6 + 1.95 * w + 1.55 * share : 18.4 + 1.67 * w + 1.1 * share);
     if (t < t_best) {
       t_best = t;
       best = {Schedule::kCut, 1};

@@ -131,6 +131,12 @@ def test_attention_plan_and_named_kernels_check_their_arguments(lib):
         s = ptd._Tree(1, 63, 63, keys, 16, 16, 16)
         assert plan(s, bf, 32, layers, lib.ptd_attention_workspace_size(ctypes.byref(s), ctypes.byref(bf), 32,
                                                                         layers))[0] in kinds, (layers, keys)
+    # many short units: a share of a few of them costs more than whole units in waves
+    for batch, nodes, keys, layers, kind in ((6, 48, 300, 9, ptd.ATTN_UNIT), (12, 48, 1000, 4, ptd.ATTN_UNIT),
+                                             (10, 8, 300, 4, ptd.ATTN_UNIT), (1, 63, 1000, 20, ptd.ATTN_CUT)):
+        s = ptd._Tree(batch, batch * nodes, nodes, keys, 16, 16, 16)
+        assert plan(s, bf, 32, layers, lib.ptd_attention_workspace_size(ctypes.byref(s), ctypes.byref(bf), 32,
+                                                                        layers))[0] == kind, (batch, nodes, keys)
     assert plan(t, bf, 30, 1, 0) == -ptd.INVALID_ARG and plan(t, bf, 32, 33, 0) == -ptd.INVALID_ARG
     named = lambda cache, kernel, csize: lib.ptd_tree_attention_as(
         ctypes.byref(t), ctypes.byref(cache), 0, 1, 16, 32, 0.0, 16, None, 0, 16, kernel, csize, None)

@@ -615,6 +615,7 @@ def test_attention_graph_replay_with_new_inputs():
     (more units than SMs) must not take the counts that the previous replay left for its own."""
     w = syn.Workload(syn.shrink(syn.CONFIGS["llama3-8b-gqa"], layers=20, ctx=(1000, 1000), vocab=100), 29)
     dw = DeviceWorkload(w, with_step_buffers=False)
+    _check_auto(dw, ptd.ATTN_CUT)
     dw.attention()
     torch.cuda.synchronize()
     graph = torch.cuda.CUDAGraph()
